@@ -210,3 +210,66 @@ def tolerance(case):
         # a token's eighth and ninth expert may be closer than the router sums' rounding
         return {"rel": 1e-2, "differ": 2e-3 if case["M"] >= 64 else 0.1}
     return {"rel": 1e-2}
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _weights64(qbits, w):
+    q, s = w
+    if qbits == 4:                # even k in the low nibble, zero point 8
+        q = torch.stack((q & 15, q >> 4), -1).flatten(-2).to(torch.int16) - 8
+    return (q.double().unflatten(-1, (-1, 32)) * s.double()[..., None]).flatten(-2)
+
+
+def _silu_mul64(gu):
+    g, u = gu.chunk(2, -1)
+    return g * torch.sigmoid(g) * u
+
+
+def _attend64(m, qkv, causal):
+    Hq, Hkv, d = m["Hq"], m["Hkv"], m["d"]
+    q, k, v = (t.unflatten(-1, (-1, d)) for t in qkv.double().split([Hq * d, Hkv * d, Hkv * d], -1))
+    out = torch.empty_like(q)
+    mask = torch.ones((len(q), len(q)), dtype=torch.bool, device=q.device).triu(1) if causal else None
+    for h in range(Hq):
+        p = q[:, h] @ k[:, h * Hkv // Hq].T / math.sqrt(d)
+        if causal:
+            p.masked_fill_(mask, -math.inf)
+        out[:, h] = torch.softmax(p, -1) @ v[:, h * Hkv // Hq]
+    return out.flatten(1)
+
+
+def _block_scaled64(x):
+    """Values of a block-scaled FP8 encoding: per 32 values a power of two, floor(log2 of the largest) - 8, and E4M3 codes."""
+    b = x.double().unflatten(-1, (-1, 32))
+    top = b.abs().amax(-1, keepdim=True)
+    scale = torch.ldexp(torch.ones_like(top), torch.frexp(top).exponent - 1 - 8)
+    code = torch.where(top > 0, b / scale, b).clamp(-448, 448).float().to(torch.float8_e4m3fn)
+    return (code.double() * scale).flatten(-2)
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    st = prepare(dict(case, kind="decode") if kind == "fp8" else case, seed)
+    if kind != "moe":
+        m = DENSE[case["model"]]
+    if kind == "attention":
+        return _attend64(m, st["qkv"], st["causal"])
+    if kind in ("decode", "fp8"):
+        enc = _block_scaled64 if kind == "fp8" else torch.Tensor.double
+        return tuple(enc(st[x]) @ enc(_weights64(m["qbits"], st[w])).T
+                     for x, w in (("x", "qkv"), ("attn", "o"), ("x2", "gate_up"), ("act", "down")))
+    if kind == "prefill":
+        W = {name: _weights64(m["qbits"], st[name]) for name, _, _ in _projections(m)}
+        qkv = st["x"].double() @ W["qkv"].T
+        h = _silu_mul64(st["x2"].double() @ W["gate_up"].T)
+        return qkv, _attend64(m, qkv, True) @ W["o"].T, h @ W["down"].T
+    x = st["x"].double()
+    top, idx = (x @ st["router"].double().T).topk(MOE["k"], -1)
+    w, y = torch.softmax(top, -1), torch.zeros_like(x)
+    for e in range(MOE["E"]):
+        t, slot = torch.nonzero(idx == e, as_tuple=True)
+        w1, w2 = (_weights64(4, (st[n][0][e], st[n][1][e])) for n in ("w1", "w2"))
+        y.index_add_(0, t, w[t, slot, None] * (_silu_mul64(x[t] @ w1.T) @ w2.T))
+    if case["shared"]:
+        y += _silu_mul64(x @ _weights64(4, st["shared1"]).T) @ _weights64(4, st["shared2"]).T
+    return dict(y=y, topk_idx=None, topk_w=w)
