@@ -65,8 +65,8 @@ int qg_create(qg_ctx** out, int device) {
         cudaMalloc(&ctx->sk_flags, sizeof(int) * 2 * ctx->sm_count) != cudaSuccess ||
         cudaMemset(ctx->sk_flags, 0, sizeof(int) * 2 * ctx->sm_count) != cudaSuccess ||
         cudaMalloc(&ctx->gemv_partial, ctx->gemv_partial_bytes) != cudaSuccess ||
-        cudaMalloc(&ctx->gemv_tickets, sizeof(int) * ctx->gemv_ticket_count) != cudaSuccess ||
-        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * ctx->gemv_ticket_count) != cudaSuccess) {
+        cudaMalloc(&ctx->gemv_tickets, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS)) != cudaSuccess ||
+        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_status); cudaFree(ctx->gemv_partial); cudaFree(ctx->gemv_tickets);
         cudaFree(ctx->sk_partial); cudaFree(ctx->sk_flags);
@@ -99,7 +99,7 @@ int qg_poll_status(qg_ctx* ctx, void* stream) {
         // next launch starts clean
         cudaMemset(ctx->d_status, 0, sizeof(int));
         cudaMemset(ctx->sk_flags, 0, sizeof(int) * 2 * ctx->sm_count);
-        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * ctx->gemv_ticket_count);
+        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS));
     }
     return host;
 }
@@ -197,9 +197,10 @@ int get_tmap_2d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 
 int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_bytes, const void* base,
                 uint64_t inner, uint64_t rows, uint64_t planes, uint64_t plane_stride_bytes, uint32_t box_inner,
-                uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz) {
+                uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz, uint64_t row_stride_bytes) {
     TmapEntry key{};
-    key.base = base; key.inner = inner; key.rows = rows; key.row_stride = inner * static_cast<uint64_t>(elem_bytes);
+    key.base = base; key.inner = inner; key.rows = rows;
+    key.row_stride = row_stride_bytes ? row_stride_bytes : inner * static_cast<uint64_t>(elem_bytes);
     key.box_inner = box_inner; key.box_rows = box_rows;
     key.planes = planes; key.plane_stride = plane_stride_bytes; key.box_planes = box_planes;
     key.dt = static_cast<int>(dt); key.elem_bytes = elem_bytes; key.swz = static_cast<int>(swz);

@@ -21,6 +21,7 @@ struct TmapEntry {
 };
 constexpr int TMAP_CACHE = 2048, TMAP_WAYS = 8;   // entries, entries per hashed set
 constexpr uint32_t DEFAULT_WAIT_LIMIT = 1u << 18;   // polls; an unsatisfied try_wait poll lasts about 4 us: about a second
+constexpr int SCHED_INTS = 2;                     // tile counters after the gemv tickets
 // Slots of qg_ctx::attr_set, one per kernel instantiation that needs the dynamic shared-memory attribute.
 enum AttrSlot {
     ATTR_GEMM = 0,          // 18 slots: format (2) x token tile (3) x epilogue (3)
@@ -33,7 +34,8 @@ enum AttrSlot {
     ATTR_MX_MOE = 32,       // 2: down, gate/up
     ATTR_MX_256 = 34,
     ATTR_GEMV_RING = 35,    // 4: format (2) x more than eight tokens (2)
-    ATTR_SLOTS = 39
+    ATTR_MOE_STREAM = 39,   // 4: down, gate/up x rows per tile (2)
+    ATTR_SLOTS = 43
 };
 }  // namespace qg
 
@@ -56,7 +58,8 @@ struct qg_ctx {
     int streamk_mode;          // QG_STREAMK at creation: -1 heuristic (default), 0 never, 1 whenever legal
     float* gemv_partial;       // K-slice partial sums of qgemm_small_m, [slices][16][N] fp32
     size_t gemv_partial_bytes;
-    int* gemv_tickets;         // one arrival counter per 64-row tile, zero between launches
+    int* gemv_tickets;         // one arrival counter per 64-row tile, then the tile counters of the grouped streaming kernel;
+                               // zero between launches
     int gemv_ticket_count;
     int gemv_mode;             // test hook (qg_test_gemv_mode): bit 0 no clusters, bit 1 always the ring kernel, bit 2 never
     int gemv_max_clusters[4][9];   // ring kernel, per instantiation and cluster size: clusters that fit at once (0 unknown, -1 none)
@@ -92,5 +95,9 @@ int get_tmap_2d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 // box_planes, which lands in shared memory plane after plane.
 int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_bytes, const void* base,
                 uint64_t inner, uint64_t rows, uint64_t planes, uint64_t plane_stride_bytes, uint32_t box_inner,
-                uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz);
+                uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz, uint64_t row_stride_bytes = 0);
+// The streaming kernel of the grouped GEMM (4-bit weights, modes 0 to 2), for a few rows per expert; QG_ERR_WORKSPACE if the
+// shape does not suit it.
+int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, const int32_t* offsets,
+                      const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st);
 }  // namespace qg

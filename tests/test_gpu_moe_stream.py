@@ -1,0 +1,82 @@
+"""The grouped GEMM's streaming kernel (4-bit weights, a few rows per expert): the edges of its tiles, stages and row groups,
+against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2607_19438_b200 import binding as qg, synth
+from tests import util
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(counts, N, K, seed):
+    E = len(counts)
+    offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    R = int(offsets[-1])
+    A = synth.activations(R, K, seed, 61)
+    Wq = synth.weights_q4(E * N, K, seed, 62).reshape(E, N, K // 2)
+    Ws = synth.scales(E * N, K // 32, 7, seed, 63).reshape(E, N, K // 32)
+    return offsets, A, Wq, Ws
+
+
+# one row; the row groups of eight and the tile of sixteen from both sides; a segment cut into three tiles; empty experts first,
+# in between and last; an odd number of stages, a single one, and more stages than the ring holds; ragged rows of weights
+SEGMENTS = [([1], 128, 256), ([0, 7, 8, 9, 0], 384, 512), ([15, 16, 17, 0, 1, 40], 256, 768),
+            ([0, 0, 3, 0, 33, 1, 0, 2], 640, 2048), ([1] * 9, 1408, 1280), ([2, 0, 5], 136, 256), ([4, 12, 6], 8, 1024)]
+
+
+@pytest.mark.parametrize("mode", [qg.MODE_PLAIN, qg.MODE_GATE_UP_SILU, qg.MODE_DOWN_WEIGHTED], ids=["plain", "gateup", "weighted"])
+@pytest.mark.parametrize("counts,N,K", SEGMENTS, ids=["-".join(map(str, c)) + f"_{n}_{k}" for c, n, k in SEGMENTS])
+def test_short_segments(counts, N, K, mode):
+    if mode == qg.MODE_GATE_UP_SILU and N % 128:
+        N = (N + 127) // 128 * 128
+    offsets, A, Wq, Ws = problem(counts, N, K, 4)
+    R = int(offsets[-1])
+    rng = np.random.default_rng(6)
+    row_pair, w = rng.permutation(R).astype(np.int32), rng.uniform(0.1, 1.0, R).astype(np.float32)
+    g = util.Guarded((R, N // 2 if mode == qg.MODE_GATE_UP_SILU else N), torch.bfloat16)
+    out = qg.moe_grouped_qgemm(mode, 4, util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws), topk_w=util.dev(w),
+                               row_pair=util.dev(row_pair), out=g.t)
+    qg.poll_status()
+    ref = orc.grouped_gemm(4, orc.bf16_to_f64(A), offsets, Wq, Ws)
+    if mode == qg.MODE_GATE_UP_SILU:
+        ref = orc.silu_mul(ref)
+    elif mode == qg.MODE_DOWN_WEIGHTED:
+        ref = ref * w[row_pair].astype(np.float64)[:, None]
+    util.assert_close(util.host_bf16_f64(out), ref, "short segments")
+    assert g.intact()
+
+
+def test_infinities_and_nan_stay_in_their_rows():
+    """A row with an infinity gives what the plain sum gives (an infinity of the weight's sign where the weight is not
+    zero), and no other row notices."""
+    counts, N, K = [3, 2, 9], 256, 512
+    offsets, A, Wq, Ws = problem(counts, N, K, 5)
+    clean = qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
+    dA = util.dev_bf16(A)
+    dA[4, 77], dA[11, 3] = float("inf"), float("nan")
+    out = qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, dA, util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
+    qg.poll_status()
+    rest = [r for r in range(14) if r not in (4, 11)]
+    assert torch.equal(out[rest], clean[rest])
+    assert bool(torch.isnan(out[11]).all())
+    q = ((Wq[1, :, 77 // 2] >> 4).astype(np.int64) - 8) * np.sign(Ws[1, :, 77 // 32].view(np.float16).astype(np.float64))
+    got, nz = out[4].float().cpu().numpy(), q != 0
+    assert np.array_equal(got[nz], np.sign(q[nz]) * np.inf)
+
+
+def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct():
+    counts, N, K = [5, 9, 2, 12], 512, 1024
+    offsets, A, Wq, Ws = problem(counts, N, K, 7)
+    args = (util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
+    try:
+        qg.test_inject(wait_limit_polls=2048, skip_kblock=6)         # the second stage's rows are never loaded
+        qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args)
+        assert qg.poll_status_code() == -7
+    finally:
+        qg.test_inject(0, -1)
+    out = qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args)
+    qg.poll_status()
+    util.assert_close(util.host_bf16_f64(out), orc.grouped_gemm(4, orc.bf16_to_f64(A), offsets, Wq, Ws), "after a timeout")
