@@ -101,12 +101,19 @@ def context(device: int | None = None):
     return _ctx[device]
 
 
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+# The current stream's handle alone.  torch.cuda.current_stream() builds a Stream object around it, 3.2 us against 0.1: a
+# quarter of the host's share of a call (12.5 us, of which the library and its launch are 3.8).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+
+
+def _here():
+    """(library, context, stream handle) of the current device: what every call starts with."""
+    device = torch.cuda.current_device()
+    return _lib or load(), _ctx.get(device) or context(device), _raw_stream(device)
 
 
 def _ptr(t):
-    return C.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _check(rc, what):
@@ -116,12 +123,14 @@ def _check(rc, what):
 
 def poll_status():
     """Synchronises the current stream and raises if a kernel recorded a device-side error."""
-    _check(load().qg_poll_status(context(), _stream()), "qg_poll_status")
+    lib, ctx, stream = _here()
+    _check(lib.qg_poll_status(ctx, stream), "qg_poll_status")
 
 
 def poll_status_code() -> int:
     """Synchronises the current stream; returns (and clears) the device status word instead of raising."""
-    return int(load().qg_poll_status(context(), _stream()))
+    lib, ctx, stream = _here()
+    return int(lib.qg_poll_status(ctx, stream))
 
 
 def test_inject(wait_limit_polls: int = 0, skip_kblock: int = -1):
@@ -157,7 +166,8 @@ def qgemm_dense(qbits, A, Wq, Wscale, out=None):
     N = Wq.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=torch.bfloat16, device=A.device)
-    _check(load().qgemm_dense(context(), qbits, M, N, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.qgemm_dense(ctx, qbits, M, N, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out), stream),
            "qgemm_dense")
     return out
 
@@ -168,7 +178,8 @@ def qgemm_small_m(qbits, A, Wq, Wscale, out=None):
     N = Wq.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=torch.bfloat16, device=A.device)
-    _check(load().qgemm_small_m(context(), qbits, M, N, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.qgemm_small_m(ctx, qbits, M, N, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out), stream),
            "qgemm_small_m")
     return out
 
@@ -179,8 +190,9 @@ def qgemm_dense_gate_up_silu(qbits, A, Wq, Wscale, out=None):
     F = Wq.shape[0] // 2
     if out is None:
         out = torch.empty((M, F), dtype=torch.bfloat16, device=A.device)
-    _check(load().qgemm_dense_gate_up_silu(context(), qbits, M, F, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out),
-                                           _stream()), "qgemm_dense_gate_up_silu")
+    lib, ctx, stream = _here()
+    _check(lib.qgemm_dense_gate_up_silu(ctx, qbits, M, F, K, _ptr(A), _ptr(Wq), _ptr(Wscale), _ptr(out),
+                                        stream), "qgemm_dense_gate_up_silu")
     return out
 
 
@@ -192,8 +204,9 @@ def prefill_attention(Q, K, V, Hq, Hkv, d, causal=True, scale=0.0, out=None):
         assert t.dim() == 2 and t.stride(1) == 1 and t.dtype == torch.bfloat16
     if out is None:
         out = torch.empty((S, Hq * d), dtype=torch.bfloat16, device=Q.device)
-    _check(load().prefill_attention(context(), S, Hq, Hkv, d, _ptr(Q), Q.stride(0), _ptr(K), K.stride(0), _ptr(V),
-                                    V.stride(0), _ptr(out), out.stride(0), 1 if causal else 0, float(scale), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.prefill_attention(ctx, S, Hq, Hkv, d, _ptr(Q), Q.stride(0), _ptr(K), K.stride(0), _ptr(V),
+                                 V.stride(0), _ptr(out), out.stride(0), 1 if causal else 0, float(scale), stream),
            "prefill_attention")
     return out
 
@@ -203,7 +216,8 @@ def mx_quantize(X):
     rows, K = X.shape
     codes = torch.empty((rows, K), dtype=torch.uint8, device=X.device)
     sf = torch.empty(max(16, int(load().qg_mx_scale_bytes(rows, K))), dtype=torch.uint8, device=X.device)
-    _check(load().qg_mx_quantize(context(), rows, K, _ptr(X), _ptr(codes), _ptr(sf), _stream()), "qg_mx_quantize")
+    lib, ctx, stream = _here()
+    _check(lib.qg_mx_quantize(ctx, rows, K, _ptr(X), _ptr(codes), _ptr(sf), stream), "qg_mx_quantize")
     return codes, sf
 
 
@@ -213,7 +227,8 @@ def mx_pack_weights(qbits, Wq, Wscale):
     K = Wscale.shape[1] * 32
     codes = torch.empty((N, K), dtype=torch.uint8, device=Wq.device)
     sf = torch.empty(max(16, int(load().qg_mx_scale_bytes(N, K))), dtype=torch.uint8, device=Wq.device)
-    _check(load().qg_mx_pack_weights(context(), qbits, N, K, _ptr(Wq), _ptr(Wscale), _ptr(codes), _ptr(sf), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.qg_mx_pack_weights(ctx, qbits, N, K, _ptr(Wq), _ptr(Wscale), _ptr(codes), _ptr(sf), stream),
            "qg_mx_pack_weights")
     return codes, sf
 
@@ -224,8 +239,9 @@ def qgemm_mx_dense(A_codes, A_sf, W_codes, W_sf, out=None):
     N = W_codes.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=torch.bfloat16, device=A_codes.device)
-    _check(load().qgemm_mx_dense(context(), M, N, K, _ptr(A_codes), _ptr(A_sf), _ptr(W_codes), _ptr(W_sf), _ptr(out),
-                                 _stream()), "qgemm_mx_dense")
+    lib, ctx, stream = _here()
+    _check(lib.qgemm_mx_dense(ctx, M, N, K, _ptr(A_codes), _ptr(A_sf), _ptr(W_codes), _ptr(W_sf), _ptr(out),
+                              stream), "qgemm_mx_dense")
     return out
 
 
@@ -235,7 +251,8 @@ def mx_quantize_grouped(X, offsets):
     E = offsets.numel() - 1
     codes = torch.empty((R, K), dtype=torch.uint8, device=X.device)
     sf = torch.zeros(max(16, load().qg_mx_grouped_scale_bytes(R, E, K)), dtype=torch.uint8, device=X.device)
-    _check(load().qg_mx_quantize_grouped(context(), R, E, K, _ptr(X), _ptr(offsets), _ptr(codes), _ptr(sf), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.qg_mx_quantize_grouped(ctx, R, E, K, _ptr(X), _ptr(offsets), _ptr(codes), _ptr(sf), stream),
            "qg_mx_quantize_grouped")
     return codes, sf
 
@@ -246,8 +263,9 @@ def moe_grouped_qgemm_mx(mode, A_codes, A_sf, offsets, W_codes, W_sf, N, topk_w=
     E = offsets.numel() - 1
     if out is None:
         out = torch.empty((R, N // 2 if mode == MODE_GATE_UP_SILU else N), dtype=torch.bfloat16, device=A_codes.device)
-    _check(load().moe_grouped_qgemm_mx(context(), mode, R, E, N, K, _ptr(A_codes), _ptr(A_sf), _ptr(offsets), _ptr(W_codes),
-                                       _ptr(W_sf), _ptr(topk_w), _ptr(row_pair), _ptr(out), _stream()), "moe_grouped_qgemm_mx")
+    lib, ctx, stream = _here()
+    _check(lib.moe_grouped_qgemm_mx(ctx, mode, R, E, N, K, _ptr(A_codes), _ptr(A_sf), _ptr(offsets), _ptr(W_codes),
+                                    _ptr(W_sf), _ptr(topk_w), _ptr(row_pair), _ptr(out), stream), "moe_grouped_qgemm_mx")
     return out
 
 
@@ -255,10 +273,13 @@ def _route_outputs(M, E, k, H, dev, X, out):
     """The output tensors of a routing call: the caller's (`out`, a dict with the same keys) or fresh ones."""
     if out is not None:
         return out
-    i32 = dict(dtype=torch.int32, device=dev)
-    o = dict(topk_idx=torch.empty((M, k), **i32), topk_w=torch.empty((M, k), dtype=torch.float32, device=dev),
-             counts=torch.empty(E, **i32), offsets=torch.empty(E + 1, **i32),
-             row_pair=torch.empty(M * k, **i32), pair_row=torch.empty(M * k, **i32))
+    # the small integer outputs (and the weights, 32 bits as well) are one allocation: seven of them cost the host more
+    # than the four launches of the call
+    n = M * k
+    idx, w, row_pair, pair_row, counts, offsets = torch.empty(4 * n + 2 * E + 1, dtype=torch.int32, device=dev).split_with_sizes(
+        (n, n, n, n, E, E + 1))
+    o = dict(topk_idx=idx.view(M, k), topk_w=w.view(torch.float32).view(M, k), counts=counts, offsets=offsets,
+             row_pair=row_pair, pair_row=pair_row)
     if X is not None:
         o["Xperm"] = torch.empty((M * k, H), dtype=torch.bfloat16, device=dev)
     return o
@@ -272,9 +293,10 @@ def moe_route(logits, k, X=None, ws=None, out=None):
     need = route_workspace_bytes(M, E, k)
     if ws is None:
         ws = torch.empty(max(need, 16), dtype=torch.uint8, device=logits.device)
-    _check(load().moe_route(context(), M, E, k, _ptr(logits), _ptr(out["topk_idx"]), _ptr(out["topk_w"]),
-                            _ptr(out["counts"]), _ptr(out["offsets"]), _ptr(out["row_pair"]), _ptr(out["pair_row"]),
-                            _ptr(X), _ptr(out.get("Xperm")), H, _ptr(ws), ws.numel(), _stream()), "moe_route")
+    lib, ctx, stream = _here()
+    _check(lib.moe_route(ctx, M, E, k, _ptr(logits), _ptr(out["topk_idx"]), _ptr(out["topk_w"]),
+                         _ptr(out["counts"]), _ptr(out["offsets"]), _ptr(out["row_pair"]), _ptr(out["pair_row"]),
+                         _ptr(X), _ptr(out.get("Xperm")), H, _ptr(ws), ws.numel(), stream), "moe_route")
     return out
 
 
@@ -286,9 +308,10 @@ def moe_route_static(logits, k, X=None, out=None):
     M, E = logits.shape
     H = X.shape[1] if X is not None else 0
     out = _route_outputs(M, E, k, H, logits.device, X, out)
-    _check(load().moe_route_static(context(), M, E, k, _ptr(logits), _ptr(out["topk_idx"]), _ptr(out["topk_w"]),
-                                   _ptr(out["counts"]), _ptr(out["offsets"]), _ptr(out["row_pair"]),
-                                   _ptr(out["pair_row"]), _ptr(X), _ptr(out.get("Xperm")), H, _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.moe_route_static(ctx, M, E, k, _ptr(logits), _ptr(out["topk_idx"]), _ptr(out["topk_w"]),
+                                _ptr(out["counts"]), _ptr(out["offsets"]), _ptr(out["row_pair"]),
+                                _ptr(out["pair_row"]), _ptr(X), _ptr(out.get("Xperm")), H, stream),
            "moe_route_static")
     return out
 
@@ -297,7 +320,8 @@ def moe_permute(X, row_pair, k, out=None):
     M, H = X.shape
     if out is None:
         out = torch.empty((M * k, H), dtype=torch.bfloat16, device=X.device)
-    _check(load().moe_permute(context(), M, k, H, _ptr(X), _ptr(row_pair), _ptr(out), _stream()), "moe_permute")
+    lib, ctx, stream = _here()
+    _check(lib.moe_permute(ctx, M, k, H, _ptr(X), _ptr(row_pair), _ptr(out), stream), "moe_permute")
     return out
 
 
@@ -313,8 +337,9 @@ def moe_grouped_qgemm(mode, qbits, Ain, offsets, Wq, Wscale, topk_w=None, row_pa
             out = torch.zeros((M if M is not None else R // k, N), dtype=torch.float32, device=dev)
         else:
             out = torch.empty((R, N), dtype=torch.bfloat16, device=dev)
-    _check(load().moe_grouped_qgemm(context(), mode, qbits, R, E, N, K, _ptr(Ain), _ptr(offsets), _ptr(Wq),
-                                    _ptr(Wscale), _ptr(topk_w), _ptr(row_pair), k, _ptr(out), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.moe_grouped_qgemm(ctx, mode, qbits, R, E, N, K, _ptr(Ain), _ptr(offsets), _ptr(Wq),
+                                 _ptr(Wscale), _ptr(topk_w), _ptr(row_pair), k, _ptr(out), stream),
            "moe_grouped_qgemm")
     return out
 
@@ -332,8 +357,9 @@ def moe_grouped_qgemm_gather(mode, qbits, X, row_pair, k, offsets, Wq, Wscale, t
             out = torch.zeros((M, N), dtype=torch.float32, device=dev)
         else:
             out = torch.empty((R, N), dtype=torch.bfloat16, device=dev)
-    _check(load().moe_grouped_qgemm_gather(context(), mode, qbits, M, R, E, N, K, _ptr(X), _ptr(row_pair), k,
-                                           _ptr(offsets), _ptr(Wq), _ptr(Wscale), _ptr(topk_w), _ptr(out), _stream()),
+    lib, ctx, stream = _here()
+    _check(lib.moe_grouped_qgemm_gather(ctx, mode, qbits, M, R, E, N, K, _ptr(X), _ptr(row_pair), k,
+                                        _ptr(offsets), _ptr(Wq), _ptr(Wscale), _ptr(topk_w), _ptr(out), stream),
            "moe_grouped_qgemm_gather")
     return out
 
@@ -348,11 +374,13 @@ def moe_combine(D, pair_row, k, topk_w=None, d_kind=D_BF16, out=None, shared=Non
     if out is None:
         out = torch.empty((M, H), dtype=torch.bfloat16, device=D.device)
     if shared is None:
-        _check(load().moe_combine(context(), M, k, H, _ptr(D), d_kind, _ptr(pair_row), _ptr(topk_w), _ptr(out), _stream()),
+        lib, ctx, stream = _here()
+        _check(lib.moe_combine(ctx, M, k, H, _ptr(D), d_kind, _ptr(pair_row), _ptr(topk_w), _ptr(out), stream),
                "moe_combine")
     else:
-        _check(load().moe_combine_shared(context(), M, k, H, _ptr(D), d_kind, _ptr(pair_row), _ptr(topk_w), _ptr(shared),
-                                         _ptr(out), _stream()), "moe_combine_shared")
+        lib, ctx, stream = _here()
+        _check(lib.moe_combine_shared(ctx, M, k, H, _ptr(D), d_kind, _ptr(pair_row), _ptr(topk_w), _ptr(shared),
+                                      _ptr(out), stream), "moe_combine_shared")
     return out
 
 
@@ -362,5 +390,6 @@ def moe_router_logits(X, Wr, out=None):
     E = Wr.shape[0]
     if out is None:
         out = torch.empty((M, E), dtype=torch.float32, device=X.device)
-    _check(load().moe_router_logits(context(), M, H, E, _ptr(X), _ptr(Wr), _ptr(out), _stream()), "moe_router_logits")
+    lib, ctx, stream = _here()
+    _check(lib.moe_router_logits(ctx, M, H, E, _ptr(X), _ptr(Wr), _ptr(out), stream), "moe_router_logits")
     return out
