@@ -237,7 +237,7 @@ moe_stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constan
         }
     } else if (warp == MS_CONS_WARPS + 1) {
         // ------------------------------------------------ segment rows: each group of eight k into the order 0, 2, 4, 6, 1, 3,
-        // 5, 7 of q4_spread, in place, and their block sums times -136
+        // 5, 7 of q4_spread, in place
         uint32_t slot = 0, phase = 0;
         int ends = 0;
         while (ends < 2 && __all_sync(0xFFFFFFFFu, ms_wait(xfull0 + 8u * slot, phase, abort_flag, p))) {
@@ -385,6 +385,9 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     const size_t fixed = 1024 + 4 * p.nt_max * 2 * 512 + 24 * MS_MAX_ST + 64 + 16 + 16 * MS_MAX_ST + (2 * static_cast<size_t>(E) + 2) * sizeof(int);
     p.n_stages = static_cast<int>((MS_SMEM_MAX - fixed) / p.stage_bytes);
     if (p.n_stages > MS_MAX_ST) p.n_stages = MS_MAX_ST;
+    // An even number, so that a slot's stages all belong to one set: with an odd one a set would see every other phase of a
+    // slot's barrier only, and a wait by parity passes too early when the phase in between is not complete yet.
+    p.n_stages &= ~1;
     if (p.n_stages < 2) return QG_ERR_WORKSPACE;
     const size_t smem = fixed + static_cast<size_t>(p.n_stages) * p.stage_bytes;
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
