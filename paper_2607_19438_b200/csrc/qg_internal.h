@@ -33,8 +33,8 @@ enum AttrSlot {
     ATTR_ROUTER_4 = 31,
     ATTR_MX_MOE = 32,       // 2: down, gate/up
     ATTR_MX_256 = 34,
-    ATTR_GEMV_RING = 35,    // 4: format (2) x more than eight tokens (2)
-    ATTR_MOE_STREAM = 39,   // 4: down, gate/up x rows per tile (2)
+    ATTR_STREAM = 35,       // 4: down, gate/up x rows per tile (2)
+    ATTR_DENSE_STREAM = 39, // 4: format (2) x more than eight tokens (2)
     ATTR_SLOTS = 43
 };
 }  // namespace qg
@@ -56,13 +56,13 @@ struct qg_ctx {
     float* sk_partial;         // stream-K: one fp32 partial tile (256 tokens x 128 rows) per CTA
     int* sk_flags;             // stream-K: two counters per CTA, zero between launches
     int streamk_mode;          // QG_STREAMK at creation: -1 heuristic (default), 0 never, 1 whenever legal
-    float* gemv_partial;       // K-slice partial sums of qgemm_small_m, [slices][16][N] fp32
+    float* gemv_partial;       // K-slice partial sums of qgemm_small_m's block kernel, [slices][16][N] fp32
     size_t gemv_partial_bytes;
-    int* gemv_tickets;         // one arrival counter per 64-row tile, then the tile counters of the grouped streaming kernel;
+    int* gemv_tickets;         // one arrival counter per 64-row tile, then the tile counters of the streaming kernel;
                                // zero between launches
     int gemv_ticket_count;
-    int gemv_mode;             // test hook (qg_test_gemv_mode): bit 0 no clusters, bit 1 always the ring kernel, bit 2 never
-    int gemv_max_clusters[4][9];   // ring kernel, per instantiation and cluster size: clusters that fit at once (0 unknown, -1 none)
+    int gemv_mode;             // test hook (qg_test_gemv_mode): bit 0 no clusters, bit 1 always the streaming kernel, bit 2 never
+    int gemv_max_clusters[4][9];   // streaming kernel, per instantiation and cluster size: clusters that fit at once (0 unknown, -1 none)
     long long* stats;          // profiling builds only
 };
 
@@ -100,4 +100,7 @@ int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 // shape does not suit it.
 int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, const int32_t* offsets,
                       const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st);
+// The same kernel for one matrix and up to sixteen tokens.
+int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void* A, const void* Wq, const void* Ws, void* Cout,
+                        cudaStream_t st);
 }  // namespace qg

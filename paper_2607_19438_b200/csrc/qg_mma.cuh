@@ -1,5 +1,5 @@
-// Warp-level pieces of the weight-streaming kernels: mma.sync with the weights as the 16-row operand, 4-bit codes as bf16
-// integers, packed fp32 arithmetic.
+// Warp-level pieces of the weight-streaming kernels: mma.sync with the weights as the 16-row operand, codes as bf16
+// integers.
 #pragma once
 #include <stdint.h>
 
@@ -13,6 +13,11 @@ __device__ __forceinline__ uint4 lds_u4(uint32_t addr) {
 __device__ __forceinline__ uint32_t lds_u1(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint2 lds_u2(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
     return v;
 }
 __device__ __forceinline__ void sts_u4(uint32_t addr, const uint4& v) {
@@ -45,6 +50,20 @@ __device__ __forceinline__ void q4_spread(uint32_t w, uint32_t (&p)[4]) {
     p[1] = sub_bf16x2(__byte_perm(e, HIGH, 0x7362), ZERO);
     p[2] = sub_bf16x2(__byte_perm(o, HIGH, 0x5140), ZERO);
     p[3] = sub_bf16x2(__byte_perm(o, HIGH, 0x7362), ZERO);
+}
+
+// four int8 codes (one word) -> two bf16 pairs of the same integers: (0, 2), (1, 3).  The low seven bits above 0x43 are the
+// bf16 number 128 + bits, the sign bit above 0x43 is 128 or 256: their difference is exact.
+__device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t mask, uint32_t base) {     // one LOP3 (two when written with operators)
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(a), "r"(mask), "r"(base));
+    return r;
+}
+__device__ __forceinline__ void q8_spread(uint32_t w, uint32_t& p02, uint32_t& p13) {
+    constexpr uint32_t LOW = 0x007F007Fu, SIGN = 0x00800080u, BASE = 0x43004300u;
+    const uint32_t v = w >> 8;
+    p02 = sub_bf16x2(and_or(w, LOW, BASE), and_or(w, SIGN, BASE));
+    p13 = sub_bf16x2(and_or(v, LOW, BASE), and_or(v, SIGN, BASE));
 }
 
 }  // namespace qg

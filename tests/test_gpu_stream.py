@@ -1,5 +1,5 @@
-"""The grouped GEMM's streaming kernel (4-bit weights, a few rows per expert): the edges of its tiles, stages and row groups,
-against the oracle."""
+"""The weight-streaming kernel (a few rows per expert, or one matrix and up to sixteen tokens): the edges of its tiles, stages,
+row groups and K slices, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -80,3 +80,56 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct():
     out = qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args)
     qg.poll_status()
     util.assert_close(util.host_bf16_f64(out), orc.grouped_gemm(4, orc.bf16_to_f64(A), offsets, Wq, Ws), "after a timeout")
+
+
+# one stage and an odd number of them; a slice of a single stage; ragged rows; more tiles than CTAs (tiles from the counter)
+# with one stage, with an odd number and with more stages than the ring holds; eight and sixteen tokens from both sides
+DENSE = [(8, 1, 64, 4096), (8, 8, 72, 768), (8, 9, 264, 1280), (4, 16, 136, 256 * 7), (4, 8, 2048, 512), (8, 16, 19016, 256),
+         (8, 3, 19136, 768), (4, 9, 38024, 256), (4, 7, 38144, 1280), (8, 2, 4096, 4096), (4, 1, 3072, 8192)]
+
+
+@pytest.mark.parametrize("mode", [2, 3], ids=["slices", "whole-k"])
+@pytest.mark.parametrize("qbits,M,N,K", DENSE, ids=[f"q{q}-{m}x{n}x{k}" for q, m, n, k in DENSE])
+def test_one_matrix(qbits, M, N, K, mode):
+    A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=15)
+    dA, dWq, dWs = util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws)
+    g = util.Guarded((M, N), torch.bfloat16)
+    qg.test_gemv_mode(mode)
+    try:
+        qg.qgemm_small_m(qbits, dA, dWq, dWs, out=g.t)
+        again = [qg.qgemm_small_m(qbits, dA, dWq, dWs) for _ in range(3)]
+        qg.poll_status()
+    finally:
+        qg.test_gemv_mode(0)
+    assert g.intact() and not bool(g.untouched_inside().any().item())
+    assert all(torch.equal(g.t, a) for a in again)
+    rows = np.unique(np.concatenate([np.arange(0, N, max(1, N // 700)), np.arange(max(0, N - 140), N)]))
+    util.assert_close(util.host_bf16_f64(g.t)[:, rows], orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows]), "one matrix")
+
+
+def test_every_8_bit_code_is_exact():
+    """Unit tokens and unit scales: the output is the code itself, for all 256 codes at every position of a 32-block."""
+    N, K = 256, 1024
+    Wq = ((np.arange(N)[:, None] + 37 * np.arange(K)[None, :]) % 256 - 128).astype(np.int8)
+    Ws = np.full((N, K // 32), np.float16(1).view(np.uint16))
+    for k0 in range(0, 32, 16):
+        A = torch.zeros((16, K), dtype=torch.bfloat16, device="cuda")
+        ks = [(k0 + m) + 32 * ((5 * m + k0) % 32) for m in range(16)]
+        for m, k in enumerate(ks):
+            A[m, k] = 1.0
+        out = qg.qgemm_small_m(8, A, util.dev(Wq), util.dev_f16(Ws))
+        qg.poll_status()
+        assert np.array_equal(util.host_bf16_f64(out), Wq[:, ks].T.astype(np.float64))
+
+
+def test_an_infinite_token_gives_infinities_of_the_codes_signs():
+    M, N, K = 3, 512, 1024
+    A, Wq, Ws = synth.dense_problem(8, M, N, K, seed=16)
+    dA = util.dev_bf16(A)
+    clean = qg.qgemm_small_m(8, dA, util.dev(Wq), util.dev_f16(Ws))
+    dA[1, 500] = float("-inf")
+    out = qg.qgemm_small_m(8, dA, util.dev(Wq), util.dev_f16(Ws))
+    qg.poll_status()
+    assert torch.equal(out[[0, 2]], clean[[0, 2]])
+    q = Wq[:, 500].astype(np.int64) * np.sign(Ws[:, 500 // 32].view(np.float16).astype(np.float64))
+    assert np.array_equal(out[1].float().cpu().numpy()[q != 0], -np.sign(q[q != 0]) * np.inf)
