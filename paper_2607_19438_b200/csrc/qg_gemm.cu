@@ -21,6 +21,8 @@
 //   warp 3      also allocates and frees TMEM
 // Barriers the MMA waits on live in the even CTA and also collect the odd CTA's arrivals (remote mbarrier
 // arrive, TMA completion bytes); barriers that free a stage are signalled in both CTAs by the commit.
+// Dense calls with few tiles cut K into slices, one per CTA pair of a larger cluster (qgemm_slices_kernel): every pair leaves
+// its fp32 tile in shared memory and the cluster adds them in slice order.
 // Every mbarrier wait is bounded; when one expires the CTA records QG_ERR_TIMEOUT and leaves.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -49,6 +51,8 @@ struct GemmParams {
                                 // pairs; tiles cut in the middle are summed through sk_partial
     float* sk_partial;          // [CTAs][BT * 128] fp32: the partial accumulator of each CTA's unfinished first tile
     int* sk_flags;              // [CTAs][2]: 16-token blocks of the partial written / consumed; zero between launches
+    int slices, kc;             // dense plain calls with few tiles: K cut into `slices` parts of kc k-blocks, one per CTA
+                                // pair of a cluster; the cluster adds the parts through distributed shared memory
     int* status;
     uint32_t wait_limit;        // polls per bounded wait (an unsatisfied poll lasts about 4 us)
     int skip_kb;                // test hook: k-block of the first tile whose activation load is left out (-1: none)
@@ -318,12 +322,66 @@ __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int t
     }
 }
 
+// K slices (SK = 2): a warp leaves the raw fp32 fragments of its 16-token blocks in this CTA's shared memory (the idle ring of
+// the activation tile, exactly as large): register r of block b and lane quarter q at ((b 4 + q) 16 + r) 32 + lane.
+__device__ __forceinline__ void dump_partial(float* part, uint32_t taddr, int n_epi, int pid, int npart, int quarter, int lane) {
+    for (int b = pid; b < (n_epi >> 4); b += npart) {
+        uint32_t v0[8], v1[8];
+        tmem_ld_16x256_x2(taddr + 16 * b, v0);
+        tmem_ld_16x256_x2(taddr + (16u << 16) + 16 * b, v1);
+        tmem_ld_wait();
+        float* dst = part + ((b * 4 + quarter) * 16) * 32 + lane;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            dst[r * 32] = __uint_as_float(v0[r]);
+            dst[(8 + r) * 32] = __uint_as_float(v1[r]);
+        }
+    }
+}
+
+// Then one warp adds a block's fragments over the slices, in slice order, and stores it (the layout and the transposition of
+// drain_plain).  part: shared::cluster-mappable address of the fragments, r_cta: which CTA of each pair holds these rows.
+__device__ __forceinline__ void sum_block(const GemmParams& p, uint32_t part, uint32_t r_cta, int unit, int tok0, int tok_end,
+                                          int n_tile, __nv_bfloat16* st, int lane) {
+    const int b = unit >> 2, quarter = unit & 3;
+    float v[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = 0.f;
+    for (int sl = 0; sl < p.slices; ++sl) {
+        const uint32_t src = map_to_cta(part + (unit * 16 * 32 + lane) * 4, 2 * sl + r_cta);
+        float x[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x[r]) : "r"(src + r * 128));
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] += x[r];
+    }
+    uint32_t pk[8];
+#pragma unroll
+    for (int gq = 0; gq < 2; ++gq) {
+        pk[4 * gq + 0] = bf16x2(v[4 * gq + 0], v[4 * gq + 1]);
+        pk[4 * gq + 1] = bf16x2(v[4 * gq + 2], v[4 * gq + 3]);
+        pk[4 * gq + 2] = bf16x2(v[8 + 4 * gq + 0], v[8 + 4 * gq + 1]);
+        pk[4 * gq + 3] = bf16x2(v[8 + 4 * gq + 2], v[8 + 4 * gq + 3]);
+    }
+    const uint32_t st_row = smem_u32(st) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
+    const int tk = lane >> 2, c4 = lane & 3, n = n_tile + quarter * 32 + c4 * 8, left = tok_end - tok0 - 16 * b - tk;
+    stmatrix_x4_trans(st_row, pk[0], pk[1], pk[2], pk[3]);
+    stmatrix_x4_trans(st_row + 512, pk[4], pk[5], pk[6], pk[7]);
+    __syncwarp();
+    const uint4* s_lo = reinterpret_cast<const uint4*>(st + tk * 32 + ((c4 ^ ((tk >> 1) & 3)) << 3));
+    __nv_bfloat16* g = static_cast<__nv_bfloat16*>(p.out) + static_cast<size_t>(tok0 + 16 * b + tk) * p.N + n;
+    if (n < p.N && left > 0) *reinterpret_cast<uint4*>(g) = *s_lo;
+    if (n < p.N && left > 8) *reinterpret_cast<uint4*>(g + static_cast<size_t>(8) * p.N) = s_lo[32];
+    __syncwarp();
+}
+
+// SK: 0 every tile is computed whole, 1 stream-K, 2 K slices of one tile on the CTA pairs of a cluster (grid = one cluster
+// per tile).
 // EPI: 0 plain / routing-weighted bf16 store, 1 gate/up + SiLU, 2 weighted fp32 atomic accumulate (compiled apart so
 // that each instantiation carries one epilogue only).
-template <int QBITS, int BT, int EPI, bool SK>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
-qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
-             const __grid_constant__ CUtensorMap tm_s, const GemmParams p) {
+template <int QBITS, int BT, int EPI, int SK>
+__device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const CUtensorMap& tm_s,
+                                          const GemmParams& p) {
     using C = Cfg<QBITS, BT>;
     extern __shared__ uint8_t smem_dyn[];
     const uint32_t sbase = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -349,7 +407,11 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
     const uint32_t last_full = bar0 + 8u * (2 * C::SX + 2 * C::SR + 4);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();          // 0: issues the MMAs, 1: its peer
+    const uint32_t crank = cluster_ctarank();
+    const uint32_t rank = (SK == 2) ? (crank & 1u) : crank;            // 0: issues the MMAs, 1: its peer
+    const uint32_t leader = (SK == 2) ? (crank & ~1u) : 0u;            // the pair's even CTA
+    const int slice = (SK == 2) ? static_cast<int>(crank >> 1) : 0;
+    const int kb_first = (SK == 2) ? slice * p.kc : 0;                 // this pair's first k-block
     // The next kernel in the stream may be scheduled as this grid's CTAs leave their SMs.  This kernel in turn may
     // have started before the previous one finished: whatever that kernel may have written (activations, expert
     // offsets, routing tables) or may still read (the output buffer) is touched only after pdl_wait().  The weights
@@ -358,8 +420,10 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
     if (warp == 0) { QG_MARK(0); }
     QG_SPAN(0);
     const bool grouped = (p.offsets != nullptr);
-    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int pair = (SK == 2) ? static_cast<int>(blockIdx.x) / (2 * p.slices) : static_cast<int>(blockIdx.x) >> 1;
+    const int n_pairs = (SK == 2) ? static_cast<int>(gridDim.x) / (2 * p.slices) : static_cast<int>(gridDim.x) >> 1;
     volatile int* abort_flag = misc + 1;
+    float* partial = reinterpret_cast<float*>(sgen + C::OFF_X);          // K slices: where the ring of the activation tile was
 
     if (warp == 0) {   // barrier initialisation spread over the lanes of one warp (a single thread needs ~50 steps)
         if (lane < C::SX) { mbar_init(full(lane), 1 + 8); mbar_init(done(lane), 1); }
@@ -412,15 +476,15 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         }
         if (lane == 0) prefix[p.E] = carry;
         __syncwarp();
-        if (!SK && pair < carry) {
+        if (SK != 1 && pair < carry) {
             const Tile tl = decode_tile(pair, prefix, p, BT);
             const int wt = 2 * tl.pw + static_cast<int>(rank);
             if (lane == 0) {
                 mbar_arrive_expect_tx(r_full(0), 4 * C::RAW_BYTES + C::SC_BYTES);
-                load_w(sbase + C::OFF_SC, &tm_s, 0, tl.e, wt, r_full(0));
+                load_w(sbase + C::OFF_SC, &tm_s, (kb_first >> 2) * 8, tl.e, wt, r_full(0));
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    load_w(sbase + C::OFF_RAW + j * C::RAW_BYTES, &tm_w, j * C::RAW_ROW, tl.e, wt, r_full(0));
+                    load_w(sbase + C::OFF_RAW + j * C::RAW_BYTES, &tm_w, (kb_first + j) * C::RAW_ROW, tl.e, wt, r_full(0));
             }
             w_pre_issued = true;
         }
@@ -441,7 +505,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
     const int nk4 = nkb >> 2;
     int my_tiles;
     uint32_t own_kb4;            // this pair's k-blocks / 4
-    if constexpr (SK) {
+    if constexpr (SK == 1) {
         // Units of four k-blocks, U = tiles * nk4 in all; pair q owns units [U q / P, U (q + 1) / P).  Piece j of this
         // pair lies in tile t_first + j (the host keeps the number of pieces within the table).
         const long long U = static_cast<long long>(total_tiles) * nk4;
@@ -468,6 +532,10 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
             ptab[j] = pc;
             tab[j] = decode_tile(t, prefix, p, BT);
         }
+    } else if constexpr (SK == 2) {
+        my_tiles = 1;                                       // one cluster per tile
+        own_kb4 = static_cast<uint32_t>(min(p.kc, nkb - kb_first)) >> 2;
+        if (threadIdx.x == 0) tab[0] = decode_tile(pair, prefix, p, BT);
     } else {
         my_tiles = (total_tiles > pair) ? (total_tiles - pair + n_pairs - 1) / n_pairs : 0;
         own_kb4 = static_cast<uint32_t>(my_tiles) * static_cast<uint32_t>(nk4);
@@ -480,9 +548,9 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         return (j < C::TAB_N) ? tab[j] : decode_tile(pair + j * n_pairs, prefix, p, BT);
     };
     auto piece_at = [&](int j) -> Piece {
-        if constexpr (SK) return ptab[j];
+        if constexpr (SK == 1) return ptab[j];
         Piece pc;
-        pc.kb0 = 0; pc.kb1 = nkb; pc.i0 = j * nkb; pc.nsrc = 0;
+        pc.kb0 = kb_first; pc.kb1 = (SK == 2) ? kb_first + 4 * static_cast<int>(own_kb4) : nkb; pc.i0 = j * nkb; pc.nsrc = 0;
         return pc;
     };
 
@@ -494,7 +562,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         // ------------------------------------------------ activation producer (this CTA's half of the token tile)
         uint32_t s = 0, ph = 0;      // first stage of the next batch (0, 2, 4, 6) and the parity of its next "done" phase
         uint32_t sent_kb = 0;        // k-blocks sent so far: the first eight find the ring empty and need no wait
-        const uint32_t full_leader = map_to_cta(full(0), 0);
+        const uint32_t full_leader = map_to_cta(full(0), leader);
         bool ok = true;
         QG_DECL();
         for (int jt = 0; jt < my_tiles && ok; ++jt) {
@@ -632,14 +700,14 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
                     if (lane == 0) {
                         umma_kblock_ts_pair(d_tmem, tmem_base + C::A_COL0 + ta * C::A_COLS,
                                             b_lo0 + st * (C::X_BYTES >> 4), b_hi, idesc, kb != pc.kb0 ? 1u : 0u);
-                        umma_commit_pair(done(st));
+                        umma_commit_pair(done(st), 3u << leader);
                     }
                     __syncwarp();
                     QG_ACC(10);
                     kb += 2;
                     i = in;
                 }
-                if (ok && lane == 0) umma_commit_pair(acc_full(a));
+                if (ok && lane == 0) umma_commit_pair(acc_full(a), 3u << leader);
                 __syncwarp();
                 if (w == 0 && static_cast<int>(j) == my_tiles - 1) { QG_MARK(3); }
             }
@@ -658,7 +726,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         const uint32_t swz = (QBITS == 8) ? ((row >> 1) & 3u) : ((row >> 2) & 1u);
         const uint32_t raw_row = row * C::RAW_ROW;
         const uint32_t a_taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + C::A_COL0;
-        const uint32_t full_leader = map_to_cta(full(0), 0);
+        const uint32_t full_leader = map_to_cta(full(0), leader);
         const uint32_t n_own = own_kb4;
         constexpr uint32_t magic = 0x43000000u;
         QG_DECL();
@@ -666,13 +734,14 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         // stage) it must have released every accumulator of an earlier tile, otherwise a single-accumulator pipeline
         // would wait for itself; at that point it has filled the ring for the next tile and would idle anyway.
         auto per_tile = [&](uint32_t t) -> uint32_t {                  // own k-blocks of the pair's t-th tile (piece)
-            if constexpr (!SK) return static_cast<uint32_t>(nk4);
+            if constexpr (SK == 0) return static_cast<uint32_t>(nk4);
+            if constexpr (SK == 2) return own_kb4;
             const Piece pc = ptab[t];
             return static_cast<uint32_t>(pc.kb1 - pc.kb0) >> 2;
         };
         uint32_t helped = 0;                                           // tiles whose accumulator this warp released
         uint32_t t2 = 0, in2 = 0;                                      // tile of own k-block n - 2, position in it
-        const uint32_t acc_empty_leader = map_to_cta(acc_empty(0), 0);
+        const uint32_t acc_empty_leader = map_to_cta(acc_empty(0), leader);
         constexpr bool plain_ep = (EPI == 0);
         __nv_bfloat16* my_st = stg16 + (warp - 8) * 512;               // private 1 KB transposition buffer
         uint32_t ta = static_cast<uint32_t>(g) % C::SA;                 // TMEM weight stage of own k-block i = i % SA
@@ -689,7 +758,10 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
             tc_fence_after_sync();
             if (plain_ep && wt < p.n_wt) {
                 const int n_mma = min(BT, (tl.tok_end - tl.tok0 + 15) & ~15);
-                drain_plain<SK>(p, tl.tok0, tl.tok_end, wt * BW + q * 32,
+                if constexpr (SK == 2)
+                    dump_partial(partial, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma, 1 + g, 5, q, lane);
+                else
+                    drain_plain<SK == 1>(p, tl.tok0, tl.tok_end, wt * BW + q * 32,
                             tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma, 1 + g, 5, my_st, lane,
                             piece_at(static_cast<int>(jt)).nsrc, q, BT * 128, abort_flag);
             }
@@ -787,7 +859,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         const int et = threadIdx.x - 128;
         __nv_bfloat16* outb = static_cast<__nv_bfloat16*>(p.out);
         float* outf = static_cast<float*>(p.out);
-        const uint32_t acc_empty_base = map_to_cta(acc_empty(0), 0);
+        const uint32_t acc_empty_base = map_to_cta(acc_empty(0), leader);
         uint32_t j = 0;
         QG_DECL();
         for (; static_cast<int>(j) < my_tiles; ++j) {
@@ -810,7 +882,8 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
             const int n_epi = (wt < p.n_wt) ? n_mma : 0;
             if constexpr (EPI == 0) {
                 // shared with the dequantising warps (participants 1..4 of this lane quarter) when they help
-                drain_plain<SK>(p, tl.tok0, tl.tok_end, wt * BW + qd * 32, taddr, n_epi, 0,
+                if constexpr (SK == 2) dump_partial(partial, taddr, n_epi, 0, 5, qd, lane);
+                else drain_plain<SK == 1>(p, tl.tok0, tl.tok_end, wt * BW + qd * 32, taddr, n_epi, 0,
                             (C::HELP || static_cast<int>(j) == my_tiles - 1) ? 5 : 1,
                             stg16 + (16 + qd) * 512, lane, piece_at(static_cast<int>(j)).nsrc, qd, BT * 128, abort_flag);
             } else {
@@ -882,6 +955,21 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
         if (et == 0) QG_FLUSH();
     }
 
+    // ---------------------------------------------------- K slices: sum over the cluster
+    if constexpr (SK == 2) {
+        __syncthreads();
+        cluster_sync_all();          // every slice's fragments are in place
+        const Tile tl = tab[0];
+        const int wt = 2 * tl.pw + static_cast<int>(rank);
+        if (warp >= 4 && wt < p.n_wt && !*abort_flag) {
+            pdl_wait();
+            const int units = ((tl.tok_end - tl.tok0 + 15) >> 4) * 4;
+            for (int u = (warp - 4) * p.slices + slice; u < units; u += 20 * p.slices)
+                sum_block(p, smem_u32(partial), rank, u, tl.tok0, tl.tok_end, wt * BW,
+                          stg16 + (warp >= 8 ? warp - 8 : warp + 12) * 512, lane);
+        }
+    }
+
     // ---------------------------------------------------- teardown
     __syncthreads();
     if (warp == 0) { QG_MARK(6); }
@@ -896,7 +984,41 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
     QG_SPAN(1);
 }
 
-template <int QBITS, int BT, int EPI, bool SK>
+template <int QBITS, int BT, int EPI, int SK>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+             const __grid_constant__ CUtensorMap tm_s, const GemmParams p) {
+    gemm_body<QBITS, BT, EPI, SK>(tm_x, tm_w, tm_s, p);
+}
+// K slices: the launch names the cluster size (two CTAs per slice)
+template <int QBITS, int BT>
+__global__ void __launch_bounds__(NTHREADS, 1)
+qgemm_slices_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                    const __grid_constant__ CUtensorMap tm_s, const GemmParams p) {
+    gemm_body<QBITS, BT, 0, 2>(tm_x, tm_w, tm_s, p);
+}
+// clusters of 2 * slices CTAs of the kernel above that fit on the GPU at once (asked once per context, kernel and size)
+template <int QBITS, int BT>
+static int slices_capacity(qg_ctx* ctx, int slices) {
+    constexpr int inst = (QBITS == 4 ? 2 : 0) + (BT == 128 ? 0 : 1);
+    int& cached = ctx->slice_clusters[inst][slices];
+    if (cached == 0) {
+        constexpr int smem = Cfg<QBITS, BT>::SMEM_BYTES;
+        auto kern = qgemm_slices_kernel<QBITS, BT>;
+        cudaLaunchConfig_t q = {};
+        cudaLaunchAttribute ca;
+        ca.id = cudaLaunchAttributeClusterDimension;
+        ca.val.clusterDim.x = 2 * slices; ca.val.clusterDim.y = 1; ca.val.clusterDim.z = 1;
+        q.gridDim = dim3(2 * slices); q.blockDim = dim3(NTHREADS); q.dynamicSmemBytes = smem; q.attrs = &ca; q.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        cached = n > 0 ? n : -1;
+    }
+    return cached;
+}
+
+template <int QBITS, int BT, int EPI, int SK>
 static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_rows, const void* Wq, const void* Ws,
                        cudaStream_t st) {
     using C = Cfg<QBITS, BT>;
@@ -920,9 +1042,27 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
                         : get_tmap_2d(ctx, &tm_s, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, Ws, p.K / 32, wrows, 8, 128,
                                       CU_TENSOR_MAP_SWIZZLE_NONE);
     if (rc != QG_OK) return rc;
+    if constexpr (SK == 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * p.slices * static_cast<unsigned>(((p.n_wt + 1) / 2) * ((p.R + BT - 1) / BT)));
+        cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2 * p.slices; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at; cfg.numAttrs = ctx->pdl ? 2 : 1;
+        if (cudaLaunchKernelEx(&cfg, qgemm_slices_kernel<QBITS, BT>, tm_x, tm_w, tm_s, p) == cudaSuccess) return QG_OK;
+        // refused although the occupancy query allowed it: remember that and leave K whole
+        cudaGetLastError();
+        ctx->slice_clusters[(QBITS == 4 ? 2 : 0) + (BT == 128 ? 0 : 1)][p.slices] = -1;
+        GemmParams whole = p;
+        whole.slices = 1;
+        return launch_gemm<QBITS, BT, EPI, 0>(ctx, whole, X, x_rows, Wq, Ws, st);
+    }
     auto kern = qgemm_kernel<QBITS, BT, EPI, SK>;
     // the shared-memory attribute belongs to the function on one device: set once per context and instantiation
-    constexpr int inst = SK ? ATTR_GEMM_SK + ((QBITS == 4) ? 3 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 1 : 2)
+    constexpr int inst = SK == 1 ? ATTR_GEMM_SK + ((QBITS == 4) ? 3 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 1 : 2)
                             : ATTR_GEMM + ((QBITS == 4) ? 9 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 3 : 6) + EPI;
     if (!ctx->attr_set[inst]) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess) {
@@ -954,13 +1094,49 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
 // removes most of a wave of long-K tiles, and the model charges it accordingly.
 struct DensePlan {
     int bt, streamk;
+    int slices, kc;      // > 1: K slices of kc k-blocks on the CTA pairs of a cluster
 };
-static DensePlan plan_dense(const qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
+static int slices_capacity(qg_ctx* ctx, int qbits, int bt, int slices) {
+    if (qbits == QG_Q8) return bt == 128 ? slices_capacity<8, 128>(ctx, slices) : slices_capacity<8, 192>(ctx, slices);
+    return bt == 128 ? slices_capacity<4, 128>(ctx, slices) : slices_capacity<4, 192>(ctx, slices);
+}
+// Few tiles leave most SM pairs idle behind a serial walk over K.  Cutting K into two to four slices, one per pair of a
+// cluster that adds its partial tiles through distributed shared memory, divides the walk; the sum costs
+// 1100 + 1300 (slices - 2) cycles and 20 + 5 (slices - 2) per token of the tile (fitted to 25 shapes at 20 to 500 tokens, a
+// k-block being 515 cycles with up to 128 tokens and 600 with 192).  Stream-K's exchange through global memory costs 22000
+// on top of its share.  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four slices, so this
+// is for at most 33 tiles.  Measured, 20 / 128 tokens: 3072 x 3072 16.5 / 17.3 us whole, 10.0 / 12.3 in four slices;
+// 5120 x 3072 16.7 / 17.7, 11.3 / 13.3 in three; 2048 x 8192 24.8 / 30.1 (stream-K), 14.1 / 16.8 in four; 4096 x 14336
+// 29.2 / 34.1 (stream-K), 26.7 / 29.6 in three.
+static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePlan& plan) {
+    if (ctx->force_bt || ctx->streamk_mode != -1) return;
+    const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
+    const int nk4 = K / (4 * BK);
+    const long long tiles0 = n_pw * ((M + plan.bt - 1) / plan.bt);
+    if (tiles0 > pairs) return;
+    auto period = [](int bt) { return bt == 128 ? 515.0 : bt == 192 ? 600.0 : 720.0; };
+    double best = plan.streamk ? (tiles0 * nk4 + pairs - 1) / pairs * 4.0 * period(plan.bt) + 22000.0 : nk4 * 4.0 * period(plan.bt);
+    best *= 0.97;
+    for (int bt = 128; bt <= 192; bt += 64) {
+        if (bt > 128 && M <= 128) break;
+        const long long tiles = n_pw * ((M + bt - 1) / bt);
+        for (int sl = 2; sl <= 4 && sl <= nk4 && tiles * sl <= pairs; ++sl) {
+            const int per = (nk4 + sl - 1) / sl;
+            if ((nk4 + per - 1) / per != sl) continue;             // the same cut as a smaller count
+            const double cost = per * 4.0 * period(bt) + 1100.0 + 1300.0 * (sl - 2) + (20.0 + 5.0 * (sl - 2)) * (M < bt ? M : bt);
+            if (cost < best && slices_capacity(ctx, qbits, bt, sl) >= tiles) {
+                best = cost;
+                plan = DensePlan{bt, 0, sl, 4 * per};
+            }
+        }
+    }
+}
+static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
     const int cand[3] = {128, 192, 256};
     const double period[3] = {630.0, 655.0, (qbits == 4) ? 760.0 : 720.0}, epilogue[3] = {0.0, 0.0, 6000.0};
     const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
     const int nk4 = K / (4 * BK);
-    DensePlan best{256, 0};
+    DensePlan best{256, 0, 1, 0};
     double best_cost = 1e300;
     for (int c = 0; c < 3; ++c) {
         if (M <= 128 && cand[c] > 128) break;
@@ -969,7 +1145,7 @@ static DensePlan plan_dense(const qg_ctx* ctx, int qbits, int M, int n_wt, int K
         const double waves = 0.5 * (static_cast<double>((tiles + pairs - 1) / pairs) + frac);
         const double dp = waves * ((K / BK) * period[c] + epilogue[c]);
         if (ctx->streamk_mode != 1 || tiles % pairs == 0)
-            if (dp < best_cost) { best_cost = dp; best = DensePlan{cand[c], 0}; }
+            if (dp < best_cost) { best_cost = dp; best = DensePlan{cand[c], 0, 1, 0}; }
     }
     if (ctx->streamk_mode == 0) return best;
     // Below K = 4096 the exchange never paid in the measurements (K = 2048 and 3072, 64 to 1024 tokens: 2 to 10 us slower).
@@ -986,10 +1162,15 @@ static DensePlan plan_dense(const qg_ctx* ctx, int qbits, int M, int n_wt, int K
         const double sk = share * 4.0 * period[c] + pieces * epilogue[c] + 10000.0;
         if (ctx->streamk_mode == 1 ? (best.streamk == 0 || sk < best_cost) : (sk < 0.95 * best_cost)) {
             best_cost = sk;
-            best = DensePlan{cand[c], 1};
+            best = DensePlan{cand[c], 1, 1, 0};
         }
     }
     return best;
+}
+static DensePlan plan_dense(qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
+    DensePlan plan = plan_whole(ctx, qbits, M, n_wt, K);
+    plan_slices(ctx, qbits, M, n_wt, K, plan);
+    return plan;
 }
 
 static int dispatch_gemm(qg_ctx* ctx, int qbits, int bt, const GemmParams& p_in, const void* X, int x_rows,
@@ -1006,11 +1187,16 @@ static int dispatch_gemm(qg_ctx* ctx, int qbits, int bt, const GemmParams& p_in,
     const int epi = (p.mode == QG_MODE_GATE_UP_SILU) ? 1 : (p.mode == QG_MODE_DOWN_ACCUM_F32) ? 2 : 0;
 #define QG_LAUNCH(Q, B)                                                                 \
     do {                                                                                \
-        if (epi == 0 && p.streamk) return launch_gemm<Q, B, 0, true>(ctx, p, X, x_rows, Wq, Ws, st);   \
-        if (epi == 0) return launch_gemm<Q, B, 0, false>(ctx, p, X, x_rows, Wq, Ws, st);                \
-        if (epi == 1) return launch_gemm<Q, B, 1, false>(ctx, p, X, x_rows, Wq, Ws, st);                \
-        return launch_gemm<Q, B, 2, false>(ctx, p, X, x_rows, Wq, Ws, st);                              \
+        if (epi == 0 && p.streamk) return launch_gemm<Q, B, 0, 1>(ctx, p, X, x_rows, Wq, Ws, st);       \
+        if (epi == 0) return launch_gemm<Q, B, 0, 0>(ctx, p, X, x_rows, Wq, Ws, st);                    \
+        if (epi == 1) return launch_gemm<Q, B, 1, 0>(ctx, p, X, x_rows, Wq, Ws, st);                    \
+        return launch_gemm<Q, B, 2, 0>(ctx, p, X, x_rows, Wq, Ws, st);                                  \
     } while (0)
+    if (p.slices > 1) {
+        if (qbits == QG_Q8)
+            return (bt == 128) ? launch_gemm<8, 128, 0, 2>(ctx, p, X, x_rows, Wq, Ws, st) : launch_gemm<8, 192, 0, 2>(ctx, p, X, x_rows, Wq, Ws, st);
+        return (bt == 128) ? launch_gemm<4, 128, 0, 2>(ctx, p, X, x_rows, Wq, Ws, st) : launch_gemm<4, 192, 0, 2>(ctx, p, X, x_rows, Wq, Ws, st);
+    }
     if (qbits == QG_Q8) {
         if (bt == 256) QG_LAUNCH(8, 256);
         if (bt == 192) QG_LAUNCH(8, 192);
@@ -1051,6 +1237,7 @@ int qgemm_dense(qg_ctx* ctx, int qbits, int M, int N, int K, const void* A, cons
     p.offsets = nullptr; p.out = Cout; p.topk_w = nullptr; p.row_pair = nullptr;
     const qg::DensePlan plan = qg::plan_dense(ctx, qbits, M, p.n_wt, K);
     p.streamk = (ctx->force_bt == 0 || ctx->streamk_mode == 1) ? plan.streamk : 0;
+    p.slices = plan.slices; p.kc = plan.kc;
     p.sk_partial = ctx->sk_partial; p.sk_flags = ctx->sk_flags;
     return qg::dispatch_gemm(ctx, qbits, plan.bt, p, A, M, Wq, Wscale, static_cast<cudaStream_t>(stream));
 }

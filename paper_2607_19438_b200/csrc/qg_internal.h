@@ -61,6 +61,7 @@ struct qg_ctx {
     int* gemv_tickets;         // one arrival counter per 64-row tile, then the tile counters of the streaming kernel;
                                // zero between launches
     int gemv_ticket_count;
+    int slice_clusters[4][5];      // dense GEMM with K slices, per format x token tile and slices: clusters that fit at once (0 unknown, -1 none)
     int gemv_mode;             // test hook (qg_test_gemv_mode): bit 0 no clusters, bit 1 always the streaming kernel, bit 2 never
     int gemv_max_clusters[4][9];   // streaming kernel, per instantiation and cluster size: clusters that fit at once (0 unknown, -1 none)
     long long* stats;          // profiling builds only

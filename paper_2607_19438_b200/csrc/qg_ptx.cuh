@@ -184,10 +184,11 @@ __device__ __forceinline__ void umma_kblock_ts_pair(uint32_t tmem_d, uint32_t tm
         ::"r"(tmem_d), "r"(tmem_a), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc0)
         : "memory");
 }
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+// ctas: the pair's two CTAs as a mask of cluster ranks (ranks 0 and 1 unless the cluster holds several pairs)
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t ctas = 3u) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        ::"r"(bar), "h"(static_cast<unsigned short>(3))
+        ::"r"(bar), "h"(static_cast<unsigned short>(ctas))
         : "memory");
 }
 

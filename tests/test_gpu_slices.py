@@ -1,0 +1,45 @@
+"""qgemm_dense with K cut into slices that a thread-block cluster adds (few tiles): every slice count and token tile, ragged
+rows and tokens, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2607_19438_b200 import binding as qg, synth
+from tests import util
+
+pytestmark = pytest.mark.gpu
+
+# slices of equal and unequal length (K = 1280: 5 units of four k-blocks), one row tile and an odd number of them, rows past
+# the end in the last tile, tokens around the edges of the 16-token blocks and of the 128- and 192-token tiles
+SHAPES = [(8, 17, 256, 2048), (4, 20, 3072, 3072), (8, 128, 2184, 2560), (4, 129, 1152, 1280), (8, 127, 136, 8192),
+          (4, 192, 2048, 2048), (8, 333, 2048, 2048), (4, 500, 2560, 2048), (8, 193, 4096, 4096), (4, 64, 5120, 3072),
+          (8, 1, 512, 1024), (4, 16, 8, 512)]
+
+
+@pytest.mark.parametrize("qbits,M,N,K", SHAPES, ids=[f"q{q}-{m}x{n}x{k}" for q, m, n, k in SHAPES])
+def test_slices_match_the_oracle(qbits, M, N, K):
+    A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=23)
+    g = util.Guarded((M, N), torch.bfloat16)
+    args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
+    for _ in range(3):                                   # back to back: a launch's start overlaps the end of the one before
+        qg.qgemm_dense(qbits, *args, out=g.t)
+    qg.poll_status()
+    assert g.intact() and not bool(g.untouched_inside().any().item())
+    rows = np.unique(np.concatenate([np.arange(0, N, max(1, N // 500)), np.arange(max(0, N - 140), N)]))
+    util.assert_close(util.host_bf16_f64(g.t)[:, rows], orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows]), "slices")
+
+
+def test_a_wait_that_runs_out_in_one_slice():
+    qbits, M, N, K = 8, 40, 2048, 4096
+    A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=24)
+    args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
+    try:
+        qg.test_inject(wait_limit_polls=2048, skip_kblock=K // 64 - 2)      # a k-block of the last slice
+        qg.qgemm_dense(qbits, *args)
+        assert qg.poll_status_code() == -7
+    finally:
+        qg.test_inject(0, -1)
+    out = qg.qgemm_dense(qbits, *args)
+    qg.poll_status()
+    util.assert_close(util.host_bf16_f64(out), orc.qgemm_dense(qbits, A, Wq, Ws), "after a timeout")
