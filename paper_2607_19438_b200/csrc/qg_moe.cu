@@ -187,6 +187,129 @@ route_scatter_kernel(int M, int E, int k, const int32_t* __restrict__ topk_idx, 
     }
 }
 
+// The whole of routing for up to 32 tokens in one block: one warp per token, at most 1024 pairs and 32 NK experts.  The three
+// kernels above are a few microseconds of latency each with next to no work then (128 experts, eight per token: 4 tokens
+// 8.7 us, 32 tokens 10.4; this one 3.3 and 6.4; with four tokens per warp it took 24 at 128 tokens against 10.4).  The
+// token's keys stay in registers, NK per lane; the selection is route_topk_kernel's.  Thread p then places pair p: its rank
+// among the pairs of its warp with the same expert, plus a prefix over the warps, plus the expert's offset, all in ascending
+// pair order.  The block has a warp for every token, for every 32 pairs and for every 32 experts.
+// Dynamic shared memory: expert of each pair [32 pair warps], pairs per pair warp and expert, [E] offsets, [32] warp sums.
+template <int NK>
+__global__ void __launch_bounds__(1024)
+route_small_kernel(int M, int E, int k, const float* __restrict__ logits, int32_t* __restrict__ topk_idx,
+                   float* __restrict__ topk_w, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
+                   int32_t* __restrict__ row_pair, int32_t* __restrict__ pair_row) {
+    extern __shared__ int rs[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x, nwarps = blockDim.x >> 5;
+    const int pw = (M * k + 31) >> 5;            // warps that hold pairs
+    int* expert = rs;
+    int* wcnt = expert + 32 * pw;
+    int* tot = wcnt + pw * E;
+    int* wsum = tot + E;
+    pdl_launch_dependents();
+    for (int i = tid; i < pw * E; i += blockDim.x) wcnt[i] = 0;
+    if (tid < 32) wsum[tid] = 0;
+    pdl_wait();
+    if (warp < M) {
+        const float* row = logits + static_cast<size_t>(warp) * E;
+        uint32_t key[NK];
+#pragma unroll
+        for (int j = 0; j < NK; ++j) key[j] = (lane + 32 * j < E) ? route_key(row[lane + 32 * j]) : 0u;
+        float mine0 = 0.f, mine1 = 0.f, top = 0.f;          // logits selected in rounds lane and lane + 32 (k <= 64)
+        for (int s = 0; s < k; ++s) {
+            uint32_t bk = 0u;
+            int bj = 0;
+#pragma unroll
+            for (int j = 0; j < NK; ++j)
+                if (key[j] > bk) { bk = key[j]; bj = j; }
+            const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, bk);
+            const int wi = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, static_cast<uint32_t>(bk == wk ? lane + 32 * bj : 0x7FFFFFFF)));
+#pragma unroll
+            for (int j = 0; j < NK; ++j)
+                if (wi == lane + 32 * j) key[j] = 0u;
+            const float v = route_unkey(wk);
+            if (s == 0) top = v;
+            if (s == lane) mine0 = v;
+            if (s == lane + 32) mine1 = v;
+            if (lane == 0) {
+                expert[warp * k + s] = wi;
+                topk_idx[warp * k + s] = wi;
+            }
+        }
+        // softmax over the k selected logits, summed as route_topk_kernel sums
+        float part = 0.f;
+        if (lane < k) part += expf(mine0 - top);
+        if (lane + 32 < k) part += expf(mine1 - top);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, off);
+        if (lane < k) topk_w[warp * k + lane] = expf(mine0 - top) / part;
+        if (lane + 32 < k) topk_w[warp * k + lane + 32] = expf(mine1 - top) / part;
+    }
+    __syncthreads();
+    const bool valid = tid < M * k;
+    const int e = valid ? expert[tid] : E + lane;
+    const uint32_t same = __match_any_sync(0xFFFFFFFFu, e);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (valid && rank == 0) wcnt[warp * E + e] = __popc(same);
+    __syncthreads();
+    int total = 0;
+    if (tid < E) {                               // exclusive prefix over the pair warps, in place
+        for (int w = 0; w < pw; ++w) {
+            const int c = wcnt[w * E + tid];
+            wcnt[w * E + tid] = total;
+            total += c;
+        }
+        counts[tid] = total;
+    }
+    int inc = total;                             // offsets: exclusive prefix of the totals over the experts
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int u = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if (lane >= off) inc += u;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < nwarps; ++w) {
+        if (32 * w >= E) break;
+        if (w < warp) before += wsum[w];
+    }
+    if (tid < E) {
+        const int o = before + inc - total;
+        offsets[tid] = o;
+        tot[tid] = o;
+        if (tid == E - 1) offsets[E] = o + total;
+    }
+    __syncthreads();
+    if (valid) {
+        const int pos = tot[e] + wcnt[warp * E + e] + rank;
+        row_pair[pos] = tid;
+        pair_row[tid] = pos;
+    }
+}
+
+// Xperm[pair_row[t k + s], :] = X[t, :]: one block per token, which reads its row once and writes it k times (a row-major
+// gather reads it k times from L2: 2048 tokens x 2048, eight rows each 13.7 us, 8192 tokens
+// 68; here 9.8 and 49).
+__global__ void __launch_bounds__(256)
+permute_tokens_kernel(int k, int H8, const int4* __restrict__ X, const int32_t* __restrict__ pair_row, int4* __restrict__ Xp) {
+    const int t = blockIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    const int32_t* rows = pair_row + static_cast<size_t>(t) * k;
+    for (int v = threadIdx.x; v < H8; v += blockDim.x) {
+        const int4 x = __ldg(X + static_cast<size_t>(t) * H8 + v);
+        for (int s0 = 0; s0 < k; s0 += 8) {
+            int row[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) row[j] = (s0 + j < k) ? rows[s0 + j] : -1;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (row[j] >= 0) Xp[static_cast<size_t>(row[j]) * H8 + v] = x;
+        }
+    }
+}
+
 // Xperm[r, :] = X[row_pair[r] / k, :]; one warp per row, 16-byte vectors.
 __global__ void __launch_bounds__(256)
 permute_rows_kernel(int R, int k, int H8, const int4* __restrict__ X, const int32_t* __restrict__ row_pair,
@@ -327,6 +450,21 @@ static int route_impl(qg_ctx* ctx, int M, int E, int k, const float* logits, int
         }
         return QG_OK;
     }
+    const auto permute = [&]() {
+        if (!gather) return static_cast<int>(QG_OK);
+        return qg::launch_rc(qg::launch_kernel(ctx, qg::permute_tokens_kernel, dim3(M), dim3(256), 0, st, k, H / 8,
+                                               static_cast<const int4*>(X), static_cast<const int32_t*>(pair_row),
+                                               static_cast<int4*>(Xperm)));
+    };
+    if (M <= 32 && M * k <= 1024 && k <= 64 && E <= 256) {
+        const auto kern = (E <= 128) ? qg::route_small_kernel<4> : qg::route_small_kernel<8>;
+        const int pw = (M * k + 31) / 32, ew = (E + 31) / 32;
+        const size_t smem = (32 * static_cast<size_t>(pw) + static_cast<size_t>(pw) * E + E + 32) * sizeof(int);
+        const int warps = max(M, max(pw, ew));
+        const int rc = qg::launch_rc(qg::launch_kernel(ctx, kern, dim3(1), dim3(32 * warps), smem, st, M, E, k, logits, topk_idx,
+                                                       topk_w, expert_counts, expert_offsets, row_pair, pair_row));
+        return rc != QG_OK ? rc : permute();
+    }
     // one token per warp when 32 warps' rows fit in 64 KB of shared memory, else 8 warps take 4 tokens each
     const int topk_warps = (32 * static_cast<size_t>(E + k) * sizeof(float) <= 64 * 1024) ? 32 : qg::ROUTE_WARPS;
     const size_t sm_topk = (static_cast<size_t>(topk_warps) * (E + k) + E) * sizeof(float);
@@ -350,8 +488,7 @@ static int route_impl(qg_ctx* ctx, int M, int E, int k, const float* logits, int
                                              static_cast<const int32_t*>(expert_offsets),
                                              static_cast<const int32_t*>(hist), row_pair, pair_row));
     if (rc != QG_OK) return rc;
-    if (gather) return moe_permute(ctx, M, k, H, X, row_pair, Xperm, stream);
-    return QG_OK;
+    return permute();
 }
 
 static int route_check(qg_ctx* ctx, int M, int E, int k, const float* logits, int32_t* topk_idx, float* topk_w,

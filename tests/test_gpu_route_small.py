@@ -1,0 +1,69 @@
+"""Routing and router projection of a small batch (one block for the whole of routing, a block per expert for the projection),
+at the edges of the sizes they serve, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2607_19438_b200 import binding as qg, synth
+from tests import util
+
+pytestmark = pytest.mark.gpu
+
+
+# one token, the most tokens, pairs that fill the last warp or not, one expert, experts around the register groups of 128 and
+# 256, every expert selected, the most slots, and just outside (33 tokens, 65 slots, 257 experts)
+CASES = [(1, 1, 1), (1, 128, 8), (2, 5, 5), (31, 127, 8), (32, 128, 8), (32, 129, 32), (16, 256, 64), (3, 64, 64), (7, 33, 33),
+         (32, 8, 2), (33, 128, 8), (4, 128, 65), (5, 257, 4)]
+
+
+@pytest.mark.parametrize("kind", ["plain", "ties", "extremes"])
+@pytest.mark.parametrize("M,E,k", CASES, ids=lambda v: str(v))
+def test_route(M, E, k, kind):
+    rng = np.random.default_rng(M * 1000 + E + k)
+    logits = rng.standard_normal((M, E)).astype(np.float32)
+    if kind == "ties":
+        logits = np.round(logits * 2) / 2 * np.where(rng.random((M, E)) < 0.2, -0.0, 1.0).astype(np.float32)
+    elif kind == "extremes":
+        pool = np.array([3.0e38, -3.0e38, 1.0e-45, -1.0e-45, 0.0, -0.0, 1.5, -np.inf], np.float32)
+        logits = pool[rng.integers(0, pool.size, (M, E))]
+        logits[:, 0] = 2.0
+    H = 136
+    X = synth.activations(M, H, seed=3)
+    r = qg.moe_route(util.dev(logits), k, X=util.dev_bf16(X))
+    qg.poll_status()
+    idx, w, _ = orc.route(logits, k)
+    counts, offsets = orc.counts_offsets(idx, E)
+    row_pair, pair_row = orc.permutation(idx, offsets)
+    for name, ref in (("topk_idx", idx), ("counts", counts), ("offsets", offsets), ("row_pair", row_pair), ("pair_row", pair_row)):
+        assert np.array_equal(r[name].cpu().numpy().reshape(ref.shape), ref), name
+    assert np.max(np.abs(r["topk_w"].cpu().numpy().astype(np.float64) - w)) <= util.TOPK_W_ATOL
+    assert np.array_equal(util.host_bf16_bits(r["Xperm"]), orc.permute(X, row_pair, k))
+
+
+def test_nan_logits_route_as_in_a_larger_batch():
+    """NaN sorts after every number: the first 32 of 40 tokens, routed alone, select what they select in the batch."""
+    rng = np.random.default_rng(8)
+    logits = rng.standard_normal((40, 64)).astype(np.float32)
+    logits[rng.random((40, 64)) < 0.9] = np.nan
+    a, b = qg.moe_route(util.dev(logits), 8), qg.moe_route(util.dev(logits[:32].copy()), 8)
+    assert torch.equal(a["topk_idx"][:32], b["topk_idx"])
+    assert torch.equal(a["topk_w"][:32].view(torch.int32), b["topk_w"].view(torch.int32))
+
+
+@pytest.mark.parametrize("M,H,E", [(1, 64, 1), (8, 2048, 128), (9, 2112, 130), (96, 512, 64), (97, 512, 64), (32, 4096, 1000)], ids=lambda v: str(v))
+def test_router_logits(M, H, E):
+    xb, wb = synth.activations(M, H, seed=M, tid=41), synth.activations(E, H, seed=H, tid=42)
+    g = util.Guarded((M, E), torch.float32)
+    dx, dw = util.dev_bf16(xb), util.dev_bf16(wb)
+    qg.moe_router_logits(dx, dw, out=g.t)
+    again = qg.moe_router_logits(dx, dw)
+    qg.poll_status()
+    assert g.intact() and not bool(g.untouched_inside().any().item()) and torch.equal(again, g.t)
+    ref = orc.router_logits(orc.bf16_to_f64(xb), orc.bf16_to_f64(wb))
+    # every product is exact; a sum of H terms in fp32, 8 per thread and then pairwise, is off by under 16 roundings of sum |x w|
+    bound = 16 * 2.0 ** -24 * orc.router_logits(np.abs(orc.bf16_to_f64(xb)), np.abs(orc.bf16_to_f64(wb))) + 1e-30
+    if M <= 96:
+        assert np.all(np.abs(g.t.cpu().numpy().astype(np.float64) - ref) <= bound * max(1, H // 2048))
+    else:
+        assert util.errors(g.t.cpu().numpy(), ref)[2] < 1e-5
