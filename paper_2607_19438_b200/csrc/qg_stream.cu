@@ -171,9 +171,12 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     uint8_t* after = ms_smem + (ring - smem_u32(ms_smem)) + p.n_stages * p.stage_bytes;
     const uint32_t xch = smem_u32(after);              // [4 warps][NTM][MT][32 lanes] float4: sums handed from set to set, or of the slice
     after += 4 * NTM * MT * 512;
-    const uint32_t full0 = smem_u32(after), empty0 = full0 + 8u * MS_MAX_ST, xfull0 = empty0 + 8u * MS_MAX_ST;
+    // full: stage i's barrier is number i mod 2 n_stages (twice the slots), so that one set waits on it every time it is used:
+    // with one barrier per slot and an odd number of slots a set would see every other phase only, and a wait by parity
+    // passes too early while the phase in between is not complete.
+    const uint32_t full0 = smem_u32(after), empty0 = full0 + 16u * MS_MAX_ST, xfull0 = empty0 + 8u * MS_MAX_ST;
     const uint32_t hfull0 = xfull0 + 8u * MS_MAX_ST, hempty0 = hfull0 + 32u;      // the hand-over of each pair of warps
-    after += 24 * MS_MAX_ST + 64;
+    after += 32 * MS_MAX_ST + 64;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(after);
     volatile StreamTile* tiles = reinterpret_cast<volatile StreamTile*>(after + 16);   // per stage: the tile it belongs to
     int* off = reinterpret_cast<int*>(after + 16 + 16 * MS_MAX_ST);      // grouped: [E + 1] segment offsets
@@ -181,7 +184,8 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pdl_launch_dependents();
     if (warp == 0) {
-        if (lane < p.n_stages) { mbar_init(full0 + 8u * lane, 2); mbar_init(empty0 + 8u * lane, MS_CONS_WARPS / 2); mbar_init(xfull0 + 8u * lane, 1); }
+        if (lane < 2 * p.n_stages) mbar_init(full0 + 8u * lane, 2);
+        if (lane < p.n_stages) { mbar_init(empty0 + 8u * lane, MS_CONS_WARPS / 2); mbar_init(xfull0 + 8u * lane, 1); }
         if (lane >= 16 && lane < 24) mbar_init(hfull0 + 8u * (lane - 16), 1);
         if (lane == 31) *abort_flag = 0;
         fence_mbar_init();
@@ -222,12 +226,12 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     if (warp == MS_CONS_WARPS) {
         // ------------------------------------------------ producer
         if (lane == 0) {
-            uint32_t slot = 0, phase = 0;
+            uint32_t slot = 0, phase = 0, fslot = 0;
             int sent = 0, ahead = 0;                   // stages filled, stages whose weights are on their way
             const int skip = (blockIdx.x == 0 && blockIdx.y == 0) ? p.skip_stage : -1;
             bool ok = true;
-            auto load_weights = [&](uint32_t at, int st, const StreamTile& tl) {
-                const uint32_t dst = ring + at * p.stage_bytes, bar = full0 + 8u * at;
+            auto load_weights = [&](uint32_t at, uint32_t bar, int st, const StreamTile& tl) {
+                const uint32_t dst = ring + at * p.stage_bytes;
                 mbar_arrive_expect_tx(bar, MS_W_BYTES + ms_s_bytes(QBITS));
                 if constexpr (GATE_UP) {
                     tma_load_3d(dst, &tm_w, st * 128, tl.wt * 64, 2 * tl.e, bar);
@@ -241,7 +245,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             };
             if (!GROUPED) {
                 const StreamTile tl{0, static_cast<int>(blockIdx.x), 0, p.R};
-                for (; ahead < min(nst, p.n_stages); ++ahead) load_weights(ahead, ahead, tl);
+                for (; ahead < min(nst, p.n_stages); ++ahead) load_weights(ahead, full0 + 8u * ahead, ahead, tl);
                 pdl_wait();
             }
             for (int t = blockIdx.x; ok; ) {
@@ -274,15 +278,16 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     d->e = tl.e; d->wt = tl.wt; d->tok0 = tl.tok0; d->n = tl.n;
                     if (tl.n == 0) {
                         mbar_arrive(xbar);
-                        mbar_arrive(full0 + 8u * slot);
+                        mbar_arrive(full0 + 8u * fslot);
                     } else {
                         mbar_arrive_expect_tx(xbar, nt * MS_X_BYTES);
                         if (sent != skip)
                             for (int i = 0; i < nt; ++i)
                                 tma_load_3d(ring + slot * p.stage_bytes + OFF_X + i * MS_X_BYTES, &tm_x, 0, tl.tok0 + 8 * i, k0 / 32 + st * 8, xbar);
-                        if (sent >= ahead) load_weights(slot, st, tl);
+                        if (sent >= ahead) load_weights(slot, full0 + 8u * fslot, st, tl);
                     }
                     if (++slot == static_cast<uint32_t>(p.n_stages)) { slot = 0; phase ^= 1u; }
+                    if (++fslot == 2u * p.n_stages) fslot = 0;
                 }
                 if (tl.n == 0) break;
                 t = next;
@@ -291,7 +296,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     } else if (warp == MS_CONS_WARPS + 1) {
         // ------------------------------------------------ token rows: every 32-block into the order of q4_spread (a lane's eight
         // k as 0, 2, 4, 6, 1, 3, 5, 7) or q8_spread (four k of each half of the block, each as 0, 2, 1, 3), in place
-        uint32_t slot = 0, phase = 0;
+        uint32_t slot = 0, phase = 0, fslot = 0;
         int ends = 0;
         const int g = lane >> 2, j = lane & 3;
         while (ends < 2 && __all_sync(0xFFFFFFFFu, ms_wait(xfull0 + 8u * slot, phase, abort_flag, p))) {
@@ -319,8 +324,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
             fence_proxy_async_smem();              // the slot's next load comes after these writes
             __syncwarp();
-            if (lane == 0) mbar_arrive(full0 + 8u * slot);
+            if (lane == 0) mbar_arrive(full0 + 8u * fslot);
             if (++slot == static_cast<uint32_t>(p.n_stages)) { slot = 0; phase ^= 1u; }
+            if (++fslot == 2u * p.n_stages) fslot = 0;
         }
     } else {
         // ------------------------------------------------ consumers: two sets of four warps, set 0 takes the even stages and
@@ -333,7 +339,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         const uint32_t sc0 = ring + OFF_S + row * 16;
         const uint32_t x0 = ring + OFF_X + lane * 16;
         const uint32_t my_xch = xch + (w4 * NTM * MT * 32 + lane) * 16, hfull = hfull0 + 8u * w4, hempty = hempty0 + 8u * w4;
-        uint32_t slot = set, phase = 0;
+        uint32_t slot = set, fslot = set, fphase = 0;
         float wl = 0.f;                       // routing weight of row `lane` of the chunk
         int have = -1;                        // first row of the chunk wl belongs to
         for (uint32_t q = 0, base = 0; ; ++q, base += nst) {              // tile and its first stage, both counted from 0
@@ -342,7 +348,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 if (sliced) break;
                 continue;
             }
-            if (!__all_sync(0xFFFFFFFFu, ms_wait(full0 + 8u * slot, phase, abort_flag, p))) break;
+            if (!__all_sync(0xFFFFFFFFu, ms_wait(full0 + 8u * fslot, fphase, abort_flag, p))) break;
             const int wt = tiles[slot].wt, tok0 = tiles[slot].tok0, n = tiles[slot].n;
             if (n == 0) break;
             const int nt_n = (n + 7) >> 3;
@@ -358,7 +364,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 for (int e = 0; e < 4 * MT; ++e) acc[nt][e >> 2][e & 3] = 0.f;
             bool ok = true;
             for (uint32_t st = first; st < base + nst; st += 2) {
-                ok = __all_sync(0xFFFFFFFFu, ms_wait(full0 + 8u * slot, phase, abort_flag, p));
+                ok = __all_sync(0xFFFFFFFFu, ms_wait(full0 + 8u * fslot, fphase, abort_flag, p));
                 if (!ok) break;
                 const uint32_t o = slot * p.stage_bytes;
                 if (NTM == 1 || nt_n == 1) ms_stage<QBITS, 1, HI, STEP>(acc, wl0 + o, x0 + o, sc0 + o);
@@ -366,7 +372,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty0 + 8u * slot);
                 slot += 2;
-                if (slot >= static_cast<uint32_t>(p.n_stages)) { slot -= p.n_stages; phase ^= 1u; }
+                if (slot >= static_cast<uint32_t>(p.n_stages)) slot -= p.n_stages;
+                fslot += 2;
+                if (fslot >= 2u * p.n_stages) { fslot -= 2u * p.n_stages; fphase ^= 1u; }
             }
             if (!ok) break;
             if (nst > 1 && !mine) {           // hand the sums to the other set's warp of the same rows
@@ -470,13 +478,10 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 // Ring depth and shared memory of a launch; false if not even two stages fit.
 static bool ms_layout(StreamParams& p, int qbits, int ntm, int n_exp, size_t& smem) {
     p.stage_bytes = (MS_W_BYTES + ms_s_bytes(qbits) + ntm * MS_X_BYTES + 1023) & ~1023;      // the codes' swizzle wants 1 KB
-    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + 24 * MS_MAX_ST + 64 + 16 + 16 * MS_MAX_ST +
+    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + 32 * MS_MAX_ST + 64 + 16 + 16 * MS_MAX_ST +
                          (2 * static_cast<size_t>(n_exp) + 2) * sizeof(int);
     p.n_stages = static_cast<int>((MS_SMEM_MAX - fixed) / p.stage_bytes);
     if (p.n_stages > MS_MAX_ST) p.n_stages = MS_MAX_ST;
-    // An even number, so that a slot's stages all belong to one set: with an odd one a set would see every other phase of a
-    // slot's barrier only, and a wait by parity passes too early when the phase in between is not complete yet.
-    p.n_stages &= ~1;
     smem = fixed + static_cast<size_t>(p.n_stages) * p.stage_bytes;
     return p.n_stages >= 2;
 }
