@@ -140,7 +140,7 @@ def test_inject(wait_limit_polls: int = 0, skip_kblock: int = -1):
 
 
 def test_gemv_mode(mode: int = 0):
-    """Testing hook: kernel choice of qgemm_small_m (bit 0 no clusters, bit 1 always the ring kernel, bit 2 never)."""
+    """Testing hook: kernel choice of qgemm_small_m (bit 0 no clusters, bit 1 always the streaming kernel, bit 2 never)."""
     _check(load().qg_test_gemv_mode(context(), mode), "qg_test_gemv_mode")
 
 

@@ -1059,29 +1059,30 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
         GemmParams whole = p;
         whole.slices = 1;
         return launch_gemm<QBITS, BT, EPI, 0>(ctx, whole, X, x_rows, Wq, Ws, st);
-    }
-    auto kern = qgemm_kernel<QBITS, BT, EPI, SK>;
-    // the shared-memory attribute belongs to the function on one device: set once per context and instantiation
-    constexpr int inst = SK == 1 ? ATTR_GEMM_SK + ((QBITS == 4) ? 3 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 1 : 2)
-                            : ATTR_GEMM + ((QBITS == 4) ? 9 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 3 : 6) + EPI;
-    if (!ctx->attr_set[inst]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess) {
+    } else {
+        auto kern = qgemm_kernel<QBITS, BT, EPI, SK>;
+        // the shared-memory attribute belongs to the function on one device: set once per context and instantiation
+        constexpr int inst = SK == 1 ? ATTR_GEMM_SK + ((QBITS == 4) ? 3 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 1 : 2)
+                                : ATTR_GEMM + ((QBITS == 4) ? 9 : 0) + ((BT == 128) ? 0 : (BT == 192) ? 3 : 6) + EPI;
+        if (!ctx->attr_set[inst]) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess) {
+                cudaGetLastError();
+                return QG_ERR_CUDA;
+            }
+            ctx->attr_set[inst] = true;
+        }
+        // Upper bound on the number of pair tiles (the exact count lives on the device for grouped calls).
+        long long max_tiles =
+            (static_cast<long long>((p.R + BT - 1) / BT) + (p.offsets ? p.E : 0)) * ((p.n_wt + 1) / 2);
+        if (p.streamk) max_tiles *= p.K / (4 * BK);      // units of four k-blocks: every pair gets at least one
+        const long long pairs_hw = ctx->sm_count / 2;
+        const int grid = 2 * static_cast<int>(max_tiles < pairs_hw ? max_tiles : pairs_hw);
+        if (launch_kernel(ctx, kern, dim3(grid), dim3(NTHREADS), C::SMEM_BYTES, st, tm_x, tm_w, tm_s, p) != cudaSuccess) {
             cudaGetLastError();
             return QG_ERR_CUDA;
         }
-        ctx->attr_set[inst] = true;
+        return QG_OK;
     }
-    // Upper bound on the number of pair tiles (the exact count lives on the device for grouped calls).
-    long long max_tiles =
-        (static_cast<long long>((p.R + BT - 1) / BT) + (p.offsets ? p.E : 0)) * ((p.n_wt + 1) / 2);
-    if (p.streamk) max_tiles *= p.K / (4 * BK);      // units of four k-blocks: every pair gets at least one
-    const long long pairs_hw = ctx->sm_count / 2;
-    const int grid = 2 * static_cast<int>(max_tiles < pairs_hw ? max_tiles : pairs_hw);
-    if (launch_kernel(ctx, kern, dim3(grid), dim3(NTHREADS), C::SMEM_BYTES, st, tm_x, tm_w, tm_s, p) != cudaSuccess) {
-        cudaGetLastError();
-        return QG_ERR_CUDA;
-    }
-    return QG_OK;
 }
 
 // Token tile and schedule of a dense call: the candidate with the smallest modelled time, the model fitted to timings
