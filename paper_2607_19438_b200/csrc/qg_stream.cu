@@ -238,8 +238,8 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     tma_load_3d(dst + OFF_S, &tm_s, st * 8, tl.wt * 64, 2 * tl.e, bar);
                 } else {
                     const int row = tl.e * p.N + tl.wt * ROWS, ks = k0 / MS_SK + st;
-                    tma_load_2d(dst, &tm_w, ks * (MS_SK * QBITS / 8), row, bar);
-                    if (QBITS == 8) tma_load_2d(dst + MS_W_BYTES / 2, &tm_w, ks * MS_SK + 128, row, bar);
+                    if (QBITS == 8) tma_load_3d(dst, &tm_w, 0, row, 2 * ks, bar);
+                    else tma_load_2d(dst, &tm_w, ks * 128, row, bar);
                     tma_load_2d(dst + OFF_S, &tm_s, ks * 8, row, bar);
                 }
             };
@@ -590,8 +590,11 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb;
     CUtensorMap tm_w, tm_s, tm_x;
-    rc = get_tmap_2d(ctx, &tm_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, static_cast<uint64_t>(K) * qbits / 8, N, 128, rows,
-                     CU_TENSOR_MAP_SWIZZLE_128B);
+    // 8-bit codes as [K / 128][N][128]: both halves of a stage are one box (an instruction less per stage for the producer)
+    rc = (qbits == 8) ? get_tmap_3d(ctx, &tm_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, 128, N, K / 128, 128, 128, rows, 2,
+                                    CU_TENSOR_MAP_SWIZZLE_128B, static_cast<uint64_t>(K))
+                      : get_tmap_2d(ctx, &tm_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, static_cast<uint64_t>(K) / 2, N, 128, rows,
+                                    CU_TENSOR_MAP_SWIZZLE_128B);
     if (rc == QG_OK) rc = get_tmap_2d(ctx, &tm_s, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, Ws, K / 32, N, 8, rows, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (rc == QG_OK)
         rc = get_tmap_3d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, A, 32, M, K / 32, 64, 32, 8, 8, CU_TENSOR_MAP_SWIZZLE_NONE,
