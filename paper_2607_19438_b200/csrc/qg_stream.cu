@@ -485,6 +485,11 @@ static bool ms_layout(StreamParams& p, int qbits, int ntm, int n_exp, size_t& sm
     smem = fixed + static_cast<size_t>(p.n_stages) * p.stage_bytes;
     return p.n_stages >= 2;
 }
+// Tile counters of a launch: zero, and left zero by the launch.  Expert GEMMs on several streams overlap, so a launch does not
+// get the pair that one of the 63 before it got.
+static int* ms_counters(qg_ctx* ctx) {
+    return ctx->gemv_tickets + ctx->gemv_ticket_count + 2 * (ctx->sched_next++ % SCHED_SLOTS);
+}
 using StreamKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const StreamParams);
 static int ms_set_smem(qg_ctx* ctx, StreamKernel kern, int inst) {
     if (ctx->attr_set[inst]) return QG_OK;
@@ -512,7 +517,7 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     if (!ms_layout(p, 4, ntm, E, smem)) return QG_ERR_WORKSPACE;
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
     p.topk_w = (mode == QG_MODE_DOWN_WEIGHTED) ? topk_w : nullptr; p.row_pair = row_pair;
-    p.sched = ctx->gemv_tickets + ctx->gemv_ticket_count;
+    p.sched = ms_counters(ctx);
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb < 0 ? -1 : ctx->skip_kb / (MS_SK / 64);
     CUtensorMap tm_w, tm_s, tm_x;
@@ -586,7 +591,7 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     }
     p.R = M; p.N = N; p.K = K; p.E = 0; p.kc = kc; p.n_wt = tiles;
     p.out = static_cast<__nv_bfloat16*>(Cout);
-    p.sched = ctx->gemv_tickets + ctx->gemv_ticket_count;
+    p.sched = ms_counters(ctx);
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb;
     CUtensorMap tm_w, tm_s, tm_x;

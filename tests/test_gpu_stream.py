@@ -133,3 +133,19 @@ def test_an_infinite_token_gives_infinities_of_the_codes_signs():
     assert torch.equal(out[[0, 2]], clean[[0, 2]])
     q = Wq[:, 500].astype(np.int64) * np.sign(Ws[:, 500 // 32].view(np.float16).astype(np.float64))
     assert np.array_equal(out[1].float().cpu().numpy()[q != 0], -np.sign(q[q != 0]) * np.inf)
+
+
+def test_expert_gemms_on_two_streams_at_once():
+    """Launches that overlap take their tiles from counters of their own."""
+    counts, N, K = [3, 7, 1, 12, 0, 5] * 8, 1536, 1024
+    offsets, A, Wq, Ws = problem(counts, N, K, 9)
+    args = (util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
+    want = qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args)
+    streams, outs = [torch.cuda.Stream(), torch.cuda.Stream()], []
+    torch.cuda.synchronize()
+    for i in range(40):
+        with torch.cuda.stream(streams[i % 2]):
+            outs.append(qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args))
+    torch.cuda.synchronize()
+    qg.poll_status()
+    assert all(torch.equal(o, want) for o in outs)
