@@ -212,10 +212,9 @@ router_small_kernel(int M, int H8, int E, const uint4* __restrict__ X, const uin
     float acc[RS_TOK];
 #pragma unroll
     for (int i = 0; i < RS_TOK; ++i) acc[i] = 0.f;
-    bool waited = false;
+    pdl_wait();                                  // X and Wr are bf16 rows as this library's other calls write them: both may be fresh
     for (int v = threadIdx.x; v < H8; v += 256) {
-        const uint4 w = __ldg(Wr + static_cast<size_t>(e) * H8 + v);       // the router's weights are constants of the model
-        if (!waited) { pdl_wait(); waited = true; }
+        const uint4 w = __ldg(Wr + static_cast<size_t>(e) * H8 + v);
         uint4 x[RS_TOK];
 #pragma unroll
         for (int i = 0; i < RS_TOK; ++i) x[i] = (i < n) ? X[static_cast<size_t>(t0 + i) * H8 + v] : make_uint4(0u, 0u, 0u, 0u);
@@ -230,7 +229,6 @@ router_small_kernel(int M, int H8, int E, const uint4* __restrict__ X, const uin
             }
         }
     }
-    if (!waited) pdl_wait();
 #pragma unroll
     for (int i = 0; i < RS_TOK; ++i) {
 #pragma unroll

@@ -67,3 +67,25 @@ def test_router_logits(M, H, E):
         assert np.all(np.abs(g.t.cpu().numpy().astype(np.float64) - ref) <= bound * max(1, H // 2048))
     else:
         assert util.errors(g.t.cpu().numpy(), ref)[2] < 1e-5
+
+
+@pytest.mark.parametrize("M,H,E", [(1, 64, 8), (8, 2048, 128), (96, 1024, 64), (97, 1024, 64)], ids=lambda v: str(v))
+def test_router_weights_written_by_the_call_before(M, H, E):
+    """The router's weights are the output of a GEMM queued on the stream just before: the projection waits for it."""
+    A, Wq, Ws = synth.dense_problem(8, E, H, 8192, seed=12)
+    dA, dWq, dWs = util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws)
+    x = util.dev_bf16(synth.activations(M, H, seed=M, tid=43))
+    want_w = qg.qgemm_dense(8, dA, dWq, dWs)
+    want = qg.moe_router_logits(x, want_w)
+    qg.poll_status()
+    wr, outs = torch.zeros_like(want_w), []
+    for _ in range(10):
+        wr.zero_()
+        qg.qgemm_dense(8, dA, dWq, dWs, out=wr)
+        outs.append((qg.moe_router_logits(x, wr), wr.clone()))
+    qg.poll_status()
+    for logits, w in outs:                       # stream-K sums of the GEMM may differ in their last bit: compare with the weights of that pass
+        ref = x.double() @ w.double().T
+        assert float((logits.double() - ref).norm() / ref.norm()) < 1e-5
+    ref = x.double() @ want_w.double().T
+    assert float((want.double() - ref).norm() / ref.norm()) < 1e-5
