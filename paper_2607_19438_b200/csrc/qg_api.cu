@@ -65,8 +65,8 @@ int qg_create(qg_ctx** out, int device) {
         cudaMalloc(&ctx->sk_flags, sizeof(int) * 2 * ctx->sm_count) != cudaSuccess ||
         cudaMemset(ctx->sk_flags, 0, sizeof(int) * 2 * ctx->sm_count) != cudaSuccess ||
         cudaMalloc(&ctx->gemv_partial, ctx->gemv_partial_bytes) != cudaSuccess ||
-        cudaMalloc(&ctx->gemv_tickets, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS)) != cudaSuccess ||
-        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS)) != cudaSuccess) {
+        cudaMalloc(&ctx->gemv_tickets, sizeof(int) * ctx->gemv_ticket_count) != cudaSuccess ||
+        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * ctx->gemv_ticket_count) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_status); cudaFree(ctx->gemv_partial); cudaFree(ctx->gemv_tickets);
         cudaFree(ctx->sk_partial); cudaFree(ctx->sk_flags);
@@ -99,7 +99,7 @@ int qg_poll_status(qg_ctx* ctx, void* stream) {
         // next launch starts clean
         cudaMemset(ctx->d_status, 0, sizeof(int));
         cudaMemset(ctx->sk_flags, 0, sizeof(int) * 2 * ctx->sm_count);
-        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * (ctx->gemv_ticket_count + qg::SCHED_INTS));
+        cudaMemset(ctx->gemv_tickets, 0, sizeof(int) * ctx->gemv_ticket_count);
     }
     return host;
 }

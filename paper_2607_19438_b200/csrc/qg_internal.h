@@ -21,8 +21,6 @@ struct TmapEntry {
 };
 constexpr int TMAP_CACHE = 2048, TMAP_WAYS = 8;   // entries, entries per hashed set
 constexpr uint32_t DEFAULT_WAIT_LIMIT = 1u << 18;   // polls; an unsatisfied try_wait poll lasts about 4 us: about a second
-constexpr int SCHED_SLOTS = 64, SCHED_INTS = 2 * SCHED_SLOTS;   // tile counters after the gemv tickets: a pair per launch, taken in turn,
-                                                  // so that launches that overlap on the GPU do not share one
 // Slots of qg_ctx::attr_set, one per kernel instantiation that needs the dynamic shared-memory attribute.
 enum AttrSlot {
     ATTR_GEMM = 0,          // 18 slots: format (2) x token tile (3) x epilogue (3)
@@ -59,10 +57,8 @@ struct qg_ctx {
     int streamk_mode;          // QG_STREAMK at creation: -1 heuristic (default), 0 never, 1 whenever legal
     float* gemv_partial;       // K-slice partial sums of qgemm_small_m's block kernel, [slices][16][N] fp32
     size_t gemv_partial_bytes;
-    int* gemv_tickets;         // one arrival counter per 64-row tile, then the tile counters of the streaming kernel;
-                               // zero between launches
+    int* gemv_tickets;         // one arrival counter per 64-row tile, zero between launches
     int gemv_ticket_count;
-    unsigned sched_next;       // pair of tile counters the next launch takes
     int slice_clusters[4][5];      // dense GEMM with K slices, per format x token tile and slices: clusters that fit at once (0 unknown, -1 none)
     int gemv_mode;             // test hook (qg_test_gemv_mode): bit 0 no clusters, bit 1 always the streaming kernel, bit 2 never
     int gemv_max_clusters[4][9];   // streaming kernel, per instantiation and cluster size: clusters that fit at once (0 unknown, -1 none)

@@ -100,6 +100,26 @@ __device__ __forceinline__ void cluster_sync_all() {   // every thread of both C
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Cluster launch control: asks the hardware for a block of this grid that has not been started; the 16-byte answer arrives at
+// `answer` (shared memory) and completes 16 bytes on `bar`.  No request may follow one that was refused.
+__device__ __forceinline__ void clc_try_cancel(uint32_t answer, uint32_t bar) {
+    asm volatile("fence.proxy.async.shared::cta;\n\t"          // the answer before was read through the generic proxy
+                 "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
+}
+// The answer: the x index of the block that is this CTA's now, or false (all blocks have been started or taken).
+__device__ __forceinline__ bool clc_block(uint32_t answer, uint32_t& x) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .b128 a;\n\t.reg .pred p;\n\t"
+        "ld.shared.b128 a, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n\t}"
+        : "=r"(ok), "=r"(x) : "r"(answer) : "memory");
+    return ok != 0;
+}
+
 // Generic-proxy writes to shared memory -> visible to the async proxy (TMA, tcgen05.mma operands).
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

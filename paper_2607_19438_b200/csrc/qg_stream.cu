@@ -13,8 +13,10 @@
 // shared memory was the limit; 8-bit codes are twice the bytes per MMA).  The set with a tile's last stage adds the
 // other's sums and writes the result.  In gate/up mode an MMA tile is eight gate rows and the eight up rows that belong
 // to them: a thread ends up with both values of its outputs.
-//   Grouped, or more tiles than CTAs: tile after tile comes from a counter in global memory (dealt out beforehand, the
-// tiles left an SM up to 16 % more than its share: nine tiles are too few to round).
+//   More tiles than CTAs fit: the grid has a block per tile, and a CTA that is done with its tile takes over the tile of a block
+// that has not been started (cluster launch control; dealt out beforehand, the tiles left an SM up to 16 % more than its
+// share: nine tiles are too few to round).  The hardware keeps the count, nothing outlives the launch, so launches may
+// overlap on the GPU in any way.
 //   One matrix with fewer tiles: K is cut into slices, the slices of a tile are a thread-block cluster, and the cluster adds
 // its sums through distributed shared memory in slice order.  All sums have a fixed order: results are reproducible.
 //
@@ -69,8 +71,7 @@ struct StreamParams {
     int n_wt;                   // weight tiles per expert (gate/up mode: 64 gate + 64 up rows each)
     int n_stages, stage_bytes;
     int kc;                     // k per CTA: K, or a slice of it when the CTAs of a cluster share a tile
-    int dynamic;                // more tiles than CTAs: the next tile comes from the counter
-    int* sched;                 // [0] tiles taken beyond the first of each CTA, [1] CTAs that are done; zero between launches
+    int dynamic;                // more blocks than fit at once: a CTA goes on with the tiles of blocks not yet started
     const int32_t* offsets;     // grouped: device expert offsets [E + 1]
     __nv_bfloat16* out;
     const float* topk_w;        // grouped: routing weights, applied to the rows named by row_pair (nullptr: none)
@@ -159,7 +160,7 @@ __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(
 // tm_w: packed codes, box 128 bytes x the tile's rows (gate/up: 64 rows x 2 planes), 128-byte swizzle; tm_s: scales, box 8 x
 // the same rows; tm_x: token rows as [K / 32][R][32], box 32 k x 8 rows x 8 blocks, so that the 16 bytes a lane of an MMA
 // fragment needs follow one another in lane order.  Rows past the end arrive as zeros.
-// grid = (tiles or fewer CTAs, K slices); the slices of a tile are one cluster.
+// grid = (tiles, K slices); the slices of a tile are one cluster.
 template <int QBITS, bool GROUPED, bool GATE_UP, int NTM>
 __global__ void __launch_bounds__(MS_THREADS, 2)
 stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
@@ -177,6 +178,8 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t full0 = smem_u32(after), empty0 = full0 + 16u * MS_MAX_ST, xfull0 = empty0 + 8u * MS_MAX_ST;
     const uint32_t hfull0 = xfull0 + 8u * MS_MAX_ST, hempty0 = hfull0 + 32u;      // the hand-over of each pair of warps
     after += 32 * MS_MAX_ST + 64;
+    const uint32_t taken = smem_u32(after), taken_bar = taken + 16;      // the hardware's answer to a request for a tile
+    after += 32;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(after);
     volatile StreamTile* tiles = reinterpret_cast<volatile StreamTile*>(after + 16);   // per stage: the tile it belongs to
     int* off = reinterpret_cast<int*>(after + 16 + 16 * MS_MAX_ST);      // grouped: [E + 1] segment offsets
@@ -187,7 +190,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (lane < 2 * p.n_stages) mbar_init(full0 + 8u * lane, 2);
         if (lane < p.n_stages) { mbar_init(empty0 + 8u * lane, MS_CONS_WARPS / 2); mbar_init(xfull0 + 8u * lane, 1); }
         if (lane >= 16 && lane < 24) mbar_init(hfull0 + 8u * (lane - 16), 1);
-        if (lane == 31) *abort_flag = 0;
+        if (lane == 31) { *abort_flag = 0; mbar_init(taken_bar, 1); }
         fence_mbar_init();
         fence_proxy_async_smem();
     }
@@ -228,6 +231,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (lane == 0) {
             uint32_t slot = 0, phase = 0, fslot = 0;
             int sent = 0, ahead = 0;                   // stages filled, stages whose weights are on their way
+            uint32_t asked = 0;                        // requests for a tile so far, each a phase of taken_bar
             const int skip = (blockIdx.x == 0 && blockIdx.y == 0) ? p.skip_stage : -1;
             bool ok = true;
             auto load_weights = [&](uint32_t at, uint32_t bar, int st, const StreamTile& tl) {
@@ -250,9 +254,11 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
             for (int t = blockIdx.x; ok; ) {
                 StreamTile tl{0, 0, 0, 0};
-                int next = total;
                 if (t < total) {
-                    if (p.dynamic) next = static_cast<int>(gridDim.x) + atomicAdd(p.sched, 1);       // asked for early, used at the end of this tile
+                    if (p.dynamic) {                   // asked for early, used at the end of this tile
+                        mbar_arrive_expect_tx(taken_bar, 16);
+                        clc_try_cancel(taken, taken_bar);
+                    }
                     if constexpr (GROUPED) {
                         int lo = 0, hi = p.E - 1;            // the last expert whose tiles start at or before t
                         while (lo < hi) {
@@ -290,7 +296,18 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     if (++fslot == 2u * p.n_stages) fslot = 0;
                 }
                 if (tl.n == 0) break;
-                t = next;
+                // the block taken over, or none.  Blocks past the last tile (their number is an upper bound) are taken too, so that
+                // none of them is started.
+                t = total;
+                while (ok && p.dynamic) {
+                    ok = ms_wait(taken_bar, asked & 1u, abort_flag, p);
+                    ++asked;
+                    uint32_t block;
+                    if (!ok || !clc_block(taken, block)) break;
+                    if (block < static_cast<uint32_t>(total)) { t = static_cast<int>(block); break; }
+                    mbar_arrive_expect_tx(taken_bar, 16);
+                    clc_try_cancel(taken, taken_bar);
+                }
             }
         }
     } else if (warp == MS_CONS_WARPS + 1) {
@@ -466,10 +483,6 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         }
         cluster_sync_all();                    // nobody reads this CTA's shared memory any more
     }
-    if (p.dynamic && threadIdx.x == 0) {       // whoever is last leaves the counters ready for the next launch
-        __threadfence();
-        if (atomicAdd(p.sched + 1, 1) == static_cast<int>(gridDim.x) - 1) { p.sched[0] = 0; p.sched[1] = 0; }
-    }
     if (*abort_flag) {
         for (int i = 0; i < 64; ++i) __nanosleep(2000);       // copies still in flight land before the memory is released
     }
@@ -478,17 +491,12 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 // Ring depth and shared memory of a launch; false if not even two stages fit.
 static bool ms_layout(StreamParams& p, int qbits, int ntm, int n_exp, size_t& smem) {
     p.stage_bytes = (MS_W_BYTES + ms_s_bytes(qbits) + ntm * MS_X_BYTES + 1023) & ~1023;      // the codes' swizzle wants 1 KB
-    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + 32 * MS_MAX_ST + 64 + 16 + 16 * MS_MAX_ST +
+    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + 32 * MS_MAX_ST + 64 + 32 + 16 + 16 * MS_MAX_ST +
                          (2 * static_cast<size_t>(n_exp) + 2) * sizeof(int);
     p.n_stages = static_cast<int>((MS_SMEM_MAX - fixed) / p.stage_bytes);
     if (p.n_stages > MS_MAX_ST) p.n_stages = MS_MAX_ST;
     smem = fixed + static_cast<size_t>(p.n_stages) * p.stage_bytes;
     return p.n_stages >= 2;
-}
-// Tile counters of a launch: zero, and left zero by the launch.  Expert GEMMs on several streams overlap, so a launch does not
-// get the pair that one of the 63 before it got.
-static int* ms_counters(qg_ctx* ctx) {
-    return ctx->gemv_tickets + ctx->gemv_ticket_count + 2 * (ctx->sched_next++ % SCHED_SLOTS);
 }
 using StreamKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const StreamParams);
 static int ms_set_smem(qg_ctx* ctx, StreamKernel kern, int inst) {
@@ -507,7 +515,7 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     const bool gate_up = mode == QG_MODE_GATE_UP_SILU;
     if (R > static_cast<long long>(MS_MAX_ROWS) * E) return QG_ERR_WORKSPACE;
     StreamParams p{};
-    p.R = R; p.N = N; p.K = K; p.E = E; p.kc = K; p.dynamic = 1;
+    p.R = R; p.N = N; p.K = K; p.E = E; p.kc = K;
     p.n_wt = gate_up ? N / 128 : (N + 127) / 128;
     // Rows per tile: eight up to five rows per expert, sixteen above.  The wider tile's ring is a stage shorter (56.1 us
     // against 53.0 at four rows per expert, gate/up); cutting a segment in two costs more from six on (60.4 with eight and
@@ -517,7 +525,6 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     if (!ms_layout(p, 4, ntm, E, smem)) return QG_ERR_WORKSPACE;
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
     p.topk_w = (mode == QG_MODE_DOWN_WEIGHTED) ? topk_w : nullptr; p.row_pair = row_pair;
-    p.sched = ms_counters(ctx);
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb < 0 ? -1 : ctx->skip_kb / (MS_SK / 64);
     CUtensorMap tm_w, tm_s, tm_x;
@@ -540,7 +547,9 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     ctx->skip_kb = -1;                                        // the test hook acts on one launch
     // at most one chunk per 8 ntm rows and one more per expert that has rows
     const long long max_tiles = static_cast<long long>(R / (8 * ntm) + (R < E ? R : E)) * p.n_wt;
-    const int grid = static_cast<int>(max_tiles < 2LL * ctx->sm_count ? max_tiles : 2LL * ctx->sm_count);
+    if (max_tiles > 0x7FFFFFFF) return QG_ERR_WORKSPACE;
+    const int grid = static_cast<int>(max_tiles);
+    p.dynamic = grid > 2 * ctx->sm_count;
     if (launch_kernel(ctx, kern, dim3(grid), dim3(MS_THREADS), smem, st, tm_w, tm_s, tm_x, p) != cudaSuccess) {
         cudaGetLastError();
         return QG_ERR_CUDA;
@@ -591,7 +600,6 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     }
     p.R = M; p.N = N; p.K = K; p.E = 0; p.kc = kc; p.n_wt = tiles;
     p.out = static_cast<__nv_bfloat16*>(Cout);
-    p.sched = ms_counters(ctx);
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb;
     CUtensorMap tm_w, tm_s, tm_x;
@@ -606,10 +614,9 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
                          static_cast<uint64_t>(K) * 2);
     if (rc != QG_OK) return rc;
     ctx->skip_kb = -1;
-    const int grid = (slices == 1 && tiles > 2 * ctx->sm_count) ? 2 * ctx->sm_count : tiles;
-    p.dynamic = tiles > grid;
+    p.dynamic = slices == 1 && tiles > 2 * ctx->sm_count;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid, slices); cfg.blockDim = dim3(MS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.gridDim = dim3(tiles, slices); cfg.blockDim = dim3(MS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute at[2];
     int n_at = 0;
     if (ctx->pdl) {

@@ -82,7 +82,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct():
     util.assert_close(util.host_bf16_f64(out), orc.grouped_gemm(4, orc.bf16_to_f64(A), offsets, Wq, Ws), "after a timeout")
 
 
-# one stage and an odd number of them; a slice of a single stage; ragged rows; more tiles than CTAs (tiles from the counter)
+# one stage and an odd number of them; a slice of a single stage; ragged rows; more tiles than CTAs (tiles taken over)
 # with one stage, with an odd number and with more stages than the ring holds; eight and sixteen tokens from both sides
 DENSE = [(8, 1, 64, 4096), (8, 8, 72, 768), (8, 9, 264, 1280), (4, 16, 136, 256 * 7), (4, 8, 2048, 512), (8, 16, 19016, 256),
          (8, 3, 19136, 768), (4, 9, 38024, 256), (4, 7, 38144, 1280), (8, 2, 4096, 4096), (4, 1, 3072, 8192)]
@@ -136,7 +136,7 @@ def test_an_infinite_token_gives_infinities_of_the_codes_signs():
 
 
 def test_expert_gemms_on_two_streams_at_once():
-    """Launches that overlap take their tiles from counters of their own."""
+    """Launches that overlap deal out their tiles independently."""
     counts, N, K = [3, 7, 1, 12, 0, 5] * 8, 1536, 1024
     offsets, A, Wq, Ws = problem(counts, N, K, 9)
     args = (util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
@@ -149,3 +149,41 @@ def test_expert_gemms_on_two_streams_at_once():
     torch.cuda.synchronize()
     qg.poll_status()
     assert all(torch.equal(o, want) for o in outs)
+
+
+@pytest.mark.parametrize("dense", [False, True], ids=["grouped", "one-matrix"])
+def test_launches_share_nothing_however_they_overlap(dense):
+    """Launches queued behind a long kernel on one stream, many more issued on a second one meanwhile, and replays of a captured
+    launch on a third: all write what a launch alone writes."""
+    if dense:
+        A, Wq, Ws = synth.dense_problem(8, 5, 38016, 512, seed=19)            # 594 tiles: more than CTAs
+        args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
+        call = lambda out: qg.qgemm_small_m(8, *args, out=out)
+        shape = (5, 38016)
+    else:
+        counts, N, K = [3, 7, 1, 12, 0, 5] * 8, 1536, 1024
+        offsets, A, Wq, Ws = problem(counts, N, K, 9)
+        args = (util.dev_bf16(A), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws))
+        call = lambda out: qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args, out=out)
+        shape = (int(offsets[-1]), N)
+    fresh = lambda: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    want = call(fresh())
+    held, busy, replay = (torch.cuda.Stream() for _ in range(3))
+    captured, graph = fresh(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(captured)
+    outs = [fresh() for _ in range(170)]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(held):
+        torch.cuda._sleep(2_000_000)                                          # about a millisecond
+        for o in outs[:20]:
+            call(o)
+    for i, o in enumerate(outs[20:]):
+        with torch.cuda.stream(busy):
+            call(o)
+        if i % 3 == 0:
+            with torch.cuda.stream(replay):
+                graph.replay()
+    torch.cuda.synchronize()
+    qg.poll_status()
+    assert torch.equal(captured, want) and all(torch.equal(o, want) for o in outs)
