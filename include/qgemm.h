@@ -131,7 +131,8 @@ int qgemm_dense_gate_up_silu(qg_ctx* ctx, int qbits, int M, int F, int K, const 
  * slice order across CTAs), so results do not depend on scheduling.  Same formats and constraints as qgemm_dense, fp32
  * accumulation.  Numerics: the streaming kernel multiplies the exact integers q and applies the block's scale to the fp32
  * sum of each 32-block, which is closer to the exact value than weights rounded to bf16 (q * scale), as the block kernel and
- * qgemm_dense multiply them (all are within the library's tolerance of it).  Uses the context's scratch, so calls on one
+ * qgemm_dense multiply them (all are within the library's tolerance of it).  An output is finite wherever the sum of the scaled
+ * products is: unscaled sums that leave fp32 (token values from 8e34 on) are computed again.  Uses the context's scratch, so calls on one
  * context must not overlap on the GPU.
  */
 int qgemm_small_m(qg_ctx* ctx, int qbits, int M, int N, int K, const void* A, const void* Wq,

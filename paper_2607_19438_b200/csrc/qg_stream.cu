@@ -33,6 +33,13 @@
 // difference is the code (42 instructions per 512 weights and eight rows, against 68 slots of the permute, packed fma and
 // round chain that produces scaled weights).
 //
+// Range.  A 32-block's unscaled sum is up to 2^12 (4-bit codes: 2^8) times its largest token value: from 2^116 (2^120) on it may
+// leave fp32 although the scaled sum would not.  Such a sum ends as an infinity or a NaN whatever is added, and so does the
+// output; a warp that has stored one computes its outputs that are not finite again, from weights scaled beforehand, unless their
+// token row is not finite itself (ms_again).  (Looking for huge values where the rows are prepared, and shrinking them by a
+// power of two, costs every stage something: 128 tokens, 128 experts 144 us against 127.  As a called function, with a stack frame,
+// the repair costs short launches 0.6 us: inlined, 1 % over 1086 shapes.)
+//
 // Measured, 128 experts x (1536 x 2048 gate/up, 2048 x 768 down), against the tensor-memory kernel: 1 token of eight
 // experts 13.3 / 9.1 us against 16 / 12, 4 tokens 22 / 13 against 33 / 21, 32 tokens 48 / 30 (3.9 / 3.2 TB/s of codes and
 // scales) against 85 / 49, 128 tokens 64 / 39 against 101 / 56, 256 tokens 91 / 54 against 102 / 57.
@@ -74,6 +81,9 @@ struct StreamParams {
     int dynamic;                // more blocks than fit at once: a CTA goes on with the tiles of blocks not yet started
     const int32_t* offsets;     // grouped: device expert offsets [E + 1]
     __nv_bfloat16* out;
+    const __nv_bfloat16* x;     // token rows, codes and scales once more, for ms_again
+    const uint8_t* wq;
+    const __half* ws;
     const float* topk_w;        // grouped: routing weights, applied to the rows named by row_pair (nullptr: none)
     const int32_t* row_pair;
     int* status;
@@ -156,6 +166,53 @@ __device__ __forceinline__ void ms_stage(float (&acc)[NTM][MT][4], uint32_t wl, 
 }
 
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
+
+// Token row x times weight row `row` (over all experts), each weight scaled before it is multiplied, in the order of k.
+template <int QBITS>
+__device__ __forceinline__ float ms_dot(const StreamParams& p, const __nv_bfloat16* x, long long row) {
+    const uint8_t* q = p.wq + row * (static_cast<long long>(p.K) * QBITS / 8);
+    const __half* s = p.ws + row * (p.K >> 5);
+    float acc = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < p.K; k += 2) {
+        const float sc = __half2float(s[k >> 5]);
+        int q0, q1;
+        if constexpr (QBITS == 8) {
+            q0 = static_cast<int8_t>(q[k]); q1 = static_cast<int8_t>(q[k + 1]);
+        } else {
+            q0 = (q[k >> 1] & 15) - 8; q1 = (q[k >> 1] >> 4) - 8;
+        }
+        acc = fmaf(__bfloat162float(x[k]), q0 * sc, acc);
+        acc = fmaf(__bfloat162float(x[k + 1]), q1 * sc, acc);
+    }
+    return acc;
+}
+__device__ __forceinline__ bool ms_finite(__nv_bfloat16 v) { return (__bfloat16_as_ushort(v) & 0x7F80) != 0x7F80; }
+// The outputs of token row `tok` in columns c and c + 8 (gate/up: column c only) again, where they are not finite.
+template <int QBITS, bool GATE_UP>
+__device__ __forceinline__ void ms_again(const StreamParams& p, int e, int tok, int c) {
+    const __nv_bfloat16* x = p.x + static_cast<size_t>(tok) * p.K;
+    const int width = GATE_UP ? p.N >> 1 : p.N;
+    __nv_bfloat16* o = p.out + static_cast<size_t>(tok) * width;
+    bool scanned = false;
+#pragma unroll 1
+    for (int h = 0; h < (GATE_UP ? 1 : 2); ++h, c += 8) {
+        if (c >= width || ms_finite(o[c])) continue;
+#pragma unroll 1
+        for (int k = 0; !scanned && k < p.K; ++k)
+            if (!ms_finite(x[k])) return;             // what the products gave stands
+        scanned = true;
+        const long long row = static_cast<long long>(e) * p.N + c;
+        float v = ms_dot<QBITS>(p, x, row);
+        if (GATE_UP) v = silu_mul(v, ms_dot<QBITS>(p, x, row + width));
+        else if (p.topk_w) v *= p.topk_w[p.row_pair[tok]];
+        o[c] = __float2bfloat16_rn(v);
+    }
+}
+// 0, or NaN if one of the four is an infinity or a NaN
+__device__ __forceinline__ float zero_if_finite(float z, float a, float b, float c, float d) {
+    return fmaf(a, 0.f, fmaf(b, 0.f, fmaf(c, 0.f, fmaf(d, 0.f, z))));
+}
 
 // tm_w: packed codes, box 128 bytes x the tile's rows (gate/up: 64 rows x 2 planes), 128-byte swizzle; tm_s: scales, box 8 x
 // the same rows; tm_x: token rows as [K / 32][R][32], box 32 k x 8 rows x 8 blocks, so that the 16 bytes a lane of an MMA
@@ -408,6 +465,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 continue;
             }
             if (nst > 1 && !__all_sync(0xFFFFFFFFu, ms_wait(hfull, q & 1u, abort_flag, p))) break;
+            float z = 0.f;
 #pragma unroll
             for (int nt = 0; nt < NTM; ++nt) {
                 if (nt >= nt_n) break;
@@ -426,6 +484,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                         sts_u4(at, make_uint4(__float_as_uint(c0), __float_as_uint(c1), __float_as_uint(c2), __float_as_uint(c3)));
                         continue;
                     }
+                    z = zero_if_finite(z, c0, c1, c2, c3);
                     __nv_bfloat16* o = p.out;
                     if constexpr (GATE_UP) {
                         const int F = p.N >> 1;
@@ -451,6 +510,16 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             if (nst > 1) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(hempty);
+            }
+            if (z != 0.f) {                   // a NaN: one of this thread's sums is not finite
+                int e = 0;
+                if (GROUPED)
+                    while (off[e + 1] <= tok0) ++e;
+#pragma unroll 1
+                for (int i = 0; i < 2 * MT * nt_n; ++i) {
+                    const int t = 8 * (i / (2 * MT)) + 2 * j + (i & 1), m = (i >> 1) % MT;
+                    if (t < n) ms_again<QBITS, GATE_UP>(p, e, tok0 + t, GATE_UP ? wt * 64 + 16 * w4 + 8 * m + g : wt * ROWS + 16 * (MT * w4 + m) + g);
+                }
             }
         }
     }
@@ -480,6 +549,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 if (r < p.N) o[p.N] = __float2bfloat16_rn(c[1]);
                 if (r + 8 < p.N) o[p.N + 8] = __float2bfloat16_rn(c[3]);
             }
+            if (zero_if_finite(0.f, c[0], c[1], c[2], c[3]) != 0.f)
+#pragma unroll 1
+                for (int u = t; u < min(t + 2, p.R); ++u) ms_again<QBITS, false>(p, 0, u, r + (l >> 2));
         }
         cluster_sync_all();                    // nobody reads this CTA's shared memory any more
     }
@@ -524,6 +596,7 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     size_t smem = 0;
     if (!ms_layout(p, 4, ntm, E, smem)) return QG_ERR_WORKSPACE;
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
+    p.x = static_cast<const __nv_bfloat16*>(Ain); p.wq = static_cast<const uint8_t*>(Wq); p.ws = static_cast<const __half*>(Ws);
     p.topk_w = (mode == QG_MODE_DOWN_WEIGHTED) ? topk_w : nullptr; p.row_pair = row_pair;
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb < 0 ? -1 : ctx->skip_kb / (MS_SK / 64);
@@ -600,6 +673,7 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     }
     p.R = M; p.N = N; p.K = K; p.E = 0; p.kc = kc; p.n_wt = tiles;
     p.out = static_cast<__nv_bfloat16*>(Cout);
+    p.x = static_cast<const __nv_bfloat16*>(A); p.wq = static_cast<const uint8_t*>(Wq); p.ws = static_cast<const __half*>(Ws);
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb;
     CUtensorMap tm_w, tm_s, tm_x;

@@ -187,3 +187,72 @@ def test_launches_share_nothing_however_they_overlap(dense):
     torch.cuda.synchronize()
     qg.poll_status()
     assert torch.equal(captured, want) and all(torch.equal(o, want) for o in outs)
+
+
+def huge_tokens(M, K, seed):
+    """Ordinary token rows, then in some 256-k stages values up to the largest bf16; the first row is the largest number for
+    which no unscaled block sum overflows, and the second an ordinary one throughout."""
+    x = synth.bf16_bits_to_f32(synth.activations(M, K, seed, 64)).copy()
+    rng = np.random.default_rng(seed)
+    for st in range(0, K // 256, 2):
+        blk = slice(256 * st, 256 * st + 256)
+        x[2:, blk] = rng.choice([-1.0, 1.0], (M - 2, 256)) * rng.uniform(0.5, 1.0, (M - 2, 256)).astype(np.float32) * np.float32(3.38e38)
+    x[0, :] = np.float32(2.0 ** 116 * (1 - 2.0 ** -8))
+    return synth.f32_to_bf16_bits(x.astype(np.float32))
+
+
+@pytest.mark.parametrize("qbits,M,N,K", [(8, 4, 1024, 768), (8, 16, 1032, 1024), (4, 5, 1024, 768), (4, 16, 2056, 256), (8, 9, 38016, 256)],
+                         ids=lambda v: str(v))
+def test_tokens_up_to_the_largest_number_stay_finite(qbits, M, N, K):
+    """Weights scaled beforehand give finite sums of huge tokens, so the exact integer products have to as well, and a zero
+    scale gives zero.  An ordinary row beside them keeps its bits."""
+    _, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=21)
+    Wq = Wq.copy()
+    Wq[:64] = -128 if qbits == 8 else 0                          # the most negative code throughout
+    Ws = np.abs(Ws.view(np.float16)).astype(np.float32)
+    Ws = (Ws / Ws.max() * 2.0 ** -15).astype(np.float16)
+    Ws[5], Ws[N - 3] = 0, 0
+    Ws = Ws.view(np.uint16)
+    xb = huge_tokens(M, K, 3)
+    args = (util.dev(Wq), util.dev_f16(Ws))
+    out = util.host_bf16_f64(qg.qgemm_small_m(qbits, util.dev_bf16(xb), *args))
+    alone = util.host_bf16_f64(qg.qgemm_small_m(qbits, util.dev_bf16(np.repeat(xb[1:2], M, 0)), *args))
+    qg.poll_status()
+    assert np.all(out[:, [5, N - 3]] == 0) and np.array_equal(out[1], alone[1])
+    rows = np.unique(np.concatenate([np.arange(0, N, max(1, N // 512)), np.arange(64)]))
+    ref = orc.qgemm_dense(qbits, xb, Wq[rows], Ws[rows])
+    inside = np.abs(ref) < 3.3e38                                # (rows of one sign and one code may leave the format's range)
+    assert inside[:, 64:].all() and inside[0].all()
+    for m in range(M):                                           # row by row: the rows differ by 38 orders of magnitude
+        util.assert_close(out[m, rows][inside[m]], ref[m][inside[m]], f"row {m}")
+
+
+@pytest.mark.parametrize("mode", [qg.MODE_PLAIN, qg.MODE_GATE_UP_SILU, qg.MODE_DOWN_WEIGHTED], ids=["plain", "gateup", "weighted"])
+def test_huge_tokens_in_short_segments(mode):
+    counts, N, K = [0, 7, 16, 1, 23], 256, 768
+    offsets, _, Wq, Ws = problem(counts, N, K, 22)
+    R = int(offsets[-1])
+    Ws = (np.abs(Ws.view(np.float16)).astype(np.float32) * 2.0 ** -7).astype(np.float16)
+    if mode == qg.MODE_GATE_UP_SILU:
+        Ws[:, N // 2:] *= np.float16(2.0 ** 7)                   # the up projection sees the ordinary stage only: the gate is huge already
+        Ws[:, N // 2:, :8], Ws[:, N // 2:, 16:] = 0, 0
+    Ws = Ws.view(np.uint16)
+    xb = huge_tokens(R, K, 5)
+    w = np.full(R, 0.5, np.float32)
+    row_pair = np.arange(R, dtype=np.int32)
+    out = qg.moe_grouped_qgemm(mode, 4, util.dev_bf16(xb), util.dev(offsets), util.dev(Wq), util.dev_f16(Ws), topk_w=util.dev(w),
+                               row_pair=util.dev(row_pair))
+    qg.poll_status()
+    ref = orc.grouped_gemm(4, orc.bf16_to_f64(xb), offsets, Wq, Ws)
+    if mode == qg.MODE_GATE_UP_SILU:
+        g, u = ref[:, :N // 2], ref[:, N // 2:]
+        ref = np.where(g > 0, g * u, 0.0)                        # |g| is beyond 100 wherever it is not the ordinary row
+        keep = (np.abs(g) > 100) & (np.abs(ref) < 3.3e38)
+    else:
+        ref = ref * (0.5 if mode == qg.MODE_DOWN_WEIGHTED else 1.0)
+        keep = np.abs(ref) < 3.3e38
+    got = util.host_bf16_f64(out)
+    for r in range(R):
+        if keep[r].sum() > 8:
+            util.assert_close(got[r][keep[r]], ref[r][keep[r]], f"row {r}")
+    assert keep.mean() > (0.3 if mode == qg.MODE_GATE_UP_SILU else 0.99)
