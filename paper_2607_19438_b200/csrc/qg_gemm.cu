@@ -1286,9 +1286,10 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     // expected rows per expert decide the token tile; 192 keeps two accumulators, so the short main loops of
     // expert tiles overlap their epilogues
     const int bt = (R / E > 100) ? 192 : 128;
-    // a few rows per expert (4-bit weights, rows in segment order, no accumulation) the streaming kernel is faster
-    if (qbits == QG_Q4 && mode <= QG_MODE_DOWN_WEIGHTED && gather_k == 0 && ctx->force_bt == 0) {
-        const int rc = qg::launch_moe_stream(ctx, mode, R, E, N, K, Ain, expert_offsets, Wq, Wscale, topk_w, row_pair, Out,
+    // a few rows per expert (4-bit weights, no accumulation) the streaming kernel is faster; the gathering form takes the same
+    // kernel as the form for sorted rows, so that they give the same numbers
+    if (qbits == QG_Q4 && mode <= QG_MODE_DOWN_WEIGHTED && ctx->force_bt == 0) {
+        const int rc = qg::launch_moe_stream(ctx, mode, R, E, N, K, Ain, in_rows, gather_k, expert_offsets, Wq, Wscale, topk_w, row_pair, Out,
                                              static_cast<cudaStream_t>(stream));
         if (rc != QG_ERR_WORKSPACE) return rc;
     }

@@ -32,9 +32,9 @@ enum AttrSlot {
     ATTR_ROUTER_4 = 31,
     ATTR_MX_MOE = 32,       // 2: down, gate/up
     ATTR_MX_256 = 34,
-    ATTR_STREAM = 35,       // 4: down, gate/up x rows per tile (2)
-    ATTR_DENSE_STREAM = 39, // 4: format (2) x more than eight tokens (2)
-    ATTR_SLOTS = 43
+    ATTR_STREAM = 35,       // 8: sorted, gathered rows x down, gate/up x rows per tile (2)
+    ATTR_DENSE_STREAM = 43, // 4: format (2) x more than eight tokens (2)
+    ATTR_SLOTS = 47
 };
 }  // namespace qg
 
@@ -97,7 +97,7 @@ int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
                 uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz, uint64_t row_stride_bytes = 0);
 // The streaming kernel of the grouped GEMM (4-bit weights, modes 0 to 2), for a few rows per expert; QG_ERR_WORKSPACE if the
 // shape does not suit it.
-int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, const int32_t* offsets,
+int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, int in_rows, int gather_k, const int32_t* offsets,
                       const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st);
 // The same kernel for one matrix and up to sixteen tokens.
 int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void* A, const void* Wq, const void* Ws, void* Cout,

@@ -1,5 +1,5 @@
 // The weight-streaming GEMM: one matrix and up to sixteen tokens (qgemm_small_m), or the 4-bit expert matrices of a routed
-// layer with a few rows per expert (moe_grouped_qgemm: plain, gate/up + SiLU, routing-weighted).
+// layer with a few rows per expert (moe_grouped_qgemm and its gathering form: plain, gate/up + SiLU, routing-weighted).
 //
 // Every weight byte is used for a handful of token rows only, so the call is a streaming read of the packed weights: 42
 // 4-bit or 22 8-bit weights per clock and SM at HBM speed.  The tensor-memory kernel of the long segments (qg_gemm.cu)
@@ -86,6 +86,7 @@ struct StreamParams {
     const __half* ws;
     const float* topk_w;        // grouped: routing weights, applied to the rows named by row_pair (nullptr: none)
     const int32_t* row_pair;
+    int gather_k;               // gathered: row r of the input is token row_pair[r] / gather_k
     int* status;
     uint32_t wait_limit;
     int skip_stage;             // test hook: stage of the first CTA whose token rows are never loaded (-1: none)
@@ -189,9 +190,9 @@ __device__ __forceinline__ float ms_dot(const StreamParams& p, const __nv_bfloat
 }
 __device__ __forceinline__ bool ms_finite(__nv_bfloat16 v) { return (__bfloat16_as_ushort(v) & 0x7F80) != 0x7F80; }
 // The outputs of token row `tok` in columns c and c + 8 (gate/up: column c only) again, where they are not finite.
-template <int QBITS, bool GATE_UP>
+template <int QBITS, bool GATE_UP, bool GATHER>
 __device__ __forceinline__ void ms_again(const StreamParams& p, int e, int tok, int c) {
-    const __nv_bfloat16* x = p.x + static_cast<size_t>(tok) * p.K;
+    const __nv_bfloat16* x = p.x + static_cast<size_t>(GATHER ? p.row_pair[tok] / p.gather_k : tok) * p.K;
     const int width = GATE_UP ? p.N >> 1 : p.N;
     __nv_bfloat16* o = p.out + static_cast<size_t>(tok) * width;
     bool scanned = false;
@@ -216,9 +217,10 @@ __device__ __forceinline__ float zero_if_finite(float z, float a, float b, float
 
 // tm_w: packed codes, box 128 bytes x the tile's rows (gate/up: 64 rows x 2 planes), 128-byte swizzle; tm_s: scales, box 8 x
 // the same rows; tm_x: token rows as [K / 32][R][32], box 32 k x 8 rows x 8 blocks, so that the 16 bytes a lane of an MMA
-// fragment needs follow one another in lane order.  Rows past the end arrive as zeros.
+// fragment needs follow one another in lane order.  Rows past the end arrive as zeros.  Gathered rows: [M][K], box 256 k x one
+// row, four rows per copy, which land row after row.
 // grid = (tiles, K slices); the slices of a tile are one cluster.
-template <int QBITS, bool GROUPED, bool GATE_UP, int NTM>
+template <int QBITS, bool GROUPED, bool GATE_UP, int NTM, bool GATHER>
 __global__ void __launch_bounds__(MS_THREADS, 2)
 stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
               const __grid_constant__ CUtensorMap tm_x, const StreamParams p) {
@@ -334,6 +336,13 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     }
                 }
                 const int nt = (tl.n + 7) >> 3;
+                int rows[TN];                          // gathered: the tile's token rows (past its end the first one: computed, never stored)
+                if (GATHER && tl.n > 0) {
+#pragma unroll
+                    for (int i = 0; i < TN; ++i) rows[i] = p.row_pair[tl.tok0 + (i < tl.n ? i : 0)];
+#pragma unroll
+                    for (int i = 0; i < TN; ++i) rows[i] /= p.gather_k;
+                }
                 for (int st = 0; st < (tl.n ? nst : 2); ++st, ++sent) {     // no more tiles: two empty stages, one for each set, say so
                     if (sent >= p.n_stages && !ms_wait(empty0 + 8u * slot, phase ^ 1u, abort_flag, p)) { ok = false; break; }
                     const uint32_t xbar = xfull0 + 8u * slot;
@@ -344,7 +353,14 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                         mbar_arrive(full0 + 8u * fslot);
                     } else {
                         mbar_arrive_expect_tx(xbar, nt * MS_X_BYTES);
-                        if (sent != skip)
+                        if (sent == skip) {
+                        } else if (GATHER) {
+#pragma unroll
+                            for (int i = 0; i < TN; i += 4)
+                                if (i < 8 * nt)
+                                    tma_gather4(ring + slot * p.stage_bytes + OFF_X + i * 512, &tm_x, st * MS_SK, rows[i], rows[i + 1], rows[i + 2],
+                                                rows[i + 3], xbar);
+                        } else
                             for (int i = 0; i < nt; ++i)
                                 tma_load_3d(ring + slot * p.stage_bytes + OFF_X + i * MS_X_BYTES, &tm_x, 0, tl.tok0 + 8 * i, k0 / 32 + st * 8, xbar);
                         if (sent >= ahead) load_weights(slot, full0 + 8u * fslot, st, tl);
@@ -383,7 +399,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     if constexpr (QBITS == 4) {
-                        const uint4 r = lds_u4(xi + u * 512 + lane * 16);
+                        const uint4 r = lds_u4(GATHER ? xi + g * 512 + u * 64 + j * 16 : xi + u * 512 + lane * 16);
                         v[u] = make_uint4(__byte_perm(r.x, r.y, 0x5410), __byte_perm(r.z, r.w, 0x5410),
                                           __byte_perm(r.x, r.y, 0x7632), __byte_perm(r.z, r.w, 0x7632));
                     } else {
@@ -392,7 +408,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                                           __byte_perm(c.x, c.y, 0x5410), __byte_perm(c.x, c.y, 0x7632));
                     }
                 }
-                if (QBITS == 8) __syncwarp();      // everything is read before anything is written
+                if (QBITS == 8 || GATHER) __syncwarp();      // everything is read before anything is written
 #pragma unroll
                 for (int u = 0; u < 8; ++u) sts_u4(xi + u * 512 + lane * 16, v[u]);
             }
@@ -518,7 +534,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll 1
                 for (int i = 0; i < 2 * MT * nt_n; ++i) {
                     const int t = 8 * (i / (2 * MT)) + 2 * j + (i & 1), m = (i >> 1) % MT;
-                    if (t < n) ms_again<QBITS, GATE_UP>(p, e, tok0 + t, GATE_UP ? wt * 64 + 16 * w4 + 8 * m + g : wt * ROWS + 16 * (MT * w4 + m) + g);
+                    if (t < n) ms_again<QBITS, GATE_UP, GATHER>(p, e, tok0 + t, GATE_UP ? wt * 64 + 16 * w4 + 8 * m + g : wt * ROWS + 16 * (MT * w4 + m) + g);
                 }
             }
         }
@@ -551,7 +567,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
             if (zero_if_finite(0.f, c[0], c[1], c[2], c[3]) != 0.f)
 #pragma unroll 1
-                for (int u = t; u < min(t + 2, p.R); ++u) ms_again<QBITS, false>(p, 0, u, r + (l >> 2));
+                for (int u = t; u < min(t + 2, p.R); ++u) ms_again<QBITS, false, false>(p, 0, u, r + (l >> 2));
         }
         cluster_sync_all();                    // nobody reads this CTA's shared memory any more
     }
@@ -582,7 +598,7 @@ static int ms_set_smem(qg_ctx* ctx, StreamKernel kern, int inst) {
 }
 
 // The grouped call.  Returns QG_ERR_WORKSPACE if the shape does not suit this kernel (the caller takes the other one).
-int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, const int32_t* offsets,
+int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, int in_rows, int gather_k, const int32_t* offsets,
                       const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st) {
     const bool gate_up = mode == QG_MODE_GATE_UP_SILU;
     if (R > static_cast<long long>(MS_MAX_ROWS) * E) return QG_ERR_WORKSPACE;
@@ -598,6 +614,7 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
     p.x = static_cast<const __nv_bfloat16*>(Ain); p.wq = static_cast<const uint8_t*>(Wq); p.ws = static_cast<const __half*>(Ws);
     p.topk_w = (mode == QG_MODE_DOWN_WEIGHTED) ? topk_w : nullptr; p.row_pair = row_pair;
+    p.gather_k = gather_k;
     p.status = ctx->d_status; p.wait_limit = ctx->wait_limit;
     p.skip_stage = ctx->skip_kb < 0 ? -1 : ctx->skip_kb / (MS_SK / 64);
     CUtensorMap tm_w, tm_s, tm_x;
@@ -610,12 +627,17 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
                                    CU_TENSOR_MAP_SWIZZLE_NONE)
                      : get_tmap_2d(ctx, &tm_s, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, Ws, ks, wrows, 8, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (rc == QG_OK)
-        rc = get_tmap_3d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ain, 32, R, K / 32, 64, 32, 8, 8, CU_TENSOR_MAP_SWIZZLE_NONE,
-                         static_cast<uint64_t>(K) * 2);
+        rc = gather_k > 0 ? get_tmap_2d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ain, K, in_rows, MS_SK, 1, CU_TENSOR_MAP_SWIZZLE_NONE)
+                          : get_tmap_3d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ain, 32, R, K / 32, 64, 32, 8, 8,
+                                        CU_TENSOR_MAP_SWIZZLE_NONE, static_cast<uint64_t>(K) * 2);
     if (rc != QG_OK) return rc;
-    const StreamKernel kern = (ntm == 1) ? (gate_up ? stream_kernel<4, true, true, 1> : stream_kernel<4, true, false, 1>)
-                                         : (gate_up ? stream_kernel<4, true, true, MS_NT> : stream_kernel<4, true, false, MS_NT>);
-    rc = ms_set_smem(ctx, kern, ATTR_STREAM + (gate_up ? 2 : 0) + ntm - 1);
+    const StreamKernel kerns[8] = {
+        stream_kernel<4, true, false, 1, false>, stream_kernel<4, true, false, MS_NT, false>, stream_kernel<4, true, true, 1, false>,
+        stream_kernel<4, true, true, MS_NT, false>, stream_kernel<4, true, false, 1, true>, stream_kernel<4, true, false, MS_NT, true>,
+        stream_kernel<4, true, true, 1, true>, stream_kernel<4, true, true, MS_NT, true>};
+    const int which = (gather_k > 0 ? 4 : 0) + (gate_up ? 2 : 0) + ntm - 1;
+    const StreamKernel kern = kerns[which];
+    rc = ms_set_smem(ctx, kern, ATTR_STREAM + which);
     if (rc != QG_OK) return rc;
     ctx->skip_kb = -1;                                        // the test hook acts on one launch
     // at most one chunk per 8 ntm rows and one more per expert that has rows
@@ -637,8 +659,8 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     StreamParams p{};
     size_t smem = 0;
     if (!ms_layout(p, qbits, ntm, 0, smem)) return QG_ERR_WORKSPACE;
-    const StreamKernel kern = (qbits == 8) ? (ntm == 1 ? stream_kernel<8, false, false, 1> : stream_kernel<8, false, false, 2>)
-                                           : (ntm == 1 ? stream_kernel<4, false, false, 1> : stream_kernel<4, false, false, 2>);
+    const StreamKernel kern = (qbits == 8) ? (ntm == 1 ? stream_kernel<8, false, false, 1, false> : stream_kernel<8, false, false, 2, false>)
+                                           : (ntm == 1 ? stream_kernel<4, false, false, 1, false> : stream_kernel<4, false, false, 2, false>);
     int rc = ms_set_smem(ctx, kern, ATTR_DENSE_STREAM + variant);
     if (rc != QG_OK) return rc;
     // clusters of `ns` CTAs of this kernel that fit on the GPU at once (asked once per context, variant and size)

@@ -256,3 +256,24 @@ def test_huge_tokens_in_short_segments(mode):
         if keep[r].sum() > 8:
             util.assert_close(got[r][keep[r]], ref[r][keep[r]], f"row {r}")
     assert keep.mean() > (0.3 if mode == qg.MODE_GATE_UP_SILU else 0.99)
+
+
+@pytest.mark.parametrize("mode", [qg.MODE_PLAIN, qg.MODE_GATE_UP_SILU, qg.MODE_DOWN_WEIGHTED], ids=["plain", "gateup", "weighted"])
+@pytest.mark.parametrize("M,E,k,N,K", [(1, 4, 1, 128, 256), (3, 8, 2, 256, 512), (37, 5, 2, 384, 768), (70, 40, 8, 256, 1280), (256, 128, 8, 1536, 256)],
+                         ids=lambda v: str(v))
+def test_gathered_rows_give_the_bits_of_sorted_rows(M, E, k, N, K, mode):
+    """Fewer rows than a copy of four, a tile of eight, a tile of sixteen; tokens used more than once; more tiles than CTAs."""
+    X, Wq, Ws = synth.activations(M, K, 31), synth.weights_q4(E * N, K, 31).reshape(E, N, K // 2), synth.scales(E * N, K // 32, 7, 31).reshape(E, N, K // 32)
+    dX, dWq, dWs = util.dev_bf16(X), util.dev(Wq), util.dev_f16(Ws)
+    r = qg.moe_route(util.dev(synth.router_logits(M, E, 31)), k, X=dX)
+    w = r["topk_w"].view(-1)
+    a = qg.moe_grouped_qgemm(mode, 4, r["Xperm"], r["offsets"], dWq, dWs, topk_w=w, row_pair=r["row_pair"])
+    g = util.Guarded(a.shape, torch.bfloat16)
+    qg.moe_grouped_qgemm_gather(mode, 4, dX, r["row_pair"], k, r["offsets"], dWq, dWs, topk_w=w, out=g.t)
+    qg.poll_status()
+    assert torch.equal(a, g.t) and g.intact()
+    dX[M // 2, K // 2] = float("inf")                      # and so they do in the rows of a token that is not finite
+    a = qg.moe_grouped_qgemm(mode, 4, qg.moe_permute(dX, r["row_pair"], k), r["offsets"], dWq, dWs, topk_w=w, row_pair=r["row_pair"])
+    b = qg.moe_grouped_qgemm_gather(mode, 4, dX, r["row_pair"], k, r["offsets"], dWq, dWs, topk_w=w)
+    qg.poll_status()
+    assert torch.equal(a.nan_to_num(7.0), b.nan_to_num(7.0))
