@@ -230,6 +230,9 @@ int moe_permute(qg_ctx* ctx, int M, int k, int H, const void* X, const int32_t* 
  * projection (N = 2F, F % 64 == 0).  Modes 2 and 3 need topk_w (f32 [M*k]) and row_pair; mode 3 also
  * needs k and adds into a caller-zeroed f32 [M, N] with atomics (sum order not fixed).
  * expert_offsets stays on the device; empty experts are legal.
+ * Two kernels serve the call.  4-bit weights with a few rows per expert, modes 0 to 2: the streaming kernel, numerics as in
+ * qgemm_small_m (exact integer products, the block's scale applied to the fp32 sum of each 32-block; fixed order).
+ * Otherwise, and whenever qg_set_schedule forces a token tile: the kernel of qgemm_dense, weights rounded to bf16 (q * scale).
  */
 int moe_grouped_qgemm(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, int K, const void* Ain,
                       const int32_t* expert_offsets, const void* Wq, const void* Wscale,
@@ -240,8 +243,10 @@ int moe_grouped_qgemm(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, int
  * projection over the tokens routed to it; here they are read where they lie, so the permuted copy Xperm and its
  * round trip through global memory never exist): row r of the input is X[row_pair[r] / k, :], X bf16 [M, K] in
  * token order.  Everything else - segments, weights, modes, outputs in sorted-row order - is as in
- * moe_grouped_qgemm; row_pair and k are always required.  Results are identical to
- * moe_permute followed by moe_grouped_qgemm.
+ * moe_grouped_qgemm; row_pair and k are always required.  Results are those of
+ * moe_permute followed by moe_grouped_qgemm: the same kernel serves both forms of a call, with the same bits where it is the
+ * streaming one (see moe_grouped_qgemm), and up to the order of the fp32 sums, which may differ from run to run in the last
+ * place, where it is the other.
  */
 int moe_grouped_qgemm_gather(qg_ctx* ctx, int mode, int qbits, int M, int R, int E, int N, int K, const void* X,
                              const int32_t* row_pair, int k, const int32_t* expert_offsets, const void* Wq,

@@ -157,7 +157,7 @@ def test_gather_in_load_equals_permute_then_gemm(name, qbits, M, H, E, F, k, ske
     util.assert_close(util.host_bf16_f64(Gp), o["GU"], "gathered plain")
     util.assert_close(util.host_bf16_f64(Hh), o["Hh"], "gathered gate/up+silu")
     util.assert_close(util.host_bf16_f64(y), o["y"], "layer (gather + accumulate)")
-    # and the two ways of feeding the kernel agree to the last bit on a stage with one k-block order per tile
+    # and the form for sorted rows against the same reference (bit equality of the two: test_gpu_stream.py)
     Xp = qg.moe_permute(dX, r["row_pair"], k)
     Hh2 = qg.moe_grouped_qgemm(qg.MODE_GATE_UP_SILU, qbits, Xp, r["offsets"], dW1q, dW1s)
     qg.poll_status()
