@@ -56,6 +56,7 @@ struct GemmParams {
     int* status;
     uint32_t wait_limit;        // polls per bounded wait (an unsatisfied poll lasts about 4 us)
     int skip_kb;                // test hook: k-block of the first tile whose activation load is left out (-1: none)
+    GroupedChoice choice;       // grouped: whether this launch has the work or the streaming kernel's in front of it
 #ifdef QG_PROFILE
     long long* stats;           // per-CTA cycle counters of a profiling build
 #endif
@@ -417,6 +418,23 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     // offsets, routing tables) or may still read (the output buffer) is touched only after pdl_wait().  The weights
     // are constants of the model, so in the dense case their producer and the dequantising warps start at once.
     pdl_launch_dependents();
+    if (SK == 0 && p.choice.on) {
+        // The streaming kernel in front lets this one start only when the offsets are there (it has waited for them), so they are
+        // read before its end, past the L1 cache, by every warp for itself: a launch that is not wanted ends before it has
+        // set anything up.
+        int chunks = 0, wide = 0;
+        for (int e = lane; e < p.E; e += 32) {
+            const int cnt = __ldcg(p.offsets + e + 1) - __ldcg(p.offsets + e);
+            chunks += (cnt + p.choice.chunk - 1) / p.choice.chunk;
+            wide += (cnt + 127) >> 7;
+        }
+        if (p.choice.streams(__reduce_add_sync(0xFFFFFFFFu, chunks), __reduce_add_sync(0xFFFFFFFFu, wide))) {
+            // the kernel behind this one waits for this one alone, so one pair waits for the kernel in front; the others
+            // leave their SMs to the kernel behind
+            if (blockIdx.x < 2) pdl_wait();
+            return;
+        }
+    }
     if (warp == 0) { QG_MARK(0); }
     QG_SPAN(0);
     const bool grouped = (p.offsets != nullptr);
@@ -1290,8 +1308,8 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     // kernel as the form for sorted rows, so that they give the same numbers
     if (qbits == QG_Q4 && mode <= QG_MODE_DOWN_WEIGHTED && ctx->force_bt == 0) {
         const int rc = qg::launch_moe_stream(ctx, mode, R, E, N, K, Ain, in_rows, gather_k, expert_offsets, Wq, Wscale, topk_w, row_pair, Out,
-                                             static_cast<cudaStream_t>(stream));
-        if (rc != QG_ERR_WORKSPACE) return rc;
+                                             p.choice, static_cast<cudaStream_t>(stream));
+        if (rc != QG_ERR_WORKSPACE && (rc != QG_OK || !p.choice.on)) return rc;
     }
     return qg::dispatch_gemm(ctx, qbits, bt, p, Ain, in_rows, Wq, Wscale, static_cast<cudaStream_t>(stream));
 }

@@ -95,10 +95,47 @@ int get_tmap_2d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_bytes, const void* base,
                 uint64_t inner, uint64_t rows, uint64_t planes, uint64_t plane_stride_bytes, uint32_t box_inner,
                 uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz, uint64_t row_stride_bytes = 0);
+// Which of its two kernels serves a grouped call with 4-bit weights: the streaming kernel when every expert has a few rows, the
+// tensor-memory kernel when they crowd into few experts, and how the rows are spread only the device knows.  The times are
+// fitted to 654 calls (14 shapes of 1 to 1024 experts; rows spread evenly, with a quarter of the experts preferred, over eight
+// experts, all with one): the faster kernel by them takes 1.02 of the faster one's time on average, 1.2 at worst.
+//   The host weighs three calls with evenly spread rows against one with all rows in one segment: the streaming kernel alone,
+// the other alone, or both, in which case each works out the same answer from the offsets and the one that is not wanted ends at
+// once.  That costs every such call 5 to 8 us (the unwanted launch keeps the next one from starting early).  128 experts,
+// 1536 x 2048: alone up to 11 rows per expert (even 63 us against 99, one segment 38 against 17 at eight rows), both up to 16,
+// the other from there (even 96 against 99, one segment 70 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
+// (even 741 us against 1117, eight segments 270 against 537 when the average alone decided).
+struct GroupedChoice {
+    enum Way { STREAM, OTHER, BOTH };
+    int on;                    // both kernels are launched
+    int chunk;                 // rows per tile of the streaming kernel, 8 or 16
+    int n_wt, stages;          // its weight tiles per expert and 256-k stages per tile
+    int sm_count;
+    // ns of each kernel; chunks: row tiles of all experts, wide: their tiles of 128 rows
+    __host__ __device__ long long stream_ns(long long chunks) const {
+        const long long ctas = 2 * sm_count, tiles = chunks * n_wt, waves = (tiles + ctas - 1) / ctas;
+        const long long halves = waves > 2 ? tiles + waves * ctas : 2 * waves * ctas;        // waves, in units of 1 / (2 ctas)
+        return 1300 + halves * stages * (chunk == 8 ? 1000 : 1300) / (2 * ctas) + waves * 1500;
+    }
+    __host__ __device__ long long other_ns(long long wide) const {
+        const long long pairs = sm_count / 2;
+        return 8000 + (wide * ((n_wt + 1) / 2) + pairs - 1) / pairs * stages * (4 * 271);
+    }
+    __host__ __device__ bool streams(long long chunks, long long wide) const { return stream_ns(chunks) <= other_ns(wide); }
+    static constexpr int MAX_ROWS = 18;       // per expert, on average: evenly spread, the other kernel is the faster one from there on
+    Way plan(long long R, long long E) const {
+        if (R > MAX_ROWS * E) return OTHER;
+        const long long used = R < E ? R : E, even = 2 * R <= chunk * E ? used : R / chunk + E / 2;
+        const long long gain = other_ns(used) - stream_ns(even), loss = stream_ns((R + chunk - 1) / chunk) - other_ns((R + 127) / 128);
+        const long long stream = loss > 0 ? loss : 0, other = gain > 0 ? 3 * gain : 0, both = 4 * (6000 + 10 * E);
+        if (stream <= other && stream <= both) return STREAM;
+        return other <= both ? OTHER : BOTH;
+    }
+};
 // The streaming kernel of the grouped GEMM (4-bit weights, modes 0 to 2), for a few rows per expert; QG_ERR_WORKSPACE if the
-// shape does not suit it.
+// shape does not suit it.  choice.on: the other kernel has to be launched behind it.
 int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, int in_rows, int gather_k, const int32_t* offsets,
-                      const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st);
+                      const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, GroupedChoice& choice, cudaStream_t st);
 // The same kernel for one matrix and up to sixteen tokens.
 int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void* A, const void* Wq, const void* Ws, void* Cout,
                         cudaStream_t st);

@@ -13,8 +13,8 @@
 // shared memory was the limit; 8-bit codes are twice the bytes per MMA).  The set with a tile's last stage adds the
 // other's sums and writes the result.  In gate/up mode an MMA tile is eight gate rows and the eight up rows that belong
 // to them: a thread ends up with both values of its outputs.
-//   More tiles than CTAs fit: the grid has a block per tile, and a CTA that is done with its tile takes over the tile of a block
-// that has not been started (cluster launch control; dealt out beforehand, the tiles left an SM up to 16 % more than its
+//   More tiles than CTAs fit: the grid has a block per tile, or per few tiles, and a CTA that is done with its block takes over
+// one that has not been started (cluster launch control; dealt out beforehand, the tiles left an SM up to 16 % more than its
 // share: nine tiles are too few to round).  The hardware keeps the count, nothing outlives the launch, so launches may
 // overlap on the GPU in any way.
 //   One matrix with fewer tiles: K is cut into slices, the slices of a tile are a thread-block cluster, and the cluster adds
@@ -68,9 +68,10 @@ constexpr int MS_X_BYTES = 8 * MS_SK * 2;             // eight token rows
 constexpr int MS_CONS_WARPS = 8, MS_THREADS = 32 * (MS_CONS_WARPS + 2);
 constexpr int MS_NT = 2;                              // most groups of eight segment rows per tile
 constexpr int MS_MAX_ST = 6;
-// Rows per expert, on average, up to which this kernel is the faster one (both projections: 145 us against 158 at sixteen
-// rows, 166 against 160 at twenty).
-constexpr int MS_MAX_ROWS = 18;
+// Most blocks of a launch, per SM: above that many tiles a block has several.  A CTA that runs out of tiles takes the blocks
+// beyond the last tile one by one, 0.33 us each, and with a block per tile there may be 50 for each of them (all rows with one
+// of 256 experts: 75 us against 60).  Fewer blocks are dealt out less evenly (8 per SM: 1946 us against 1506 for 17000 tiles).
+constexpr int MS_BLOCKS_PER_SM = 64;
 constexpr size_t MS_SMEM_MAX = 115712;                // half of an SM's shared memory: two CTAs per SM
 
 struct StreamParams {
@@ -79,6 +80,7 @@ struct StreamParams {
     int n_stages, stage_bytes;
     int kc;                     // k per CTA: K, or a slice of it when the CTAs of a cluster share a tile
     int dynamic;                // more blocks than fit at once: a CTA goes on with the tiles of blocks not yet started
+    GroupedChoice choice;       // grouped: whether this launch has the work or the one behind it
     const int32_t* offsets;     // grouped: device expert offsets [E + 1]
     __nv_bfloat16* out;
     const __nv_bfloat16* x;     // token rows, codes and scales once more, for ms_again
@@ -244,7 +246,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     int* off = reinterpret_cast<int*>(after + 16 + 16 * MS_MAX_ST);      // grouped: [E + 1] segment offsets
     int* prefix = off + p.E + 1;                                         // grouped: [E + 1] tiles before an expert
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_launch_dependents();
+    if (!GROUPED || !p.choice.on) pdl_launch_dependents();
     if (warp == 0) {
         if (lane < 2 * p.n_stages) mbar_init(full0 + 8u * lane, 2);
         if (lane < p.n_stages) { mbar_init(empty0 + 8u * lane, MS_CONS_WARPS / 2); mbar_init(xfull0 + 8u * lane, 1); }
@@ -257,13 +259,15 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     int total = p.n_wt;
     if constexpr (GROUPED) {
         pdl_wait();
+        if (p.choice.on) pdl_launch_dependents();      // the kernel behind this one reads the offsets as soon as it runs
         for (int e = threadIdx.x; e <= p.E; e += MS_THREADS) off[e] = p.offsets[e];
         __syncthreads();
         if (warp == 0) {
-            int carry = 0;
+            int carry = 0, wide = 0;
             for (int e0 = 0; e0 < p.E; e0 += 32) {
                 const int e = e0 + lane;
                 const int n = (e < p.E) ? (off[e + 1] - off[e] + TN - 1) / TN * p.n_wt : 0;
+                wide += (e < p.E) ? (off[e + 1] - off[e] + 127) >> 7 : 0;
                 int inc = n;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -273,6 +277,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 if (e < p.E) prefix[e] = carry + inc - n;
                 carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
             }
+            if (p.choice.on && !p.choice.streams(carry / p.n_wt, __reduce_add_sync(0xFFFFFFFFu, wide))) carry = 0;     // nothing to do
             if (lane == 0) prefix[p.E] = carry;
         }
         __syncthreads();
@@ -290,7 +295,8 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (lane == 0) {
             uint32_t slot = 0, phase = 0, fslot = 0;
             int sent = 0, ahead = 0;                   // stages filled, stages whose weights are on their way
-            uint32_t asked = 0;                        // requests for a tile so far, each a phase of taken_bar
+            uint32_t asked = 0;                        // answers to requests for a block so far, each a phase of taken_bar
+            bool more = p.dynamic, waiting = false;    // there may be blocks that have not been started; a request is on its way
             const int skip = (blockIdx.x == 0 && blockIdx.y == 0) ? p.skip_stage : -1;
             bool ok = true;
             auto load_weights = [&](uint32_t at, uint32_t bar, int st, const StreamTile& tl) {
@@ -312,12 +318,22 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 pdl_wait();
             }
             for (int t = blockIdx.x; ok; ) {
+                if (more && !waiting) {                // asked for early, used at the end of this block's tiles
+                    mbar_arrive_expect_tx(taken_bar, 16);
+                    clc_try_cancel(taken, taken_bar);
+                    waiting = true;
+                }
+                if (more && t >= total) {              // (blocks past the last tile are taken as well: started, they would cost more)
+                    uint32_t block = 0;
+                    ok = ms_wait(taken_bar, asked & 1u, abort_flag, p);
+                    ++asked;
+                    waiting = false;
+                    more = ok && clc_block(taken, block);
+                    if (more) t = static_cast<int>(block);
+                    continue;
+                }
                 StreamTile tl{0, 0, 0, 0};
                 if (t < total) {
-                    if (p.dynamic) {                   // asked for early, used at the end of this tile
-                        mbar_arrive_expect_tx(taken_bar, 16);
-                        clc_try_cancel(taken, taken_bar);
-                    }
                     if constexpr (GROUPED) {
                         int lo = 0, hi = p.E - 1;            // the last expert whose tiles start at or before t
                         while (lo < hi) {
@@ -369,18 +385,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     if (++fslot == 2u * p.n_stages) fslot = 0;
                 }
                 if (tl.n == 0) break;
-                // the block taken over, or none.  Blocks past the last tile (their number is an upper bound) are taken too, so that
-                // none of them is started.
-                t = total;
-                while (ok && p.dynamic) {
-                    ok = ms_wait(taken_bar, asked & 1u, abort_flag, p);
-                    ++asked;
-                    uint32_t block;
-                    if (!ok || !clc_block(taken, block)) break;
-                    if (block < static_cast<uint32_t>(total)) { t = static_cast<int>(block); break; }
-                    mbar_arrive_expect_tx(taken_bar, 16);
-                    clc_try_cancel(taken, taken_bar);
-                }
+                t += gridDim.x;
             }
         }
     } else if (warp == MS_CONS_WARPS + 1) {
@@ -597,11 +602,11 @@ static int ms_set_smem(qg_ctx* ctx, StreamKernel kern, int inst) {
     return QG_OK;
 }
 
-// The grouped call.  Returns QG_ERR_WORKSPACE if the shape does not suit this kernel (the caller takes the other one).
+// The grouped call, alone or (choice.on) with the other kernel behind it.  Returns QG_ERR_WORKSPACE if the shape does not suit
+// this kernel (the caller takes the other one).
 int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const void* Ain, int in_rows, int gather_k, const int32_t* offsets,
-                      const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, cudaStream_t st) {
+                      const void* Wq, const void* Ws, const float* topk_w, const int32_t* row_pair, void* Out, GroupedChoice& choice, cudaStream_t st) {
     const bool gate_up = mode == QG_MODE_GATE_UP_SILU;
-    if (R > static_cast<long long>(MS_MAX_ROWS) * E) return QG_ERR_WORKSPACE;
     StreamParams p{};
     p.R = R; p.N = N; p.K = K; p.E = E; p.kc = K;
     p.n_wt = gate_up ? N / 128 : (N + 127) / 128;
@@ -611,6 +616,14 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     const int ntm = (R <= 5LL * E) ? 1 : MS_NT;
     size_t smem = 0;
     if (!ms_layout(p, 4, ntm, E, smem)) return QG_ERR_WORKSPACE;
+    // at most one chunk per 8 ntm rows and one more per expert that has rows
+    const long long max_tiles = static_cast<long long>(R / (8 * ntm) + (R < E ? R : E)) * p.n_wt;
+    if (max_tiles > 0x3FFFFFFF) return QG_ERR_WORKSPACE;
+    p.choice.chunk = 8 * ntm; p.choice.n_wt = p.n_wt; p.choice.stages = K / MS_SK; p.choice.sm_count = ctx->sm_count;
+    const int way = p.choice.plan(R, E);
+    if (way == GroupedChoice::OTHER) return QG_ERR_WORKSPACE;
+    p.choice.on = way == GroupedChoice::BOTH;
+    choice = p.choice;
     p.offsets = offsets; p.out = static_cast<__nv_bfloat16*>(Out);
     p.x = static_cast<const __nv_bfloat16*>(Ain); p.wq = static_cast<const uint8_t*>(Wq); p.ws = static_cast<const __half*>(Ws);
     p.topk_w = (mode == QG_MODE_DOWN_WEIGHTED) ? topk_w : nullptr; p.row_pair = row_pair;
@@ -640,10 +653,8 @@ int launch_moe_stream(qg_ctx* ctx, int mode, int R, int E, int N, int K, const v
     rc = ms_set_smem(ctx, kern, ATTR_STREAM + which);
     if (rc != QG_OK) return rc;
     ctx->skip_kb = -1;                                        // the test hook acts on one launch
-    // at most one chunk per 8 ntm rows and one more per expert that has rows
-    const long long max_tiles = static_cast<long long>(R / (8 * ntm) + (R < E ? R : E)) * p.n_wt;
-    if (max_tiles > 0x7FFFFFFF) return QG_ERR_WORKSPACE;
-    const int grid = static_cast<int>(max_tiles);
+    const long long max_blocks = static_cast<long long>(MS_BLOCKS_PER_SM) * ctx->sm_count;
+    const int grid = static_cast<int>(max_tiles < max_blocks ? max_tiles : max_blocks);
     p.dynamic = grid > 2 * ctx->sm_count;
     if (launch_kernel(ctx, kern, dim3(grid), dim3(MS_THREADS), smem, st, tm_w, tm_s, tm_x, p) != cudaSuccess) {
         cudaGetLastError();
@@ -711,8 +722,9 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     if (rc != QG_OK) return rc;
     ctx->skip_kb = -1;
     p.dynamic = slices == 1 && tiles > 2 * ctx->sm_count;
+    const int blocks_x = tiles < MS_BLOCKS_PER_SM * ctx->sm_count ? tiles : MS_BLOCKS_PER_SM * ctx->sm_count;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles, slices); cfg.blockDim = dim3(MS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.gridDim = dim3(blocks_x, slices); cfg.blockDim = dim3(MS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute at[2];
     int n_at = 0;
     if (ctx->pdl) {

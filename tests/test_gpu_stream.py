@@ -259,7 +259,7 @@ def test_huge_tokens_in_short_segments(mode):
 
 
 @pytest.mark.parametrize("mode", [qg.MODE_PLAIN, qg.MODE_GATE_UP_SILU, qg.MODE_DOWN_WEIGHTED], ids=["plain", "gateup", "weighted"])
-@pytest.mark.parametrize("M,E,k,N,K", [(1, 4, 1, 128, 256), (3, 8, 2, 256, 512), (37, 5, 2, 384, 768), (70, 40, 8, 256, 1280), (256, 128, 8, 1536, 256)],
+@pytest.mark.parametrize("M,E,k,N,K", [(1, 4, 1, 128, 256), (3, 8, 2, 256, 512), (37, 5, 2, 384, 768), (70, 40, 8, 256, 1280), (100, 128, 8, 1536, 1024)],
                          ids=lambda v: str(v))
 def test_gathered_rows_give_the_bits_of_sorted_rows(M, E, k, N, K, mode):
     """Fewer rows than a copy of four, a tile of eight, a tile of sixteen; tokens used more than once; more tiles than CTAs."""
@@ -277,3 +277,111 @@ def test_gathered_rows_give_the_bits_of_sorted_rows(M, E, k, N, K, mode):
     b = qg.moe_grouped_qgemm_gather(mode, 4, dX, r["row_pair"], k, r["offsets"], dWq, dWs, topk_w=w)
     qg.poll_status()
     assert torch.equal(a.nan_to_num(7.0), b.nan_to_num(7.0))
+
+
+def spread(kind, R, E):
+    """R rows over E experts: evenly, preferring a few, all with one (not the first)."""
+    counts = np.zeros(E, np.int64)
+    if kind == "even":
+        counts[:] = R // E
+        counts[:R % E] += 1
+    elif kind == "few":
+        counts[::E // 4] = R // 4
+        counts[E - 1] += R - counts.sum()
+    else:
+        counts[E // 2] = R
+    return counts.tolist()
+
+
+@pytest.mark.parametrize("mode", [qg.MODE_PLAIN, qg.MODE_GATE_UP_SILU, qg.MODE_DOWN_WEIGHTED], ids=["plain", "gateup", "weighted"])
+@pytest.mark.parametrize("kind", ["even", "few", "one"])
+@pytest.mark.parametrize("R,E,N,K", [(449, 32, 3072, 3072), (160, 32, 6144, 3072), (320, 32, 2944, 3072)], ids=lambda v: str(v))
+def test_either_kernel_serves_uneven_segments(R, E, N, K, kind, mode):
+    """Sizes around which both kernels are launched and the offsets decide."""
+    counts = spread(kind, R, E)
+    offsets, A, _, _ = problem(counts, 8, K, 41)
+    Wq, Ws = synth.weights_q4(N, K, 41, 62), synth.scales(N, K // 32, 7, 41, 63)
+    Wq, Ws = np.stack([np.roll(Wq, e, 0) for e in range(E)]), np.stack([np.roll(Ws, e, 0) for e in range(E)])
+    rng = np.random.default_rng(42)
+    row_pair, w = rng.permutation(R).astype(np.int32), rng.uniform(0.1, 1.0, R).astype(np.float32)
+    X = np.empty_like(A)
+    X[row_pair] = A                                        # token order: row r is token row_pair[r]
+    dW, dO, dw, drp = (util.dev(Wq), util.dev_f16(Ws)), util.dev(offsets), util.dev(w), util.dev(row_pair)
+    g = util.Guarded((R, N // 2 if mode == qg.MODE_GATE_UP_SILU else N), torch.bfloat16)
+    for _ in range(3):                                     # back to back: a call's kernels overlap the next one's
+        qg.moe_grouped_qgemm(mode, 4, util.dev_bf16(A), dO, *dW, topk_w=dw, row_pair=drp, out=g.t)
+    b = qg.moe_grouped_qgemm_gather(mode, 4, util.dev_bf16(X), drp, 1, dO, *dW, topk_w=dw)
+    qg.poll_status()
+    assert g.intact() and not bool(g.untouched_inside().any().item())
+    cols = np.unique(np.concatenate([np.arange(0, N // 2, 29), np.arange(N // 2 - 130, N // 2)]))
+    if mode != qg.MODE_GATE_UP_SILU:
+        cols = np.concatenate([cols, cols + N // 2])
+    es = [e for e in range(E) if counts[e]][:: max(1, E // 8)]
+    for e in es:
+        seg = slice(int(offsets[e]), int(offsets[e + 1]))
+        rows = np.concatenate([cols, cols + N // 2]) if mode == qg.MODE_GATE_UP_SILU else cols
+        ref = orc.qgemm_dense(4, A[seg], np.ascontiguousarray(Wq[e][rows]), np.ascontiguousarray(Ws[e][rows]))
+        if mode == qg.MODE_GATE_UP_SILU:
+            ref = orc.silu_mul(ref)
+        elif mode == qg.MODE_DOWN_WEIGHTED:
+            ref = ref * w[row_pair[seg]].astype(np.float64)[:, None]
+        util.assert_close(util.host_bf16_f64(g.t[seg])[:, cols], ref, f"expert {e}")
+        util.assert_close(util.host_bf16_f64(b[seg])[:, cols], ref, f"expert {e}, gathered")
+
+
+def test_several_tiles_per_block():
+    """More tiles than a launch has blocks: a block's second tile, and blocks beyond the last tile."""
+    R, E, N, K = 64, 8, 131072, 256
+    A = util.dev_bf16(synth.activations(R, K, 44))
+    Wq = torch.randint(0, 256, (E, N, K // 2), dtype=torch.uint8, device="cuda")
+    Ws = torch.rand((E, N, K // 32), device="cuda").mul_(0.01).to(torch.float16)
+    for counts in (spread("even", R, E), spread("one", R, E)):
+        offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+        g = util.Guarded((R, N), torch.bfloat16)
+        qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, A, util.dev(offsets), Wq, Ws, out=g.t)
+        qg.poll_status()
+        assert g.intact() and not bool(g.untouched_inside().any().item())
+        for e in range(E):
+            q = torch.stack((Wq[e] & 15, Wq[e] >> 4), -1).flatten(-2).to(torch.float32) - 8
+            w = (q.unflatten(-1, (-1, 32)) * Ws[e].float()[..., None]).flatten(-2)
+            seg = slice(int(offsets[e]), int(offsets[e + 1]))
+            if counts[e]:
+                util.assert_close(util.host_bf16_f64(g.t[seg]), (A[seg].double() @ w.double().T).cpu().numpy(), f"expert {e}")
+
+
+@pytest.mark.parametrize("R,E,N,K", [(2304, 128, 1536, 2048), (1024, 256, 4096, 2048), (128, 8, 28672, 4096)], ids=lambda v: str(v))
+@pytest.mark.parametrize("kind", ["few", "one"])
+def test_uneven_segments_do_not_fall_behind_the_tensor_memory_kernel(R, E, N, K, kind):
+    """Rows that crowd into a few experts: the call takes about the time of the kernel that suits them, whatever their average
+    (1.5 times and 16 us are the cost of launching both, with room; the wrong kernel takes 2.7 to 4 times as long)."""
+    counts = spread(kind, R, E)
+    offsets, A, Wq, Ws = problem([R], 8, K, 43)            # random rows; any codes will do
+    offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    Wq = torch.randint(0, 256, (E, N, K // 2), dtype=torch.uint8, device="cuda")
+    Ws = torch.full((E, N, K // 32), 0.01, dtype=torch.float16, device="cuda")
+    args = (util.dev_bf16(A), util.dev(offsets), Wq, Ws)
+    out = torch.empty((R, N), dtype=torch.bfloat16, device="cuda")
+
+    def best():
+        graph = torch.cuda.CUDAGraph()
+        qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args, out=out)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            for _ in range(10):
+                qg.moe_grouped_qgemm(qg.MODE_PLAIN, 4, *args, out=out)
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(); graph.replay(); b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return min(times)
+
+    own = best()
+    qg.set_schedule(128, -1)
+    try:
+        forced = best()
+    finally:
+        qg.set_schedule(0, -1)
+    qg.poll_status()
+    assert own <= 1.5 * forced + 16.0, (own, forced)
