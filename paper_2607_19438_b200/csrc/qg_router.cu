@@ -199,10 +199,22 @@ router_logits_kernel_4(const __grid_constant__ CUtensorMap tm_x, const __grid_co
 
 // A few tokens: one block of eight warps per expert.  A thread multiplies its 16-byte pieces of the expert's row with every
 // token's (the tokens come from L2) and keeps RS_TOK sums in fp32; warps add by shuffles, then the block in warp order.  The
-// tensor-core kernel is four CTAs and their hand-overs here (128 experts x 2048, 4 / 32 / 64 / 128 tokens: 6.5 / 9.5 / 9.6 /
-// 9.9 us; this one 1.5 / 2.6 / 4.7 / 8.5).
+// tensor-core kernel is four CTAs and their hand-overs here (128 experts x 2048, 4 / 32 / 64 / 96 tokens: 5.9 / 8.9 / 9.1 /
+// 9.2 us; this one 2.5 / 4.1 / 5.8 / 8.1).
 constexpr int RS_TOK = 8;
 constexpr int RS_MAX_M = 96;
+// This kernel reads 9 rows of H per block of eight tokens and one expert from L2, the tensor-core kernel's time grows with its
+// up to 256 columns and, up to 32 tokens, with its rows.  Times in ns, fitted to 21 router shapes (8 to 1024 experts, H 64 to
+// 16384) of 1 to 96 tokens; the line lies at 80 tokens for 128 x 4096 (9.6 against 11.1 us; 96 tokens 12.3 against 11.2), 64 for 256 x
+// 4096, 48 for 256 x 7168 and at 8 for 1024 x 8192 (14.2 against 16.1; 96 tokens 115 against 21).  Below 256 columns of H the other
+// kernel has no slices to add and is the faster one from 1024 blocks on.
+static bool router_small(long long M, long long E, long long H) {
+    const long long blocks = E * ((M + RS_TOK - 1) / RS_TOK);
+    if (M > RS_MAX_M || (H < 256 && blocks > 1024)) return false;
+    const long long small = 1800 + H * 3 / 10 + blocks * (2200 + H * 83 / 100) / 1000;
+    const long long other = 2500 + H * 21 / 20 + (E < 256 ? E : 256) * (12 + 25 * (M < 32 ? M : 32) / 32);
+    return small <= other;
+}
 __global__ void __launch_bounds__(256)
 router_small_kernel(int M, int H8, int E, const uint4* __restrict__ X, const uint4* __restrict__ Wr, float* __restrict__ L) {
     __shared__ float part[8][RS_TOK];
@@ -255,7 +267,7 @@ int moe_router_logits(qg_ctx* ctx, int M, int H, int E, const void* X, const voi
     if (!X || !Wr || !logits) return QG_ERR_NULL;
     if (!qg::aligned16(X) || !qg::aligned16(Wr)) return QG_ERR_ALIGN;
     if (const int rc = qg::check_device(ctx)) return rc;
-    if (M <= qg::RS_MAX_M) {
+    if (qg::router_small(M, E, H)) {
         const cudaError_t le = qg::launch_kernel(ctx, qg::router_small_kernel, dim3(E, (M + qg::RS_TOK - 1) / qg::RS_TOK), dim3(256), 0,
                                                  static_cast<cudaStream_t>(stream), M, H / 8, E, static_cast<const uint4*>(X),
                                                  static_cast<const uint4*>(Wr), logits);
