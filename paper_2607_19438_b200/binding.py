@@ -269,19 +269,17 @@ def moe_grouped_qgemm_mx(mode, A_codes, A_sf, offsets, W_codes, W_sf, N, topk_w=
     return out
 
 
-def _route_outputs(M, E, k, H, dev, X, out):
+def _route_outputs(logits, k, X, out):
     """The output tensors of a routing call: the caller's (`out`, a dict with the same keys) or fresh ones."""
     if out is not None:
         return out
-    # the small integer outputs (and the weights, 32 bits as well) are one allocation: seven of them cost the host more
-    # than the four launches of the call
-    n = M * k
-    idx, w, row_pair, pair_row, counts, offsets = torch.empty(4 * n + 2 * E + 1, dtype=torch.int32, device=dev).split_with_sizes(
-        (n, n, n, n, E, E + 1))
-    o = dict(topk_idx=idx.view(M, k), topk_w=w.view(torch.float32).view(M, k), counts=counts, offsets=offsets,
-             row_pair=row_pair, pair_row=pair_row)
+    # One allocation each: 16-byte aligned as the header wants them, and a caller who changes one in place (scaled weights)
+    # touches no other's autograd version.  Views of a single one would save 2.3 us of host time (10.2 against 7.9).
+    (M, E), empty, i32 = logits.shape, logits.new_empty, torch.int32
+    o = dict(topk_idx=empty((M, k), dtype=i32), topk_w=empty((M, k), dtype=torch.float32), counts=empty(E, dtype=i32),
+             offsets=empty(E + 1, dtype=i32), row_pair=empty(M * k, dtype=i32), pair_row=empty(M * k, dtype=i32))
     if X is not None:
-        o["Xperm"] = torch.empty((M * k, H), dtype=torch.bfloat16, device=dev)
+        o["Xperm"] = empty((M * k, X.shape[1]), dtype=torch.bfloat16)
     return o
 
 
@@ -289,7 +287,7 @@ def moe_route(logits, k, X=None, ws=None, out=None):
     """logits f32 [M,E] -> dict(topk_idx, topk_w, counts, offsets, row_pair, pair_row[, Xperm])."""
     M, E = logits.shape
     H = X.shape[1] if X is not None else 0
-    out = _route_outputs(M, E, k, H, logits.device, X, out)
+    out = _route_outputs(logits, k, X, out)
     need = route_workspace_bytes(M, E, k)
     if ws is None:
         ws = torch.empty(max(need, 16), dtype=torch.uint8, device=logits.device)
@@ -307,7 +305,7 @@ def moe_route_static(logits, k, X=None, out=None):
     it allocates them for convenience.  Calls that overlap on the GPU share the array and would race."""
     M, E = logits.shape
     H = X.shape[1] if X is not None else 0
-    out = _route_outputs(M, E, k, H, logits.device, X, out)
+    out = _route_outputs(logits, k, X, out)
     lib, ctx, stream = _here()
     _check(lib.moe_route_static(ctx, M, E, k, _ptr(logits), _ptr(out["topk_idx"]), _ptr(out["topk_w"]),
                                 _ptr(out["counts"]), _ptr(out["offsets"]), _ptr(out["row_pair"]),
