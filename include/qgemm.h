@@ -83,13 +83,15 @@ size_t qg_route_workspace_bytes(int M, int E, int k);
  * Launch configuration of qgemm_dense (host only, nothing is launched): the token tile (128, 192 or 256) and whether
  * the call runs as stream-K, i.e. with the k-blocks of all output tiles dealt out evenly over the SM pairs and the
  * tiles that are cut in the middle summed through the context's scratch in a fixed order.  (With few tiles K may instead be
- * cut into slices that a thread-block cluster adds; that is reported as not stream-K, and any override of the two values
- * turns it off.)  The library chooses both per call from (M, N, K) with a cost model; qg_set_schedule overrides the choice for sweeps and tests:
+ * cut into slices that a thread-block cluster adds; that is reported as not stream-K, qg_plan_slices tells how many slices
+ * (1: none), and any override of the two values turns it off.  A launch of slices that the GPU refuses is done without, and its
+ * slice count is not planned again.)  The library chooses both per call from (M, N, K) with a cost model; qg_set_schedule overrides the choice for sweeps and tests:
  * token_tile 0 = model, else 128 / 192 / 256 (also applies to the grouped calls); streamk_mode -1 = model, 0 = never,
  * 1 = whenever the tile count is not a multiple of the SM-pair count.  The environment variables QG_FORCE_BT and
  * QG_STREAMK set the same two values when the context is created.
  */
 int qg_plan_dense(qg_ctx* ctx, int qbits, int M, int N, int K, int* token_tile, int* streamk);
+int qg_plan_slices(qg_ctx* ctx, int qbits, int M, int N, int K, int* slices);
 int qg_set_schedule(qg_ctx* ctx, int token_tile, int streamk_mode);
 
 /*

@@ -18,7 +18,7 @@ QG_Q8, QG_Q4 = 8, 4
 MODE_PLAIN, MODE_GATE_UP_SILU, MODE_DOWN_WEIGHTED, MODE_DOWN_ACCUM_F32 = 0, 1, 2, 3
 D_BF16, D_F32_ACC = 0, 1
 
-EXPORTS = ["qg_create", "qg_destroy", "qg_strerror", "qg_poll_status", "qg_test_inject", "qg_test_gemv_mode", "qg_plan_dense", "qg_set_schedule", "qg_route_workspace_bytes",
+EXPORTS = ["qg_create", "qg_destroy", "qg_strerror", "qg_poll_status", "qg_test_inject", "qg_test_gemv_mode", "qg_plan_dense", "qg_plan_slices", "qg_set_schedule", "qg_route_workspace_bytes",
            "qgemm_dense", "qgemm_small_m", "qgemm_dense_gate_up_silu", "prefill_attention",
            "qg_mx_scale_bytes", "qg_mx_quantize", "qg_mx_pack_weights", "qgemm_mx_dense",
            "moe_route", "moe_route_static", "moe_permute", "moe_grouped_qgemm", "moe_grouped_qgemm_gather", "moe_combine",
@@ -53,6 +53,7 @@ def load():
         lib.qg_test_inject.argtypes = [C.c_void_p, C.c_uint, C.c_int]
         lib.qg_test_gemv_mode.argtypes = [C.c_void_p, C.c_int]
         lib.qg_plan_dense.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int)]
+        lib.qg_plan_slices.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
         lib.qg_set_schedule.argtypes = [C.c_void_p, C.c_int, C.c_int]
         vp, ci = C.c_void_p, C.c_int
         lib.qgemm_dense.argtypes = [vp, ci, ci, ci, ci, vp, vp, vp, vp, vp]
@@ -149,6 +150,13 @@ def plan_dense(qbits, M, N, K):
     bt, sk = C.c_int(0), C.c_int(0)
     _check(load().qg_plan_dense(context(), qbits, M, N, K, C.byref(bt), C.byref(sk)), "qg_plan_dense")
     return bt.value, bool(sk.value)
+
+
+def plan_slices(qbits, M, N, K):
+    """K slices qgemm_dense would use for this shape (1: none)."""
+    n = C.c_int(0)
+    _check(load().qg_plan_slices(context(), qbits, M, N, K, C.byref(n)), "qg_plan_slices")
+    return n.value
 
 
 def set_schedule(token_tile: int = 0, streamk_mode: int = -1):

@@ -1029,7 +1029,9 @@ static int slices_capacity(qg_ctx* ctx, int slices) {
         ca.val.clusterDim.x = 2 * slices; ca.val.clusterDim.y = 1; ca.val.clusterDim.z = 1;
         q.gridDim = dim3(2 * slices); q.blockDim = dim3(NTHREADS); q.dynamicSmemBytes = smem; q.attrs = &ca; q.numAttrs = 1;
         int n = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        // a plan may be asked for with another device current: attribute and answer are those of the context's device
+        const OnDevice here(ctx->device);
+        if (!here.ok || cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess) { cudaGetLastError(); n = 0; }
         cached = n > 0 ? n : -1;
     }
@@ -1238,6 +1240,14 @@ int qg_plan_dense(qg_ctx* ctx, int qbits, int M, int N, int K, int* token_tile, 
     const qg::DensePlan plan = qg::plan_dense(ctx, qbits, M, (N + qg::BW - 1) / qg::BW, K);
     if (token_tile) *token_tile = ctx->force_bt ? ctx->force_bt : plan.bt;
     if (streamk) *streamk = (ctx->force_bt == 0 || ctx->streamk_mode == 1) ? plan.streamk : 0;
+    return QG_OK;
+}
+
+int qg_plan_slices(qg_ctx* ctx, int qbits, int M, int N, int K, int* slices) {
+    if (!ctx || !slices) return QG_ERR_NULL;
+    if (qbits != QG_Q8 && qbits != QG_Q4) return QG_ERR_SHAPE;
+    if (M < 1 || N < 8 || N % 8 || K < 256 || K % 256) return QG_ERR_SHAPE;
+    *slices = qg::plan_dense(ctx, qbits, M, (N + qg::BW - 1) / qg::BW, K).slices;
     return QG_OK;
 }
 

@@ -84,6 +84,17 @@ inline cudaError_t launch_kernel(const qg_ctx* ctx, void (*kern)(KArgs...), dim3
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 // QG_OK if the calling thread's current device is the context's, else QG_ERR_DEVICE.
 int check_device(const qg_ctx* ctx);
+// Makes the context's device the current one for a question about it, and leaves the caller's as it was.
+struct OnDevice {
+    int prev = -1;
+    bool ok;
+    explicit OnDevice(int device) {
+        ok = cudaGetDevice(&prev) == cudaSuccess && (prev == device || cudaSetDevice(device) == cudaSuccess);
+        if (prev == device) prev = -1;
+        if (!ok) cudaGetLastError();
+    }
+    ~OnDevice() { if (prev >= 0) cudaSetDevice(prev); }
+};
 // A 2-D row-major tensor map (inner = contiguous extent in elements, box in elements, row_stride_bytes = distance
 // between rows, 0 = packed): looked up in the context's cache, encoded on a miss, and copied to *out (the caller's own
 // copy: a later lookup may replace the cached entry).

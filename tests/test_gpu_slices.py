@@ -43,3 +43,27 @@ def test_a_wait_that_runs_out_in_one_slice():
     out = qg.qgemm_dense(qbits, *args)
     qg.poll_status()
     util.assert_close(util.host_bf16_f64(out), orc.qgemm_dense(qbits, A, Wq, Ws), "after a timeout")
+
+
+def test_a_plan_needs_no_current_device_and_leaves_it_alone():
+    """Planning on a fresh context, before any launch; with a second GPU, while that one is current: the plan is the same, and
+    the sliced launch that follows is not refused (the plan then still names its slices)."""
+    import ctypes as C
+    lib, shape = qg.load(), (8, 20, 2048, 4096)
+    want = qg.plan_slices(*shape)
+    assert want > 1
+    for dev in range(min(2, torch.cuda.device_count())):
+        h, n = C.c_void_p(), C.c_int(0)
+        assert lib.qg_create(C.byref(h), 0) == 0
+        with torch.cuda.device(dev):
+            assert lib.qg_plan_slices(h, *shape, C.byref(n)) == 0 and n.value == want
+            assert torch.cuda.current_device() == dev
+        A, Wq, Ws = synth.dense_problem(*shape, seed=25)
+        dA, dWq, dWs, out = util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws), torch.empty((20, 2048), dtype=torch.bfloat16, device="cuda")
+        assert lib.qgemm_dense(h, *shape, dA.data_ptr(), dWq.data_ptr(), dWs.data_ptr(), out.data_ptr(), None) == 0
+        assert lib.qg_poll_status(h, None) == 0
+        util.assert_close(util.host_bf16_f64(out), orc.qgemm_dense(8, A, Wq, Ws), "a context of its own")
+        assert lib.qg_plan_slices(h, *shape, C.byref(n)) == 0 and n.value == want
+        lib.qg_destroy(h)
+    assert lib.qg_plan_slices(qg.context(), 8, 20, 2044, 4096, C.byref(C.c_int(0))) == -2
+    assert lib.qg_plan_slices(qg.context(), *shape, None) == -1
