@@ -56,7 +56,6 @@ struct GemmParams {
     int* status;
     uint32_t wait_limit;        // polls per bounded wait (an unsatisfied poll lasts about 4 us)
     int skip_kb;                // test hook: k-block of the first tile whose activation load is left out (-1: none)
-    GroupedChoice choice;       // grouped: whether this launch has the work or the streaming kernel's in front of it
 #ifdef QG_PROFILE
     long long* stats;           // per-CTA cycle counters of a profiling build
 #endif
@@ -418,23 +417,6 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     // offsets, routing tables) or may still read (the output buffer) is touched only after pdl_wait().  The weights
     // are constants of the model, so in the dense case their producer and the dequantising warps start at once.
     pdl_launch_dependents();
-    if (SK == 0 && p.choice.on) {
-        // The streaming kernel in front lets this one start only when the offsets are there (it has waited for them), so they are
-        // read before its end, past the L1 cache, by every warp for itself: a launch that is not wanted ends before it has
-        // set anything up.
-        int chunks = 0, wide = 0;
-        for (int e = lane; e < p.E; e += 32) {
-            const int cnt = __ldcg(p.offsets + e + 1) - __ldcg(p.offsets + e);
-            chunks += (cnt + p.choice.chunk - 1) / p.choice.chunk;
-            wide += (cnt + 127) >> 7;
-        }
-        if (p.choice.streams(__reduce_add_sync(0xFFFFFFFFu, chunks), __reduce_add_sync(0xFFFFFFFFu, wide))) {
-            // the kernel behind this one waits for this one alone, so one pair waits for the kernel in front; the others
-            // leave their SMs to the kernel behind
-            if (blockIdx.x < 2) pdl_wait();
-            return;
-        }
-    }
     if (warp == 0) { QG_MARK(0); }
     QG_SPAN(0);
     const bool grouped = (p.offsets != nullptr);
@@ -1008,6 +990,28 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ C
              const __grid_constant__ CUtensorMap tm_s, const GemmParams p) {
     gemm_body<QBITS, BT, EPI, SK>(tm_x, tm_w, tm_s, p);
 }
+// Grouped, behind a launch of the streaming kernel: whether this one has the work follows from the offsets.
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+qgemm_choice_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                    const __grid_constant__ CUtensorMap tm_s, const GemmParams p, const GroupedChoice choice) {
+    pdl_launch_dependents();
+    // The kernel in front lets this one start only when the offsets are there (it has waited for them), so they are read before its
+    // end, past the L1 cache, by every warp for itself: a launch that is not wanted ends before it has set anything up.
+    int chunks = 0, wide = 0;
+    for (int e = threadIdx.x & 31; e < p.E; e += 32) {
+        const int cnt = __ldcg(p.offsets + e + 1) - __ldcg(p.offsets + e);
+        chunks += (cnt + choice.chunk - 1) / choice.chunk;
+        wide += (cnt + 127) >> 7;
+    }
+    if (choice.streams(__reduce_add_sync(0xFFFFFFFFu, chunks), __reduce_add_sync(0xFFFFFFFFu, wide))) {
+        // the kernel behind this one waits for this one alone, so one pair waits for the kernel in front; the others leave their
+        // SMs to the kernel behind
+        if (blockIdx.x < 2) pdl_wait();
+        return;
+    }
+    gemm_body<4, 128, EPI, 0>(tm_x, tm_w, tm_s, p);
+}
 // K slices: the launch names the cluster size (two CTAs per slice)
 template <int QBITS, int BT>
 __global__ void __launch_bounds__(NTHREADS, 1)
@@ -1040,7 +1044,7 @@ static int slices_capacity(qg_ctx* ctx, int slices) {
 
 template <int QBITS, int BT, int EPI, int SK>
 static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_rows, const void* Wq, const void* Ws,
-                       cudaStream_t st) {
+                       cudaStream_t st, const GroupedChoice* choice = nullptr) {
     using C = Cfg<QBITS, BT>;
     static_assert(C::SMEM_BYTES <= 232448, "shared memory budget");
     CUtensorMap tm_x, tm_w, tm_s;       // cached in the context: the same buffers recur every layer and step
@@ -1097,11 +1101,22 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
         if (p.streamk) max_tiles *= p.K / (4 * BK);      // units of four k-blocks: every pair gets at least one
         const long long pairs_hw = ctx->sm_count / 2;
         const int grid = 2 * static_cast<int>(max_tiles < pairs_hw ? max_tiles : pairs_hw);
-        if (launch_kernel(ctx, kern, dim3(grid), dim3(NTHREADS), C::SMEM_BYTES, st, tm_x, tm_w, tm_s, p) != cudaSuccess) {
-            cudaGetLastError();
-            return QG_ERR_CUDA;
+        cudaError_t e = cudaSuccess;
+        if constexpr (QBITS == 4 && BT == 128 && SK == 0 && EPI < 2) {
+            if (choice) {
+                if (!ctx->attr_set[ATTR_GEMM_CHOICE + EPI]) {
+                    e = cudaFuncSetAttribute(qgemm_choice_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+                    ctx->attr_set[ATTR_GEMM_CHOICE + EPI] = e == cudaSuccess;
+                }
+                if (e == cudaSuccess)
+                    e = launch_kernel(ctx, qgemm_choice_kernel<EPI>, dim3(grid), dim3(NTHREADS), C::SMEM_BYTES, st, tm_x, tm_w, tm_s, p, *choice);
+                if (e != cudaSuccess) cudaGetLastError();
+                return e == cudaSuccess ? QG_OK : QG_ERR_CUDA;
+            }
         }
-        return QG_OK;
+        e = launch_kernel(ctx, kern, dim3(grid), dim3(NTHREADS), C::SMEM_BYTES, st, tm_x, tm_w, tm_s, p);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess ? QG_OK : QG_ERR_CUDA;
     }
 }
 
@@ -1195,7 +1210,7 @@ static DensePlan plan_dense(qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
 }
 
 static int dispatch_gemm(qg_ctx* ctx, int qbits, int bt, const GemmParams& p_in, const void* X, int x_rows,
-                         const void* Wq, const void* Ws, cudaStream_t st) {
+                         const void* Wq, const void* Ws, cudaStream_t st, const GroupedChoice* choice = nullptr) {
     GemmParams p = p_in;
     if (ctx->force_bt) bt = ctx->force_bt;       // QG_FORCE_BT, read when the context was created (tile-shape sweeps)
     p.status = ctx->d_status;
@@ -1209,8 +1224,8 @@ static int dispatch_gemm(qg_ctx* ctx, int qbits, int bt, const GemmParams& p_in,
 #define QG_LAUNCH(Q, B)                                                                 \
     do {                                                                                \
         if (epi == 0 && p.streamk) return launch_gemm<Q, B, 0, 1>(ctx, p, X, x_rows, Wq, Ws, st);       \
-        if (epi == 0) return launch_gemm<Q, B, 0, 0>(ctx, p, X, x_rows, Wq, Ws, st);                    \
-        if (epi == 1) return launch_gemm<Q, B, 1, 0>(ctx, p, X, x_rows, Wq, Ws, st);                    \
+        if (epi == 0) return launch_gemm<Q, B, 0, 0>(ctx, p, X, x_rows, Wq, Ws, st, choice);            \
+        if (epi == 1) return launch_gemm<Q, B, 1, 0>(ctx, p, X, x_rows, Wq, Ws, st, choice);            \
         return launch_gemm<Q, B, 2, 0>(ctx, p, X, x_rows, Wq, Ws, st);                                  \
     } while (0)
     if (p.slices > 1) {
@@ -1316,12 +1331,13 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     const int bt = (R / E > 100) ? 192 : 128;
     // a few rows per expert (4-bit weights, no accumulation) the streaming kernel is faster; the gathering form takes the same
     // kernel as the form for sorted rows, so that they give the same numbers
+    qg::GroupedChoice choice{};
     if (qbits == QG_Q4 && mode <= QG_MODE_DOWN_WEIGHTED && ctx->force_bt == 0) {
         const int rc = qg::launch_moe_stream(ctx, mode, R, E, N, K, Ain, in_rows, gather_k, expert_offsets, Wq, Wscale, topk_w, row_pair, Out,
-                                             p.choice, static_cast<cudaStream_t>(stream));
-        if (rc != QG_ERR_WORKSPACE && (rc != QG_OK || !p.choice.on)) return rc;
+                                             choice, static_cast<cudaStream_t>(stream));
+        if (rc != QG_ERR_WORKSPACE && (rc != QG_OK || !choice.on)) return rc;
     }
-    return qg::dispatch_gemm(ctx, qbits, bt, p, Ain, in_rows, Wq, Wscale, static_cast<cudaStream_t>(stream));
+    return qg::dispatch_gemm(ctx, qbits, bt, p, Ain, in_rows, Wq, Wscale, static_cast<cudaStream_t>(stream), choice.on ? &choice : nullptr);
 }
 
 int moe_grouped_qgemm(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, int K, const void* Ain,

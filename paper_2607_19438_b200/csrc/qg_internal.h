@@ -34,7 +34,8 @@ enum AttrSlot {
     ATTR_MX_256 = 34,
     ATTR_STREAM = 35,       // 8: sorted, gathered rows x down, gate/up x rows per tile (2)
     ATTR_DENSE_STREAM = 43, // 4: format (2) x more than eight tokens (2)
-    ATTR_SLOTS = 47
+    ATTR_GEMM_CHOICE = 47,  // 2: epilogue
+    ATTR_SLOTS = 49
 };
 }  // namespace qg
 
