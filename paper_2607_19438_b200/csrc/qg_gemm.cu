@@ -1140,9 +1140,11 @@ static int slices_capacity(qg_ctx* ctx, int qbits, int bt, int slices) {
 // cluster that adds its partial tiles through distributed shared memory, divides the walk; the sum costs
 // 1100 + 1300 (slices - 2) cycles and 20 + 5 (slices - 2) per token of the tile (fitted to 25 shapes at 20 to 500 tokens, a
 // k-block being 515 cycles with up to 128 tokens and 600 with 192).  Stream-K's exchange through global memory costs 22000
-// on top of its share.  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four slices, so this
-// is for at most 33 tiles.  Measured, 20 / 128 tokens: 3072 x 3072 16.5 / 17.3 us whole, 10.0 / 12.3 in four slices;
-// 5120 x 3072 16.7 / 17.7, 11.3 / 13.3 in three; 2048 x 8192 24.8 / 30.1 (stream-K), 14.1 / 16.8 in four; 4096 x 14336
+// on top of its share.  Unless the alternative is stream-K, slices take SMs that the next launch could start on: 800 cycles from a
+// quarter of the SM pairs on and 3000 from 0.45 of them on (two slices, K = 1024, 17 tokens: 24 tiles 8.0 us against 7.5 whole, 32 tiles
+// 8.8 against 7.9, 16 tiles 6.7 against 7.4).  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four
+// slices, so this is for at most 33 tiles.  Measured, 20 / 128 tokens: 3072 x 3072 16.5 / 17.3 us whole, 10.0 / 12.3 in four
+// slices; 5120 x 3072 16.7 / 17.7, 11.3 / 13.3 in three; 2048 x 8192 24.8 / 30.1 (stream-K), 14.1 / 16.8 in four; 4096 x 14336
 // 29.2 / 34.1 (stream-K), 26.7 / 29.6 in three.
 static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePlan& plan) {
     if (ctx->force_bt || ctx->streamk_mode != -1) return;
@@ -1153,13 +1155,15 @@ static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePla
     auto period = [](int bt) { return bt == 128 ? 515.0 : bt == 192 ? 600.0 : 720.0; };
     double best = plan.streamk ? (tiles0 * nk4 + pairs - 1) / pairs * 4.0 * period(plan.bt) + 22000.0 : nk4 * 4.0 * period(plan.bt);
     best *= 0.97;
+    const bool streamk = plan.streamk != 0;
     for (int bt = 128; bt <= 192; bt += 64) {
         if (bt > 128 && M <= 128) break;
         const long long tiles = n_pw * ((M + bt - 1) / bt);
         for (int sl = 2; sl <= 4 && sl <= nk4 && tiles * sl <= pairs; ++sl) {
             const int per = (nk4 + sl - 1) / sl;
             if ((nk4 + per - 1) / per != sl) continue;             // the same cut as a smaller count
-            const double cost = per * 4.0 * period(bt) + 1100.0 + 1300.0 * (sl - 2) + (20.0 + 5.0 * (sl - 2)) * (M < bt ? M : bt);
+            const double cost = per * 4.0 * period(bt) + 1100.0 + 1300.0 * (sl - 2) + (20.0 + 5.0 * (sl - 2)) * (M < bt ? M : bt) +
+                                (streamk || 4 * tiles * sl < pairs ? 0.0 : 20 * tiles * sl < 9 * pairs ? 800.0 : 3000.0);
             if (cost < best && slices_capacity(ctx, qbits, bt, sl) >= tiles) {
                 best = cost;
                 plan = DensePlan{bt, 0, sl, 4 * per};
