@@ -129,7 +129,7 @@ int qgemm_dense_gate_up_silu(qg_ctx* ctx, int qbits, int M, int F, int K, const 
  * The same product for 1 <= M <= 16 tokens (else QG_ERR_SHAPE): the decode-side and small verification-batch
  * regime that Sec. 2.3 describes as bound by memory bandwidth and Sec. 5.2 names as future work for the tensor
  * path.  Every weight byte is used once, so this call streams the packed weights: a kernel whose weights arrive through a
- * TMA-fed shared-memory ring, and for matrices below 256 K codes a block kernel.  Both add in a fixed order (K slices in
+ * TMA-fed shared-memory ring, and a block kernel for matrices below 256 K codes, of K = 256 or of a few very long rows.  Both add in a fixed order (K slices in
  * slice order across CTAs), so results do not depend on scheduling.  Same formats and constraints as qgemm_dense, fp32
  * accumulation.  Numerics: the streaming kernel multiplies the exact integers q and applies the block's scale to the fp32
  * sum of each 32-block, which is closer to the exact value than weights rounded to bf16 (q * scale), as the block kernel and

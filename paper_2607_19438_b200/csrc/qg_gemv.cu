@@ -1,5 +1,5 @@
 // Small-batch (1..16 tokens) block-quantised GEMM for sm_100a: the entry point of qgemm_small_m and the kernel that serves
-// its smallest matrices (qg_stream.cu serves the others).
+// its smallest, shallowest and longest matrices (qg_stream.cu serves the others).
 //
 // Operation: C[m, n] = sum_k A[m, k] * q[n, k] * scale[n, k/32], the definition of qgemm_dense, for M <= 16.
 //
@@ -39,11 +39,6 @@ __device__ __forceinline__ uint4 ldg_stream128(const void* p) {
 __device__ __forceinline__ uint2 ldg_stream64(const void* p) {
     uint2 v;
     asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ uint32_t ldg_stream32(const void* p) {
-    uint32_t v;
-    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 
@@ -212,10 +207,17 @@ extern "C" int qgemm_small_m(qg_ctx* ctx, int qbits, int M, int N, int K, const 
     if (!A || !Wq || !Wscale || !Cout) return QG_ERR_NULL;
     if (!qg::aligned16(A) || !qg::aligned16(Wq) || !qg::aligned16(Wscale) || !qg::aligned16(Cout)) return QG_ERR_ALIGN;
     if (const int rc = qg::check_device(ctx)) return rc;
-    // The streaming kernel (qg_stream.cu) serves all but the smallest matrices: below 256 K codes there is nothing to keep
-    // a ring busy with, and its set-up costs more than the block kernel above takes (256 x 256, one token: 2.9 us against
-    // 2.1; 512 x 512 4.6 either way; 2048 x 1024 4.8 against 5.8; 1024 x 8192 6.9 against 11.8).
-    const bool small = static_cast<long long>(N) * K < (1LL << 18);
+    // The streaming kernel (qg_stream.cu) serves all but three kinds of matrices, 1 / 16 tokens, stream against block:
+    //  - below 256 K codes there is nothing to keep a ring busy with, and its set-up costs more than the block kernel above
+    //    takes (256 x 256 2.9 us against 2.1; 512 x 512 3.6 / 4.0 against 4.2 / 5.1; 1024 x 1024 3.6 / 4.7 against 4.3 / 5.3);
+    //  - K = 256 is one stage per tile, two barrier round trips for 16 KB, as long as the rows fill the GPU no more than about
+    //    once: 8 bit 8192 rows 3.4 / 4.2 us against 2.9 / 2.9, 24576 5.2 / 5.5 against 3.4 / 3.8, 32768 5.4 / 5.9 against 6.0 / 6.8; 4 bit
+    //    12288 3.5 / 4.3 against 2.6 / 2.9, 16384 3.7 / 4.5 against 3.9 / 4.3;
+    //  - a long K over a few rows: eight slices of a cluster against up to 32 of the block kernel (16 x 16384 6.7 / 8.6 us against
+    //    8.1 / 8.7, 16 x 32768 10.3 / 13.8 against 8.7 / 9.3, 128 x 32768 10.3 / 13.9 against 10.5 / 12.0, 128 x 65536 17.9 / 23.6
+    //    against 14.3 / 16.8, 256 x 32768 10.6 / 13.9 against 13.8 / 15.6).
+    const bool small = static_cast<long long>(N) * K < (1LL << 18) || (K == 256 && N <= (qbits == QG_Q8 ? 24576 : 12288)) ||
+                       (K <= 32 * qg::GV_MAX_KS && ((N <= 32 && K >= 24576) || (N <= 128 && K >= 32768)));
     const bool always_stream = (ctx->gemv_mode & 2) != 0, never_stream = (ctx->gemv_mode & 4) != 0;
     if ((!small || always_stream) && !never_stream)
         return qg::launch_dense_stream(ctx, qbits, M, N, K, A, Wq, Wscale, Cout, static_cast<cudaStream_t>(stream));

@@ -155,3 +155,36 @@ def test_gemv_mode_hook_rejects_contradictory_bits():
         assert e.value.code == -2
     qg.test_gemv_mode(5)          # never the ring kernel, and no clusters: accepted
     qg.test_gemv_mode(0)
+
+
+@pytest.mark.parametrize("qbits,M,N,K", [(8, 16, 1536, 256), (4, 16, 1536, 256), (8, 3, 24576, 256), (4, 16, 16, 32768), (8, 16, 128, 32768), (8, 1, 8, 65536),
+                                         (8, 2, 16, 65792)], ids=lambda v: str(v))
+def test_shallow_and_long_matrices(qbits, M, N, K):
+    """One stage per tile, and a few rows of a very long K (the last one beyond the slices of the block kernel): right, the same
+    bits again, and no slower than the faster of the two kernels by more than 1.25 times and 0.5 us (the wrong one takes 1.4 times)."""
+    A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=26)
+    args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
+    g = util.Guarded((M, N), torch.bfloat16)
+    qg.qgemm_small_m(qbits, *args, out=g.t)
+    again = qg.qgemm_small_m(qbits, *args)
+    qg.poll_status()
+    assert g.intact() and torch.equal(again, g.t)
+    util.assert_close(util.host_bf16_f64(g.t), orc.qgemm_dense(qbits, A, Wq, Ws), "shallow or long")
+    times = {}
+    for mode in (0, 2, 4):
+        if mode == 4 and K > 65536:
+            continue
+        qg.test_gemv_mode(mode)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(20):
+                qg.qgemm_small_m(qbits, *args, out=g.t)
+        best = 1e9
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(); graph.replay(); b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 50)
+        times[mode] = best
+    qg.poll_status()
+    assert times[0] <= 1.25 * min(times.values()) + 0.5, times
