@@ -116,3 +116,49 @@ def test_router_time_does_not_fall_with_the_97th_token(E, H):
     limit = 1.3 * best(97) + 1.0
     assert best(96) <= limit and best(32) <= limit
     qg.poll_status()
+
+
+@pytest.mark.parametrize("M,E,k,H", [(1, 4, 1, 8), (300, 16, 1, 64), (257, 8, 2, 520), (5, 64, 9, 136), (33, 256, 64, 4096), (600, 16, 16, 1032), (40, 16, 3, 24576), (2047, 8, 2, 512), (2048, 8, 2, 512)],
+                         ids=lambda v: str(v))
+def test_row_copies(M, E, k, H):
+    """Rows of fewer vectors than a block has threads and of more, slots in one group of eight, in a group and one, in eight groups,
+    on both sides of the sizes that a warp per row serves: bit copies, and nothing outside."""
+    logits, X = synth.router_logits(M, E, 51), synth.activations(M, H, 51)
+    r = qg.moe_route(util.dev(logits), k)
+    g = util.Guarded((M * k, H), torch.bfloat16)
+    qg.moe_route(util.dev(logits), k, X=util.dev_bf16(X), out=dict(r, Xperm=g.t))
+    qg.poll_status()
+    assert g.intact()
+    assert np.array_equal(util.host_bf16_bits(g.t), X[r["row_pair"].cpu().numpy() // k])
+
+
+@pytest.mark.parametrize("M,E,k,H", [(8192, 16, 1, 64), (8192, 8, 1, 128), (32, 256, 64, 4096), (128, 16, 16, 8192), (8192, 16, 2, 512)], ids=lambda v: str(v))
+def test_row_copies_are_no_slower_than_a_gather(M, E, k, H):
+    """Routing with the row copy against routing and moe_permute (a warp per row): 1.1 times and 1 us are several times what the
+    timings scatter; one block per token took up to 1.57 times as long."""
+    logits, X = torch.randn((M, E), device="cuda"), torch.randn((M, H), device="cuda").to(torch.bfloat16)
+    r = qg.moe_route(logits, k, X=X)
+    ws = torch.empty(max(16, qg.route_workspace_bytes(M, E, k)), dtype=torch.uint8, device="cuda")
+    plain = {n: t for n, t in r.items() if n != "Xperm"}
+
+    def best(call):
+        graph = torch.cuda.CUDAGraph()
+        call()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            for _ in range(20):
+                call()
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(); graph.replay(); b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 50)
+        return min(times)
+
+    def apart():
+        qg.moe_route(logits, k, ws=ws, out=plain)
+        qg.moe_permute(X, r["row_pair"], k, out=r["Xperm"])
+
+    assert best(lambda: qg.moe_route(logits, k, X=X, ws=ws, out=r)) <= 1.1 * best(apart) + 1.0
+    qg.poll_status()
