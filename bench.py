@@ -866,8 +866,8 @@ def run_ours(args):
         }
         if cpu is not None:
             line["cpu_baseline"] = cpu
-        if sweep is not None:
-            line["sweep"] = sweep
+        # The result is one short line; the per-call and per-configuration tables, tens of kilobytes, go to the error output.
+        print(json.dumps({"kernels": line.pop("kernels"), "sweep": sweep}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()

@@ -14,7 +14,12 @@
  *     (a cudaStream_t passed as void*; NULL = the legacy default stream);
  *   - the context's device must be the calling thread's current device (else QG_ERR_DEVICE); a
  *     context and its calls belong to one host thread and one stream at a time (it caches tensor
- *     maps and owns the partial-sum scratch of qgemm_small_m and qgemm_dense);
+ *     maps and owns the partial-sum scratch of qgemm_small_m's block kernel and of stream-K qgemm_dense calls; launches of
+ *     the other kernels share nothing);
+ *   - a call may start while the kernel before it on its stream still runs; it reads and writes nothing that kernel may touch
+ *     until it has ended, with one exception: the quantised weights (Wq, Wscale) of qgemm_dense, qgemm_dense_gate_up_silu
+ *     and qgemm_small_m are taken for constants and may be read earlier, so whoever writes them has to be done before the call
+ *     in front of the reading one starts (a model is loaded, then any other call: that is enough);
  *   - return value: QG_OK (0) or a negative QG_ERR_* code; an error is detected before anything is
  *     launched, so the outputs are untouched; nothing aborts, traps or throws;
  *   - there is no fallback path: a shape the kernels do not accept is an error (the paper's

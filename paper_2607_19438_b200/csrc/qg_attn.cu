@@ -31,7 +31,7 @@ namespace qg {
 constexpr int AT_BQ = 128, AT_BKV = 128, AT_THREADS = 320;
 // One pair of exponentials in eight goes to the FMA pipe.  The row's warp is bound by the chain of its own instructions as much
 // as by the 16 exponentials per clock and SM, and a polynomial is thirteen instructions for a pair: with one in eight 1500
-// positions take 31.9 us against 32.5 and 8192 (causal, 32 heads) 488 against 497, with two 34.6 and 525, with four 38.5 and 590.
+// positions take 31.7 us against 32.3 and 8192 (causal, 32 heads) 488 against 497, with two 34.6 and 525, with four 38.5 and 590.
 constexpr int AT_POLY_OF = 8;
 
 struct AttnParams {

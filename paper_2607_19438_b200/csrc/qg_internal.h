@@ -68,8 +68,9 @@ struct qg_ctx {
 
 namespace qg {
 // Launches `kern`; with ctx->pdl the launch carries the programmatic-serialization attribute, so the kernel's prologue
-// may overlap the tail of the kernel before it in the stream (every kernel of this library calls pdl_wait() before it
-// reads or writes anything an earlier kernel may touch).
+// may overlap the tail of the kernel before it in the stream.  Every kernel of this library calls pdl_wait() before it reads
+// or writes anything an earlier kernel may touch, except quantised weights, which no kernel of this library writes: the GEMMs
+// that take codes and scales request their first ones before the wait.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(const qg_ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                  cudaStream_t st, Args&&... args) {

@@ -140,7 +140,7 @@ SMALL_M = [(8, M, N, K) for M in (1, 4, 16) for N, K in ((2560, 2048), (2048, 20
 
 @pytest.mark.parametrize("qbits,M,N,K", SMALL_M, ids=[f"q{c[0]}-{c[1]}x{c[2]}x{c[3]}" for c in SMALL_M])
 def test_small_m_full_size_sampled_rows(qbits, M, N, K):
-    """All tokens against a sample of weight rows: a few in every 128-row tile (the unit a CTA of the ring kernel owns),
+    """All tokens against a sample of weight rows: a few in every 128-row tile (the unit a CTA of the streaming kernel owns),
     the first and the last rows."""
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=3)
     out = qg.qgemm_small_m(qbits, util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))

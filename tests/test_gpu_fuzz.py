@@ -128,9 +128,9 @@ def test_fuzz_route_and_layer(i):
 
 @pytest.mark.parametrize("i", range(24))
 def test_fuzz_small_m(i):
-    """Random ragged shapes through qgemm_small_m with the kernel choice forced in turn (library's choice, ring kernel
-    with clusters, ring kernel with the scratch): tiles that end inside a 128-row block, K that does not divide into
-    equal slices or phases, every token count."""
+    """Random ragged shapes through qgemm_small_m with the kernel choice forced in turn (library's choice, streaming
+    kernel with K slices, with K whole): tiles that end inside a 128-row block, K that does not divide into equal slices, every
+    token count."""
     r = _rng(500 + i)
     qbits = int(r.choice([4, 8]))
     M = int(r.integers(1, 17)); N = 8 * int(r.integers(1, 400)); K = 256 * int(r.integers(1, 25))

@@ -1,5 +1,6 @@
-"""qgemm_dense with K cut into slices that a thread-block cluster adds (few tiles): every slice count and token tile, ragged
-rows and tokens, against the oracle."""
+"""qgemm_dense with K cut into slices that a thread-block cluster adds (few tiles): two to four slices, token tiles of 128 and 192
+rows in both formats, ragged rows and tokens, against the oracle.  Each case first asks whether the call will be sliced, and
+afterwards that the GPU has not refused the launch."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +15,8 @@ pytestmark = pytest.mark.gpu
 # the end in the last tile, tokens around the edges of the 16-token blocks and of the 128- and 192-token tiles
 SHAPES = [(8, 17, 256, 2048), (4, 20, 3072, 3072), (8, 128, 2184, 2560), (4, 129, 1152, 1280), (8, 127, 136, 8192),
           (4, 192, 2048, 2048), (8, 333, 2048, 2048), (4, 500, 2560, 2048), (8, 193, 4096, 4096), (4, 64, 5120, 3072),
-          (8, 1, 512, 1024), (4, 16, 8, 512)]
+          (8, 1, 512, 1024), (4, 16, 8, 512), (8, 500, 2560, 2048), (8, 64, 136, 8192)]
+WHOLE = (8, 127, 136, 8192)                              # stream-K is expected to be faster there
 
 
 @pytest.mark.parametrize("qbits,M,N,K", SHAPES, ids=[f"q{q}-{m}x{n}x{k}" for q, m, n, k in SHAPES])
@@ -22,9 +24,12 @@ def test_slices_match_the_oracle(qbits, M, N, K):
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=23)
     g = util.Guarded((M, N), torch.bfloat16)
     args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
+    planned = qg.plan_slices(qbits, M, N, K)
+    assert (planned > 1) == ((qbits, M, N, K) != WHOLE)
     for _ in range(3):                                   # back to back: a launch's start overlaps the end of the one before
         qg.qgemm_dense(qbits, *args, out=g.t)
     qg.poll_status()
+    assert qg.plan_slices(qbits, M, N, K) == planned     # a refused launch would not be planned again
     assert g.intact() and not bool(g.untouched_inside().any().item())
     rows = np.unique(np.concatenate([np.arange(0, N, max(1, N // 500)), np.arange(max(0, N - 140), N)]))
     util.assert_close(util.host_bf16_f64(g.t)[:, rows], orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows]), "slices")
@@ -32,6 +37,7 @@ def test_slices_match_the_oracle(qbits, M, N, K):
 
 def test_a_wait_that_runs_out_in_one_slice():
     qbits, M, N, K = 8, 40, 2048, 4096
+    assert qg.plan_slices(qbits, M, N, K) > 1
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=24)
     args = (util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws))
     try:
@@ -76,3 +82,10 @@ def test_short_k_over_many_tiles_is_not_sliced(M, N, K):
     whole, 10.1 against 8.5 at 128 tokens)."""
     assert qg.plan_slices(8, M, N, K) == 1 and qg.plan_slices(4, M, N, K) == 1
     assert qg.plan_slices(8, M, 4096, 4096) > 1 and qg.plan_slices(8, M, 5120, 3072) > 1
+
+
+def test_the_cases_cover_every_instantiation():
+    """Both formats with both token tiles, and two, three and four slices."""
+    plans = {(q, qg.plan_dense(q, m, n, k)[0]) for q, m, n, k in SHAPES if (q, m, n, k) != WHOLE}
+    assert plans == {(8, 128), (8, 192), (4, 128), (4, 192)}
+    assert {qg.plan_slices(*s) for s in SHAPES} == {1, 2, 3, 4}

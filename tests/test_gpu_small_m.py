@@ -1,6 +1,6 @@
 """GPU parity of qgemm_small_m (1..16 tokens, the weight-streaming call) against the fp64 oracle, through each of the
-kernels that can serve it: the TMA-fed ring kernel with its K slices added through a thread-block cluster or through
-the scratch, the small-block kernel, and the library's own choice."""
+kernels that can serve it: the streaming kernel with K in slices that a thread-block cluster adds or left whole, the block
+kernel, and the library's own choice."""
 import numpy as np
 import pytest
 import torch
@@ -17,8 +17,8 @@ SHAPES = [
     (4, 3, 136, 768), (8, 7, 2560, 2048), (4, 16, 72, 4096), (8, 2, 2048, 8192), (4, 9, 1536, 2304),
     (8, 8, 1096, 5120),        # K slices of unequal length, a ragged last tile
 ]
-# qg_test_gemv_mode: the library's choice, the ring kernel with and without clusters, the other kernels
-MODES = [(0, "auto"), (2, "ring"), (3, "ring-scratch"), (4, "no-ring")]
+# qg_test_gemv_mode: the library's choice, the streaming kernel with K slices and with K whole, the block kernel
+MODES = [(0, "auto"), (2, "stream"), (3, "stream-whole-k"), (4, "block")]
 
 
 @pytest.fixture(autouse=True)
@@ -40,18 +40,17 @@ def test_small_m_parity_and_guards(qbits, M, N, K, mode, mname):
     ref = orc.qgemm_dense(qbits, A, Wq, Ws)
     mx, rmax, fro = util.assert_close(util.host_bf16_f64(g.t), ref, f"small-M q{qbits} {M}x{N}x{K} {mname}")
     assert fro > 1e-4
-    # fixed-order sums over the K phases and slices: a second run gives the same bits
+    # fixed-order sums over the K slices: a second run gives the same bits
     again = qg.qgemm_small_m(qbits, dA, dWq, dWs)
     qg.poll_status()
     assert torch.equal(again, g.t)
 
 
 @pytest.mark.parametrize("qbits,M,N,K", [(4, 3, 19200, 4096), (8, 8, 19072, 6144), (8, 12, 18944, 2304)],
-                         ids=["q4-two-phases", "q8-three-phases", "q8-16-tokens-two-phases"])
-def test_small_m_ring_kernel_many_tiles_and_k_phases(qbits, M, N, K):
-    """As many row tiles as SMs and K longer than the token slice a CTA keeps in shared memory: every CTA walks its
-    tiles once per K phase and carries fp32 sums from phase to phase.  Sampled rows against the oracle, guards, and
-    the same bits on a second run."""
+                         ids=["q4", "q8", "q8-16-tokens"])
+def test_small_m_many_tiles_and_stages(qbits, M, N, K):
+    """About as many row tiles as the GPU has places for CTAs, or a few more, and more stages than the ring holds.  Sampled rows
+    against the oracle, guards, and the same bits on a second run."""
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=9)
     dA, dWq, dWs = util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws)
     g = util.Guarded((M, N), torch.bfloat16)
@@ -62,16 +61,16 @@ def test_small_m_ring_kernel_many_tiles_and_k_phases(qbits, M, N, K):
     rng = np.random.default_rng(5)
     rows = np.unique(np.concatenate([rng.integers(0, N, 600), np.arange(0, 300), np.arange(N - 300, N)]))
     ref = orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows])
-    util.assert_close(util.host_bf16_f64(g.t)[:, rows], ref, f"ring kernel q{qbits} {M}x{N}x{K}")
+    util.assert_close(util.host_bf16_f64(g.t)[:, rows], ref, f"streaming kernel q{qbits} {M}x{N}x{K}")
     again = qg.qgemm_small_m(qbits, dA, dWq, dWs)
     qg.poll_status()
     assert torch.equal(again, g.t)
 
 
 @pytest.mark.parametrize("qbits,M,N,K,mode,skip", [(8, 4, 2048, 2048, 2, 1), (4, 16, 3072, 8192, 3, 0), (8, 3, 19072, 4096, 2, 5)],
-                         ids=["cluster", "scratch-and-tickets", "phases"])
-def test_small_m_ring_kernel_wait_that_runs_out(qbits, M, N, K, mode, skip):
-    """The ring kernel's bounded waits: its first CTA never loads one weight stage, the consumers' wait for it expires,
+                         ids=["slices", "whole-k", "many-tiles"])
+def test_small_m_wait_that_runs_out(qbits, M, N, K, mode, skip):
+    """The streaming kernel's bounded waits: its first CTA never loads one stage's token rows, the consumers' wait for it expires,
     the launch ends with QG_ERR_TIMEOUT in the status word (every warp walks through the remaining barriers, the other
     CTAs of its cluster are not left waiting), and the next call on the context is correct."""
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=14)
@@ -90,7 +89,7 @@ def test_small_m_ring_kernel_wait_that_runs_out(qbits, M, N, K, mode, skip):
     util.assert_close(util.host_bf16_f64(out)[:, rows], orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows]), "after a timeout")
 
 
-@pytest.mark.parametrize("mode", [2, 4], ids=["ring", "no-ring"])
+@pytest.mark.parametrize("mode", [2, 4], ids=["stream", "block"])
 @pytest.mark.parametrize("qbits", [8, 4])
 def test_small_m_integer_exact_is_bit_exact(qbits, mode):
     M, N, K = 11, 264, 512
@@ -111,7 +110,7 @@ def test_small_m_integer_exact_is_bit_exact(qbits, mode):
     assert np.array_equal(util.host_bf16_bits(out), orc.f64_to_bf16(ref))
 
 
-@pytest.mark.parametrize("mode", [2, 4], ids=["ring", "no-ring"])
+@pytest.mark.parametrize("mode", [2, 4], ids=["stream", "block"])
 @pytest.mark.parametrize("qbits", [8, 4])
 def test_small_m_extreme_scales_and_argument_checks(qbits, mode):
     M, N, K = 4, 128, 512
@@ -137,15 +136,14 @@ def test_small_m_extreme_scales_and_argument_checks(qbits, mode):
 
 @pytest.mark.parametrize("qbits,M,N,K", [(8, 16, 16384, 2048), (4, 16, 6144, 8192), (8, 12, 4096, 14336)],
                          ids=["q8-many-rows", "q4-48M-weights", "q8-long-k"])
-def test_small_m_large_matrices_take_the_prefill_kernel(qbits, M, N, K):
-    """With more than eight tokens, at 16384 rows or 48 M weights and more, the call is served by qgemm_dense's kernel (same numerics; the last bf16
-    place may differ between runs, so only the oracle comparison and the guards are asserted)."""
+def test_small_m_large_matrices(qbits, M, N, K):
+    """Large matrices and more than eight tokens: every row against the oracle, and the guards."""
     A, Wq, Ws = synth.dense_problem(qbits, M, N, K, seed=7)
     g = util.Guarded((M, N), torch.bfloat16)
     qg.qgemm_small_m(qbits, util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws), out=g.t)
     qg.poll_status()
     assert g.intact() and not bool(g.untouched_inside().any().item())
-    util.assert_close(util.host_bf16_f64(g.t), orc.qgemm_dense(qbits, A, Wq, Ws), f"small-M via prefill kernel q{qbits} {M}x{N}x{K}")
+    util.assert_close(util.host_bf16_f64(g.t), orc.qgemm_dense(qbits, A, Wq, Ws), f"large small-M q{qbits} {M}x{N}x{K}")
 
 
 def test_gemv_mode_hook_rejects_contradictory_bits():
@@ -153,7 +151,7 @@ def test_gemv_mode_hook_rejects_contradictory_bits():
         with pytest.raises(qg.QGemmError) as e:
             qg.test_gemv_mode(bad)
         assert e.value.code == -2
-    qg.test_gemv_mode(5)          # never the ring kernel, and no clusters: accepted
+    qg.test_gemv_mode(5)          # never the streaming kernel, and no clusters: accepted
     qg.test_gemv_mode(0)
 
 
