@@ -692,7 +692,9 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     // K slices.  A CTA streams at its own pace as long as it has an SM to itself and at 0.8 of that with a second one beside
     // it, so more and shorter slices are faster until the sum over the cluster (about 60 k of a tile per slice) takes it
     // back.  4096 x 14336, 8 bit, one token: 36.8 / 24.7 / 19.1 / 16.4 us with one to four slices; 2048 x 2048: 6.6 / 6.3 /
-    // 5.6 / 6.2 with one, two, four and eight; 3072 x 8192, 4 bit: 22.0 / 16.7 / 12.1 / 9.0.  All clusters have to be resident at once.
+    // 5.6 / 6.2 with one, two, four and eight; 3072 x 8192, 4 bit: 22.0 / 16.7 / 12.1 / 9.0.  Clusters of eight that fill the GPU
+    // start late behind one another, and seven or six slices are faster then (32 tiles of 8 bit, K = 8192: 9.0 us with eight, 8.2
+    // with seven; 4 bit, K = 4096: 7.8 with eight, 7.1 with six).  All clusters have to be resident at once.
     const int tiles = (N + rows - 1) / rows, blocks = K / MS_SK;
     int slices = 1, kc = K;
     long long best = -1;
@@ -701,7 +703,9 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
         if ((blocks + per - 1) / per != ns) continue;          // the same cut as a smaller count
         if (ns > 1 && (ctx->gemv_mode & 1 || cluster_capacity(ns) < tiles)) continue;
         const long long alone = static_cast<long long>(per) * MS_SK;
-        const long long cost = (static_cast<long long>(tiles) * ns <= ctx->sm_count ? alone : alone + alone / 4) + (ns > 1 ? 60 * ns : 0);
+        const long long ctas = static_cast<long long>(tiles) * ns;
+        const int beside = ctas <= ctx->sm_count ? 100 : ns == 8 && 5 * ctas > 8 * ctx->sm_count ? 170 : 125;     // percent
+        const long long cost = alone * beside / 100 + (ns > 1 ? 60 * ns : 0);
         if (best < 0 || cost < best) { best = cost; slices = ns; kc = per * MS_SK; }
     }
     p.R = M; p.N = N; p.K = K; p.E = 0; p.kc = kc; p.n_wt = tiles;
