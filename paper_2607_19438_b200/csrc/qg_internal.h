@@ -117,7 +117,8 @@ int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 // once.  That costs every such call 5 to 8 us (the unwanted launch keeps the next one from starting early).  128 experts,
 // 1536 x 2048: alone up to 11 rows per expert (even 63 us against 99, one segment 38 against 17 at eight rows), both up to 16,
 // the other from there (even 96 against 99, one segment 70 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
-// (even 741 us against 1117, eight segments 270 against 537 when the average alone decided).
+// (even 917 us against 1605 of the other alone; eight segments 183 against 622 when the average alone decided, and 154 of the
+// other alone).
 struct GroupedChoice {
     enum Way { STREAM, OTHER, BOTH };
     int on;                    // both kernels are launched
