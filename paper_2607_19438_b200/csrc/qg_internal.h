@@ -139,7 +139,8 @@ struct GroupedChoice {
     static constexpr int MAX_ROWS = 18;       // per expert, on average: evenly spread, the other kernel is the faster one from there on
     Way plan(long long R, long long E) const {
         if (R > MAX_ROWS * E) return OTHER;
-        const long long used = R < E ? R : E, even = 2 * R <= chunk * E ? used : R / chunk + E / 2;
+        // rows drawn evenly (Poisson): a tile per expert up to 5/8 of a tile's rows, then 3/8 of a tile more than the rows fill
+        const long long used = R < E ? R : E, even = 8 * R <= 5 * chunk * E ? used : R / chunk + 3 * E / 8;
         const long long gain = other_ns(used) - stream_ns(even), loss = stream_ns((R + chunk - 1) / chunk) - other_ns((R + 127) / 128);
         const long long stream = loss > 0 ? loss : 0, other = gain > 0 ? 3 * gain : 0, both = 4 * (6000 + 10 * E);
         if (stream <= other && stream <= both) return STREAM;

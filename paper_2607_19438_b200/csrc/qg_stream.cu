@@ -1,8 +1,8 @@
 // The weight-streaming GEMM: one matrix and up to sixteen tokens (qgemm_small_m), or the 4-bit expert matrices of a routed
 // layer with a few rows per expert (moe_grouped_qgemm and its gathering form: plain, gate/up + SiLU, routing-weighted).
 //
-// Every weight byte is used for a handful of token rows only, so the call is a streaming read of the packed weights: 42
-// 4-bit or 22 8-bit weights per clock and SM at HBM speed.  The tensor-memory kernel of the long segments (qg_gemm.cu)
+// Every weight byte is used for a handful of token rows only, so the call is a streaming read of the packed weights: 39
+// 4-bit or 21 8-bit weights per clock and SM at HBM speed.  The tensor-memory kernel of the long segments (qg_gemm.cu)
 // passes 13 weights per clock and SM from stage to stage whatever the row count; here mma.sync takes them directly.
 //
 // A CTA (eight consumer warps, a producer warp and one that prepares the rows; two CTAs per SM, so that the next kernel's
