@@ -479,7 +479,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         if (SK != 1 && pair < carry) {
             const Tile tl = decode_tile(pair, prefix, p, BT);
             const int wt = 2 * tl.pw + static_cast<int>(rank);
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_arrive_expect_tx(r_full(0), 4 * C::RAW_BYTES + C::SC_BYTES);
                 load_w(sbase + C::OFF_SC, &tm_s, (kb_first >> 2) * 8, tl.e, wt, r_full(0));
 #pragma unroll
@@ -600,7 +600,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                             tma_gather4_pair(sbase + C::OFF_X + (s + j) * C::X_BYTES + lane * 512, &tm_x, (kb + j) * BK,
                                              g0, g1, g2, g3, full_leader + 8u * (s + j));
                     }
-                } else if (lane == 0) {
+                } else if (elect_one()) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         if (jt == 0 && kb + j == p.skip_kb) continue;      // test hook: this stage never fills
@@ -633,7 +633,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                 if (jt == 0 && kb == pc.kb0) { QG_MARK(8); }
                 const bool sent = (batches == 0 && w_pre_issued);       // the first batch left in the prologue
                 ++batches;
-                if (lane == 0 && !sent) {
+                if (!sent && elect_one()) {
                     // five copies and one barrier per batch: the 8 scales per row that cover these four k-blocks,
                     // then the packed codes of each k-block
                     mbar_arrive_expect_tx(r_full(s), 4 * C::RAW_BYTES + C::SC_BYTES);
@@ -697,7 +697,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                     // start the wait for this warp's next k-block before issuing, so its latency is hidden
                     const uint32_t in = i + 2u;
                     ready = (kb + 2 < pc.kb1) && mbar_test_wait_cluster(full(in & 7u), (in >> 3) & 1u);
-                    if (lane == 0) {
+                    if (elect_one()) {
                         umma_kblock_ts_pair(d_tmem, tmem_base + C::A_COL0 + ta * C::A_COLS,
                                             b_lo0 + st * (C::X_BYTES >> 4), b_hi, idesc, kb != pc.kb0 ? 1u : 0u);
                         umma_commit_pair(done(st), 3u << leader);
@@ -707,7 +707,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                     kb += 2;
                     i = in;
                 }
-                if (ok && lane == 0) umma_commit_pair(acc_full(a), 3u << leader);
+                if (ok && elect_one()) umma_commit_pair(acc_full(a), 3u << leader);
                 __syncwarp();
                 if (w == 0 && static_cast<int>(j) == my_tiles - 1) { QG_MARK(3); }
             }
