@@ -207,7 +207,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         bool ok = true;
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_arrive_expect_tx(q_full, 2 * C::TILE_BYTES);       // rows past the sequence end arrive as zeros
 #pragma unroll
             for (int t = 0; t < 2; ++t)
@@ -220,7 +220,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int s = j & 1;
             const uint32_t ph = (j >> 1) & 1u;
             if (!at_wait(k_empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_arrive_expect_tx(k_full(s), C::TILE_BYTES);
 #pragma unroll
                 for (int a = 0; a < C::NBOX; ++a)
@@ -228,7 +228,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                                 j * AT_BKV, k_full(s));
             }
             if (!at_wait(v_empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_arrive_expect_tx(v_full(s), C::TILE_BYTES);
 #pragma unroll
                 for (int a = 0; a < C::NBOX; ++a)

@@ -326,7 +326,7 @@ qgemm_mx_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         uint32_t s = 0, ph = 0;
         for (uint32_t g = 0; g < total; ++g) {
             if (g >= C::ST && !mx_wait(empty(s), ph ^ 1u, abort_flag, p)) break;
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t fb = full_leader + 8u * s;
                 if (warp == 0) {
                     if (rank == 0) mbar_arrive_expect_tx(full(s), 2u * C::LOADED);

@@ -197,7 +197,7 @@ qgemm_mx_moe_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             bool ok = true;
             for (int j = 0; j < nch; ++j, ++g) {
                 if (g >= MG_ST && !mg_wait(empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t st = sbase + s * MG_STAGE, sf = sbase + MG_OFF_SF + s * MG_SF_STAGE;
                     if (warp == 0) {
                         mbar_arrive_expect_tx(full(s), MG_STAGE + MG_SF_STAGE);

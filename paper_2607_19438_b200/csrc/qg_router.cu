@@ -99,7 +99,7 @@ __device__ __forceinline__ void router_body(const CUtensorMap& tm_x, const CUten
         for (int kb = kb0; kb < kb1; ++kb, ++i) {
             const uint32_t s = i % RT_ST;
             if (i >= RT_ST && !rt_wait(empty(s), ((i / RT_ST) & 1u) ^ 1u, abort_flag, p)) break;
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t st = sbase + s * RT_STAGE;
                 mbar_arrive_expect_tx(full(s), RT_A_BYTES + n_boxes * (RT_B_BYTES / 2));
                 tma_load_2d(st, &tm_x, kb * RT_BK, t0, full(s));

@@ -292,7 +292,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 
     if (warp == MS_CONS_WARPS) {
         // ------------------------------------------------ producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t slot = 0, phase = 0, fslot = 0;
             int sent = 0, ahead = 0;                   // stages filled, stages whose weights are on their way
             uint32_t asked = 0;                        // answers to requests for a block so far, each a phase of taken_bar
