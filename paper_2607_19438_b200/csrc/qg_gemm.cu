@@ -728,7 +728,6 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         const uint32_t a_taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + C::A_COL0;
         const uint32_t full_leader = map_to_cta(full(0), leader);
         const uint32_t n_own = own_kb4;
-        constexpr uint32_t magic = 0x43000000u;
         QG_DECL();
         // Helping with the epilogue.  Before this warp waits for the MMAs of own k-block n - 2 (to reuse their TMEM
         // stage) it must have released every accumulator of an earlier tile, otherwise a single-accumulator pipeline
@@ -800,24 +799,24 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                 if constexpr (QBITS == 8) {
                     const uint4 v0 = lds128(raw + (((2 * h) ^ swz) << 4));
                     const uint4 v1 = lds128(raw + (((2 * h + 1) ^ swz) << 4));
-                    const float m1 = 256.f * sc, c1 = -32896.f * sc;
-                    const uint64_t m = pack_f32x2(m1, m1), c = pack_f32x2(c1, c1);
-                    dq8_word(v0.x, m, c, magic, oh[0], oh[1]);
-                    dq8_word(v0.y, m, c, magic, oh[2], oh[3]);
-                    dq8_word(v0.z, m, c, magic, oh[4], oh[5]);
-                    dq8_word(v0.w, m, c, magic, oh[6], oh[7]);
-                    dq8_word(v1.x, m, c, magic, oh[8], oh[9]);
-                    dq8_word(v1.y, m, c, magic, oh[10], oh[11]);
-                    dq8_word(v1.z, m, c, magic, oh[12], oh[13]);
-                    dq8_word(v1.w, m, c, magic, oh[14], oh[15]);
+                    uint64_t m, c;
+                    dq8_consts(sc, m, c);
+                    dq8_word(v0.x, m, c, DQ_MAGIC, oh[0], oh[1]);
+                    dq8_word(v0.y, m, c, DQ_MAGIC, oh[2], oh[3]);
+                    dq8_word(v0.z, m, c, DQ_MAGIC, oh[4], oh[5]);
+                    dq8_word(v0.w, m, c, DQ_MAGIC, oh[6], oh[7]);
+                    dq8_word(v1.x, m, c, DQ_MAGIC, oh[8], oh[9]);
+                    dq8_word(v1.y, m, c, DQ_MAGIC, oh[10], oh[11]);
+                    dq8_word(v1.z, m, c, DQ_MAGIC, oh[12], oh[13]);
+                    dq8_word(v1.w, m, c, DQ_MAGIC, oh[14], oh[15]);
                 } else {
                     const uint4 v = lds128(raw + ((h ^ swz) << 4));
-                    const float m1 = 256.f * sc, c1 = -32776.f * sc;
-                    const uint64_t m = pack_f32x2(m1, m1), c = pack_f32x2(c1, c1);
-                    dq4_word(v.x, m, c, magic, oh);
-                    dq4_word(v.y, m, c, magic, oh + 4);
-                    dq4_word(v.z, m, c, magic, oh + 8);
-                    dq4_word(v.w, m, c, magic, oh + 12);
+                    uint32_t hi2, lo2;
+                    dq4_consts(sc, hi2, lo2);
+                    dq4_word(v.x, hi2, lo2, oh);
+                    dq4_word(v.y, hi2, lo2, oh + 4);
+                    dq4_word(v.z, hi2, lo2, oh + 8);
+                    dq4_word(v.w, hi2, lo2, oh + 12);
                 }
             }
             __syncwarp();

@@ -122,17 +122,19 @@ qgemv_kernel(const GemvParams p) {
             for (int u = 0; u < GV_BATCH; ++u) {
                 const int c = c0 + u;
                 const float sc = __half2float(srow[2 * c]);     // the 32-block that holds k = 16 j .. 16 j + 15
-                uint64_t m2, c2;
-                dq_consts(sc, QBITS == 8, m2, c2);
                 uint32_t w[8];                                   // 16 bf16: k = 16 j .. 16 j + 15 of this chunk, row g
                 if constexpr (QBITS == 8) {
+                    uint64_t m2, c2;
+                    dq8_consts(sc, m2, c2);
                     dq8_word(raw[u].x, m2, c2, DQ_MAGIC, w[0], w[1]);
                     dq8_word(raw[u].y, m2, c2, DQ_MAGIC, w[2], w[3]);
                     dq8_word(raw[u].z, m2, c2, DQ_MAGIC, w[4], w[5]);
                     dq8_word(raw[u].w, m2, c2, DQ_MAGIC, w[6], w[7]);
                 } else {
-                    dq4_word(raw[u].x, m2, c2, DQ_MAGIC, w);
-                    dq4_word(raw[u].y, m2, c2, DQ_MAGIC, w + 4);
+                    uint32_t hi2, lo2;
+                    dq4_consts(sc, hi2, lo2);
+                    dq4_word(raw[u].x, hi2, lo2, w);
+                    dq4_word(raw[u].y, hi2, lo2, w + 4);
                 }
                 const uint4 lo0 = *reinterpret_cast<const uint4*>(a_lo + c * 64);       // A[g][k .. k + 7]
                 const uint4 lo1 = *reinterpret_cast<const uint4*>(a_lo + c * 64 + 8);   // A[g][k + 8 .. k + 15]
