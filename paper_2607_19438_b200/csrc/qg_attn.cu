@@ -136,7 +136,7 @@ __device__ __forceinline__ uint64_t exp2_poly2(uint64_t x2) {
 __device__ __forceinline__ bool at_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, const AttnParams& p) {
     const uint32_t limit = p.wait_limit;
     for (int it = 0; it < 16; ++it)
-        if (mbar_test_wait_cluster(bar, parity)) return true;
+        if (mbar_test_wait(bar, parity)) return true;
     for (uint32_t it = 0; it < limit; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((it & 255u) == 255u && *abort_flag) return false;

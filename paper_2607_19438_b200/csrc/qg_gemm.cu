@@ -12,13 +12,13 @@
 // Persistent CTA of 24 warps, one tile at a time.  BT <= 192: two TMEM accumulators (the epilogue of tile j overlaps
 // the main loop of tile j+1); BT = 256: one accumulator and eight TMEM weight stages, the exposed epilogue is shared
 // with the dequantising warps.
-//   warp 0      TMA producer of this CTA's half activation tile X[BT/2, 64] (128-byte swizzle)    -> x ring
+//   warp 0      TMA producer of this CTA's half activation tile, 2 x X[BT/2, 64] (128-byte swizzle) -> x ring
 //   warp 2      TMA producer of packed weights [128, 64] (+ scales every 4 k-blocks)              -> raw ring
 //   warps 8-23  dequantise raw -> bf16, written with tcgen05.st into TMEM weight stages (4 groups x 4 warps,
 //               group g converts every 4th k-block)
-//   warps 1, 3  (even CTA only) issue tcgen05.mma.cta_group::2 for the even / odd k-blocks and commit to both CTAs
+//   warp 1      (even CTA only) issues tcgen05.mma.cta_group::2, two k-blocks at a time, and commits to both CTAs
 //   warps 4-7   epilogue: tcgen05.ld, fused activation / routing weight, staged 16-byte bf16 stores
-//   warp 3      also allocates and frees TMEM
+//   warp 3      allocates and frees TMEM
 // Barriers the MMA waits on live in the even CTA and also collect the odd CTA's arrivals (remote mbarrier
 // arrive, TMA completion bytes); barriers that free a stage are signalled in both CTAs by the commit.
 // Dense calls with few tiles cut K into slices, one per CTA pair of a larger cluster (qgemm_slices_kernel): every pair leaves
@@ -64,7 +64,7 @@ struct GemmParams {
 template <int QBITS, int BT>
 struct Cfg {
     static constexpr int SX = 8;                                   // k-block stages: ring of the activation tile (smem)
-                                                                   // and of the full/done barriers
+    static constexpr int SP = SX / 2;                              // ... in pairs: what the full/done barriers count
     static constexpr int SR = (QBITS == 4 && BT <= 192) ? 16 : 8;  // packed-weight stages (smem, refilled four at a time):
                                                                    // twice as deep for 4-bit tiles where shared memory allows
     static constexpr int NACC = (BT > 192) ? 1 : 2;                // accumulators in tensor memory
@@ -89,7 +89,7 @@ struct Cfg {
     static constexpr int TAB_N = 128;                              // decoded tiles of this pair kept in shared memory
     static constexpr int OFF_TAB = OFF_PREFIX + (MAX_E + 4) * 4;
     static constexpr int OFF_BAR = OFF_TAB + TAB_N * 16;
-    static constexpr int NBAR = 2 * SX + 2 * SR + 5;
+    static constexpr int NBAR = 2 * SP + 2 * SR + 5;
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;        // + slack for 1024-byte alignment
     static constexpr int TMEM_COLS = 512;                          // accumulator(s) + SX weight stages
@@ -98,7 +98,7 @@ struct Cfg {
     static_assert(NACC * BT + SA * 32 <= 512, "tensor memory budget");
     static_assert(X_BYTES % 1024 == 0, "swizzled stages must stay 1024-byte aligned");
     static_assert(SX == 8, "stage arithmetic below assumes a ring of eight");
-    static_assert(SA >= 4 && (!HELP || SA == 8), "weight stages");
+    static_assert(SA >= 4 && SA % 2 == 0 && (!HELP || SA == 8), "weight stages");
 };
 
 struct __align__(16) Tile {
@@ -131,12 +131,13 @@ __device__ __forceinline__ Tile decode_tile(int t, const int* prefix, const Gemm
     return r;
 }
 
-// Bounded wait on an mbarrier phase.  Returns false if the CTA is giving up.
-template <bool CLUSTER>
+// Bounded wait on an mbarrier phase, first without suspending: a phase that is complete already is the common case, and the
+// plain test tells it sooner (3 % of a grouped GEMM).  Returns false if the CTA is giving up.
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag, const GemmParams& p) {
     const uint32_t limit = p.wait_limit;
+    if (mbar_test_wait(bar, parity)) return true;
     for (uint32_t it = 0; it < limit; ++it) {
-        if (CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if ((it & 255u) == 255u && *abort_flag) return false;
     }
     *abort_flag = 1;
@@ -148,8 +149,8 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
 // the bounded blocking wait.
 __device__ __forceinline__ bool spin_wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag, const GemmParams& p) {
     for (int it = 0; it < 64; ++it)
-        if (mbar_test_wait_cluster(bar, parity)) return true;
-    return wait_bar<true>(bar, parity, abort_flag, p);
+        if (mbar_test_wait(bar, parity)) return true;
+    return wait_bar(bar, parity, abort_flag, p);
 }
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
@@ -391,20 +392,20 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     __nv_bfloat16* stg16 = reinterpret_cast<__nv_bfloat16*>(sgen + C::OFF_STG);
     volatile int* misc = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC);  // [0] tmem base, [1] abort, [2..3] epilogue go/stop
     const uint32_t bar0 = sbase + C::OFF_BAR;
-    // full[s]   (even CTA): k-block in stage s is ready: both halves of the activation tile have landed (TMA bytes)
-    //           and all eight dequantising warps of the pair (4 per CTA) have written its weights to TMEM.
-    // done[s]   (both CTAs, by commit): the MMAs of the k-block in stage s have completed.
+    // full[s]   (even CTA): the two k-blocks of stage pair s are ready: both halves of the activation tile have landed (TMA
+    //           bytes) and all sixteen dequantising warps of the pair (4 per CTA and k-block) have written their weights to TMEM.
+    // done[s]   (both CTAs, by commit): the MMAs of the two k-blocks in stage pair s have completed.
     // r_full / r_empty: this CTA's packed-weight ring.   acc_full (both CTAs) / acc_empty (even CTA): accumulators.
     auto full = [&](int s) { return bar0 + 8u * s; };
-    auto done = [&](int s) { return bar0 + 8u * (C::SX + s); };
-    auto r_full = [&](int s) { return bar0 + 8u * (2 * C::SX + s); };
-    auto r_empty = [&](int s) { return bar0 + 8u * (2 * C::SX + C::SR + s); };
-    auto acc_full = [&](int s) { return bar0 + 8u * (2 * C::SX + 2 * C::SR + s); };
-    auto acc_empty = [&](int s) { return bar0 + 8u * (2 * C::SX + 2 * C::SR + 2 + s); };
+    auto done = [&](int s) { return bar0 + 8u * (C::SP + s); };
+    auto r_full = [&](int s) { return bar0 + 8u * (2 * C::SP + s); };
+    auto r_empty = [&](int s) { return bar0 + 8u * (2 * C::SP + C::SR + s); };
+    auto acc_full = [&](int s) { return bar0 + 8u * (2 * C::SP + 2 * C::SR + s); };
+    auto acc_empty = [&](int s) { return bar0 + 8u * (2 * C::SP + 2 * C::SR + 2 + s); };
     // last_full (this CTA, one phase): the epilogue warps, which consume every accumulator phase in order, have seen the
     // last tile's accumulator complete.  The dequantising warps that help with that last epilogue wait here instead
     // of on acc_full, whose parity they cannot tell apart from the phase two tiles earlier when K is short.
-    const uint32_t last_full = bar0 + 8u * (2 * C::SX + 2 * C::SR + 4);
+    const uint32_t last_full = bar0 + 8u * (2 * C::SP + 2 * C::SR + 4);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t crank = cluster_ctarank();
@@ -426,9 +427,9 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     float* partial = reinterpret_cast<float*>(sgen + C::OFF_X);          // K slices: where the ring of the activation tile was
 
     if (warp == 0) {   // barrier initialisation spread over the lanes of one warp (a single thread needs ~50 steps)
-        if (lane < C::SX) { mbar_init(full(lane), 1 + 8); mbar_init(done(lane), 1); }
+        if (lane < C::SP) { mbar_init(full(lane), 1 + 16); mbar_init(done(lane), 1); }
         // an accumulator is released by the 4 epilogue + 16 dequantising warps of both CTAs
-        if (lane >= 16 && lane < 18) { mbar_init(acc_full(lane - 16), 2); mbar_init(acc_empty(lane - 16), C::HELP ? 40 : 8); }
+        if (lane >= 16 && lane < 18) { mbar_init(acc_full(lane - 16), 1); mbar_init(acc_empty(lane - 16), C::HELP ? 40 : 8); }
         if (lane == 31) { misc[1] = 0; mbar_init(last_full, 1); }
         fence_mbar_init();
         fence_proxy_async_smem();
@@ -554,14 +555,15 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         return pc;
     };
 
-    // Control warps walk their loops with all 32 lanes (converged) and keep the per-k-block instruction count small:
-    // a lone thread retires only one dependent instruction every few cycles and an mbarrier round trip costs a few
-    // hundred cycles, so the producers work in batches of four k-blocks and the MMA warp does one wait, one
-    // four-MMA statement and one commit per k-block.
+    // Control warps walk their loops with all 32 lanes (converged) and issue behind elect.sync.  Each shares its scheduler with
+    // four converting warps, so an iteration of a few dozen dependent instructions lasts some hundred cycles, the price of a wait
+    // that succeeds at once (200) among them: a k-block at a time the activation producer was the pace of the kernel (128
+    // experts, 1536 x 2048, 512 tokens: 116 us).  So it hands over two k-blocks at a time, as one copy and one barrier, the
+    // packed-weight producer four.
     if (warp == 0) {
         // ------------------------------------------------ activation producer (this CTA's half of the token tile)
-        uint32_t s = 0, ph = 0;      // first stage of the next batch (0, 2, 4, 6) and the parity of its next "done" phase
-        uint32_t sent_kb = 0;        // k-blocks sent so far: the first eight find the ring empty and need no wait
+        uint32_t s = 0, ph = 0;      // next stage pair and the parity of its next "done" phase
+        uint32_t sent = 0;           // pairs sent so far: the first ones find the ring empty and need no wait
         const uint32_t full_leader = map_to_cta(full(0), leader);
         bool ok = true;
         QG_DECL();
@@ -583,34 +585,26 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             }
             for (int kb = pc.kb0; kb < pc.kb1; kb += 2) {
                 QG_T0();
-                // a stage is free once the MMAs that read it eight k-blocks ago are done (even and odd stages
-                // belong to different MMA warps, so both are checked)
-                if (sent_kb >= 8u &&
-                    (!wait_bar<false>(done(s), ph ^ 1u, abort_flag, p) ||
-                     !wait_bar<false>(done(s + 1), ph ^ 1u, abort_flag, p))) { ok = false; break; }
-                sent_kb += 2u;
+                // a stage pair is free once the MMAs that read it eight k-blocks ago are done
+                if (sent >= C::SP && !wait_bar(done(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
+                ++sent;
                 QG_ACC(0);
                 if (jt == 0 && kb == pc.kb0) { QG_MARK(7); }
-                if (p.gather_k > 0) {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        if (jt == 0 && kb + j == p.skip_kb) continue;      // test hook: this stage never fills
-                        if (lane == 0 && rank == 0) mbar_arrive_expect_tx(full(s + j), 2u * groups * 512u);
-                        if (lane < groups)
-                            tma_gather4_pair(sbase + C::OFF_X + (s + j) * C::X_BYTES + lane * 512, &tm_x, (kb + j) * BK,
-                                             g0, g1, g2, g3, full_leader + 8u * (s + j));
-                    }
-                } else if (elect_one()) {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        if (jt == 0 && kb + j == p.skip_kb) continue;      // test hook: this stage never fills
-                        if (rank == 0) mbar_arrive_expect_tx(full(s + j), 2 * C::X_BYTES);
-                        tma_load_2d_pair(sbase + C::OFF_X + (s + j) * C::X_BYTES, &tm_x, (kb + j) * BK, row0,
-                                         full_leader + 8u * (s + j));
+                const uint32_t dst = sbase + C::OFF_X + s * (2 * C::X_BYTES);
+                if (!(jt == 0 && kb == (p.skip_kb & ~1))) {                 // test hook: that pair never fills
+                    if (p.gather_k > 0) {
+                        if (lane == 0 && rank == 0) mbar_arrive_expect_tx(full(s), 4u * groups * 512u);
+                        if (lane < groups) {
+                            tma_gather4_pair(dst + lane * 512, &tm_x, kb * BK, g0, g1, g2, g3, full_leader + 8u * s);
+                            tma_gather4_pair(dst + C::X_BYTES + lane * 512, &tm_x, (kb + 1) * BK, g0, g1, g2, g3, full_leader + 8u * s);
+                        }
+                    } else if (elect_one()) {
+                        if (rank == 0) mbar_arrive_expect_tx(full(s), 4 * C::X_BYTES);
+                        tma_load_3d_pair(dst, &tm_x, 0, row0, kb, full_leader + 8u * s);
                     }
                 }
                 __syncwarp();
-                s = (s + 2u) & 7u;
+                s = (s + 1u) % C::SP;
                 if (s == 0) ph ^= 1u;
             }
         }
@@ -628,7 +622,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             const int wt = 2 * tl.pw + static_cast<int>(rank);
             for (int kb = pc.kb0; kb < pc.kb1; kb += 4) {
                 QG_T0();
-                if (batches >= C::SR / 4 && !wait_bar<false>(r_empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
+                if (batches >= C::SR / 4 && !wait_bar(r_empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
                 QG_ACC(1);
                 if (jt == 0 && kb == pc.kb0) { QG_MARK(8); }
                 const bool sent = (batches == 0 && w_pre_issued);       // the first batch left in the prologue
@@ -650,69 +644,52 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         }
         __syncwarp();
         if (lane == 0) QG_FLUSH();
-    } else if (warp == 1 || warp == 3) {
-        // ------------------------------------------------ MMA issuers (even CTA of the pair only)
-        // One warp needs about 500-560 cycles to issue the four TMEM-operand MMAs, the commit and the wait of a
-        // k-block, more than the 256-512 cycles the tensor cores need for it, and two warps issue concurrently at
-        // full speed; so warps 1 and 3 take the even and the odd k-blocks.  MMAs of different threads are ordered
-        // only through completion, so the odd warp starts a tile after the "done" of the tile's first k-block (which
-        // overwrites the accumulator); within a tile the order of the accumulating k-blocks does not matter.
-        // (Alternating pairs of k-blocks instead, so that the second warp's wait is covered by the first warp's two
-        // k-blocks, was measured slower: 5 % on the dense and 16 % on the short-K grouped GEMMs.)
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer (even CTA of the pair only)
+        // Two k-blocks per barrier: eight MMAs and one commit take about 350 cycles to issue, less than the tensor cores need for
+        // them from 48 tokens on.  One issuing thread also fixes the order in which a tile's k-blocks are added.
         if (rank == 0) {
-            const uint32_t w = (warp == 3) ? 1u : 0u;
             bool ok = true;
             QG_DECL();
             const uint32_t b_hi = (1024u >> 4) | (1u << 14) | (2u << 29);   // stride, version, 128-byte swizzle
             const uint32_t b_lo0 = ((sbase + C::OFF_X) >> 4) | (1u << 16);
-            uint32_t j = 0;
-            for (; static_cast<int>(j) < my_tiles && ok; ++j) {
+            for (uint32_t j = 0; static_cast<int>(j) < my_tiles && ok; ++j) {
                 const Tile tl = tile_at(static_cast<int>(j));
                 const Piece pc = piece_at(static_cast<int>(j));
                 const int n_mma = min(BT, (tl.tok_end - tl.tok0 + 15) & ~15);
                 const uint32_t idesc = umma_idesc_bf16(2 * BW, n_mma);
                 const uint32_t a = (C::NACC == 2) ? (j & 1u) : 0u;
                 const uint32_t aph = (C::NACC == 2) ? ((j >> 1) & 1u) : (j & 1u);
-                const uint32_t i0 = static_cast<uint32_t>(pc.i0);             // first k-block of the piece (ring index)
                 QG_T0();
-                if (w == 0) {
-                    if (!spin_wait_bar(acc_empty(a), aph ^ 1u, abort_flag, p)) { ok = false; break; }
-                } else {
-                    if (!spin_wait_bar(done(i0 & 7u), (i0 >> 3) & 1u, abort_flag, p)) { ok = false; break; }
-                }
+                if (!spin_wait_bar(acc_empty(a), aph ^ 1u, abort_flag, p)) { ok = false; break; }
                 QG_ACC(2);
                 const uint32_t d_tmem = tmem_base + a * BT;
-                // this warp's k-blocks of the piece: every other one, starting at kb0 + w
-                int kb = pc.kb0 + static_cast<int>(w);
-                uint32_t i = i0 + w;
-                bool ready = mbar_test_wait_cluster(full(i & 7u), (i >> 3) & 1u);
-                while (kb < pc.kb1) {
-                    const uint32_t st = i & 7u;
-                    const uint32_t ta = i % C::SA;                               // TMEM weight stage of k-block i
+                uint32_t i = static_cast<uint32_t>(pc.i0);                    // ring index of k-block kb
+                bool ready = mbar_test_wait(full((i >> 1) % C::SP), (i >> 3) & 1u);
+                for (int kb = pc.kb0; kb < pc.kb1; kb += 2, i += 2) {
+                    const uint32_t sp = (i >> 1) % C::SP;
                     QG_T0();
-                    if (!ready && !spin_wait_bar(full(st), (i >> 3) & 1u, abort_flag, p)) { ok = false; break; }
+                    if (!ready && !spin_wait_bar(full(sp), (i >> 3) & 1u, abort_flag, p)) { ok = false; break; }
                     QG_ACC(3);
-                    if (w == 0 && j == 0 && kb == pc.kb0) { QG_MARK(2); }
+                    if (j == 0 && kb == pc.kb0) { QG_MARK(2); }
                     tc_fence_after_sync();
-                    // start the wait for this warp's next k-block before issuing, so its latency is hidden
-                    const uint32_t in = i + 2u;
-                    ready = (kb + 2 < pc.kb1) && mbar_test_wait_cluster(full(in & 7u), (in >> 3) & 1u);
+                    // start the wait for the next pair before issuing, so its latency is hidden
+                    ready = (kb + 2 < pc.kb1) && mbar_test_wait(full((sp + 1) % C::SP), ((i + 2) >> 3) & 1u);
                     if (elect_one()) {
-                        umma_kblock_ts_pair(d_tmem, tmem_base + C::A_COL0 + ta * C::A_COLS,
-                                            b_lo0 + st * (C::X_BYTES >> 4), b_hi, idesc, kb != pc.kb0 ? 1u : 0u);
-                        umma_commit_pair(done(st), 3u << leader);
+                        const uint32_t ta = tmem_base + C::A_COL0 + (i % C::SA) * C::A_COLS;     // TMEM weight stage
+                        const uint32_t b_lo = b_lo0 + sp * (2 * C::X_BYTES >> 4);
+                        umma_kblock_ts_pair(d_tmem, ta, b_lo, b_hi, idesc, kb != pc.kb0 ? 1u : 0u);
+                        umma_kblock_ts_pair(d_tmem, ta + C::A_COLS, b_lo + (C::X_BYTES >> 4), b_hi, idesc, 1u);
+                        umma_commit_pair(done(sp), 3u << leader);
+                        if (kb + 2 >= pc.kb1) umma_commit_pair(acc_full(a), 3u << leader);
                     }
                     __syncwarp();
                     QG_ACC(10);
-                    kb += 2;
-                    i = in;
                 }
-                if (ok && elect_one()) umma_commit_pair(acc_full(a), 3u << leader);
-                __syncwarp();
-                if (w == 0 && static_cast<int>(j) == my_tiles - 1) { QG_MARK(3); }
+                if (static_cast<int>(j) == my_tiles - 1) { QG_MARK(3); }
             }
             __syncwarp();
-            if (lane == 0 && w == 0) QG_FLUSH();
+            if (lane == 0) QG_FLUSH();
         }
     } else if (warp >= 8) {
         // ------------------------------------------------ dequantise: raw ring -> TMEM weight stages
@@ -753,7 +730,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             const uint32_t aph = (C::NACC == 2) ? ((jt >> 1) & 1u) : (jt & 1u);
             // single accumulator: every tile is helped, so the phases of acc_full are consumed in order; two
             // accumulators: only the last tile is helped, through the one-shot barrier
-            if (!wait_bar<false>(C::HELP ? acc_full(a) : last_full, C::HELP ? aph : 0u, abort_flag, p)) return false;
+            if (!wait_bar(C::HELP ? acc_full(a) : last_full, C::HELP ? aph : 0u, abort_flag, p)) return false;
             tc_fence_after_sync();
             if (plain_ep && wt < p.n_wt) {
                 const int n_mma = min(BT, (tl.tok_end - tl.tok0 + 15) & ~15);
@@ -783,7 +760,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             }
             QG_T0();
             // the four k-blocks of a batch and their scales arrive on the barrier of the batch's first stage
-            if (!wait_bar<false>(r_full((n % NB) << 2), phr, abort_flag, p)) break;
+            if (!wait_bar(r_full((n % NB) << 2), phr, abort_flag, p)) break;
             QG_ACC(5);
             if (n == 0 && warp == 8) { QG_MARK(10); }
             const uint32_t raw = sbase + C::OFF_RAW + sr * C::RAW_BYTES + raw_row;
@@ -825,7 +802,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             // its TMEM stage (i % SA) is free once the MMAs of k-block i - SA have completed
             {
                 const uint32_t i = 4u * n + g;
-                if (i >= C::SA && !wait_bar<false>(done((i - C::SA) & 7u), ((i - C::SA) >> 3) & 1u, abort_flag, p)) break;
+                if (i >= C::SA && !wait_bar(done(((i - C::SA) >> 1) % C::SP), ((i - C::SA) >> 3) & 1u, abort_flag, p)) break;
             }
             QG_ACC(6);
             tc_fence_after_sync();
@@ -840,7 +817,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             tmem_st_wait();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(full_leader + 8u * (((n & 1u) << 2) + g));   // k-block stage i % 8
+            if (lane == 0) mbar_arrive_cluster(full_leader + 8u * (((n & 1u) << 1) + (g >> 1)));   // stage pair (i / 2) % 4
             if (n == 0 && warp == 8) { QG_MARK(9); }
             ta += 4;
             if (ta >= C::SA) ta -= C::SA;
@@ -868,7 +845,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             const uint32_t aph = (C::NACC == 2) ? ((j >> 1) & 1u) : (j & 1u);
             const uint32_t fl = j & 1u;       // flag slot: alternates so a slow warp never reads a newer flag
             QG_T0();
-            if (et == 0) misc[2 + fl] = wait_bar<false>(acc_full(a), aph, abort_flag, p) ? 1 : 0;
+            if (et == 0) misc[2 + fl] = wait_bar(acc_full(a), aph, abort_flag, p) ? 1 : 0;
             tc_fence_before_sync();
             named_bar_sync(1, 128);
             if (!misc[2 + fl]) break;
@@ -1048,9 +1025,11 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
     static_assert(C::SMEM_BYTES <= 232448, "shared memory budget");
     CUtensorMap tm_x, tm_w, tm_s;       // cached in the context: the same buffers recur every layer and step
     const uint64_t wrows = static_cast<uint64_t>(p.E) * p.N;
-    // activations: a box of half a token tile, or of a single row when the rows are gathered four at a time
-    int rc = get_tmap_2d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, p.K, x_rows, BK,
-                         p.gather_k > 0 ? 1 : C::XH_ROWS, CU_TENSOR_MAP_SWIZZLE_128B);
+    // activations: a box of half a token tile and two k-blocks, which land one after the other (a view [K / 64][rows][64]), or
+    // of a single row when the rows are gathered four at a time
+    int rc = p.gather_k > 0 ? get_tmap_2d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, p.K, x_rows, BK, 1, CU_TENSOR_MAP_SWIZZLE_128B)
+                            : get_tmap_3d(ctx, &tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, BK, x_rows, p.K / BK, 2 * BK, BK,
+                                          C::XH_ROWS, 2, CU_TENSOR_MAP_SWIZZLE_128B, 2ull * p.K);
     // weights and scales: a box of this CTA's 128 rows; in gate/up mode 64 gate rows + 64 up rows, as two planes of a
     // 3-D view (k, row within a half, half of an expert's matrix)
     const uint64_t kbytes = (QBITS == 8) ? p.K : p.K / 2;

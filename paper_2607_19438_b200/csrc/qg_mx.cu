@@ -218,7 +218,7 @@ struct MxParams {
 // Bounded wait: a few non-blocking tests first (the barrier is usually complete or about to be).
 __device__ __forceinline__ bool mx_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, const MxParams& p) {
     for (int it = 0; it < 16; ++it)
-        if (mbar_test_wait_cluster(bar, parity)) return true;
+        if (mbar_test_wait(bar, parity)) return true;
     for (uint32_t it = 0; it < p.wait_limit; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((it & 255u) == 255u && *abort_flag) return false;
