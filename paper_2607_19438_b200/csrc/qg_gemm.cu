@@ -79,13 +79,17 @@ struct Cfg {
     static constexpr int RAW_ROW = (QBITS == 8) ? 64 : 32;         // packed bytes per row per stage
     static constexpr int RAW_BYTES = BW * RAW_ROW;
     static constexpr int SC_BYTES = BW * 16;                       // 8 fp16 scales per row
-    static constexpr int STG_BYTES = 32 * 128 * 4 + 4 * 1024;      // [32 tokens][128 rows] fp32 (gate/up), also used as 16
-                                                                   // private 1 KB transposition buffers; + 4 more of those
+    // transposition buffers: 1 KB for each dequantising warp, then the epilogue warps'; theirs are 2 KB, used in turn, where they
+    // drain most tiles alone
+    static constexpr int EPI_ST = HELP ? 1024 : 2048;
+    static constexpr int STG_BYTES = 16 * 1024 + 4 * EPI_ST;
+    static constexpr int WT_BYTES = HELP ? 0 : 2 * BT * 4;         // routing weights of a tile's tokens, two tiles in turn
     static constexpr int OFF_X = 0;
     static constexpr int OFF_RAW = OFF_X + SX * X_BYTES;
     static constexpr int OFF_SC = OFF_RAW + SR * RAW_BYTES;
     static constexpr int OFF_STG = OFF_SC + NSB * SC_BYTES;
-    static constexpr int OFF_PREFIX = OFF_STG + STG_BYTES;
+    static constexpr int OFF_WT = OFF_STG + STG_BYTES;
+    static constexpr int OFF_PREFIX = OFF_WT + WT_BYTES;
     static constexpr int TAB_N = 128;                              // decoded tiles of this pair kept in shared memory
     static constexpr int OFF_TAB = OFF_PREFIX + (MAX_E + 4) * 4;
     static constexpr int OFF_BAR = OFF_TAB + TAB_N * 16;
@@ -174,11 +178,14 @@ __device__ __forceinline__ float lds_scale(uint32_t addr) {
 // token pairs), scaled, packed to bf16x2 and written with two transposing matrix stores into a private
 // [16 tokens][32 rows] buffer (16-byte chunks XOR-swizzled by the token pair, conflict-free both ways), from which
 // every thread moves two 16-byte pieces to global memory (64 contiguous bytes per token).  The next block's TMEM
-// loads are in flight while the current one is stored.  Called by the four epilogue warps and, for a
-// single-accumulator tile, by the sixteen dequantising warps, which would otherwise idle at the tile boundary.
-template <bool SK>
+// loads are in flight while the current one is stored.  Called by the four epilogue warps (TWO: with two buffers in turn, so
+// that a block need not wait until the one before it has left) and by the sixteen dequantising warps: for a
+// single-accumulator tile, and for a pair's last tile, when they would otherwise idle.
+// WS: the tile's routing weights are in shared memory (wts, by token); otherwise every warp fetches them, two dependent loads from
+// global memory in front of its first block (with 12 k-blocks a tile, 1500 of the 6500 cycles of an epilogue that was the pace).
+template <bool SK, bool WS, bool TWO>
 __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int tok_end, int n_base, uint32_t taddr,
-                                            int n_epi, int pid, int npart, __nv_bfloat16* st, int lane, int nsrc_in,
+                                            int n_epi, int pid, int npart, __nv_bfloat16* st, const float* wts, int lane, int nsrc_in,
                                             int quarter, int slot_floats, volatile int* abort_flag) {
     const int nsrc = SK ? nsrc_in : 0;       // without stream-K all of the partial-tile handling below compiles away
     // The loop is issue-bound (five warps of a scheduler drain together), so everything that does not depend on the
@@ -220,20 +227,20 @@ __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int t
     // Routing weights of the whole tile, fetched once (two dependent global loads, all in flight together): lane l
     // holds the weights of tokens l, l + 32, ... of the tile.
     float wt8[8];
-    if (weighted) {
+    if (!WS && weighted) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int tokl = tok0 + 32 * j + lane;
             wt8[j] = (32 * j < n_epi && tokl < tok_end) ? p.topk_w[p.row_pair[tokl]] : 0.f;
         }
     }
-    const uint32_t st_row = smem_u32(st) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);   // matrix lane>>3, token lane&7
+    uint32_t st_row = smem_u32(st) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);   // matrix lane>>3, token lane&7
     const int c = 2 * (lane & 3);                // this thread's token pairs: c, c + 1 and 8 + c, 9 + c of the block
     // store side: this lane moves tokens tk and 8 + tk of every block, 16 bytes (8 rows from n) each
     const int tk = lane >> 2, c4 = lane & 3;
     const int n = n_base + c4 * 8;
-    const uint4* s_lo = reinterpret_cast<const uint4*>(st + tk * 32 + ((c4 ^ ((tk >> 1) & 3)) << 3));
-    const uint4* s_hi = s_lo + 32;               // token 8 + tk: 512 bytes on, same swizzle
+    uint32_t s_lo = smem_u32(st) + tk * 64 + ((c4 ^ ((tk >> 1) & 3)) << 4);      // token 8 + tk: 512 bytes on, same swizzle
+    int flip = 1024;                             // to the other buffer and back
     const size_t row8 = static_cast<size_t>(8) * p.N;
     __nv_bfloat16* g = static_cast<__nv_bfloat16*>(p.out) + static_cast<size_t>(tok0 + 16 * b + tk) * p.N + n;
     const size_t g_step = 2 * row8 * npart;
@@ -269,13 +276,19 @@ __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int t
         }
         uint32_t pk[8];
         if (weighted) {
-            const int j = b >> 1;                // tokens 16 b .. 16 b + 15 live in register j, lanes 16 (b & 1) ..
-            float wv = wt8[0];
+            float w0, w1, w2, w3;                // weights of tokens 16 b + c, + 1, + 8, + 9
+            if constexpr (WS) {
+                const float2 wa = *reinterpret_cast<const float2*>(wts + 16 * b + c), wb = *reinterpret_cast<const float2*>(wts + 16 * b + 8 + c);
+                w0 = wa.x; w1 = wa.y; w2 = wb.x; w3 = wb.y;
+            } else {
+                const int j = b >> 1;            // tokens 16 b .. 16 b + 15 live in register j, lanes 16 (b & 1) ..
+                float wv = wt8[0];
 #pragma unroll
-            for (int jj = 1; jj < 8; ++jj) wv = (j == jj) ? wt8[jj] : wv;
-            const int src = 16 * (b & 1) + c;
-            const float w0 = __shfl_sync(0xFFFFFFFFu, wv, src), w1 = __shfl_sync(0xFFFFFFFFu, wv, src + 1);
-            const float w2 = __shfl_sync(0xFFFFFFFFu, wv, src + 8), w3 = __shfl_sync(0xFFFFFFFFu, wv, src + 9);
+                for (int jj = 1; jj < 8; ++jj) wv = (j == jj) ? wt8[jj] : wv;
+                const int src = 16 * (b & 1) + c;
+                w0 = __shfl_sync(0xFFFFFFFFu, wv, src); w1 = __shfl_sync(0xFFFFFFFFu, wv, src + 1);
+                w2 = __shfl_sync(0xFFFFFFFFu, wv, src + 8); w3 = __shfl_sync(0xFFFFFFFFu, wv, src + 9);
+            }
 #pragma unroll
             for (int gq = 0; gq < 2; ++gq) {     // tokens 8 gq .. 8 gq + 7
                 const float wa = gq ? w2 : w0, wb = gq ? w3 : w1;
@@ -301,13 +314,20 @@ __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int t
         stmatrix_x4_trans(st_row, pk[0], pk[1], pk[2], pk[3]);
         stmatrix_x4_trans(st_row + 512, pk[4], pk[5], pk[6], pk[7]);
         __syncwarp();
-        if (left > 0) *reinterpret_cast<uint4*>(g) = *s_lo;
-        if (left > 8) *reinterpret_cast<uint4*>(g + row8) = *s_hi;
-        __syncwarp();
+        if (left > 0) *reinterpret_cast<uint4*>(g) = lds128(s_lo);
+        if (left > 8) *reinterpret_cast<uint4*>(g + row8) = lds128(s_lo + 512);
+        if constexpr (TWO) {
+            st_row += flip;
+            s_lo += flip;
+            flip = -flip;
+        } else {
+            __syncwarp();
+        }
         g += g_step;
         left -= left_step;
         b = bn;
     }
+    __syncwarp();                                // the buffers may be written again
     if (SK && nsrc < 0) {
         __threadfence();
         __syncwarp();
@@ -321,6 +341,53 @@ __device__ __forceinline__ void drain_plain(const GemmParams& p, int tok0, int t
             }
         }
     }
+}
+
+// Gate/up epilogue of one warp.  The tile's weight rows were dequantised into such an order (see the dequantising warps) that the
+// lanes 0-15 of a quarter are gate rows and lanes 16-31 the up rows that belong to them, so the two fragments of a 16-token block hold
+// a thread's gates and ups in the same places: SiLU(gate) * up in registers, one transposing matrix store into a [16 tokens][16
+// rows] buffer, 32 contiguous bytes per token from there.  Blocks as in drain_plain; two buffers of 512 bytes in turn.  (Gates and ups in
+// different warps met through a [32 tokens][128 rows] fp32 buffer and two barriers of all four: 8000 cycles a tile of 192 tokens.)
+__device__ __forceinline__ void drain_gate_up(const GemmParams& p, int tok0, int tok_end, int f_base, uint32_t taddr, int n_epi, int pid,
+                                              int npart, __nv_bfloat16* st, int lane) {
+    const int nblk = n_epi >> 4, F = p.N >> 1;
+    int b = pid;
+    if (b >= nblk) return;
+    uint32_t v0[8], v1[8];
+    tmem_ld_16x256_x2(taddr + 16 * b, v0);
+    tmem_ld_16x256_x2(taddr + (16u << 16) + 16 * b, v1);
+    // write side: matrix m = lane / 8 holds rows 8 (m % 2) .. of tokens 8 (m / 2) ..; this lane names token 8 (m / 2) + lane % 8
+    const int wtok = ((lane >> 4) << 3) + (lane & 7), whalf = (lane >> 3) & 1;
+    uint32_t st_row = smem_u32(st) + wtok * 32 + ((whalf ^ ((wtok >> 2) & 1)) << 4);
+    const int tk = lane >> 1, half = lane & 1;   // store side: 16 bytes (8 rows) of one token
+    uint32_t s_at = smem_u32(st) + tk * 32 + ((half ^ ((tk >> 2) & 1)) << 4);
+    __nv_bfloat16* g = static_cast<__nv_bfloat16*>(p.out) + static_cast<size_t>(tok0 + 16 * b + tk) * F + f_base + 8 * half;
+    const size_t g_step = static_cast<size_t>(16 * npart) * F;
+    int left = tok_end - tok0 - 16 * b - tk, flip = 512;
+    while (b < nblk) {
+        tmem_ld_wait();
+        float h[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float gt = __uint_as_float(v0[i]);
+            h[i] = __fdividef(gt, 1.0f + __expf(-gt)) * __uint_as_float(v1[i]);
+        }
+        const int bn = b + npart;
+        if (bn < nblk) {                         // next block, overlapped with the rest of this one
+            tmem_ld_16x256_x2(taddr + 16 * bn, v0);
+            tmem_ld_16x256_x2(taddr + (16u << 16) + 16 * bn, v1);
+        }
+        stmatrix_x4_trans(st_row, bf16x2(h[0], h[1]), bf16x2(h[2], h[3]), bf16x2(h[4], h[5]), bf16x2(h[6], h[7]));
+        __syncwarp();
+        if (left > 0) *reinterpret_cast<uint4*>(g) = lds128(s_at);
+        st_row += flip;
+        s_at += flip;
+        flip = -flip;
+        g += g_step;
+        left -= 16 * npart;
+        b = bn;
+    }
+    __syncwarp();
 }
 
 // K slices (SK = 2): a warp leaves the raw fp32 fragments of its 16-token blocks in this CTA's shared memory (the idle ring of
@@ -388,8 +455,8 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     const uint32_t sbase = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     uint8_t* sgen = smem_dyn + (sbase - smem_u32(smem_dyn));
     int* prefix = reinterpret_cast<int*>(sgen + C::OFF_PREFIX);
-    float* stg32 = reinterpret_cast<float*>(sgen + C::OFF_STG);
     __nv_bfloat16* stg16 = reinterpret_cast<__nv_bfloat16*>(sgen + C::OFF_STG);
+    float* wts = reinterpret_cast<float*>(sgen + C::OFF_WT);
     volatile int* misc = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC);  // [0] tmem base, [1] abort, [2..3] epilogue go/stop
     const uint32_t bar0 = sbase + C::OFF_BAR;
     // full[s]   (even CTA): the two k-blocks of stage pair s are ready: both halves of the activation tile have landed (TMA
@@ -459,21 +526,28 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         fence_proxy_async_smem();
         if (grouped) pdl_wait();
         int carry = 0;
-        for (int e0 = 0; e0 < p.E; e0 += 32) {
-            const int e = e0 + lane;
-            int n = 0;
-            if (e < p.E) {
-                const int cnt = p.offsets ? (p.offsets[e + 1] - p.offsets[e]) : p.R;
-                n = ((cnt + BT - 1) / BT) * n_pw;
-            }
-            int inc = n;
+        constexpr int PB = 4;                    // experts per lane whose offsets travel together
+        for (int e0 = 0; e0 < p.E; e0 += 32 * PB) {
+            int cnt[PB];
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
-                if (lane >= off) inc += v;
+            for (int i = 0; i < PB; ++i) {
+                const int e = e0 + 32 * i + lane;
+                cnt[i] = (e >= p.E) ? 0 : p.offsets ? p.offsets[e + 1] - p.offsets[e] : p.R;
             }
-            if (e < p.E) prefix[e] = carry + inc - n;
-            carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
+#pragma unroll
+            for (int i = 0; i < PB; ++i) {
+                const int e = e0 + 32 * i + lane;
+                if (e0 + 32 * i >= p.E) break;
+                const int n = ((cnt[i] + BT - 1) / BT) * n_pw;
+                int inc = n;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+                    if (lane >= off) inc += v;
+                }
+                if (e < p.E) prefix[e] = carry + inc - n;
+                carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
+            }
         }
         if (lane == 0) prefix[p.E] = carry;
         __syncwarp();
@@ -699,7 +773,9 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         // thread = one row, all 64 k of the k-block: 64 bytes (Q8) or 32 bytes (Q4) of packed codes, read from the
         // swizzled raw tile without bank conflicts, 2 scales, 32 TMEM columns out.
         const int g = (warp - 8) >> 2, q = warp & 3;
-        const int row = q * 32 + lane;
+        // In gate/up mode lanes 0-15 of a quarter take gate rows and lanes 16-31 the up rows that belong to them (the raw tile is 64
+        // gate rows, then 64 up rows).
+        const int row = (EPI == 1) ? ((lane >> 4) << 6) + q * 16 + (lane & 15) : q * 32 + lane;
         const uint32_t swz = (QBITS == 8) ? ((row >> 1) & 3u) : ((row >> 2) & 1u);
         const uint32_t raw_row = row * C::RAW_ROW;
         const uint32_t a_taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + C::A_COL0;
@@ -718,7 +794,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         uint32_t helped = 0;                                           // tiles whose accumulator this warp released
         uint32_t t2 = 0, in2 = 0;                                      // tile of own k-block n - 2, position in it
         const uint32_t acc_empty_leader = map_to_cta(acc_empty(0), leader);
-        constexpr bool plain_ep = (EPI == 0);
+        constexpr bool shared_ep = (EPI < 2);
         __nv_bfloat16* my_st = stg16 + (warp - 8) * 512;               // private 1 KB transposition buffer
         uint32_t ta = static_cast<uint32_t>(g) % C::SA;                 // TMEM weight stage of own k-block i = i % SA
         bool dq_ok = true;
@@ -732,13 +808,17 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             // accumulators: only the last tile is helped, through the one-shot barrier
             if (!wait_bar(C::HELP ? acc_full(a) : last_full, C::HELP ? aph : 0u, abort_flag, p)) return false;
             tc_fence_after_sync();
-            if (plain_ep && wt < p.n_wt) {
+            if (shared_ep && wt < p.n_wt) {
                 const int n_mma = min(BT, (tl.tok_end - tl.tok0 + 15) & ~15);
-                if constexpr (SK == 2)
+                if constexpr (EPI == 1)
+                    drain_gate_up(p, tl.tok0, tl.tok_end, wt * 64 + q * 16, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma,
+                                  1 + g, 5, my_st, lane);
+                else if constexpr (SK == 2)
                     dump_partial(partial, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma, 1 + g, 5, q, lane);
                 else
-                    drain_plain<SK == 1>(p, tl.tok0, tl.tok_end, wt * BW + q * 32,
-                            tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma, 1 + g, 5, my_st, lane,
+                    drain_plain<SK == 1, !C::HELP, false>(p, tl.tok0, tl.tok_end, wt * BW + q * 32,
+                            tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BT, n_mma, 1 + g, 5, my_st,
+                            C::HELP ? nullptr : wts + (jt & 1u) * BT, lane,
                             piece_at(static_cast<int>(jt)).nsrc, q, BT * 128, abort_flag);
             }
             tc_fence_before_sync();
@@ -826,21 +906,47 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         while (C::HELP && dq_ok && helped < static_cast<uint32_t>(my_tiles)) dq_ok = help_tile(helped++, true);
         // With two accumulators the epilogues overlap the main loops, except the last one: these warps have nothing
         // left to do then and take four fifths of it (nobody waits for that accumulator again: no release).
-        if (!C::HELP && plain_ep && dq_ok && my_tiles > 0) help_tile(static_cast<uint32_t>(my_tiles - 1), false);
+        if (!C::HELP && shared_ep && dq_ok && my_tiles > 0) help_tile(static_cast<uint32_t>(my_tiles - 1), false);
         __syncwarp();
         if (warp == 8 && lane == 0) QG_FLUSH();
     } else if (warp >= 4) {
         // ------------------------------------------------ epilogue (warps 4..7 <-> TMEM lanes 32 (warp-4) ..)
         const int qd = warp - 4;
         const int et = threadIdx.x - 128;
-        __nv_bfloat16* outb = static_cast<__nv_bfloat16*>(p.out);
         float* outf = static_cast<float*>(p.out);
         const uint32_t acc_empty_base = map_to_cta(acc_empty(0), leader);
         uint32_t j = 0;
+        // Routing weights are fetched ahead, a thread the token et (and et + 128) of a tile: the pairs' numbers two tiles ahead, the
+        // weights they name one tile ahead.
+        const bool weighted = EPI == 0 && !C::HELP && p.mode == QG_MODE_DOWN_WEIGHTED;
+        int pr0 = -1, pr1 = -1;
+        float w0 = 0.f, w1 = 0.f;
+        auto fetch_pairs = [&](int jt) {
+            pr0 = pr1 = -1;
+            if (jt >= my_tiles) return;
+            const Tile tn = tile_at(jt);
+            if (tn.tok0 + et < tn.tok_end) pr0 = p.row_pair[tn.tok0 + et];
+            if (BT > 128 && tn.tok0 + 128 + et < tn.tok_end) pr1 = p.row_pair[tn.tok0 + 128 + et];
+        };
+        auto fetch_weights = [&]() {
+            w0 = pr0 >= 0 ? p.topk_w[pr0] : 0.f;
+            w1 = (BT > 128 && pr1 >= 0) ? p.topk_w[pr1] : 0.f;
+        };
+        if (weighted) {
+            fetch_pairs(0);
+            fetch_weights();
+            fetch_pairs(1);
+        }
         QG_DECL();
         for (; static_cast<int>(j) < my_tiles; ++j) {
             const Tile tl = tile_at(static_cast<int>(j));
             const int wt = 2 * tl.pw + static_cast<int>(rank);     // may be one past the last tile: nothing is stored
+            if (weighted) {
+                if (et < BT) wts[(j & 1u) * BT + et] = w0;
+                if (BT > 128 && et + 128 < BT) wts[(j & 1u) * BT + 128 + et] = w1;
+                fetch_weights();
+                fetch_pairs(static_cast<int>(j) + 2);
+            }
             const uint32_t a = (C::NACC == 2) ? (j & 1u) : 0u;
             const uint32_t aph = (C::NACC == 2) ? ((j >> 1) & 1u) : (j & 1u);
             const uint32_t fl = j & 1u;       // flag slot: alternates so a slow warp never reads a newer flag
@@ -859,66 +965,33 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             if constexpr (EPI == 0) {
                 // shared with the dequantising warps (participants 1..4 of this lane quarter) when they help
                 if constexpr (SK == 2) dump_partial(partial, taddr, n_epi, 0, 5, qd, lane);
-                else drain_plain<SK == 1>(p, tl.tok0, tl.tok_end, wt * BW + qd * 32, taddr, n_epi, 0,
+                else drain_plain<SK == 1, !C::HELP, !C::HELP>(p, tl.tok0, tl.tok_end, wt * BW + qd * 32, taddr, n_epi, 0,
                             (C::HELP || static_cast<int>(j) == my_tiles - 1) ? 5 : 1,
-                            stg16 + (16 + qd) * 512, lane, piece_at(static_cast<int>(j)).nsrc, qd, BT * 128, abort_flag);
+                            stg16 + 16 * 512 + qd * (C::EPI_ST / 2), C::HELP ? nullptr : wts + (j & 1u) * BT, lane, piece_at(static_cast<int>(j)).nsrc, qd, BT * 128, abort_flag);
+            } else if constexpr (EPI == 1) {
+                drain_gate_up(p, tl.tok0, tl.tok_end, wt * 64 + qd * 16, taddr, n_epi, 0,
+                              (C::HELP || static_cast<int>(j) == my_tiles - 1) ? 5 : 1, stg16 + 16 * 512 + qd * (C::EPI_ST / 2), lane);
             } else {
                 for (int c = 0; c < n_epi; c += 32) {
                     uint32_t v[32];
                     tmem_ld_32x32(taddr + c, v);
                     tmem_ld_wait();
-                    const int row = qd * 32 + lane;          // weight row of this thread inside the tile
-                    if constexpr (EPI == 2) {
-                        // y[token, n] += w * acc: lanes are consecutive n, so each warp-wide red covers 128 bytes
-                        const int n = wt * BW + row;
-                        const int tokl = tl.tok0 + c + lane;
-                        int trow = 0;
-                        float wv = 0.f;
-                        if (tokl < tl.tok_end) {
-                            const int pr = p.row_pair[tokl];
-                            wv = p.topk_w[pr];
-                            trow = pr / p.k;
-                        }
+                    // y[token, n] += w * acc: lanes are consecutive n, so each warp-wide red covers 128 bytes
+                    const int n = wt * BW + qd * 32 + lane;
+                    const int tokl = tl.tok0 + c + lane;
+                    int trow = 0;
+                    float wv = 0.f;
+                    if (tokl < tl.tok_end) {
+                        const int pr = p.row_pair[tokl];
+                        wv = p.topk_w[pr];
+                        trow = pr / p.k;
+                    }
 #pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) {
-                            const float w = __shfl_sync(0xFFFFFFFFu, wv, jj);
-                            const int tr = __shfl_sync(0xFFFFFFFFu, trow, jj);
-                            if (tl.tok0 + c + jj < tl.tok_end && n < p.N)
-                                atomicAdd(outf + static_cast<size_t>(tr) * p.N + n, w * __uint_as_float(v[jj]));
-                        }
-                    } else {
-                        // lanes 0..63 hold gate rows, 64..127 the matching up rows: transpose through shared memory
-                        // ([32 tokens][128 rows] fp32), then every thread finishes 16 outputs of one token.
-                        const int F = p.N / 2;
-                        // The 16-byte chunk index of a row is XOR-ed with (chunk / 8) % 2 and 2 (token % 2), so that
-                        // the eight threads of a quarter warp below (two tokens x four 64-byte spans) hit eight
-                        // different bank groups instead of two.
-                        const int wchunk = ((row >> 2) ^ ((row >> 5) & 1)) << 2 | (row & 3);
-#pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) stg32[jj * 128 + (wchunk ^ ((jj & 1) << 3))] = __uint_as_float(v[jj]);
-                        named_bar_sync(2, 128);
-                        const int tk = et >> 2, f0 = (et & 3) * 16;
-                        const int tok = tl.tok0 + c + tk;
-                        const int rsw = ((et & 3) >> 1) ^ ((tk & 1) << 1);      // swizzle of this thread's chunks 4 (et & 3) + i
-                        const float4* g4 = reinterpret_cast<const float4*>(stg32 + tk * 128 + f0);
-                        const float4* u4 = reinterpret_cast<const float4*>(stg32 + tk * 128 + 64 + f0);
-                        uint32_t o[8];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float4 g = g4[i ^ rsw], u = u4[i ^ rsw];
-                            const float h0 = __fdividef(g.x, 1.0f + __expf(-g.x)) * u.x;
-                            const float h1 = __fdividef(g.y, 1.0f + __expf(-g.y)) * u.y;
-                            const float h2 = __fdividef(g.z, 1.0f + __expf(-g.z)) * u.z;
-                            const float h3 = __fdividef(g.w, 1.0f + __expf(-g.w)) * u.w;
-                            o[2 * i] = bf16x2(h0, h1);
-                            o[2 * i + 1] = bf16x2(h2, h3);
-                        }
-                        if (tok < tl.tok_end) {
-                            uint4* dst = reinterpret_cast<uint4*>(outb + static_cast<size_t>(tok) * F + wt * 64 + f0);
-                            dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                            dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
-                        }
-                        named_bar_sync(2, 128);
+                    for (int jj = 0; jj < 32; ++jj) {
+                        const float w = __shfl_sync(0xFFFFFFFFu, wv, jj);
+                        const int tr = __shfl_sync(0xFFFFFFFFu, trow, jj);
+                        if (tl.tok0 + c + jj < tl.tok_end && n < p.N)
+                            atomicAdd(outf + static_cast<size_t>(tr) * p.N + n, w * __uint_as_float(v[jj]));
                     }
                 }
             }
@@ -942,7 +1015,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             const int units = ((tl.tok_end - tl.tok0 + 15) >> 4) * 4;
             for (int u = (warp - 4) * p.slices + slice; u < units; u += 20 * p.slices)
                 sum_block(p, smem_u32(partial), rank, u, tl.tok0, tl.tok_end, wt * BW,
-                          stg16 + (warp >= 8 ? warp - 8 : warp + 12) * 512, lane);
+                          stg16 + (warp >= 8 ? (warp - 8) * 512 : 16 * 512 + (warp - 4) * (C::EPI_ST / 2)), lane);
         }
     }
 
