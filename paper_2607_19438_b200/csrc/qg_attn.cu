@@ -53,11 +53,15 @@ struct AttnCfg {
     static constexpr int OFF_K = OFF_Q + 2 * TILE_BYTES;
     static constexpr int OFF_V = OFF_K + NST * TILE_BYTES;
     static constexpr int OFF_BAR = OFF_V + NST * TILE_BYTES;
-    static constexpr int NBAR = 20;
+    static constexpr int NBAR = 19;
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
-    static constexpr int COL_S = 0;                             // S / P of tile t at 128 t
-    static constexpr int COL_O = 256;                           // O of tile t at 256 + D t
+    // tensor memory: heads of 64 have room for S of both query tiles, heads of 128 for one that the tiles use in turn
+    static constexpr bool ONE_S = (D == 128);
+    static constexpr int COL_S = 0;                             // S of tile t at 128 t, or of both at 0
+    static constexpr int COL_P = ONE_S ? 128 : 256;             // P of tile t at COL_P + 64 t
+    static constexpr int COL_O = COL_P + 128;                   // O of tile t at COL_O + D t
+    static constexpr int S_STEP = ONE_S ? 0 : 128;
     static constexpr int TMEM_COLS = 512;
     static constexpr int ROW_BYTES = D * 2;                     // staged output row (16-byte chunks XOR-swizzled by row)
     static_assert(D == 64 || D == 128, "head dimension");
@@ -166,6 +170,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     auto p_full = [&](int t, int h) { return bar0 + 8u * (11 + 2 * t + h); };   // P(j) of keys 64 h .. written (and O
                                                                                  // rescaled): 4 warps arrive
     auto pv_done = [&](int t) { return bar0 + 8u * (15 + t); };    // P(j) V(j) complete
+    auto s_free = [&](int t) { return bar0 + 8u * (17 + t); };     // S(j) is in the registers of its group: 4 warps arrive
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_qb = (p.S + 2 * AT_BQ - 1) / (2 * AT_BQ);
@@ -183,8 +188,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
     pdl_launch_dependents();
     if (warp == 0) {
-        if (lane < 17) {
-            const uint32_t cnt = (lane >= 11 && lane <= 14) ? 4u : 1u;      // p_full: one arrival per softmax warp
+        if (lane < C::NBAR) {
+            const uint32_t cnt = (lane >= 11 && lane <= 14) || lane >= 17 ? 4u : 1u;      // p_full, s_free: one arrival per softmax warp
             mbar_init(bar0 + 8u * lane, cnt);
         }
         if (lane == 31) misc[1] = 0;
@@ -239,23 +244,30 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        // Order of issue: S_A(0), S_B(0); then for every key tile j: P_A(j) V(j), S_A(j + 1), P_B(j) V(j), S_B(j + 1).
-        // MMAs of one thread execute in order, so S_t(j + 1), which overwrites the columns that held P_t(j), cannot
-        // overtake P_t(j) V(j); while the softmax group of one tile works, the MMAs of the other tile run.
+        // Order of issue: S_A(0), S_B(0); then for every key tile j: S_A(j + 1), P_A(j) V(j), S_B(j + 1), P_B(j) V(j).  A group holds
+        // its scores in registers and writes P to columns of its own, so S_t(j + 1) waits neither for P_t(j) nor for its
+        // product: only until the scores that were in its columns have been read.  With one S for both tiles (heads of 128) that
+        // is the other group's read, which takes less than the product issued in between.
         const uint32_t idesc_s = umma_idesc_bf16_major(AT_BQ, AT_BKV, 0u);
         const uint32_t idesc_o = umma_idesc_bf16_major(AT_BQ, D, 1u);
         bool ok = at_wait(q_full, 0u, abort_flag, p);
         const uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);     // group stride, version, 128-byte swizzle
+        int used_t = -1, used_j = 0;                                    // whose scores were put into the shared S last
         auto issue_s = [&](int t, int j, bool last_on_k) -> bool {      // S_t(j) = Q_t K(j)^T
             const int s = j & 1;
             if (!at_wait(k_full(s), (j >> 1) & 1u, abort_flag, p)) return false;
+            if (C::ONE_S ? used_t >= 0 : j > 0) {
+                if (!at_wait(s_free(C::ONE_S ? used_t : t), (C::ONE_S ? used_j : j - 1) & 1u, abort_flag, p)) return false;
+            }
+            used_t = t;
+            used_j = j;
             tc_fence_after_sync();
             if (elect_one()) {
                 const uint32_t q_lo = ((sbase + C::OFF_Q + t * C::TILE_BYTES) >> 4) | (1u << 16);
                 const uint32_t k_lo = ((sbase + C::OFF_K + s * C::TILE_BYTES) >> 4) | (1u << 16);
 #pragma unroll
                 for (int b = 0; b < C::NBOX; ++b)          // 64 head dimensions (one box) per statement
-                    umma_ss_x4(tmem_base + C::COL_S + t * 128, q_lo + b * (C::BOX_BYTES >> 4), k_lo + b * (C::BOX_BYTES >> 4),
+                    umma_ss_x4(tmem_base + C::COL_S + t * C::S_STEP, q_lo + b * (C::BOX_BYTES >> 4), k_lo + b * (C::BOX_BYTES >> 4),
                                desc_hi, idesc_s, b ? 1u : 0u);
                 umma_commit(s_full(t));
                 if (last_on_k) umma_commit(k_empty(s));
@@ -272,12 +284,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (!at_wait(p_full(t, 0), j & 1u, abort_flag, p) || !at_wait(v_full(s), (j >> 1) & 1u, abort_flag, p)) return false;
             tc_fence_after_sync();
             if (elect_one())
-                umma_ts_x4(tmem_base + C::COL_O + t * D, tmem_base + C::COL_S + t * 128, v_lo, desc_hi, idesc_o, j > 0 ? 1u : 0u);
+                umma_ts_x4(tmem_base + C::COL_O + t * D, tmem_base + C::COL_P + t * 64, v_lo, desc_hi, idesc_o, j > 0 ? 1u : 0u);
             __syncwarp();
             if (!at_wait(p_full(t, 1), j & 1u, abort_flag, p)) return false;
             tc_fence_after_sync();
             if (elect_one()) {
-                umma_ts_x4(tmem_base + C::COL_O + t * D, tmem_base + C::COL_S + t * 128 + 32, v_lo + 512, desc_hi, idesc_o, 1u);
+                umma_ts_x4(tmem_base + C::COL_O + t * D, tmem_base + C::COL_P + t * 64 + 32, v_lo + 512, desc_hi, idesc_o, 1u);
                 umma_commit(pv_done(t));
                 if (last_on_v) umma_commit(v_empty(s));
             }
@@ -287,10 +299,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (ok && n_a > 0) ok = issue_s(0, 0, n_b == 0);
         if (ok && n_b > 0) ok = issue_s(1, 0, true);
         for (int j = 0; j < n_loop && ok; ++j) {
-            if (j < n_a && !issue_pv(0, j, !(j < n_b))) { ok = false; break; }
             if (j + 1 < n_a && !issue_s(0, j + 1, !(j + 1 < n_b))) { ok = false; break; }
-            if (j < n_b && !issue_pv(1, j, true)) { ok = false; break; }
+            if (j < n_a && !issue_pv(0, j, !(j < n_b))) { ok = false; break; }
             if (j + 1 < n_b && !issue_s(1, j + 1, true)) { ok = false; break; }
+            if (j < n_b && !issue_pv(1, j, true)) { ok = false; break; }
         }
     } else {
         // ------------------------------------------------ softmax groups (thread = one query row)
@@ -300,7 +312,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int row = quarter * 32 + lane;
         const int qi = q0 + t * AT_BQ + row;                           // query position of this thread
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-        const uint32_t s_addr = lane_addr + C::COL_S + t * 128;
+        const uint32_t s_addr = lane_addr + C::COL_S + t * C::S_STEP, p_addr = lane_addr + C::COL_P + t * 64;
         const uint32_t o_addr = lane_addr + C::COL_O + t * D;
         const float cl = p.scale_log2;
         float m = -INFINITY, l = 0.f;
@@ -312,6 +324,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld_32x32(s_addr + 32 * c, *reinterpret_cast<uint32_t (*)[32]>(v + 32 * c));
             tmem_ld_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free(t));
             const int key0 = j * AT_BKV;
             // keys this row may see in the tile: below `lim` (all 128 except on the diagonal and at the sequence end)
             int lim = p.S - key0;
@@ -378,13 +393,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
                         pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&pb);
                     }
-                    tmem_st_32x32_x8(s_addr + 8 * c, pk);             // P over the columns S came from
+                    if (c == 0 && j > 0) {                             // P's columns are free once the product that read them has completed
+                        ok = at_wait(pv_done(t), (j - 1) & 1u, abort_flag, p);
+                        tc_fence_after_sync();
+                    }
+                    tmem_st_32x32_x8(p_addr + 8 * c, pk);
                 }
                 tmem_st_wait();
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_full(t, hh));
             }
+            if (!ok) break;
             float s0, s1;
             asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(sum2));
             l = l * alpha + (s0 + s1);
