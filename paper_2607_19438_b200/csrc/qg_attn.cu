@@ -9,16 +9,21 @@
 // tile: S = Q K^T is a tcgen05.mma with both operands in shared memory (K-major, 128-byte swizzle, staged by TMA
 // straight from the caller's strided Q / K / V, e.g. the output of a fused QKV projection) and its fp32 result in
 // tensor memory; a group of four softmax warps (one thread per query row, the whole row of 128 scores in registers)
-// keeps the running row maximum and sum and writes P = exp2(...) as bf16 over the tensor-memory columns S came from;
+// keeps the running row maximum and sum and writes P = exp2(...) as bf16 to tensor-memory columns of the tile's own;
 // O += P V is a tcgen05.mma whose A operand is P in tensor memory and whose B operand is the V tile in shared memory
 // read N-major (V's head dimension is contiguous), accumulated in the tile's own tensor-memory region.  The two
-// query tiles share every K / V tile and take turns on the tensor cores: while group A works on its scores the MMAs of
-// tile B run, and the other way round.  When a row maximum grows, the group rescales its O in tensor memory before the
-// next P V is issued.
+// query tiles share every K / V tile and take turns on the tensor cores: while a group works on its scores the other tile's MMAs
+// run and then the tile's own next scores, whose columns are free once the group holds the last ones in registers.  When a row
+// maximum grows, the group rescales its O in tensor memory before the next P V is issued.
 //   warp 0      TMA producer: both Q tiles once, then K and V tiles through two-stage rings
 //   warp 1      MMA issuer, allocates and frees tensor memory
 //   warps 2-5   softmax group A (TMEM lane quarter = warp % 4), O rescaling, final normalisation and store
 //   warps 6-9   the same for tile B
+// What bounds it.  Heads of 128: the tensor pipe, per key tile 16 S instructions of 111 cycles (both operands from shared memory)
+// and 16 P V instructions of 79, 3040 cycles of the 3200 a key tile takes.  Heads of 64: the softmax, 2 x 128 exponentials per
+// row at 16 per clock and SM, 2048 cycles of 2600.  (While P lay over S and a tile's softmax, product and next scores were one
+// chain, a polynomial on the FMA pipe for one exponential in eight shortened it; now it only adds instructions: 24 heads of 128, 4096
+// positions, full 195.6 us with it, 190.5 without; 32 heads of 64 227.8 and 225.8.)  4096 positions before both: 207.9 and 237.
 // Every mbarrier wait is bounded; when one expires the CTA records QG_ERR_TIMEOUT and leaves.
 #include <cuda_bf16.h>
 #include <math.h>
@@ -29,10 +34,6 @@
 namespace qg {
 
 constexpr int AT_BQ = 128, AT_BKV = 128, AT_THREADS = 320;
-// One pair of exponentials in eight goes to the FMA pipe.  The row's warp is bound by the chain of its own instructions as much
-// as by the 16 exponentials per clock and SM, and a polynomial is thirteen instructions for a pair: with one in eight 1500
-// positions take 31.7 us against 32.3 and 8192 (causal, 32 heads) 488 against 497, with two 34.6 and 525, with four 38.5 and 590.
-constexpr int AT_POLY_OF = 8;
 
 struct AttnParams {
     int S, Hq, Hkv, causal;
@@ -53,7 +54,7 @@ struct AttnCfg {
     static constexpr int OFF_K = OFF_Q + 2 * TILE_BYTES;
     static constexpr int OFF_V = OFF_K + NST * TILE_BYTES;
     static constexpr int OFF_BAR = OFF_V + NST * TILE_BYTES;
-    static constexpr int NBAR = 19;
+    static constexpr int NBAR = 20;
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
     // tensor memory: heads of 64 have room for S of both query tiles, heads of 128 for one that the tiles use in turn
@@ -101,42 +102,6 @@ __device__ __forceinline__ float fast_exp2(float x) {     // 2^x, exp2(-inf) = 0
     return y;
 }
 
-// 2^x of a packed pair on the FMA pipe: x = n + f with n by the rounding of x + 1.5 2^23 (whose low bits then are n), 2^f by the
-// degree-5 polynomial with the smallest largest relative error on [-1/2, 1/2] (Remez exchange; 2.1e-7 evaluated in fp32,
-// ex2.approx has 2.4e-7), times 2^n.  From -127 down (masked keys among them) n = -127 makes the factor a zero; a NaN stays one.
-__device__ __forceinline__ uint64_t exp2_poly2(uint64_t x2) {
-    uint64_t r;
-    asm("{\n\t.reg .b64 x, t, n, f, p, s, m1, big, nbig;\n\t.reg .b32 a, b;\n\t"
-        "mov.b64 {a, b}, %1;\n\t"
-        "max.NaN.f32 a, a, 0fC2FE0000;\n\t"              // -127
-        "max.NaN.f32 b, b, 0fC2FE0000;\n\t"
-        "mov.b64 x, {a, b};\n\t"
-        "mov.b64 big, %2;\n\t"
-        "mov.b64 nbig, %3;\n\t"
-        "mov.b64 m1, %4;\n\t"
-        "add.rn.f32x2 t, x, big;\n\t"
-        "add.rn.f32x2 n, t, nbig;\n\t"
-        "fma.rn.f32x2 f, n, m1, x;\n\t"
-        "fma.rn.f32x2 p, f, %5, %6;\n\t"
-        "fma.rn.f32x2 p, p, f, %7;\n\t"
-        "fma.rn.f32x2 p, p, f, %8;\n\t"
-        "fma.rn.f32x2 p, p, f, %9;\n\t"
-        "fma.rn.f32x2 p, p, f, %10;\n\t"
-        "mov.b64 {a, b}, t;\n\t"
-        "shl.b32 a, a, 23;\n\t"
-        "shl.b32 b, b, 23;\n\t"
-        "add.s32 a, a, 0x3F800000;\n\t"
-        "add.s32 b, b, 0x3F800000;\n\t"
-        "mov.b64 s, {a, b};\n\t"
-        "mul.rn.f32x2 %0, p, s;\n\t}"
-        : "=l"(r)
-        : "l"(x2), "l"(pack2(12582912.f, 12582912.f)), "l"(pack2(-12582912.f, -12582912.f)), "l"(pack2(-1.f, -1.f)),
-          "l"(pack2(1.3276472e-3f, 1.3276472e-3f)), "l"(pack2(9.6755410e-3f, 9.6755410e-3f)),
-          "l"(pack2(5.5507131e-2f, 5.5507131e-2f)), "l"(pack2(2.4022120e-1f, 2.4022120e-1f)),
-          "l"(pack2(6.9314694e-1f, 6.9314694e-1f)), "l"(pack2(1.0000001f, 1.0000001f)));
-    return r;
-}
-
 __device__ __forceinline__ bool at_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, const AttnParams& p) {
     const uint32_t limit = p.wait_limit;
     for (int it = 0; it < 16; ++it)
@@ -161,7 +126,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     volatile int* misc = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC);   // [0] tmem base, [1] abort
     volatile int* abort_flag = misc + 1;
     const uint32_t bar0 = sbase + C::OFF_BAR;
-    const uint32_t q_full = bar0;
+    auto q_full = [&](int t) { return bar0 + (t ? 8u * 19u : 0u); };
     auto k_full = [&](int s) { return bar0 + 8u * (1 + s); };
     auto v_full = [&](int s) { return bar0 + 8u * (3 + s); };
     auto k_empty = [&](int s) { return bar0 + 8u * (5 + s); };
@@ -189,7 +154,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     pdl_launch_dependents();
     if (warp == 0) {
         if (lane < C::NBAR) {
-            const uint32_t cnt = (lane >= 11 && lane <= 14) || lane >= 17 ? 4u : 1u;      // p_full, s_free: one arrival per softmax warp
+            const uint32_t cnt = (lane >= 11 && lane <= 14) || lane == 17 || lane == 18 ? 4u : 1u;      // p_full, s_free: one arrival per softmax warp
             mbar_init(bar0 + 8u * lane, cnt);
         }
         if (lane == 31) misc[1] = 0;
@@ -212,15 +177,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         bool ok = true;
-        if (elect_one()) {
-            mbar_arrive_expect_tx(q_full, 2 * C::TILE_BYTES);       // rows past the sequence end arrive as zeros
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
+        // Query tile A and the first keys come first: they are all that the first scores need, and 32 KB take an SM 800 cycles.
+        auto load_q = [&](int t) {
+            if (elect_one()) {
+                mbar_arrive_expect_tx(q_full(t), C::TILE_BYTES);    // rows past the sequence end arrive as zeros
 #pragma unroll
                 for (int a = 0; a < C::NBOX; ++a)
                     tma_load_2d(sbase + C::OFF_Q + t * C::TILE_BYTES + a * C::BOX_BYTES, &tm_q, h * D + 64 * a,
-                                q0 + t * AT_BQ, q_full);
-        }
+                                q0 + t * AT_BQ, q_full(t));
+            }
+            __syncwarp();
+        };
+        load_q(0);
         for (int j = 0; j < n_loop && ok; ++j) {
             const int s = j & 1;
             const uint32_t ph = (j >> 1) & 1u;
@@ -232,6 +200,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     tma_load_2d(sbase + C::OFF_K + s * C::TILE_BYTES + a * C::BOX_BYTES, &tm_k, g * D + 64 * a,
                                 j * AT_BKV, k_full(s));
             }
+            __syncwarp();
+            if (j == 0 && n_b > 0) load_q(1);
             if (!at_wait(v_empty(s), ph ^ 1u, abort_flag, p)) { ok = false; break; }
             if (elect_one()) {
                 mbar_arrive_expect_tx(v_full(s), C::TILE_BYTES);
@@ -250,11 +220,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // is the other group's read, which takes less than the product issued in between.
         const uint32_t idesc_s = umma_idesc_bf16_major(AT_BQ, AT_BKV, 0u);
         const uint32_t idesc_o = umma_idesc_bf16_major(AT_BQ, D, 1u);
-        bool ok = at_wait(q_full, 0u, abort_flag, p);
+        bool ok = true;
         const uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);     // group stride, version, 128-byte swizzle
         int used_t = -1, used_j = 0;                                    // whose scores were put into the shared S last
         auto issue_s = [&](int t, int j, bool last_on_k) -> bool {      // S_t(j) = Q_t K(j)^T
             const int s = j & 1;
+            if (j == 0 && !at_wait(q_full(t), 0u, abort_flag, p)) return false;
             if (!at_wait(k_full(s), (j >> 1) & 1u, abort_flag, p)) return false;
             if (C::ONE_S ? used_t >= 0 : j > 0) {
                 if (!at_wait(s_free(C::ONE_S ? used_t : t), (C::ONE_S ? used_j : j - 1) & 1u, abort_flag, p)) return false;
@@ -382,13 +353,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     for (int i = 0; i < 16; i += 2) {
                         float e0, e1;
                         fma2(e0, e1, __uint_as_float(v[16 * c + i]), __uint_as_float(v[16 * c + i + 1]), cl2, mc2);
-                        float p0, p1;
-                        if ((i >> 1) % AT_POLY_OF == 0) {
-                            const uint64_t pp = exp2_poly2(pack2(e0, e1));
-                            asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(pp));
-                        } else {
-                            p0 = fast_exp2(e0); p1 = fast_exp2(e1);
-                        }
+                        const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
                         sum2 = add2(sum2, p0, p1);
                         const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
                         pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&pb);

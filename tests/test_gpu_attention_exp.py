@@ -1,4 +1,4 @@
-"""The two ways the attention kernel takes its exponentials (one pair of keys in eight on the FMA pipe): scores over the whole
+"""The attention kernel's exponentials: scores over the whole
 range of the exponent, keys that must not count, and NaN, at every position of a group of sixteen keys."""
 import numpy as np
 import pytest
