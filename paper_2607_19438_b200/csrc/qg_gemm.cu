@@ -1171,14 +1171,16 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
     }
 }
 
-// Token tile and schedule of a dense call: the candidate with the smallest modelled time, the model fitted to timings
-// of eleven layer shapes (Q8 and Q4, K from 2048 to 14336, M = 1024 and 2048) on B200.  Data-parallel: a tile costs nkb
-// k-blocks of `period` cycles plus, for the single-accumulator 256-token tile, an exposed epilogue; tiles come in
-// waves of one per SM pair, but a ragged last wave costs less than a full one (the pairs that are done leave L2,
-// HBM and power to the others), so the wave count is taken half-way between the rounded-up and the fractional one.
-// Stream-K: every pair gets the same share of all k-blocks and pays an epilogue per tile it touches plus the exchange
-// of partial tiles; measured, that exchange and the extra epilogues cost 4-8 us per call, so it only wins where it
-// removes most of a wave of long-K tiles, and the model charges it accordingly.
+// Token tile and schedule of a dense call: the candidate with the smallest modelled time, in ns under the power cap, fitted to 121
+// plain shapes (Q8 and Q4, N from 2048 to 16384, K from 768 to 14336, 200 to 4096 tokens) and 25 gate/up shapes on B200.
+// Data-parallel: a tile costs nkb k-blocks of `period` plus, for the single-accumulator 256-token tile, an exposed epilogue;
+// tiles come in waves of one per SM pair, but a ragged last wave costs less than a full one (the pairs that are done leave L2,
+// HBM and power to the others), so the wave count is taken half-way between the rounded-up and the fractional one, and of a
+// single wave as 0.58 + 0.42 of the share of the pairs that have a tile.  16384 x 3072 gate/up, 4 bit, 200 tokens: 29.4 us with 192-token
+// tiles, 20.3 with 256; 1024 tokens 80.1 and 74.8; 4096 x 4096, 8 bit, 4096 tokens: 92.7 and 99.9.
+// Stream-K: every pair gets the same share of all k-blocks and pays an epilogue per tile it touches plus the exchange of partial
+// tiles, 5 us and a tenth of its time, as all pairs draw power to the end.  4096 x 14336: at 256 tokens 42.5 us against 55.7
+// data-parallel, at 1500 143.6 against 128.5.
 struct DensePlan {
     int bt, streamk;
     int slices, kc;      // > 1: K slices of kc k-blocks on the CTA pairs of a cluster
@@ -1190,7 +1192,7 @@ static int slices_capacity(qg_ctx* ctx, int qbits, int bt, int slices) {
 // Few tiles leave most SM pairs idle behind a serial walk over K.  Cutting K into two to four slices, one per pair of a
 // cluster that adds its partial tiles through distributed shared memory, divides the walk; the sum costs
 // 1100 + 1300 (slices - 2) cycles and 20 + 5 (slices - 2) per token of the tile (fitted to 25 shapes at 20 to 500 tokens, a
-// k-block being 515 cycles with up to 128 tokens and 600 with 192).  Stream-K's exchange through global memory costs 22000
+// k-block being 515 cycles with up to 128 tokens and 600 with 192, and 570 of a whole walk of several 128-token tiles).  Stream-K's exchange through global memory costs 22000
 // on top of its share.  Unless the alternative is stream-K, slices take SMs that the next launch could start on: 800 cycles from a
 // quarter of the SM pairs on and 3000 from 0.45 of them on (two slices, K = 1024, 17 tokens: 24 tiles 8.0 us against 7.5 whole, 32 tiles
 // 8.8 against 7.9, 16 tiles 6.7 against 7.4).  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four
@@ -1204,7 +1206,8 @@ static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePla
     const long long tiles0 = n_pw * ((M + plan.bt - 1) / plan.bt);
     if (tiles0 > pairs) return;
     auto period = [](int bt) { return bt == 128 ? 515.0 : bt == 192 ? 600.0 : 720.0; };
-    double best = plan.streamk ? (tiles0 * nk4 + pairs - 1) / pairs * 4.0 * period(plan.bt) + 22000.0 : nk4 * 4.0 * period(plan.bt);
+    double best = plan.streamk ? (tiles0 * nk4 + pairs - 1) / pairs * 4.0 * period(plan.bt) + 22000.0
+                                : nk4 * 4.0 * (plan.bt == 128 && M > 128 ? 570.0 : period(plan.bt));
     best *= 0.97;
     const bool streamk = plan.streamk != 0;
     for (int bt = 128; bt <= 192; bt += 64) {
@@ -1222,9 +1225,9 @@ static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePla
         }
     }
 }
-static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
+static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool streamk) {
     const int cand[3] = {128, 192, 256};
-    const double period[3] = {630.0, 655.0, (qbits == 4) ? 760.0 : 720.0}, epilogue[3] = {0.0, 0.0, 6000.0};
+    const double period[3] = {275.0, 298.0, 365.0}, epilogue[3] = {0.0, 0.0, 2400.0};
     const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
     const int nk4 = K / (4 * BK);
     DensePlan best{256, 0, 1, 0};
@@ -1233,12 +1236,13 @@ static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K
         if (M <= 128 && cand[c] > 128) break;
         const long long tiles = n_pw * ((M + cand[c] - 1) / cand[c]);
         const double frac = static_cast<double>(tiles) / pairs;
-        const double waves = 0.5 * (static_cast<double>((tiles + pairs - 1) / pairs) + frac);
-        const double dp = waves * ((K / BK) * period[c] + epilogue[c]);
-        if (ctx->streamk_mode != 1 || tiles % pairs == 0)
+        const double waves = tiles <= pairs ? 0.58 + 0.42 * frac : 0.5 * (static_cast<double>((tiles + pairs - 1) / pairs) + frac);
+        // (gate/up: the single accumulator has to be clearly faster; at 3000 tokens and more the two are level within the clock's drift)
+        const double dp = waves * ((K / BK) * period[c] + epilogue[c]) * (!streamk && cand[c] == 256 ? 1.03 : 1.0);
+        if (!streamk || ctx->streamk_mode != 1 || tiles % pairs == 0)
             if (dp < best_cost) { best_cost = dp; best = DensePlan{cand[c], 0, 1, 0}; }
     }
-    if (ctx->streamk_mode == 0) return best;
+    if (!streamk || ctx->streamk_mode == 0) return best;
     // Below K = 4096 the exchange never paid in the measurements (K = 2048 and 3072, 64 to 1024 tokens: 2 to 10 us slower).
     if (ctx->streamk_mode != 1 && nk4 < 16) return best;
     for (int c = 0; c < 3; ++c) {
@@ -1250,7 +1254,7 @@ static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K
         const long long share = (units + P - 1) / P;                        // units of the busiest pair
         const double pieces = static_cast<double>(share) / nk4 + 1.5;       // tiles it touches, on average
         if (share / nk4 + 2 > 120) continue;                                // the piece table has 128 entries
-        const double sk = share * 4.0 * period[c] + pieces * epilogue[c] + 10000.0;
+        const double sk = 1.1 * (share * 4.0 * period[c] + pieces * epilogue[c]) + 5000.0;
         if (ctx->streamk_mode == 1 ? (best.streamk == 0 || sk < best_cost) : (sk < 0.95 * best_cost)) {
             best_cost = sk;
             best = DensePlan{cand[c], 1, 1, 0};
@@ -1259,7 +1263,7 @@ static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K
     return best;
 }
 static DensePlan plan_dense(qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
-    DensePlan plan = plan_whole(ctx, qbits, M, n_wt, K);
+    DensePlan plan = plan_whole(ctx, M, n_wt, K, true);
     plan_slices(ctx, qbits, M, n_wt, K, plan);
     return plan;
 }
@@ -1354,8 +1358,7 @@ int qgemm_dense_gate_up_silu(qg_ctx* ctx, int qbits, int M, int F, int K, const 
     p.mode = QG_MODE_GATE_UP_SILU; p.R = M; p.N = 2 * F; p.K = K; p.E = 1; p.k = 1;
     p.n_wt = (2 * F) / 128;
     p.offsets = nullptr; p.out = Out; p.topk_w = nullptr; p.row_pair = nullptr;
-    // this epilogue always overlaps the next tile (two accumulators), so the 256-token tile is not a candidate
-    const int bt = (M > 128) ? 192 : 128;
+    const int bt = qg::plan_whole(ctx, M, p.n_wt, K, false).bt;
     return qg::dispatch_gemm(ctx, qbits, bt, p, A, M, Wq, Wscale, static_cast<cudaStream_t>(stream));
 }
 
