@@ -1384,9 +1384,12 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     p.n_wt = (mode == QG_MODE_GATE_UP_SILU) ? (N / 128) : (N + qg::BW - 1) / qg::BW;
     p.gather_k = gather_k;
     p.offsets = expert_offsets; p.out = Out; p.topk_w = topk_w; p.row_pair = row_pair;
-    // expected rows per expert decide the token tile; 192 keeps two accumulators, so the short main loops of
-    // expert tiles overlap their epilogues
-    const int bt = (R / E > 100) ? 192 : 128;
+    // Expected rows per expert decide the token tile.  A 192-token tile keeps two accumulators, and an expert with more rows than the
+    // average converts its weights once instead of twice.  128 experts, 1536 x 2048 / 2048 x 768, 192 against 128 tokens: 4 bit,
+    // 32 rows per expert 95.6 / 52.2 us against 97.6 / 52.5, 64 rows 99.0 / 55.0 against 100.7 / 55.0, with a quarter of the
+    // experts preferred 99.7 / 55.7 against 116.7 / 66.2; 8 bit, 64 rows 104.5 / 57.4 against 103.4 / 57.3.  (Behind the streaming
+    // kernel the tile is 128 tokens: those calls have up to 18 rows per expert.)
+    const int bt = (R / E > (qbits == QG_Q4 ? qg::GroupedChoice::MAX_ROWS : 50)) ? 192 : 128;
     // a few rows per expert (4-bit weights, no accumulation) the streaming kernel is faster; the gathering form takes the same
     // kernel as the form for sorted rows, so that they give the same numbers
     qg::GroupedChoice choice{};
