@@ -33,9 +33,9 @@ enum AttrSlot {
     ATTR_MX_MOE = 32,       // 2: down, gate/up
     ATTR_MX_256 = 34,
     ATTR_STREAM = 35,       // 8: sorted, gathered rows x down, gate/up x rows per tile (2)
-    ATTR_DENSE_STREAM = 43, // 4: format (2) x more than eight tokens (2)
-    ATTR_GEMM_CHOICE = 47,  // 2: epilogue
-    ATTR_SLOTS = 49
+    ATTR_DENSE_STREAM = 43, // 8: K whole, in slices x format (2) x more than eight tokens (2)
+    ATTR_GEMM_CHOICE = 51,  // 2: epilogue
+    ATTR_SLOTS = 53
 };
 }  // namespace qg
 

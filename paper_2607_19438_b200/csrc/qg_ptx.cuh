@@ -77,6 +77,15 @@ __device__ __forceinline__ void cluster_sync_all() {   // every thread of both C
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same in two halves, for threads that do not arrive together.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// 16 bytes to a shared::cluster address, counted on the barrier `bar_cluster` of the same CTA when they are there.
+__device__ __forceinline__ void st_async_v4(uint32_t dst_cluster, float a, float b, float c, float d, uint32_t bar_cluster) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(dst_cluster), "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar_cluster) : "memory");
+}
+
 // Cluster launch control: asks the hardware for a block of this grid that has not been started; the 16-byte answer arrives at
 // `answer` (shared memory) and completes 16 bytes on `bar`.  No request may follow one that was refused.
 __device__ __forceinline__ void clc_try_cancel(uint32_t answer, uint32_t bar) {

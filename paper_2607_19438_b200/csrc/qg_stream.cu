@@ -65,6 +65,8 @@ constexpr int MS_W_BYTES = 16384;                     // codes per stage: 128 ro
 __host__ __device__ constexpr int ms_rows(int qbits) { return qbits == 4 ? 128 : 64; }        // weight rows per tile
 __host__ __device__ constexpr int ms_s_bytes(int qbits) { return ms_rows(qbits) * 16; }       // eight scales per row
 constexpr int MS_X_BYTES = 8 * MS_SK * 2;             // eight token rows
+// Room for the fragments that a CTA adds, of all slices: each slice sends a share of 4 x 32 fragments of 16 bytes per MMA tile.
+__host__ __device__ constexpr int ms_recv_bytes(int mma_tiles) { return (4 * 32 * mma_tiles + 8 * 7) * 16; }
 constexpr int MS_CONS_WARPS = 8, MS_THREADS = 32 * (MS_CONS_WARPS + 2);
 constexpr int MS_NT = 2;                              // most groups of eight segment rows per tile
 constexpr int MS_MAX_ST = 6;
@@ -222,7 +224,7 @@ __device__ __forceinline__ float zero_if_finite(float z, float a, float b, float
 // fragment needs follow one another in lane order.  Rows past the end arrive as zeros.  Gathered rows: [M][K], box 256 k x one
 // row, four rows per copy, which land row after row.
 // grid = (tiles, K slices); the slices of a tile are one cluster.
-template <int QBITS, bool GROUPED, bool GATE_UP, int NTM, bool GATHER>
+template <int QBITS, bool GROUPED, bool GATE_UP, int NTM, bool GATHER, bool SLICED = false>
 __global__ void __launch_bounds__(MS_THREADS, 2)
 stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
               const __grid_constant__ CUtensorMap tm_x, const StreamParams p) {
@@ -233,6 +235,8 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     uint8_t* after = ms_smem + (ring - smem_u32(ms_smem)) + p.n_stages * p.stage_bytes;
     const uint32_t xch = smem_u32(after);              // [4 warps][NTM][MT][32 lanes] float4: sums handed from set to set, or of the slice
     after += 4 * NTM * MT * 512;
+    const uint32_t recv = smem_u32(after);             // K slices: [slices][fragments this CTA adds] float4, written by the cluster's CTAs
+    if (SLICED) after += ms_recv_bytes(NTM * MT);
     // full: stage i's barrier is number i mod 2 n_stages (twice the slots), so that one set waits on it every time it is used:
     // with one barrier per slot and an odd number of slots a set would see every other phase only, and a wait by parity
     // passes too early while the phase in between is not complete.
@@ -240,6 +244,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t hfull0 = xfull0 + 8u * MS_MAX_ST, hempty0 = hfull0 + 32u;      // the hand-over of each pair of warps
     after += 32 * MS_MAX_ST + 64;
     const uint32_t taken = smem_u32(after), taken_bar = taken + 16;      // the hardware's answer to a request for a tile
+    const uint32_t recv_bar = taken + 24;              // the fragments of all slices are there
     after += 32;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(after);
     volatile StreamTile* tiles = reinterpret_cast<volatile StreamTile*>(after + 16);   // per stage: the tile it belongs to
@@ -251,7 +256,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (lane < 2 * p.n_stages) mbar_init(full0 + 8u * lane, 2);
         if (lane < p.n_stages) { mbar_init(empty0 + 8u * lane, MS_CONS_WARPS / 2); mbar_init(xfull0 + 8u * lane, 1); }
         if (lane >= 16 && lane < 24) mbar_init(hfull0 + 8u * (lane - 16), 1);
-        if (lane == 31) { *abort_flag = 0; mbar_init(taken_bar, 1); }
+        if (lane == 31) { *abort_flag = 0; mbar_init(taken_bar, 1); mbar_init(recv_bar, 1); }
         fence_mbar_init();
         fence_proxy_async_smem();
     }
@@ -288,7 +293,16 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     }
     const int k0 = static_cast<int>(blockIdx.y) * p.kc;
     const int nst = min(p.kc, p.K - k0) / MS_SK;       // stages of a tile
-    const bool sliced = p.kc < p.K;                    // then this CTA has one tile
+    // K slices (SLICED: p.kc < p.K, and a CTA has one tile): the CTAs of a cluster hold one slice's sums of the same tile each.  Every CTA adds a share of the tile's fragments (16
+    // bytes: rows lo / hi x two tokens): the others send theirs to its shared memory, and a barrier there counts the bytes.
+    const uint32_t n_frag = 4 * MT * 32 * ((p.R + 7) >> 3), share = (n_frag + gridDim.y - 1) / gridDim.y, rank = blockIdx.y;
+    const uint32_t my_frags = rank * share < n_frag ? min(share, n_frag - rank * share) : 0;
+    if constexpr (SLICED) {
+        if (threadIdx.x == 0) mbar_arrive_expect_tx(recv_bar, my_frags * gridDim.y * 16);
+        __syncwarp();
+        cluster_arrive();
+        if (warp < MS_CONS_WARPS) cluster_wait();      // the others' barriers are set up
+    }
 
     if (warp == MS_CONS_WARPS) {
         // ------------------------------------------------ producer
@@ -440,7 +454,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         for (uint32_t q = 0, base = 0; ; ++q, base += nst) {              // tile and its first stage, both counted from 0
             const uint32_t first = base + ((base ^ set) & 1u);            // this set's first stage of the tile
             if (first >= base + nst) {                                    // a tile of one stage: every other one is the other set's
-                if (sliced) break;
+                if (SLICED) break;
                 continue;
             }
             if (!__all_sync(0xFFFFFFFFu, ms_wait(full0 + 8u * fslot, fphase, abort_flag, p))) break;
@@ -501,8 +515,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                         const uint4 v = lds_u4(at);
                         c0 += __uint_as_float(v.x); c1 += __uint_as_float(v.y); c2 += __uint_as_float(v.z); c3 += __uint_as_float(v.w);
                     }
-                    if (sliced) {             // this slice's sum: added over the cluster below
-                        sts_u4(at, make_uint4(__float_as_uint(c0), __float_as_uint(c1), __float_as_uint(c2), __float_as_uint(c3)));
+                    if constexpr (SLICED) {   // this slice's sum: to the CTA that adds this fragment
+                        const uint32_t i = ((nt * 4 + w4) * MT + m) * 32 + lane, to = i / share;
+                        st_async_v4(map_to_cta(recv + (rank * share + i - to * share) * 16, to), c0, c1, c2, c3, map_to_cta(recv_bar, to));
                         continue;
                     }
                     z = zero_if_finite(z, c0, c1, c2, c3);
@@ -527,7 +542,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                     }
                 }
             }
-            if (sliced) break;
+            if (SLICED) break;
             if (nst > 1) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(hempty);
@@ -544,21 +559,18 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
         }
     }
-    __syncthreads();
-    if (!GROUPED && sliced) {
-        // The CTAs of a cluster hold one slice's sums of the same tile each: a fragment (16 bytes: rows lo / hi x two tokens) is
-        // added over all of them in slice order, so results are reproducible, by one thread of one of them.
-        cluster_sync_all();
-        const uint32_t ns = gridDim.y, n_frag = 4 * MT * 32 * ((p.R + 7) >> 3);
-        for (uint32_t i = cluster_ctarank() * MS_THREADS + threadIdx.x; i < n_frag; i += ns * MS_THREADS) {
-            // i = (((token group) 4 + warp) MT + MMA tile) 32 + lane
+    if constexpr (SLICED) {
+        // A fragment's slices are added in order, so results are reproducible.  Nobody leaves before everybody has sent, which this CTA
+        // waits for anyway.  (Until all had met, read each other's sums and met again: 0.9 us of 5 to 9.)
+        if (warp >= MS_CONS_WARPS) cluster_wait();
+        cluster_arrive();
+        if (threadIdx.x < my_frags && ms_wait(recv_bar, 0u, abort_flag, p)) {
+            const uint32_t i = rank * share + threadIdx.x;               // (((token group) 4 + warp) MT + MMA tile) 32 + lane
             const uint32_t l = i & 31u, m = (i >> 5) % MT, w4 = (i / (32u * MT)) & 3u, nt = i / (128u * MT);
-            const uint32_t at = xch + ((w4 * NTM + nt) * MT + m) * 512 + l * 16;
             float c[4] = {0.f, 0.f, 0.f, 0.f};
-            for (uint32_t sl = 0; sl < ns; ++sl) {
-                float4 v;
-                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(map_to_cta(at, sl)));
-                c[0] += v.x; c[1] += v.y; c[2] += v.z; c[3] += v.w;
+            for (uint32_t sl = 0; sl < gridDim.y; ++sl) {
+                const uint4 v = lds_u4(recv + (sl * share + threadIdx.x) * 16);
+                c[0] += __uint_as_float(v.x); c[1] += __uint_as_float(v.y); c[2] += __uint_as_float(v.z); c[3] += __uint_as_float(v.w);
             }
             const int t = 8 * nt + 2 * (l & 3), r = blockIdx.x * ROWS + 16 * (MT * w4 + m);
             __nv_bfloat16* o = p.out + static_cast<size_t>(t) * p.N + r + (l >> 2);
@@ -574,8 +586,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll 1
                 for (int u = t; u < min(t + 2, p.R); ++u) ms_again<QBITS, false, false>(p, 0, u, r + (l >> 2));
         }
-        cluster_sync_all();                    // nobody reads this CTA's shared memory any more
+        cluster_wait();
     }
+    __syncthreads();
     if (*abort_flag) {
         for (int i = 0; i < 64; ++i) __nanosleep(2000);       // copies still in flight land before the memory is released
     }
@@ -584,7 +597,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 // Ring depth and shared memory of a launch; false if not even two stages fit.
 static bool ms_layout(StreamParams& p, int qbits, int ntm, int n_exp, size_t& smem) {
     p.stage_bytes = (MS_W_BYTES + ms_s_bytes(qbits) + ntm * MS_X_BYTES + 1023) & ~1023;      // the codes' swizzle wants 1 KB
-    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + 32 * MS_MAX_ST + 64 + 32 + 16 + 16 * MS_MAX_ST +
+    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + (n_exp ? 0 : ms_recv_bytes(ntm * (ms_rows(qbits) / 64))) + 32 * MS_MAX_ST + 64 + 32 + 16 + 16 * MS_MAX_ST +
                          (2 * static_cast<size_t>(n_exp) + 2) * sizeof(int);
     p.n_stages = static_cast<int>((MS_SMEM_MAX - fixed) / p.stage_bytes);
     if (p.n_stages > MS_MAX_ST) p.n_stages = MS_MAX_ST;
@@ -670,9 +683,12 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
     StreamParams p{};
     size_t smem = 0;
     if (!ms_layout(p, qbits, ntm, 0, smem)) return QG_ERR_WORKSPACE;
-    const StreamKernel kern = (qbits == 8) ? (ntm == 1 ? stream_kernel<8, false, false, 1, false> : stream_kernel<8, false, false, 2, false>)
-                                           : (ntm == 1 ? stream_kernel<4, false, false, 1, false> : stream_kernel<4, false, false, 2, false>);
-    int rc = ms_set_smem(ctx, kern, ATTR_DENSE_STREAM + variant);
+    const StreamKernel whole[4] = {stream_kernel<8, false, false, 1, false>, stream_kernel<8, false, false, 2, false>,
+                                   stream_kernel<4, false, false, 1, false>, stream_kernel<4, false, false, 2, false>};
+    const StreamKernel cut[4] = {stream_kernel<8, false, false, 1, false, true>, stream_kernel<8, false, false, 2, false, true>,
+                                 stream_kernel<4, false, false, 1, false, true>, stream_kernel<4, false, false, 2, false, true>};
+    int rc = ms_set_smem(ctx, whole[variant], ATTR_DENSE_STREAM + variant);
+    if (rc == QG_OK) rc = ms_set_smem(ctx, cut[variant], ATTR_DENSE_STREAM + 4 + variant);
     if (rc != QG_OK) return rc;
     // clusters of `ns` CTAs of this kernel that fit on the GPU at once (asked once per context, variant and size)
     auto cluster_capacity = [&](int ns) {
@@ -684,7 +700,7 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
             ca.val.clusterDim.x = 1; ca.val.clusterDim.y = ns; ca.val.clusterDim.z = 1;
             q.gridDim = dim3(1, ns); q.blockDim = dim3(MS_THREADS); q.dynamicSmemBytes = smem; q.attrs = &ca; q.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess) { cudaGetLastError(); n = 0; }
+            if (cudaOccupancyMaxActiveClusters(&n, cut[variant], &q) != cudaSuccess) { cudaGetLastError(); n = 0; }
             cached = n > 0 ? n : -1;
         }
         return cached;
@@ -742,7 +758,7 @@ int launch_dense_stream(qg_ctx* ctx, int qbits, int M, int N, int K, const void*
         ++n_at;
     }
     cfg.attrs = at; cfg.numAttrs = n_at;
-    if (cudaLaunchKernelEx(&cfg, kern, tm_w, tm_s, tm_x, p) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, slices > 1 ? cut[variant] : whole[variant], tm_w, tm_s, tm_x, p) != cudaSuccess) {
         cudaGetLastError();
         if (slices == 1) return QG_ERR_CUDA;
         // the cluster launch was refused although the occupancy query allowed it: remember that and leave K whole
