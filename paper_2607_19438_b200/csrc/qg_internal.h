@@ -115,8 +115,8 @@ int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
 //   The host weighs three calls with evenly spread rows against one with all rows in one segment: the streaming kernel alone,
 // the other alone, or both, in which case each works out the same answer from the offsets and the one that is not wanted ends at
 // once.  That costs every such call 5 to 8 us (the unwanted launch keeps the next one from starting early).  128 experts,
-// 1536 x 2048: alone up to 11 rows per expert (even 63 us against 99, one segment 38 against 17 at eight rows), both up to 16,
-// the other from there (even 96 against 99, one segment 70 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
+// 1536 x 2048: alone up to 11 rows per expert (even 62 us against 95, one segment 38 against 17 at eight rows), both up to 16,
+// the other from there (even 95 against 95, one segment 70 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
 // (even 917 us against 1605 of the other alone; eight segments 183 against 622 when the average alone decided, and 154 of the
 // other alone).
 struct GroupedChoice {

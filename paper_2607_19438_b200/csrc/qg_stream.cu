@@ -47,6 +47,8 @@
 // rounded scaled 8-bit weights, a block kernel and the tensor-memory kernel, whichever was fastest: 28672 x 4096 8 bit
 // 32.3 / 38.2 us (3.9 / 3.3 TB/s) against 34.3 / 39.5; 4096 x 14336 16.4 / 19.8 against 19.0 / 28.7; 4096 x 4096 8.0 / 9.6
 // against 8.6 / 13.2; 2048 x 2048 5.6 / 6.6 against 5.9 / 7.0; 3072 x 8192 4 bit 9.0 / 12.1 against 15.4 / 26.3.
+// K slices send their sums to the CTA that adds them (st.async); while they met, read each other's and met again, 1 / 16 tokens back to back in
+// a graph: 2048 x 2048 8 bit 4.8 / 5.9 us, now 4.35 / 4.95; 3072 x 8192 4 bit 8.7 / 10.75, now 7.7 / 9.8; 5120 x 3072 6.7 / 8.3, now 6.1 / 7.3.
 // What bounds it: without its arithmetic the 28672 x 4096 launch takes 26.4 us, with the codes' loads alone 22.1 (5.65 TB/s);
 // supply and arithmetic overlap, but with 16 consumer warps per SM neither hides the other fully.
 // Every mbarrier wait is bounded.
