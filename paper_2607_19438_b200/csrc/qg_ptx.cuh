@@ -44,11 +44,37 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // Non-blocking test of a phase: returns at once, so a spinning warp sees the completion within one poll instead of after the
 // wake-up of a suspended try_wait.  CTA scope also where the phase may be completed by the peer CTA of a pair: what those
 // barriers order are tensor-memory accesses and asynchronous copies, and an acquire of cluster scope costs every poll 30 cycles.
+// Not where another CTA's st.async is read by ordinary loads afterwards: that takes the two below.
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred P;\n\t"
         "mbarrier.test_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// The same two with an acquire of cluster scope: what other CTAs of the cluster stored (st.async, whose completion is a release of
+// that scope) may be read by ordinary loads once the phase is complete.
+__device__ __forceinline__ bool mbar_test_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
         "selp.b32 %0, 1, 0, P;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)

@@ -98,10 +98,11 @@ struct StreamParams {
     int skip_stage;             // test hook: stage of the first CTA whose token rows are never loaded (-1: none)
 };
 
+template <bool CLUSTER = false>         // other CTAs' stores are read after the wait
 __device__ __forceinline__ bool ms_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, const StreamParams& p) {
-    if (mbar_test_wait(bar, parity)) return true;
+    if (CLUSTER ? mbar_test_wait_cluster(bar, parity) : mbar_test_wait(bar, parity)) return true;
     for (uint32_t it = 0; it < p.wait_limit; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
         if ((it & 255u) == 255u && *abort_flag) return false;
     }
     *abort_flag = 1;
@@ -566,7 +567,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         // waits for anyway.  (Until all had met, read each other's sums and met again: 0.9 us of 5 to 9.)
         if (warp >= MS_CONS_WARPS) cluster_wait();
         cluster_arrive();
-        if (threadIdx.x < my_frags && ms_wait(recv_bar, 0u, abort_flag, p)) {
+        if (threadIdx.x < my_frags && ms_wait<true>(recv_bar, 0u, abort_flag, p)) {
             const uint32_t i = rank * share + threadIdx.x;               // (((token group) 4 + warp) MT + MMA tile) 32 + lane
             const uint32_t l = i & 31u, m = (i >> 5) % MT, w4 = (i / (32u * MT)) & 3u, nt = i / (128u * MT);
             float c[4] = {0.f, 0.f, 0.f, 0.f};

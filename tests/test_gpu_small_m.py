@@ -89,6 +89,29 @@ def test_small_m_wait_that_runs_out(qbits, M, N, K, mode, skip):
     util.assert_close(util.host_bf16_f64(out)[:, rows], orc.qgemm_dense(qbits, A, Wq[rows], Ws[rows]), "after a timeout")
 
 
+@pytest.mark.parametrize("M", [3, 16])
+@pytest.mark.parametrize("qbits,N,K", [(8, 72, 512), (8, 4096, 768), (8, 2048, 2048), (4, 2560, 1280), (8, 1024, 1536), (4, 136, 1792), (8, 2048, 8192),
+                                       (8, 264, 2048), (4, 3072, 8192)], ids=["2", "3", "4", "5", "6", "7", "7-deep", "8", "8-deep"])
+def test_sums_that_slices_send_one_another(qbits, N, K, M):
+    """Two to eight K slices.  Every call has other tokens, so a sum read before it arrived (shared memory still holds an earlier launch's)
+    would show; integer products and power-of-two scales, so the sums are exact and the bits are those of K left whole."""
+    rng = np.random.default_rng(23)
+    if qbits == 8:
+        Wq = rng.integers(-127, 128, (N, K)).astype(np.int8)
+    else:
+        Wq = rng.integers(0, 256, (N, K // 2)).astype(np.uint8)
+    dWq, dWs = util.dev(Wq), util.dev_f16(np.full((N, K // 32), 0.125, np.float16).view(np.uint16))
+    xs = [util.dev_bf16(synth.f32_to_bf16_bits(rng.integers(-1, 2, (M, K)).astype(np.float32))) for _ in range(48)]
+    qg.test_gemv_mode(3)
+    whole = [qg.qgemm_small_m(qbits, x, dWq, dWs) for x in xs]
+    qg.test_gemv_mode(2)
+    cut = [qg.qgemm_small_m(qbits, x, dWq, dWs) for x in xs]
+    qg.poll_status()
+    assert all(torch.equal(a, b) for a, b in zip(whole, cut))
+    ref = orc.qgemm_dense(qbits, util.host_bf16_bits(xs[-1]), Wq, util.host_bf16_bits(dWs))
+    assert np.array_equal(util.host_bf16_bits(cut[-1]), orc.f64_to_bf16(ref))
+
+
 @pytest.mark.parametrize("mode", [2, 4], ids=["stream", "block"])
 @pytest.mark.parametrize("qbits", [8, 4])
 def test_small_m_integer_exact_is_bit_exact(qbits, mode):
