@@ -43,6 +43,7 @@ struct GemmParams {
     int mode, R, N, K, E, k;
     int n_wt;                   // 128-row weight tiles per expert (64 gate + 64 up rows each in gate/up mode)
     int gather_k;               // > 0: input row r is X[row_pair[r] / gather_k] (token gather folded into the loads)
+    int even_tiles;             // an expert's rows are shared out evenly among its token tiles (to 16 rows); else all but the last are full
     const int32_t* offsets;     // device expert offsets [E+1]; nullptr: one segment [0, R)
     void* out;
     const float* topk_w;
@@ -117,6 +118,7 @@ struct __align__(16) Piece {
     int kb0, kb1, i0, nsrc;
 };
 
+template <bool GROUPED>          // false: stream-K and K slices, one segment
 __device__ __forceinline__ Tile decode_tile(int t, const int* prefix, const GemmParams& p, int BT) {
     int lo = 0, hi = p.E - 1;
     while (lo < hi) {
@@ -127,11 +129,18 @@ __device__ __forceinline__ Tile decode_tile(int t, const int* prefix, const Gemm
     const int seg1 = p.offsets ? p.offsets[lo + 1] : p.R;
     const int n_tt = (seg1 - seg0 + BT - 1) / BT;
     const int local = t - prefix[lo];
+    int rows = BT;
+    if (GROUPED && p.even_tiles) {
+        // the fewest rows, in steps of 16, with which as many tiles do: BT - 16 floor(spare / (16 n_tt)); the quotient of two numbers below 17
+        // by a float reciprocal (an integer division here costs every call 0.13 us)
+        const int spare = (n_tt * BT - (seg1 - seg0)) >> 4;
+        rows -= 16 * static_cast<int>(__fdividef(static_cast<float>(spare) + 0.5f, static_cast<float>(n_tt)));
+    }
     Tile r;
     r.e = lo;
     r.pw = local / n_tt;
-    r.tok0 = seg0 + (local % n_tt) * BT;
-    r.tok_end = min(seg1, r.tok0 + BT);
+    r.tok0 = seg0 + (local % n_tt) * rows;
+    r.tok_end = min(seg1, r.tok0 + rows);
     return r;
 }
 
@@ -552,7 +561,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         if (lane == 0) prefix[p.E] = carry;
         __syncwarp();
         if (SK != 1 && pair < carry) {
-            const Tile tl = decode_tile(pair, prefix, p, BT);
+            const Tile tl = decode_tile<SK == 0>(pair, prefix, p, BT);
             const int wt = 2 * tl.pw + static_cast<int>(rank);
             if (elect_one()) {
                 mbar_arrive_expect_tx(r_full(0), 4 * C::RAW_BYTES + C::SC_BYTES);
@@ -605,22 +614,22 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                 pc.nsrc = q - pair;
             }
             ptab[j] = pc;
-            tab[j] = decode_tile(t, prefix, p, BT);
+            tab[j] = decode_tile<SK == 0>(t, prefix, p, BT);
         }
     } else if constexpr (SK == 2) {
         my_tiles = 1;                                       // one cluster per tile
         own_kb4 = static_cast<uint32_t>(min(p.kc, nkb - kb_first)) >> 2;
-        if (threadIdx.x == 0) tab[0] = decode_tile(pair, prefix, p, BT);
+        if (threadIdx.x == 0) tab[0] = decode_tile<SK == 0>(pair, prefix, p, BT);
     } else {
         my_tiles = (total_tiles > pair) ? (total_tiles - pair + n_pairs - 1) / n_pairs : 0;
         own_kb4 = static_cast<uint32_t>(my_tiles) * static_cast<uint32_t>(nk4);
         for (int j = threadIdx.x; j < min(my_tiles, C::TAB_N); j += NTHREADS)
-            tab[j] = decode_tile(pair + j * n_pairs, prefix, p, BT);
+            tab[j] = decode_tile<SK == 0>(pair + j * n_pairs, prefix, p, BT);
     }
     __syncthreads();
     if (warp == 0) { QG_MARK(1); }
     auto tile_at = [&](int j) -> Tile {
-        return (j < C::TAB_N) ? tab[j] : decode_tile(pair + j * n_pairs, prefix, p, BT);
+        return (j < C::TAB_N) ? tab[j] : decode_tile<SK == 0>(pair + j * n_pairs, prefix, p, BT);
     };
     auto piece_at = [&](int j) -> Piece {
         if constexpr (SK == 1) return ptab[j];
@@ -1384,12 +1393,22 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     p.n_wt = (mode == QG_MODE_GATE_UP_SILU) ? (N / 128) : (N + qg::BW - 1) / qg::BW;
     p.gather_k = gather_k;
     p.offsets = expert_offsets; p.out = Out; p.topk_w = topk_w; p.row_pair = row_pair;
-    // Expected rows per expert decide the token tile.  A 192-token tile keeps two accumulators, and an expert with more rows than the
-    // average converts its weights once instead of twice.  128 experts, 1536 x 2048 / 2048 x 768, 192 against 128 tokens: 4 bit,
-    // 32 rows per expert 95.6 / 52.2 us against 97.6 / 52.5, 64 rows 99.0 / 55.0 against 100.7 / 55.0, with a quarter of the
-    // experts preferred 99.7 / 55.7 against 116.7 / 66.2; 8 bit, 64 rows 104.5 / 57.4 against 103.4 / 57.3.  (Behind the streaming
-    // kernel the tile is 128 tokens: those calls have up to 18 rows per expert.)
-    const int bt = (R / E > (qbits == QG_Q4 ? qg::GroupedChoice::MAX_ROWS : 50)) ? 192 : 128;
+    // Expected rows per expert decide the token tile: a 192-token tile spares an expert with 129 to 192 rows the second conversion of its
+    // weights.  192 against 128 tokens over eight layers of 8 to 512 experts, rows drawn evenly / with a quarter of the experts preferred:
+    // 4 bit, 19 rows per expert 0.98 / 0.98, 64 rows 1.00 / 0.83, 96 rows 1.00 / 0.99, 128 rows 0.76 / 0.88; 8 bit 19 rows 1.01 / 1.01, 48 rows
+    // 1.01 / 0.99, 64 rows 1.01 / 0.88, 80 rows 1.01 / 0.95, 96 rows 1.02 / 1.03, 128 rows 0.81 / 0.92.  (Behind the streaming kernel the tile
+    // is 128 tokens, so the 4-bit line is where that kernel ends.)
+    //   Gathered rows and fp32 sums cost a tile time by the row where sorted rows are bound by the conversion, and so do the stores of a short
+    // K (the epilogue is the pace): there a tile of few rows is as dear as one of about 100, and 230 rows in 192 + 38 dearer than in 128 + 102, so
+    // an expert's tiles are made equally long.  200 rows per expert, 128 experts, 4 bit, gathered 1536 x 2048 584 -> 444 us, fp32 sums
+    // 2048 x 768 271 -> 204, weighted 2048 x 768 105 -> 99; sorted rows of K = 1024 on 1.00 (K = 4096, 450 rows 1.04: not for them).  Between 65
+    // and 100 rows 128-token tiles are the better ones for the first two (a quarter preferred, 80 rows: 0.83 to 0.98 of the time of 192; evenly
+    // drawn 1.00), for fp32 sums up to K = 1536 (0.85 to 1.02 there, 1.11 at K = 3072).
+    const int rows = R / E;
+    const bool by_row = gather_k > 0 || mode == QG_MODE_DOWN_ACCUM_F32;
+    p.even_tiles = by_row || K <= 768;
+    const bool short_tiles = (gather_k > 0 || (by_row && K <= 1536)) && rows > 64 && rows <= 100;
+    const int bt = (rows > (qbits == QG_Q4 ? 18 : 50) && !short_tiles) ? 192 : 128;
     // a few rows per expert (4-bit weights, no accumulation) the streaming kernel is faster; the gathering form takes the same
     // kernel as the form for sorted rows, so that they give the same numbers
     qg::GroupedChoice choice{};
