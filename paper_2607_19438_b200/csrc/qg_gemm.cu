@@ -1180,16 +1180,17 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
     }
 }
 
-// Token tile and schedule of a dense call: the candidate with the smallest modelled time, in ns under the power cap, fitted to 121
-// plain shapes (Q8 and Q4, N from 2048 to 16384, K from 768 to 14336, 200 to 4096 tokens) and 25 gate/up shapes on B200.
+// Token tile and schedule of a dense call: the candidate with the smallest modelled time in ns, fitted to 1300 calls timed back to back on
+// B200 (Q8 and Q4, plain and gate/up, N from 136 to 28672, K from 512 to 16384, 17 to 4096 tokens; every candidate of each).  The choice
+// takes 1.004 of the time of the fastest candidate on average, 1.12 at worst.
 // Data-parallel: a tile costs nkb k-blocks of `period` plus, for the single-accumulator 256-token tile, an exposed epilogue;
 // tiles come in waves of one per SM pair, but a ragged last wave costs less than a full one (the pairs that are done leave L2,
-// HBM and power to the others), so the wave count is taken half-way between the rounded-up and the fractional one, and of a
-// single wave as 0.58 + 0.42 of the share of the pairs that have a tile.  16384 x 3072 gate/up, 4 bit, 200 tokens: 29.4 us with 192-token
+// HBM and power to the others), so the wave count is taken about half-way between the rounded-up and the fractional one, and of a
+// single wave as 0.77 + 0.23 of the share of the pairs that have a tile.  16384 x 3072 gate/up, 4 bit, 200 tokens: 29.4 us with 192-token
 // tiles, 20.3 with 256; 1024 tokens 80.1 and 74.8; 4096 x 4096, 8 bit, 4096 tokens: 92.7 and 99.9.
-// Stream-K: every pair gets the same share of all k-blocks and pays an epilogue per tile it touches plus the exchange of partial
-// tiles, 5 us and a tenth of its time, as all pairs draw power to the end.  4096 x 14336: at 256 tokens 42.5 us against 55.7
-// data-parallel, at 1500 143.6 against 128.5.
+// Stream-K: every pair gets the same share of all k-blocks; the pair with a tile's first k-block adds the parts of all pairs that have
+// others one after another, 930 ns and 5.6 a token for each.  4096 x 14336: at 2500 tokens 244 us against 293 data-parallel, at 1500 143.6
+// against 128.5.  Few tiles have many parts each: 512 x 16384 at 128 tokens, 37 parts, 73 us against 60 whole and 21 in four slices.
 struct DensePlan {
     int bt, streamk;
     int slices, kc;      // > 1: K slices of kc k-blocks on the CTA pairs of a cluster
@@ -1199,34 +1200,33 @@ static int slices_capacity(qg_ctx* ctx, int qbits, int bt, int slices) {
     return bt == 128 ? slices_capacity<4, 128>(ctx, slices) : slices_capacity<4, 192>(ctx, slices);
 }
 // Few tiles leave most SM pairs idle behind a serial walk over K.  Cutting K into two to four slices, one per pair of a
-// cluster that adds its partial tiles through distributed shared memory, divides the walk; the sum costs
-// 1100 + 1300 (slices - 2) cycles and 20 + 5 (slices - 2) per token of the tile (fitted to 25 shapes at 20 to 500 tokens, a
-// k-block being 515 cycles with up to 128 tokens and 600 with 192, and 570 of a whole walk of several 128-token tiles).  Stream-K's exchange through global memory costs 22000
-// on top of its share.  Unless the alternative is stream-K, slices take SMs that the next launch could start on: 800 cycles from a
-// quarter of the SM pairs on and 3000 from 0.45 of them on (two slices, K = 1024, 17 tokens: 24 tiles 8.0 us against 7.5 whole, 32 tiles
-// 8.8 against 7.9, 16 tiles 6.7 against 7.4).  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four
+// cluster that adds its partial tiles through distributed shared memory, divides the walk; the sum costs 525 + 620 (slices - 2) ns and
+// 9.5 + 2.4 (slices - 2) per token of the tile (a k-block of such a short walk being 245 ns with up to 128 tokens and 286 with 192, and 271
+// of a whole walk of several 128-token tiles).  Unless the alternative is stream-K, slices take SMs that the next launch could start on:
+// 380 ns from a quarter of the SM pairs on and 1430 from 0.45 of them on (two slices, K = 1024, 17 tokens: 24 tiles 8.0 us against 7.5 whole,
+// 32 tiles 8.8 against 7.9, 16 tiles 6.7 against 7.4).  All clusters have to be resident at once: 33 / 22 / 15 with two / three / four
 // slices, so this is for at most 33 tiles.  Measured, 20 / 128 tokens: 3072 x 3072 16.5 / 17.3 us whole, 10.0 / 12.3 in four
 // slices; 5120 x 3072 16.7 / 17.7, 11.3 / 13.3 in three; 2048 x 8192 24.8 / 30.1 (stream-K), 14.1 / 16.8 in four; 4096 x 14336
 // 29.2 / 34.1 (stream-K), 26.7 / 29.6 in three.
-static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePlan& plan) {
+constexpr double PLAN_START = 5000.0;        // start and end of any call
+// `whole_ns`: the time of the plan as it is, PLAN_START included
+static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, double whole_ns, DensePlan& plan) {
     if (ctx->force_bt || ctx->streamk_mode != -1) return;
     const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
     const int nk4 = K / (4 * BK);
     const long long tiles0 = n_pw * ((M + plan.bt - 1) / plan.bt);
     if (tiles0 > pairs) return;
-    auto period = [](int bt) { return bt == 128 ? 515.0 : bt == 192 ? 600.0 : 720.0; };
-    double best = plan.streamk ? (tiles0 * nk4 + pairs - 1) / pairs * 4.0 * period(plan.bt) + 22000.0
-                                : nk4 * 4.0 * (plan.bt == 128 && M > 128 ? 570.0 : period(plan.bt));
-    best *= 0.97;
+    auto period = [](int bt) { return bt == 128 ? 245.0 : bt == 192 ? 286.0 : 343.0; };
     const bool streamk = plan.streamk != 0;
+    double best = 0.97 * (streamk ? whole_ns - PLAN_START : nk4 * 4.0 * (plan.bt == 128 && M > 128 ? 271.0 : period(plan.bt)));
     for (int bt = 128; bt <= 192; bt += 64) {
         if (bt > 128 && M <= 128) break;
         const long long tiles = n_pw * ((M + bt - 1) / bt);
         for (int sl = 2; sl <= 4 && sl <= nk4 && tiles * sl <= pairs; ++sl) {
             const int per = (nk4 + sl - 1) / sl;
             if ((nk4 + per - 1) / per != sl) continue;             // the same cut as a smaller count
-            const double cost = per * 4.0 * period(bt) + 1100.0 + 1300.0 * (sl - 2) + (20.0 + 5.0 * (sl - 2)) * (M < bt ? M : bt) +
-                                (streamk || 4 * tiles * sl < pairs ? 0.0 : 20 * tiles * sl < 9 * pairs ? 800.0 : 3000.0);
+            const double cost = per * 4.0 * period(bt) + 525.0 + 620.0 * (sl - 2) + (9.5 + 2.4 * (sl - 2)) * (M < bt ? M : bt) +
+                                (streamk || 4 * tiles * sl < pairs ? 0.0 : 20 * tiles * sl < 9 * pairs ? 380.0 : 1430.0);
             if (cost < best && slices_capacity(ctx, qbits, bt, sl) >= tiles) {
                 best = cost;
                 plan = DensePlan{bt, 0, sl, 4 * per};
@@ -1234,9 +1234,10 @@ static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, DensePla
         }
     }
 }
-static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool streamk) {
+static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool streamk, double* ns = nullptr) {
     const int cand[3] = {128, 192, 256};
-    const double period[3] = {275.0, 298.0, 365.0}, epilogue[3] = {0.0, 0.0, 2400.0};
+    const double period[3] = {285.0, 300.0, 377.0}, epilogue[3] = {0.0, 0.0, 2200.0}, start[3] = {PLAN_START, PLAN_START, PLAN_START - 1750.0};
+    const double sk_period[3] = {295.0, 311.0, 394.0}, sk_start[3] = {8400.0, 8400.0, 11000.0};
     const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
     const int nk4 = K / (4 * BK);
     DensePlan best{256, 0, 1, 0};
@@ -1245,35 +1246,36 @@ static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool stre
         if (M <= 128 && cand[c] > 128) break;
         const long long tiles = n_pw * ((M + cand[c] - 1) / cand[c]);
         const double frac = static_cast<double>(tiles) / pairs;
-        const double waves = tiles <= pairs ? 0.58 + 0.42 * frac : 0.5 * (static_cast<double>((tiles + pairs - 1) / pairs) + frac);
+        const double waves = tiles <= pairs ? 0.77 + 0.23 * frac : 0.55 * static_cast<double>((tiles + pairs - 1) / pairs) + 0.45 * frac;
         // (gate/up: the single accumulator has to be clearly faster; at 3000 tokens and more the two are level within the clock's drift)
-        const double dp = waves * ((K / BK) * period[c] + epilogue[c]) * (!streamk && cand[c] == 256 ? 1.03 : 1.0);
+        const double dp = (start[c] + waves * ((K / BK) * period[c] + epilogue[c])) * (!streamk && cand[c] == 256 ? 1.03 : 1.0);
         if (!streamk || ctx->streamk_mode != 1 || tiles % pairs == 0)
             if (dp < best_cost) { best_cost = dp; best = DensePlan{cand[c], 0, 1, 0}; }
     }
-    if (!streamk || ctx->streamk_mode == 0) return best;
     // Below K = 4096 the exchange never paid in the measurements (K = 2048 and 3072, 64 to 1024 tokens: 2 to 10 us slower).
-    if (ctx->streamk_mode != 1 && nk4 < 16) return best;
+    const double whole_cost = best_cost;
     for (int c = 0; c < 3; ++c) {
+        if (!streamk || ctx->streamk_mode == 0 || (ctx->streamk_mode != 1 && nk4 < 16)) break;
         if (M <= 128 && cand[c] > 128) break;
         const long long tiles = n_pw * ((M + cand[c] - 1) / cand[c]);
         if (tiles % pairs == 0) continue;
         const long long units = tiles * nk4;
         const long long P = units < pairs ? units : pairs;
         const long long share = (units + P - 1) / P;                        // units of the busiest pair
-        const double pieces = static_cast<double>(share) / nk4 + 1.5;       // tiles it touches, on average
         if (share / nk4 + 2 > 120) continue;                                // the piece table has 128 entries
-        const double sk = 1.1 * (share * 4.0 * period[c] + pieces * epilogue[c]) + 5000.0;
-        if (ctx->streamk_mode == 1 ? (best.streamk == 0 || sk < best_cost) : (sk < 0.95 * best_cost)) {
+        const double sk = sk_start[c] + share * 4.0 * sk_period[c] + static_cast<double>(P) / tiles * (930.0 + 5.6 * (M < cand[c] ? M : cand[c]));
+        if (ctx->streamk_mode == 1 ? (best.streamk == 0 || sk < best_cost) : (sk < best_cost && sk < 0.96 * whole_cost)) {
             best_cost = sk;
             best = DensePlan{cand[c], 1, 1, 0};
         }
     }
+    if (ns) *ns = best_cost;
     return best;
 }
 static DensePlan plan_dense(qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
-    DensePlan plan = plan_whole(ctx, M, n_wt, K, true);
-    plan_slices(ctx, qbits, M, n_wt, K, plan);
+    double ns = 0.0;
+    DensePlan plan = plan_whole(ctx, M, n_wt, K, true, &ns);
+    plan_slices(ctx, qbits, M, n_wt, K, ns, plan);
     return plan;
 }
 

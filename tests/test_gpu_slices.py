@@ -15,8 +15,9 @@ pytestmark = pytest.mark.gpu
 # the end in the last tile, tokens around the edges of the 16-token blocks and of the 128- and 192-token tiles
 SHAPES = [(8, 17, 256, 2048), (4, 20, 3072, 3072), (8, 128, 2184, 2560), (4, 129, 1152, 1280), (8, 127, 136, 8192),
           (4, 192, 2048, 2048), (8, 333, 2048, 2048), (4, 500, 2560, 2048), (8, 193, 4096, 4096), (4, 64, 5120, 3072),
-          (8, 1, 512, 1024), (4, 16, 8, 512), (8, 500, 2560, 2048), (8, 64, 136, 8192)]
-WHOLE = (8, 127, 136, 8192)                              # stream-K is expected to be faster there
+          (8, 1, 512, 1024), (4, 16, 8, 512), (8, 500, 2560, 2048), (8, 64, 136, 8192), (8, 64, 8192, 512)]
+WHOLE = (8, 64, 8192, 512)                               # 32 row tiles and two units of K: two slices would fill the GPU
+# (8 x 127 x 136 x 8192 was expected whole, by stream-K: 57 us there, 30 data-parallel and 13 in four slices.)
 
 
 @pytest.mark.parametrize("qbits,M,N,K", SHAPES, ids=[f"q{q}-{m}x{n}x{k}" for q, m, n, k in SHAPES])
@@ -82,6 +83,14 @@ def test_short_k_over_many_tiles_is_not_sliced(M, N, K):
     whole, 10.1 against 8.5 at 128 tokens)."""
     assert qg.plan_slices(8, M, N, K) == 1 and qg.plan_slices(4, M, N, K) == 1
     assert qg.plan_slices(8, M, 4096, 4096) > 1 and qg.plan_slices(8, M, 5120, 3072) > 1
+
+
+@pytest.mark.parametrize("qbits,M,N,K", [(8, 128, 512, 16384), (4, 192, 136, 14336), (8, 17, 1024, 16384), (4, 333, 512, 8192), (8, 150, 4096, 14336)],
+                         ids=lambda v: str(v))
+def test_long_k_over_few_tiles_is_sliced(qbits, M, N, K):
+    """Under stream-K, whose tiles of up to 64 parts are added by one pair each, these took 71, 119, 36, 52 and 34 us; in slices 21, 19, 19,
+    14 and 29."""
+    assert qg.plan_slices(qbits, M, N, K) > 1
 
 
 def test_the_cases_cover_every_instantiation():

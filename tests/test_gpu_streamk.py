@@ -65,3 +65,9 @@ def test_the_cost_model_follows_the_measured_best_tile():
         got_bt, sk = qg.plan_dense(qbits, M, N, K)
         assert got_bt == bt and not sk, (qbits, M, N, K, got_bt, sk)
     assert qg.plan_dense(8, 64, 2048, 2048)[0] == 128
+
+
+def test_long_calls_with_a_nearly_empty_last_wave_take_streamk():
+    """2500 tokens of 4096 x 14336: 160 tiles of 256 tokens on 74 pairs, 311 us data-parallel, 244 by stream-K."""
+    qg.set_schedule(0, -1)
+    assert qg.plan_dense(8, 2500, 4096, 14336)[1]
