@@ -251,9 +251,8 @@ int moe_grouped_qgemm(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, int
  * round trip through global memory never exist): row r of the input is X[row_pair[r] / k, :], X bf16 [M, K] in
  * token order.  Everything else - segments, weights, modes, outputs in sorted-row order - is as in
  * moe_grouped_qgemm; row_pair and k are always required.  Results are those of
- * moe_permute followed by moe_grouped_qgemm: the same kernel serves both forms of a call, with the same bits where it is the
- * streaming one (see moe_grouped_qgemm), and up to the order of the fp32 sums, which may differ from run to run in the last
- * place, where it is the other.
+ * moe_permute followed by moe_grouped_qgemm, bit for bit in modes 0 to 2: the same kernel serves both forms of a call, and every
+ * sum has a fixed order (mode 3 adds with atomics).
  */
 int moe_grouped_qgemm_gather(qg_ctx* ctx, int mode, int qbits, int M, int R, int E, int N, int K, const void* X,
                              const int32_t* row_pair, int k, const int32_t* expert_offsets, const void* Wq,
