@@ -154,7 +154,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     pdl_launch_dependents();
     if (warp == 0) {
         if (lane < C::NBAR) {
-            const uint32_t cnt = (lane >= 11 && lane <= 14) || lane == 17 || lane == 18 ? 4u : 1u;      // p_full, s_free: one arrival per softmax warp
+            // p_full, s_free: one arrival per softmax warp
+            const uint32_t cnt = (lane >= 11 && lane <= 14) || lane == 17 || lane == 18 ? 4u : 1u;
             mbar_init(bar0 + 8u * lane, cnt);
         }
         if (lane == 31) misc[1] = 0;

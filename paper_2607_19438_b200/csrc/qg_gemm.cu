@@ -97,7 +97,7 @@ struct Cfg {
     static constexpr int NBAR = 2 * SP + 2 * SR + 5;
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;        // + slack for 1024-byte alignment
-    static constexpr int TMEM_COLS = 512;                          // accumulator(s) + SX weight stages
+    static constexpr int TMEM_COLS = 512;                          // accumulator(s) + SA weight stages
     static constexpr int A_COL0 = NACC * BT;                       // first column of the weight stages
     static constexpr int A_COLS = 32;                              // 64 bf16 per lane = 32 columns per stage
     static_assert(NACC * BT + SA * 32 <= 512, "tensor memory budget");
@@ -158,7 +158,7 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
     return false;
 }
 
-// Same for the MMA warps: a short non-blocking spin first (the barrier is usually complete or about to be), then
+// Same for the MMA warp: a short non-blocking spin first (the barrier is usually complete or about to be), then
 // the bounded blocking wait.
 __device__ __forceinline__ bool spin_wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag, const GemmParams& p) {
     for (int it = 0; it < 64; ++it)
@@ -170,16 +170,6 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t addr) {
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ float lds_scale(uint32_t addr) {
-    unsigned short h;
-    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(addr));
-    return __half2float(__ushort_as_half(h));
 }
 
 // Plain / routing-weighted epilogue of one warp: drains the 16-column (token) blocks b = pid, pid + npart, ... of
@@ -729,8 +719,9 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
         if (lane == 0) QG_FLUSH();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (even CTA of the pair only)
-        // Two k-blocks per barrier: eight MMAs and one commit take about 350 cycles to issue, less than the tensor cores need for
-        // them from 48 tokens on.  One issuing thread also fixes the order in which a tile's k-blocks are added.
+        // Two k-blocks per barrier.  Four MMAs take 120 cycles to issue and the commit 113, about 350 for a pair, and the tensor cores
+        // 8 (15 + N / 2) for its eight MMAs, more than that from 64 tokens on (an iteration with its wait: 450).  One issuing thread also
+        // fixes the order in which a tile's k-blocks are added.
         if (rank == 0) {
             bool ok = true;
             QG_DECL();
@@ -898,10 +889,8 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
             {
                 uint32_t (&o0)[16] = *reinterpret_cast<uint32_t (*)[16]>(o);
                 uint32_t (&o1)[16] = *reinterpret_cast<uint32_t (*)[16]>(o + 16);
-                {
-                    tmem_st_32x32_x16(a_taddr + ta * C::A_COLS, o0);
-                    tmem_st_32x32_x16(a_taddr + ta * C::A_COLS + 16, o1);
-                }
+                tmem_st_32x32_x16(a_taddr + ta * C::A_COLS, o0);
+                tmem_st_32x32_x16(a_taddr + ta * C::A_COLS + 16, o1);
             }
             tmem_st_wait();
             tc_fence_before_sync();
@@ -976,7 +965,8 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
                 if constexpr (SK == 2) dump_partial(partial, taddr, n_epi, 0, 5, qd, lane);
                 else drain_plain<SK == 1, !C::HELP, !C::HELP>(p, tl.tok0, tl.tok_end, wt * BW + qd * 32, taddr, n_epi, 0,
                             (C::HELP || static_cast<int>(j) == my_tiles - 1) ? 5 : 1,
-                            stg16 + 16 * 512 + qd * (C::EPI_ST / 2), C::HELP ? nullptr : wts + (j & 1u) * BT, lane, piece_at(static_cast<int>(j)).nsrc, qd, BT * 128, abort_flag);
+                            stg16 + 16 * 512 + qd * (C::EPI_ST / 2), C::HELP ? nullptr : wts + (j & 1u) * BT, lane,
+                            piece_at(static_cast<int>(j)).nsrc, qd, BT * 128, abort_flag);
             } else if constexpr (EPI == 1) {
                 drain_gate_up(p, tl.tok0, tl.tok_end, wt * 64 + qd * 16, taddr, n_epi, 0,
                               (C::HELP || static_cast<int>(j) == my_tiles - 1) ? 5 : 1, stg16 + 16 * 512 + qd * (C::EPI_ST / 2), lane);
@@ -1189,8 +1179,8 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
 // single wave as 0.77 + 0.23 of the share of the pairs that have a tile.  16384 x 3072 gate/up, 4 bit, 200 tokens: 29.4 us with 192-token
 // tiles, 20.3 with 256; 1024 tokens 80.1 and 74.8; 4096 x 4096, 8 bit, 4096 tokens: 92.7 and 99.9.
 // Stream-K: every pair gets the same share of all k-blocks; the pair with a tile's first k-block adds the parts of all pairs that have
-// others one after another, 930 ns and 5.6 a token for each.  4096 x 14336: at 2500 tokens 244 us against 293 data-parallel, at 1500 143.6
-// against 128.5.  Few tiles have many parts each: 512 x 16384 at 128 tokens, 37 parts, 73 us against 60 whole and 21 in four slices.
+// others one after another, 930 ns and 5.6 a token for each.  4096 x 14336: at 2500 tokens (2.2 waves) 244 us against 293 data-parallel, at
+// 1500 (1.7) 154 and 154.  Few tiles have many parts each: 512 x 16384 at 128 tokens, 37 parts, 73 us against 60 whole and 21 in four slices.
 struct DensePlan {
     int bt, streamk;
     int slices, kc;      // > 1: K slices of kc k-blocks on the CTA pairs of a cluster
@@ -1399,7 +1389,7 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     // weights.  192 against 128 tokens over eight layers of 8 to 512 experts, rows drawn evenly / with a quarter of the experts preferred:
     // 4 bit, 19 rows per expert 0.98 / 0.98, 64 rows 1.00 / 0.83, 96 rows 1.00 / 0.99, 128 rows 0.76 / 0.88; 8 bit 19 rows 1.01 / 1.01, 48 rows
     // 1.01 / 0.99, 64 rows 1.01 / 0.88, 80 rows 1.01 / 0.95, 96 rows 1.02 / 1.03, 128 rows 0.81 / 0.92.  (Behind the streaming kernel the tile
-    // is 128 tokens, so the 4-bit line is where that kernel ends.)
+    // is 128 tokens, so the 4-bit line is where that kernel ends: GroupedChoice::MAX_ROWS.)
     //   Gathered rows and fp32 sums cost a tile time by the row where sorted rows are bound by the conversion, and so do the stores of a short
     // K (the epilogue is the pace): there a tile of few rows is as dear as one of about 100, and 230 rows in 192 + 38 dearer than in 128 + 102, so
     // an expert's tiles are made equally long.  200 rows per expert, 128 experts, 4 bit, gathered 1536 x 2048 584 -> 444 us, fp32 sums
@@ -1410,7 +1400,7 @@ static int grouped_impl(qg_ctx* ctx, int mode, int qbits, int R, int E, int N, i
     const bool by_row = gather_k > 0 || mode == QG_MODE_DOWN_ACCUM_F32;
     p.even_tiles = by_row || K <= 768;
     const bool short_tiles = (gather_k > 0 || (by_row && K <= 1536)) && rows > 64 && rows <= 100;
-    const int bt = (rows > (qbits == QG_Q4 ? 18 : 50) && !short_tiles) ? 192 : 128;
+    const int bt = (rows > (qbits == QG_Q4 ? qg::GroupedChoice::MAX_ROWS : 50) && !short_tiles) ? 192 : 128;
     // a few rows per expert (4-bit weights, no accumulation) the streaming kernel is faster; the gathering form takes the same
     // kernel as the form for sorted rows, so that they give the same numbers
     qg::GroupedChoice choice{};

@@ -109,16 +109,18 @@ int get_tmap_3d(qg_ctx* ctx, CUtensorMap* out, CUtensorMapDataType dt, int elem_
                 uint64_t inner, uint64_t rows, uint64_t planes, uint64_t plane_stride_bytes, uint32_t box_inner,
                 uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swz, uint64_t row_stride_bytes = 0);
 // Which of its two kernels serves a grouped call with 4-bit weights: the streaming kernel when every expert has a few rows, the
-// tensor-memory kernel when they crowd into few experts, and how the rows are spread only the device knows.  The times are
-// fitted to 654 calls (14 shapes of 1 to 1024 experts; rows spread evenly, with a quarter of the experts preferred, over eight
-// experts, all with one): the faster kernel by them takes 1.02 of the faster one's time on average, 1.2 at worst.
+// tensor-memory kernel when they crowd into few experts, and how the rows are spread only the device knows.  By the times below the faster
+// kernel is chosen in 758 of 780 calls or missed by less than 5 % (eight layers of 8 to 512 experts, a quarter of a row to 32 rows per
+// expert; rows spread evenly, with a quarter of the experts preferred, over eight experts, all with one); 1.004 of the faster one's time on
+// average, 1.27 at worst.  (The times of the other kernel lie 7 % above what it takes by now.  Fitted anew, 773 of the 780 calls are within
+// 5 %, but the host's choice, which knows the averages only, is no better: 1.011 and 1.012 of the fastest with even and uneven rows, now 1.012
+// and 1.011, and its worst uneven call 1.39 instead of 1.20.)
 //   The host weighs three calls with evenly spread rows against one with all rows in one segment: the streaming kernel alone,
 // the other alone, or both, in which case each works out the same answer from the offsets and the one that is not wanted ends at
-// once.  That costs every such call 5 to 8 us (the unwanted launch keeps the next one from starting early).  128 experts,
-// 1536 x 2048: alone up to 11 rows per expert (even 62 us against 95, one segment 38 against 17 at eight rows), both up to 16,
-// the other from there (even 95 against 95, one segment 70 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
-// (even 917 us against 1605 of the other alone; eight segments 183 against 622 when the average alone decided, and 154 of the
-// other alone).
+// once.  That costs every such call 3 to 14 us (the unwanted launch keeps the next one from starting early).  128 experts,
+// 1536 x 2048: alone up to 12 rows per expert (even 62 us against 91, one segment 39 against 16 at eight rows), both up to 17,
+// the other from there (even 100 against 91, one segment 71 against 25 at eighteen).  256 experts, 4096 x 7168, eight rows: both
+// (even 1009 us against 1680 of the other alone; eight segments 173 against 562 of the streaming kernel and 126 of the other).
 struct GroupedChoice {
     enum Way { STREAM, OTHER, BOTH };
     int on;                    // both kernels are launched
@@ -136,7 +138,9 @@ struct GroupedChoice {
         return 8000 + (wide * ((n_wt + 1) / 2) + pairs - 1) / pairs * stages * (4 * 271);
     }
     __host__ __device__ bool streams(long long chunks, long long wide) const { return stream_ns(chunks) <= other_ns(wide); }
-    static constexpr int MAX_ROWS = 18;       // per expert, on average: evenly spread, the other kernel is the faster one from there on
+    // Rows per expert, on average.  Evenly spread and sorted, the streaming kernel takes 0.94 of the other one's time at 14, 1.05 at 16 and
+    // 1.13 at 18 (eight layers); gathered, 0.93 at 16 and 0.96 at 18, and both forms take the same kernel.
+    static constexpr int MAX_ROWS = 18;
     Way plan(long long R, long long E) const {
         if (R > MAX_ROWS * E) return OTHER;
         // rows drawn evenly (Poisson): a tile per expert up to 5/8 of a tile's rows, then 3/8 of a tile more than the rows fill

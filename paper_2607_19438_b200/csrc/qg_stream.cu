@@ -17,8 +17,8 @@
 // one that has not been started (cluster launch control; dealt out beforehand, the tiles left an SM up to 16 % more than its
 // share: nine tiles are too few to round).  The hardware keeps the count, nothing outlives the launch, so launches may
 // overlap on the GPU in any way.
-//   One matrix with fewer tiles: K is cut into slices, the slices of a tile are a thread-block cluster, and the cluster adds
-// its sums through distributed shared memory in slice order.  All sums have a fixed order: results are reproducible.
+//   One matrix with fewer tiles: K is cut into slices, the slices of a tile are a thread-block cluster, and each of its CTAs sends its
+// sums to the one that adds them, in slice order.  All sums have a fixed order: results are reproducible.
 //
 // Arithmetic.  A weight costs as few instructions as possible: a nibble becomes the bf16 number 128 + code by a byte
 // permute (0x43 above the code), in the order in which byte operations deliver them, and half a packed subtraction makes
@@ -47,8 +47,9 @@
 // rounded scaled 8-bit weights, a block kernel and the tensor-memory kernel, whichever was fastest: 28672 x 4096 8 bit
 // 32.3 / 38.2 us (3.9 / 3.3 TB/s) against 34.3 / 39.5; 4096 x 14336 16.4 / 19.8 against 19.0 / 28.7; 4096 x 4096 8.0 / 9.6
 // against 8.6 / 13.2; 2048 x 2048 5.6 / 6.6 against 5.9 / 7.0; 3072 x 8192 4 bit 9.0 / 12.1 against 15.4 / 26.3.
-// K slices send their sums to the CTA that adds them (st.async); while they met, read each other's and met again, 1 / 16 tokens back to back in
-// a graph: 2048 x 2048 8 bit 4.8 / 5.9 us, now 4.35 / 4.95; 3072 x 8192 4 bit 8.7 / 10.75, now 7.7 / 9.8; 5120 x 3072 6.7 / 8.3, now 6.1 / 7.3.
+// K slices send their sums to the CTA that adds them (st.async); while they met, read each other's and met again, 1 / 16 tokens back
+// to back in a graph: 2048 x 2048 8 bit 4.8 / 5.9 us, now 4.35 / 4.95; 3072 x 8192 4 bit 8.7 / 10.75, now 7.7 / 9.8; 5120 x 3072
+// 6.7 / 8.3, now 6.1 / 7.3.
 // What bounds it: without its arithmetic the 28672 x 4096 launch takes 26.4 us, with the codes' loads alone 22.1 (5.65 TB/s);
 // supply and arithmetic overlap, but with 16 consumer warps per SM neither hides the other fully.
 // Every mbarrier wait is bounded.
@@ -236,7 +237,7 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     extern __shared__ uint8_t ms_smem[];
     const uint32_t ring = (smem_u32(ms_smem) + 1023u) & ~1023u;
     uint8_t* after = ms_smem + (ring - smem_u32(ms_smem)) + p.n_stages * p.stage_bytes;
-    const uint32_t xch = smem_u32(after);              // [4 warps][NTM][MT][32 lanes] float4: sums handed from set to set, or of the slice
+    const uint32_t xch = smem_u32(after);              // [4 warps][NTM][MT][32 lanes] float4: sums handed from set to set
     after += 4 * NTM * MT * 512;
     const uint32_t recv = smem_u32(after);             // K slices: [slices][fragments this CTA adds] float4, written by the cluster's CTAs
     if (SLICED) after += ms_recv_bytes(NTM * MT);
@@ -296,8 +297,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     }
     const int k0 = static_cast<int>(blockIdx.y) * p.kc;
     const int nst = min(p.kc, p.K - k0) / MS_SK;       // stages of a tile
-    // K slices (SLICED: p.kc < p.K, and a CTA has one tile): the CTAs of a cluster hold one slice's sums of the same tile each.  Every CTA adds a share of the tile's fragments (16
-    // bytes: rows lo / hi x two tokens): the others send theirs to its shared memory, and a barrier there counts the bytes.
+    // K slices (SLICED: p.kc < p.K, and a CTA has one tile): the CTAs of a cluster hold one slice's sums of the same tile each.  Every
+    // CTA adds a share of the tile's fragments (16 bytes: rows lo / hi x two tokens): the others send theirs to its shared memory, and
+    // a barrier there counts the bytes.
     const uint32_t n_frag = 4 * MT * 32 * ((p.R + 7) >> 3), share = (n_frag + gridDim.y - 1) / gridDim.y, rank = blockIdx.y;
     const uint32_t my_frags = rank * share < n_frag ? min(share, n_frag - rank * share) : 0;
     if constexpr (SLICED) {
@@ -600,8 +602,9 @@ stream_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 // Ring depth and shared memory of a launch; false if not even two stages fit.
 static bool ms_layout(StreamParams& p, int qbits, int ntm, int n_exp, size_t& smem) {
     p.stage_bytes = (MS_W_BYTES + ms_s_bytes(qbits) + ntm * MS_X_BYTES + 1023) & ~1023;      // the codes' swizzle wants 1 KB
-    const size_t fixed = 1024 + 4 * ntm * (ms_rows(qbits) / 64) * 512 + (n_exp ? 0 : ms_recv_bytes(ntm * (ms_rows(qbits) / 64))) + 32 * MS_MAX_ST + 64 + 32 + 16 + 16 * MS_MAX_ST +
-                         (2 * static_cast<size_t>(n_exp) + 2) * sizeof(int);
+    const int mma_tiles = ntm * (ms_rows(qbits) / 64);
+    const size_t fixed = 1024 + 4 * mma_tiles * 512 + (n_exp ? 0 : ms_recv_bytes(mma_tiles)) + 32 * MS_MAX_ST + 64 + 32 + 16 +
+                         16 * MS_MAX_ST + (2 * static_cast<size_t>(n_exp) + 2) * sizeof(int);
     p.n_stages = static_cast<int>((MS_SMEM_MAX - fixed) / p.stage_bytes);
     if (p.n_stages > MS_MAX_ST) p.n_stages = MS_MAX_ST;
     smem = fixed + static_cast<size_t>(p.n_stages) * p.stage_bytes;
