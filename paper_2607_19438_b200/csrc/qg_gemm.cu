@@ -720,8 +720,8 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& tm_x, const CUtenso
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (even CTA of the pair only)
         // Two k-blocks per barrier.  Four MMAs take 120 cycles to issue and the commit 113, about 350 for a pair, and the tensor cores
-        // 8 (15 + N / 2) for its eight MMAs, more than that from 64 tokens on (an iteration with its wait: 450).  One issuing thread also
-        // fixes the order in which a tile's k-blocks are added.
+        // 8 (15 + N / 2) for its eight MMAs, more than that from 64 tokens on (with the test of the next pair's barrier, in a profiling
+        // build, 430 to 500).  One issuing thread also fixes the order in which a tile's k-blocks are added.
         if (rank == 0) {
             bool ok = true;
             QG_DECL();
