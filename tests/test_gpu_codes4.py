@@ -25,17 +25,35 @@ def test_all_codes_times_all_scales(rows):
     Ws = np.ascontiguousarray(s[:N * 8].reshape(N, 8))
     codes = np.arange(K, dtype=np.uint8) % 16       # each 32-block holds every code twice
     Wq = np.broadcast_to((codes[0::2] | (codes[1::2] << 4)).astype(np.uint8), (N, K // 2)).copy()
-    dWq, dWs = util.dev(Wq), util.dev_f16(Ws)
+    A = np.zeros((rows, K), np.uint16)
+    i = np.arange(rows)
+    A[i, i * (K // rows) + i % (K // rows)] = 0x3F80
     call = qg.qgemm_dense if rows > 16 else qg.qgemm_small_m
-    step = K // rows                                # a call shows each scale 32 / step codes: as many calls as it takes for all sixteen
-    for shift in range(step):
-        k = np.arange(rows) * step + (np.arange(rows) + shift) % step
-        A = np.zeros((rows, K), np.uint16)
-        A[np.arange(rows), k] = 0x3F80
-        out = util.host_bf16_bits(call(4, util.dev_bf16(A), dWq, dWs))
-        qg.poll_status()
-        w = (codes[k].astype(np.float64) - 8)[:, None] * Ws.view(np.float16).astype(np.float64)[:, k // 32].T
-        ref = orc.f64_to_bf16(w)
-        zero = (out & 0x7FFF) == 0                  # a zero's sign is not part of the contract
-        assert np.array_equal(zero, (ref & 0x7FFF) == 0)
-        assert np.array_equal(out[~zero], ref[~zero])
+    out = util.host_bf16_bits(call(4, util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws)))
+    qg.poll_status()
+    k = np.argmax(A != 0, axis=1)
+    w = (codes[k].astype(np.float64) - 8)[:, None] * Ws.view(np.float16).astype(np.float64)[:, k // 32].T
+    ref = orc.f64_to_bf16(w)
+    zero = (out & 0x7FFF) == 0                      # a zero's sign is not part of the contract
+    assert np.array_equal(zero, (ref & 0x7FFF) == 0)
+    assert np.array_equal(out[~zero], ref[~zero])
+
+
+@pytest.mark.parametrize("shift", range(16))
+def test_every_code_with_every_scale_in_the_block_kernel(shift):
+    """Sixteen tokens show each scale two codes; moved on by one sixteen times, all of them."""
+    K = 256
+    s = scales()
+    N = len(s) // 8
+    Ws = np.ascontiguousarray(s[:N * 8].reshape(N, 8))
+    codes = np.arange(K, dtype=np.uint8) % 16
+    Wq = np.broadcast_to((codes[0::2] | (codes[1::2] << 4)).astype(np.uint8), (N, K // 2)).copy()
+    k = np.arange(16) * 16 + (np.arange(16) + shift) % 16
+    A = np.zeros((16, K), np.uint16)
+    A[np.arange(16), k] = 0x3F80
+    out = util.host_bf16_bits(qg.qgemm_small_m(4, util.dev_bf16(A), util.dev(Wq), util.dev_f16(Ws)))
+    qg.poll_status()
+    ref = orc.f64_to_bf16((codes[k].astype(np.float64) - 8)[:, None] * Ws.view(np.float16).astype(np.float64)[:, k // 32].T)
+    zero = (out & 0x7FFF) == 0                      # a zero's sign is not part of the contract
+    assert np.array_equal(zero, (ref & 0x7FFF) == 0)
+    assert np.array_equal(out[~zero], ref[~zero])
