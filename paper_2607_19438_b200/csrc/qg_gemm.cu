@@ -1171,8 +1171,9 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
 }
 
 // Token tile and schedule of a dense call: the candidate with the smallest modelled time in ns, fitted to 1300 calls timed back to back on
-// B200 (Q8 and Q4, plain and gate/up, N from 136 to 28672, K from 512 to 16384, 17 to 4096 tokens; every candidate of each).  The choice
-// takes 1.004 of the time of the fastest candidate on average, 1.12 at worst.
+// B200 (Q8 and Q4, plain and gate/up, N from 136 to 28672, K from 512 to 16384, 17 to 4096 tokens; every candidate of each).  There the choice
+// takes 1.004 of the time of the fastest candidate on average, 1.12 at worst; over 904 unsliced calls of 24 layers timed afterwards, five of
+// them new to the model, 1.008 and 1.17 (4096 x 14336, 4 bit, 1800 tokens: 195 us, by stream-K 167).
 // Data-parallel: a tile costs nkb k-blocks of `period` plus, for the single-accumulator 256-token tile, an exposed epilogue;
 // tiles come in waves of one per SM pair, but a ragged last wave costs less than a full one (the pairs that are done leave L2,
 // HBM and power to the others), so the wave count is taken about half-way between the rounded-up and the fractional one, and of a
@@ -1181,6 +1182,9 @@ static int launch_gemm(qg_ctx* ctx, const GemmParams& p, const void* X, int x_ro
 // Stream-K: every pair gets the same share of all k-blocks; the pair with a tile's first k-block adds the parts of all pairs that have
 // others one after another, 930 ns and 5.6 a token for each.  4096 x 14336: at 2500 tokens (2.2 waves) 244 us against 293 data-parallel, at
 // 1500 (1.7) 154 and 154.  Few tiles have many parts each: 512 x 16384 at 128 tokens, 37 parts, 73 us against 60 whole and 21 in four slices.
+// Not from 5.5 waves on: what a ragged last one leaves idle is a tenth of the call at most, and its idle pairs leave their power to the others.
+// 28672 x 4096, 8 bit: 1024 tokens (6.05 waves of 256-token tiles) 195 us by stream-K, 179 data-parallel, 2500 tokens 466 and 425; 14336 x 4096,
+// 2048 tokens 179 and 170; three waves (28672 x 4096, 400 tokens) 91.7 and 106.
 struct DensePlan {
     int bt, streamk;
     int slices, kc;      // > 1: K slices of kc k-blocks on the CTA pairs of a cluster
@@ -1224,9 +1228,12 @@ static void plan_slices(qg_ctx* ctx, int qbits, int M, int n_wt, int K, double w
         }
     }
 }
-static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool streamk, double* ns = nullptr) {
+static DensePlan plan_whole(const qg_ctx* ctx, int qbits, int M, int n_wt, int K, bool streamk, double* ns = nullptr) {
     const int cand[3] = {128, 192, 256};
-    const double period[3] = {285.0, 300.0, 377.0}, epilogue[3] = {0.0, 0.0, 2200.0}, start[3] = {PLAN_START, PLAN_START, PLAN_START - 1750.0};
+    // 128-token tiles: with 4 bit 0.90 to 1.06 of the time of 192-token ones where both are a single wave, with 8 bit 0.02 less.  4 bit, 3072 x 3072,
+    // 512 tokens 18.4 us with 128, 17.5 with 192; 8 bit, 8192 x 8192, 256 tokens 37.0 whole with 128, 38.8 by stream-K with 256.
+    const double period[3] = {!streamk ? 285.0 : qbits == QG_Q8 ? 279.0 : 288.0, 300.0, 377.0};
+    const double epilogue[3] = {0.0, 0.0, 2200.0}, start[3] = {PLAN_START, PLAN_START, PLAN_START - 1750.0};
     const double sk_period[3] = {295.0, 311.0, 394.0}, sk_start[3] = {8400.0, 8400.0, 11000.0};
     const long long pairs = ctx->sm_count / 2, n_pw = (n_wt + 1) / 2;
     const int nk4 = K / (4 * BK);
@@ -1248,7 +1255,7 @@ static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool stre
         if (!streamk || ctx->streamk_mode == 0 || (ctx->streamk_mode != 1 && nk4 < 16)) break;
         if (M <= 128 && cand[c] > 128) break;
         const long long tiles = n_pw * ((M + cand[c] - 1) / cand[c]);
-        if (tiles % pairs == 0) continue;
+        if (tiles % pairs == 0 || (ctx->streamk_mode != 1 && 2 * tiles > 11 * pairs)) continue;
         const long long units = tiles * nk4;
         const long long P = units < pairs ? units : pairs;
         const long long share = (units + P - 1) / P;                        // units of the busiest pair
@@ -1264,7 +1271,7 @@ static DensePlan plan_whole(const qg_ctx* ctx, int M, int n_wt, int K, bool stre
 }
 static DensePlan plan_dense(qg_ctx* ctx, int qbits, int M, int n_wt, int K) {
     double ns = 0.0;
-    DensePlan plan = plan_whole(ctx, M, n_wt, K, true, &ns);
+    DensePlan plan = plan_whole(ctx, qbits, M, n_wt, K, true, &ns);
     plan_slices(ctx, qbits, M, n_wt, K, ns, plan);
     return plan;
 }
@@ -1359,7 +1366,7 @@ int qgemm_dense_gate_up_silu(qg_ctx* ctx, int qbits, int M, int F, int K, const 
     p.mode = QG_MODE_GATE_UP_SILU; p.R = M; p.N = 2 * F; p.K = K; p.E = 1; p.k = 1;
     p.n_wt = (2 * F) / 128;
     p.offsets = nullptr; p.out = Out; p.topk_w = nullptr; p.row_pair = nullptr;
-    const int bt = qg::plan_whole(ctx, M, p.n_wt, K, false).bt;
+    const int bt = qg::plan_whole(ctx, qbits, M, p.n_wt, K, false).bt;
     return qg::dispatch_gemm(ctx, qbits, bt, p, A, M, Wq, Wscale, static_cast<cudaStream_t>(stream));
 }
 

@@ -71,3 +71,19 @@ def test_long_calls_with_a_nearly_empty_last_wave_take_streamk():
     """2500 tokens of 4096 x 14336: 160 tiles of 256 tokens on 74 pairs, 311 us data-parallel, 244 by stream-K."""
     qg.set_schedule(0, -1)
     assert qg.plan_dense(8, 2500, 4096, 14336)[1]
+
+
+@pytest.mark.parametrize("qbits,M,N,K", [(8, 1024, 28672, 4096), (8, 2500, 28672, 4096), (4, 4096, 28672, 4096), (8, 2048, 14336, 4096), (4, 4096, 7168, 4096)],
+                         ids=lambda v: str(v))
+def test_calls_of_many_waves_stay_data_parallel(qbits, M, N, K):
+    """Stream-K took 1.04 to 1.09 times as long."""
+    qg.set_schedule(0, -1)
+    assert not qg.plan_dense(qbits, M, N, K)[1]
+
+
+@pytest.mark.parametrize("qbits,M,N,K,bt", [(4, 400, 3072, 3072, 192), (4, 512, 3072, 3072, 192), (8, 256, 8192, 8192, 128), (8, 640, 3072, 8192, 128)],
+                         ids=lambda v: str(v))
+def test_128_token_tiles_are_cheaper_with_8_bit(qbits, M, N, K, bt):
+    """The other tile took 1.03 to 1.06 times as long."""
+    qg.set_schedule(0, -1)
+    assert qg.plan_dense(qbits, M, N, K) == (bt, False)
